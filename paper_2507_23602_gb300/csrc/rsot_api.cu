@@ -161,6 +161,7 @@ void rsot_destroy(rsot_problem *p) {
     trunc_free(p);
     compensated_free(p);
     cutoff_free(p);
+    fx64_free(p);
     dense_free(p);
     cudaFree(p->xs);
     cudaFree(p->x64);
@@ -347,20 +348,30 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     const bool dense = mode == 0 || (mode == 1 && (!(arg > 0.0) || isinf(arg) ||
                                                     arg * arg > p->diam2 * (1.0 + 1e-12)));
     if (!e && !dense) e = mode == 1 ? cutoffs_uniform(p, 0.5 * arg * arg) : cutoffs_separable(p, psid, eps, arg);
+    // dense FP64: fixed-point exponents where they can hold the range, the FP64
+    // passes otherwise (or when the device finds that they cannot, kErrRange64)
+    bool fx = prec == RSOT_FP64 && dense && !e && fx64_ready(p, eps);
     if (!e) {
         if (prec == RSOT_COMPENSATED)
             e = launch_compensated(p, psid, eps, !dense, gd);
         else if (dense)
             e = (prec == RSOT_MIXED) ? launch_dense_mixed(p, psid, eps, gd)
+                : fx                 ? launch_dense_fx64(p, psid, eps, gd)
                                      : launch_dense_fp64(p, psid, eps, gd);
         else
             e = trunc_eval(p, psid, eps, prec == RSOT_MIXED, gd);
     }
-    if (!e && gdev && grad_out != gd)
-        e = launch_commit_grad(gd, grad_out, p->n, p->res_dev, dense ? 0 : 1, st);
-    if (!e && !gdev) e = cudaMemcpyAsync(p->grad_host, gd, nb, cudaMemcpyDeviceToHost, st);
-    if (!e) e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(EvalResult), cudaMemcpyDeviceToHost, st);
-    if (!e) e = cudaStreamSynchronize(st);
+    for (;;) {
+        if (!e && gdev && grad_out != gd)
+            e = launch_commit_grad(gd, grad_out, p->n, p->res_dev, dense ? 0 : 1, st);
+        if (!e && !gdev) e = cudaMemcpyAsync(p->grad_host, gd, nb, cudaMemcpyDeviceToHost, st);
+        if (!e) e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(EvalResult), cudaMemcpyDeviceToHost, st);
+        if (!e) e = cudaStreamSynchronize(st);
+        if (e || !fx || !(p->res_host->flags & kErrRange64)) break;
+        fx = false;
+        e = cudaMemsetAsync(p->res_dev, 0, sizeof(EvalResult), st);
+        if (!e) e = launch_dense_fp64(p, psid, eps, gd);
+    }
     if (e) {
         cudaGetLastError();
         p->tr_open.clear();

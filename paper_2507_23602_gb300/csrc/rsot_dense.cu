@@ -1169,6 +1169,36 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi, double eps, d
     return p->d == 3 ? launch_mixed_d<3>(p, psi, eps, grad) : launch_mixed_d<2>(p, psi, eps, grad);
 }
 
+// the FP32 pass 1 alone (records and per-chunk partials), for the fixed-point passes
+cudaError_t launch_mixed_pass1(rsot_problem *p, const double *psi, double eps) {
+    cudaStream_t st = p->stream;
+    trace_begin(p, "prep_targets_mixed");
+    k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
+                                                      p->d, eps, p->tdup, p->tpair, p->psinu,
+                                                      p->flags, nullptr, 1.0, nullptr);
+    trace_end(p);
+    dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)p->k1);
+    const int n_p1 = (int)round_up(p->n, P1_TS);
+    trace_begin(p, "lse_mixed");
+    if (p->d == 3)
+        k_lse_mixed<3><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tdup, n_p1, p->chunk1, p->part1,
+                                                  p->flags);
+    else
+        k_lse_mixed<2><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tdup, n_p1, p->chunk1, p->part1,
+                                                  p->flags);
+    trace_end(p);
+    return cudaGetLastError();
+}
+
+// J from pass-1 block partials of sum_q m_q eps L_q (FP64 forms)
+cudaError_t launch_finalize_J64(rsot_problem *p, const double *psi, double eps, int nbj) {
+    trace_begin(p, "finalize_J");
+    k_finalize_J<<<1, 256, 0, p->stream>>>(p->blockJ, nbj, p->psinu, p->nblk_prep, psi, eps, p->msum,
+                                           0.0, 0, p->res_dev);
+    trace_end(p);
+    return cudaGetLastError();
+}
+
 template <int D>
 static cudaError_t launch_fp64_d(rsot_problem *p, const double *psi, double eps, double *grad,
                                  const double *alpha, const double *beta) {
@@ -1204,11 +1234,7 @@ static cudaError_t launch_fp64_d(rsot_problem *p, const double *psi, double eps,
     k_finalize_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(p->part2_64, p->s2_64,
                                                                     p->n_pad, p->nu, p->n, grad);
     trace_end(p);
-    trace_begin(p, "finalize_J");
-    k_finalize_J<<<1, 256, 0, st>>>(p->blockJ, (int)nb1, p->psinu, p->nblk_prep, psi, eps, p->msum,
-                                    0.0, 0, p->res_dev);
-    trace_end(p);
-    return cudaGetLastError();
+    return launch_finalize_J64(p, psi, eps, (int)nb1);
 }
 
 cudaError_t launch_dense_fp64(rsot_problem *p, const double *psi, double eps, double *grad) {

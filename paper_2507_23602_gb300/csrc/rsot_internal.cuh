@@ -33,6 +33,7 @@ enum : int {
     kErrTimeout = 1,        // an mbarrier wait exceeded its iteration limit
     kErrNonfinitePsi = 2,   // psi had a NaN / Inf entry
     kErrBadCell = 4,        // a cell index fell outside the grid (truncated path)
+    kErrRange64 = 8,        // the fixed-point passes cannot hold the exponents: FP64 passes instead
 };
 
 struct __align__(16) Rec8 {   // 32-byte record: two float4
@@ -48,10 +49,14 @@ struct EvalResult {
     long long empty;
     int flags;
     int gate;           // bit 0: an f16 operand is out of range (both passes take the FP32 kernels)
+    unsigned fx_key[3]; // fixed-point passes (rsot_fx64.cu): largest -t*_q, B_j, |B_j| as ordered keys
+    int fx_F;           // their fraction bits
+    float fx_E;         // error bound of their FP32 exponent estimate
 };
 
 struct Grid;  // truncated-path cell grid (rsot_trunc.cu)
 struct Rec16; // tensor-core operand record (rsot_tc.cuh)
+struct FxRec; // fixed-point operand record (rsot_fx64.cu)
 
 }  // namespace rsot
 
@@ -112,6 +117,17 @@ struct rsot_problem {
     int s2_64 = 0;
     int64_t chunk2_64 = 0;
     double *part2_64 = nullptr;     // [s2_64][n_pad]
+    // fixed-point passes of the dense FP64 path (rsot_fx64.cu): one allocation on first use
+    void *fx_buf = nullptr;
+    rsot::FxRec *fx_prec = nullptr, *fx_trec = nullptr;   // integer operands of points, targets
+    float4 *fx_ptrow = nullptr, *fx_ptcol = nullptr;      // FP32 operands of the estimate
+    float4 *fx_tgrow = nullptr, *fx_tgcol = nullptr;
+    int *fx_ptshift = nullptr, *fx_tgshift = nullptr;     // integral row shifts
+    double *fx_tgscale = nullptr;                         // 2^(fraction of B_j)
+    double *fx_tab = nullptr;                             // 2^(-i/2048)
+    double *fx_part1 = nullptr, *fx_part2 = nullptr;      // row sums per column chunk
+    int fx_k1 = 0, fx_s2 = 0;
+    int64_t fx_chunk1 = 0, fx_chunk2 = 0;
     // compensated path scratch (rsot_df.cu), allocated on first use
     void *df_prec = nullptr;        // [nq_pad] point head/tail records (64 B)
     void *df_trec = nullptr;        // [n_pad] target head/tail records (64 B)
@@ -204,6 +220,13 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi_dev, double ep
                                double *grad_dev);
 cudaError_t launch_dense_fp64(rsot_problem *p, const double *psi_dev, double eps,
                               double *grad_dev);
+cudaError_t launch_mixed_pass1(rsot_problem *p, const double *psi_dev, double eps);
+cudaError_t launch_finalize_J64(rsot_problem *p, const double *psi_dev, double eps, int nbj);
+// dense FP64 evaluation with fixed-point exponents (rsot_fx64.cu); fx64_ready:
+// its buffers exist and the sizes of the exponents allow it
+bool fx64_ready(rsot_problem *p, double eps);
+cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
+void fx64_free(rsot_problem *p);
 cudaError_t launch_trunc_fp64(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
 cudaError_t launch_covering_cost(rsot_problem *p, double *C0_dev);
 cudaError_t launch_psi_stats(rsot_problem *p, const double *psi_dev, double *out3_dev);
