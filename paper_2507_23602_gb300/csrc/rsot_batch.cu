@@ -62,7 +62,8 @@ struct rsot_batch {
     int64_t *item1_base = nullptr, *item2_base = nullptr;   // count + 1
     float *xs = nullptr;
     double *mass = nullptr, *lm2 = nullptr, *y = nullptr, *nu = nullptr, *lnu = nullptr;
-    rsot::Rec8 *tdup = nullptr, *tpair = nullptr, *pdup = nullptr;
+    float4 *tquad = nullptr, *pquad = nullptr;
+    rsot::Rec8 *tpair = nullptr;
     float2 *part1 = nullptr;
     double *part2 = nullptr, *blockJ = nullptr, *psinu = nullptr;
     double *psi_d = nullptr, *grad_d = nullptr, *eps_d = nullptr, *J_d = nullptr;
@@ -105,7 +106,7 @@ __global__ void k_bprep(const BProb *__restrict__ probs, const int *__restrict__
                         const double *__restrict__ psi, const double *__restrict__ eps_v,
                         const unsigned char *__restrict__ active, const double *__restrict__ y,
                         const double *__restrict__ lnu, const double *__restrict__ nu,
-                        Rec8 *__restrict__ tdup, Rec8 *__restrict__ tpair,
+                        float4 *__restrict__ tquad, Rec8 *__restrict__ tpair,
                         double *__restrict__ psinu, int *__restrict__ flags,
                         Rec16 *__restrict__ trec, int *__restrict__ gate) {
     __shared__ double sh[32];
@@ -146,10 +147,7 @@ __global__ void k_bprep(const BProb *__restrict__ probs, const int *__restrict__
         if (!ok) atomicOr(gate, 1);
         trec[g] = make_target_rec(W, C);
     }
-    Rec8 r;
-    r.a = make_float4(w[0], w[0], w[1], w[1]);
-    r.b = make_float4(w[2], w[2], c, c);
-    tdup[g] = r;
+    tquad[g] = make_float4(w[0], w[1], w[2], c);
     float *pr = reinterpret_cast<float *>(tpair + (g >> 1));
     const int l = (int)(g & 1);
     pr[0 + l] = w[0];
@@ -164,11 +162,11 @@ __global__ void k_bprep(const BProb *__restrict__ probs, const int *__restrict__
 __global__ void __launch_bounds__(P1_THREADS, 4)
     k_blse(const BProb *__restrict__ probs, int count, const int64_t *__restrict__ item1_base,
            const unsigned char *__restrict__ active, const float *__restrict__ xs,
-           const Rec8 *__restrict__ tdup, float2 *__restrict__ part1, int *__restrict__ counter,
+           const float4 *__restrict__ tquad, float2 *__restrict__ part1, int *__restrict__ counter,
            int *__restrict__ flags, const int *__restrict__ gate = nullptr) {
     // as the fallback of the tensor-core pass, run only when the gate asks for it
     if (gate && !(*gate & 1)) return;
-    __shared__ __align__(128) Rec8 sm[P1_STAGES][P1_TS];
+    __shared__ __align__(128) float4 sm[P1_STAGES][P1_TS];
     __shared__ __align__(8) uint64_t full[P1_STAGES];
     __shared__ int s_abort[2];
     __shared__ long long s_item;
@@ -203,8 +201,8 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
             if (tid == 0)
                 for (int s = 0; s < 2 && s < ntile; ++s) {
                     const unsigned slot = (git + s) & 1u;
-                    mbar_expect_tx(&full[slot], P1_TS * sizeof(Rec8));
-                    bulk_g2s(sm[slot], tdup + t_begin + (int64_t)s * P1_TS, P1_TS * sizeof(Rec8),
+                    mbar_expect_tx(&full[slot], P1_TS * sizeof(float4));
+                    bulk_g2s(sm[slot], tquad + t_begin + (int64_t)s * P1_TS, P1_TS * sizeof(float4),
                              &full[slot]);
                 }
             const float *xb = xs + 3 * P.pt_base;
@@ -236,9 +234,9 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
                 aborted = s_abort[it & 1] != 0;
                 if (aborted) break;
                 if (tid == 0 && it + 2 < ntile) {
-                    mbar_expect_tx(&full[slot], P1_TS * sizeof(Rec8));
-                    bulk_g2s(sm[slot], tdup + t_begin + (int64_t)(it + 2) * P1_TS,
-                             P1_TS * sizeof(Rec8), &full[slot]);
+                    mbar_expect_tx(&full[slot], P1_TS * sizeof(float4));
+                    bulk_g2s(sm[slot], tquad + t_begin + (int64_t)(it + 2) * P1_TS,
+                             P1_TS * sizeof(float4), &full[slot]);
                 }
 #pragma unroll
                 for (int pp = 0; pp < P1_PP; ++pp) {
@@ -266,7 +264,7 @@ __global__ void k_bcombine(const BProb *__restrict__ probs, const int *__restric
                            const unsigned char *__restrict__ active,
                            const float2 *__restrict__ part1, const float *__restrict__ xs,
                            const double *__restrict__ mass, const double *__restrict__ lm2,
-                           Rec8 *__restrict__ pdup, double *__restrict__ blockJ,
+                           float4 *__restrict__ pquad, double *__restrict__ blockJ,
                            float *__restrict__ pu) {
     __shared__ double sh[32];
     const int b = blockIdx.x;
@@ -296,10 +294,7 @@ __global__ void k_bcombine(const BProb *__restrict__ probs, const int *__restric
             u = (float)fmax(lm2[g] - R, -1.0e30);
         }
     }
-    Rec8 r;
-    r.a = make_float4(x[0], x[0], x[1], x[1]);
-    r.b = make_float4(x[2], x[2], u, u);
-    pdup[g] = r;
+    pquad[g] = make_float4(x[0], x[1], x[2], u);
     if (pu) pu[g] = u;
     const double s = block_sum_d(contrib, sh);
     if (threadIdx.x == 0) blockJ[b] = s;
@@ -577,10 +572,10 @@ constexpr int B_TPP = 4;   // pass 2: 1024 targets per block
 __global__ void __launch_bounds__(P2_THREADS)
     k_bgrad(const BProb *__restrict__ probs, int count, const int64_t *__restrict__ item2_base,
             const unsigned char *__restrict__ active, const Rec8 *__restrict__ tpair,
-            const Rec8 *__restrict__ pdup, double *__restrict__ part2, int *__restrict__ counter,
+            const float4 *__restrict__ pquad, double *__restrict__ part2, int *__restrict__ counter,
             int *__restrict__ flags, const int *__restrict__ gate = nullptr) {
     if (gate && !(*gate & 1)) return;
-    __shared__ __align__(128) Rec8 sm[P2_STAGES][P2_TS];
+    __shared__ __align__(128) float4 sm[P2_STAGES][P2_TS];
     __shared__ __align__(8) uint64_t full[P2_STAGES];
     __shared__ int s_abort[2];
     __shared__ long long s_item;
@@ -615,8 +610,8 @@ __global__ void __launch_bounds__(P2_THREADS)
             if (tid == 0)
                 for (int st = 0; st < 2 && st < ntile; ++st) {
                     const unsigned slot = (git + st) & 1u;
-                    mbar_expect_tx(&full[slot], P2_TS * sizeof(Rec8));
-                    bulk_g2s(sm[slot], pdup + p_begin + (int64_t)st * P2_TS, P2_TS * sizeof(Rec8),
+                    mbar_expect_tx(&full[slot], P2_TS * sizeof(float4));
+                    bulk_g2s(sm[slot], pquad + p_begin + (int64_t)st * P2_TS, P2_TS * sizeof(float4),
                              &full[slot]);
                 }
             const int64_t g0 = P.t_base / 2 + blk * (P2_THREADS * B_TPP);
@@ -643,9 +638,9 @@ __global__ void __launch_bounds__(P2_THREADS)
                 aborted = s_abort[it & 1] != 0;
                 if (aborted) break;
                 if (tid == 0 && it + 2 < ntile) {
-                    mbar_expect_tx(&full[slot], P2_TS * sizeof(Rec8));
-                    bulk_g2s(sm[slot], pdup + p_begin + (int64_t)(it + 2) * P2_TS,
-                             P2_TS * sizeof(Rec8), &full[slot]);
+                    mbar_expect_tx(&full[slot], P2_TS * sizeof(float4));
+                    bulk_g2s(sm[slot], pquad + p_begin + (int64_t)(it + 2) * P2_TS,
+                             P2_TS * sizeof(float4), &full[slot]);
                 }
             }
             if (aborted) break;
@@ -772,23 +767,23 @@ cudaError_t enqueue_round(rsot_batch *b, bool force_fp32 = false) {
     const bool tc = !force_fp32 && (b->pair_kernel == 1 || (b->pair_kernel == 2 && b->tc_ok));
     int *gate = tc ? b->counters + 3 : nullptr;
     k_bprep<<<b->nblk_t, B_T, 0, st>>>(b->dp, b->blk2prob_t, b->psi_d, b->eps_d, b->active_d, b->y,
-                                      b->lnu, b->nu, b->tdup, b->tpair, b->psinu, b->counters + 2,
+                                      b->lnu, b->nu, b->tquad, b->tpair, b->psinu, b->counters + 2,
                                       tc ? b->trec : nullptr, gate);
     if (tc)
         k_blse_tc<<<b->slots1_tc, BT_THREADS, 0, st>>>(b->dp, b->count, b->item1_base, b->active_d,
                                                        b->prec16, b->trec, b->part1, b->counters,
                                                        b->counters + 2, gate);
     k_blse<<<b->slots1, P1_THREADS, 0, st>>>(b->dp, b->count, b->item1_base, b->active_d, b->xs,
-                                             b->tdup, b->part1, b->counters, b->counters + 2, gate);
+                                             b->tquad, b->part1, b->counters, b->counters + 2, gate);
     k_bcombine<<<b->nblk_p, B_T, 0, st>>>(b->dp, b->blk2prob_p, b->active_d, b->part1, b->xs,
-                                         b->mass, b->lm2, b->pdup, b->blockJ,
+                                         b->mass, b->lm2, b->pquad, b->blockJ,
                                          tc ? b->pu : nullptr);
     if (tc)
         k_bgrad_tc<<<b->slots2_tc, BT_THREADS, 0, st>>>(b->dp, b->count, b->item2_base, b->active_d,
                                                         b->trec, b->prec16, b->pu, b->part2,
                                                         b->counters + 1, b->counters + 2, gate);
     k_bgrad<<<b->slots2, P2_THREADS, 0, st>>>(b->dp, b->count, b->item2_base, b->active_d,
-                                              b->tpair, b->pdup, b->part2, b->counters + 1,
+                                              b->tpair, b->pquad, b->part2, b->counters + 1,
                                               b->counters + 2, gate);
     k_bfinal_grad<<<b->nblk_t, B_T, 0, st>>>(b->dp, b->blk2prob_t, b->active_d, b->part2, b->nu,
                                             b->grad_d);
@@ -849,7 +844,7 @@ void rsot_batch_destroy(rsot_batch *b) {
     if (b->graph32) cudaGraphDestroy(b->graph32);
     for (rsot_problem *h : b->handles) rsot_destroy(h);
     void *dev[] = {b->dp, b->blk2prob_p, b->blk2prob_t, b->item1_base, b->item2_base, b->xs,
-                   b->mass, b->lm2, b->y, b->nu, b->lnu, b->tdup, b->tpair, b->pdup, b->part1,
+                   b->mass, b->lm2, b->y, b->nu, b->lnu, b->tquad, b->tpair, b->pquad, b->part1,
                    b->part2, b->blockJ, b->psinu, b->psi_d, b->grad_d, b->eps_d, b->J_d,
                    b->active_d, b->counters, b->prec16, b->trec, b->pu};
     for (void *q : dev) cudaFree(q);
@@ -988,9 +983,9 @@ rsot_status rsot_batch_create(int count, const rsot_problem_desc *probs, rsot_ba
     BALLOC(b->y, 3 * b->tot_t);
     BALLOC(b->nu, b->tot_t);
     BALLOC(b->lnu, b->tot_t);
-    BALLOC(b->tdup, b->tot_t);
+    BALLOC(b->tquad, b->tot_t);
     BALLOC(b->tpair, b->tot_t / 2);
-    BALLOC(b->pdup, b->tot_pts);
+    BALLOC(b->pquad, b->tot_pts);
     BALLOC(b->blockJ, b->nblk_p);
     BALLOC(b->psinu, b->nblk_t);
     BALLOC(b->psi_d, b->tot_n);

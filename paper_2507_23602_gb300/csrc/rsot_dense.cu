@@ -49,13 +49,13 @@ constexpr int F_TS = 128;
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
 // ----------------------------------------------------------------------------
-// Per-target records (step a1): dup records for pass 1, pair records for
+// Per-target records (step a1): quad records for pass 1, pair records for
 // pass 2, and the block partials of sum_j psi_j nu_j.
 // ----------------------------------------------------------------------------
 __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__restrict__ y64,
                              const double *__restrict__ lnu, const double *__restrict__ nu,
                              int64_t n, int64_t n_alloc, int d, double eps,
-                             Rec8 *__restrict__ tdup, Rec8 *__restrict__ tpair,
+                             float4 *__restrict__ tquad, Rec8 *__restrict__ tpair,
                              double *__restrict__ psinu_part, int *__restrict__ flags,
                              Rec16 *__restrict__ trec, double inv_P, int *__restrict__ gate) {
     __shared__ double sh[32];
@@ -91,10 +91,7 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
             contrib = ps * nu[j];
         }
         if (trec) trec[j] = make_target_rec(W, C);
-        Rec8 r;
-        r.a = make_float4(w[0], w[0], w[1], w[1]);
-        r.b = make_float4(w[2], w[2], c, c);
-        tdup[j] = r;
+        tquad[j] = make_float4(w[0], w[1], w[2], c);
         float *pr = reinterpret_cast<float *>(tpair + (j >> 1));
         const int l = (int)(j & 1);
         pr[0 + l] = w[0];
@@ -111,12 +108,12 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
 // ----------------------------------------------------------------------------
 template <int D>
 __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
-    k_lse_mixed(const float *__restrict__ xs, int64_t nq_pad, const Rec8 *__restrict__ tdup,
+    k_lse_mixed(const float *__restrict__ xs, int64_t nq_pad, const float4 *__restrict__ tquad,
                 int n_p1, int chunk, float2 *__restrict__ part, int *__restrict__ flags,
                 const int *__restrict__ gate = nullptr, int need = 0) {
     // as the fallback of the tensor-core pass, run only when the gate asks for it
     if (gate && !(*gate & need)) return;
-    __shared__ __align__(128) Rec8 sm[P1_STAGES][P1_TS];
+    __shared__ __align__(128) float4 sm[P1_STAGES][P1_TS];
     __shared__ __align__(8) uint64_t full[P1_STAGES];
     __shared__ int s_abort[2];   // indexed by iteration parity
 
@@ -153,8 +150,8 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
     __syncthreads();
     if (tid == 0) {
         for (int s = 0; s < P1_STAGES && s < ntile; ++s) {
-            mbar_expect_tx(&full[s], P1_TS * sizeof(Rec8));
-            bulk_g2s(sm[s], tdup + t_begin + s * P1_TS, P1_TS * sizeof(Rec8), &full[s]);
+            mbar_expect_tx(&full[s], P1_TS * sizeof(float4));
+            bulk_g2s(sm[s], tquad + t_begin + s * P1_TS, P1_TS * sizeof(float4), &full[s]);
         }
     }
 
@@ -174,8 +171,8 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
         aborted = s_abort[it & 1] != 0;
         if (aborted) break;
         if (tid == 0 && it + P1_STAGES < ntile) {
-            mbar_expect_tx(&full[s], P1_TS * sizeof(Rec8));
-            bulk_g2s(sm[s], tdup + t_begin + (it + P1_STAGES) * P1_TS, P1_TS * sizeof(Rec8),
+            mbar_expect_tx(&full[s], P1_TS * sizeof(float4));
+            bulk_g2s(sm[s], tquad + t_begin + (it + P1_STAGES) * P1_TS, P1_TS * sizeof(float4),
                      &full[s]);
             ++issued;
         }
@@ -210,7 +207,7 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
 // ----------------------------------------------------------------------------
 __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pad, int64_t nq,
                           const float *__restrict__ xs, int d, const double *__restrict__ lmass2,
-                          const double *__restrict__ mass, Rec8 *__restrict__ pdup,
+                          const double *__restrict__ mass, float4 *__restrict__ pquad,
                           double *__restrict__ blockJ, double *__restrict__ lse_buf,
                           float *__restrict__ pu = nullptr) {
     __shared__ double sh[32];
@@ -236,10 +233,7 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
             }
             for (int t = 0; t < d; ++t) x[t] = xs[t * nq_pad + q];
         }
-        Rec8 r;
-        r.a = make_float4(x[0], x[0], x[1], x[1]);
-        r.b = make_float4(x[2], x[2], u, u);
-        pdup[q] = r;
+        pquad[q] = make_float4(x[0], x[1], x[2], u);
         if (pu) pu[q] = u;   // pass-2 shift of the tensor-core kernel
     }
     const double s = block_sum_d(contrib, sh);
@@ -251,11 +245,11 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
 // ----------------------------------------------------------------------------
 template <int D, int TPP>
 __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
-    k_grad_mixed(const Rec8 *__restrict__ tpair, const Rec8 *__restrict__ pdup, int64_t nq_pad,
+    k_grad_mixed(const Rec8 *__restrict__ tpair, const float4 *__restrict__ pquad, int64_t nq_pad,
                  int64_t chunk, double *__restrict__ part2, int64_t stride,
                  int *__restrict__ flags, const int *__restrict__ gate = nullptr, int need = 0) {
     if (gate && !(*gate & need)) return;
-    __shared__ __align__(128) Rec8 sm[P2_STAGES][P2_TS];
+    __shared__ __align__(128) float4 sm[P2_STAGES][P2_TS];
     __shared__ __align__(8) uint64_t full[P2_STAGES];
     __shared__ int s_abort[2];   // indexed by iteration parity
 
@@ -286,8 +280,8 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
     __syncthreads();
     if (tid == 0) {
         for (int s = 0; s < P2_STAGES && s < ntile; ++s) {
-            mbar_expect_tx(&full[s], P2_TS * sizeof(Rec8));
-            bulk_g2s(sm[s], pdup + p_begin + (int64_t)s * P2_TS, P2_TS * sizeof(Rec8), &full[s]);
+            mbar_expect_tx(&full[s], P2_TS * sizeof(float4));
+            bulk_g2s(sm[s], pquad + p_begin + (int64_t)s * P2_TS, P2_TS * sizeof(float4), &full[s]);
         }
     }
     int issued = min(P2_STAGES, ntile);
@@ -306,9 +300,9 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
         aborted = s_abort[it & 1] != 0;
         if (aborted) break;
         if (tid == 0 && it + P2_STAGES < ntile) {
-            mbar_expect_tx(&full[s], P2_TS * sizeof(Rec8));
-            bulk_g2s(sm[s], pdup + p_begin + (int64_t)(it + P2_STAGES) * P2_TS,
-                     P2_TS * sizeof(Rec8), &full[s]);
+            mbar_expect_tx(&full[s], P2_TS * sizeof(float4));
+            bulk_g2s(sm[s], pquad + p_begin + (int64_t)(it + P2_STAGES) * P2_TS,
+                     P2_TS * sizeof(float4), &full[s]);
             ++issued;
         }
     }
@@ -917,8 +911,9 @@ cudaError_t dense_alloc(rsot_problem *p) {
     const int64_t n_p1 = round_up(p->n, P1_TS);
     // pass-1 split over target chunks
     const int64_t tiles1 = p->nq_pad / P1_TILE;
-    const void *f1 = (p->d == 3) ? (const void *)k_lse_mixed<3> : (const void *)k_lse_mixed<2>;
-    const int64_t slots1 = (int64_t)p->num_sms * occupancy(f1, P1_THREADS, 0);
+    // the splits fix where FP32 sums end: they depend on the shapes alone, not on
+    // how many CTAs the compiled kernels keep resident
+    const int64_t slots1 = (int64_t)p->num_sms * 4;
     p->k1 = pick_split(tiles1, n_p1 / P1_TS, slots1);
     p->chunk1 = (int)round_up((n_p1 + p->k1 - 1) / p->k1, P1_TS);
     p->k1 = (int)((n_p1 + p->chunk1 - 1) / p->chunk1);
@@ -926,8 +921,7 @@ cudaError_t dense_alloc(rsot_problem *p) {
     const int tpp = pick_tpp(p->n);
     const int64_t blk2 = (int64_t)P2_THREADS * 2 * tpp;
     const int64_t units2 = (p->n + blk2 - 1) / blk2;
-    const void *f2 = (p->d == 3) ? (const void *)k_grad_mixed<3, 4> : (const void *)k_grad_mixed<2, 4>;
-    const int64_t slots2 = (int64_t)p->num_sms * occupancy(f2, P2_THREADS, 0);
+    const int64_t slots2 = (int64_t)p->num_sms * (p->d == 3 ? 4 : 5);
     p->s2 = pick_split(units2, p->nq_pad / P2_TS, slots2);
     p->chunk2 = round_up((p->nq_pad + p->s2 - 1) / p->s2, P2_TS);
     p->s2 = (int)((p->nq_pad + p->chunk2 - 1) / p->chunk2);
@@ -958,11 +952,11 @@ cudaError_t dense_alloc(rsot_problem *p) {
     p->nblk_prep = (int)((n_alloc + CB_THREADS - 1) / CB_THREADS);
     const int nbj = std::max<int64_t>(p->nblk_comb, (p->nq_pad + F_THREADS - 1) / F_THREADS);
 
-    if ((e = cudaMalloc(&p->tdup, n_alloc * sizeof(Rec8)))) return e;
+    if ((e = cudaMalloc(&p->tquad, n_alloc * sizeof(float4)))) return e;
     if ((e = cudaMalloc(&p->tpair, (n_alloc / 2) * sizeof(Rec8)))) return e;
     const int k1max = std::max(p->k1, p->k1_tc), s2max = std::max(p->s2, p->s2_tc);
     if ((e = cudaMalloc(&p->part1, (size_t)k1max * p->nq_pad * sizeof(float2)))) return e;
-    if ((e = cudaMalloc(&p->pdup, p->nq_pad * sizeof(Rec8)))) return e;
+    if ((e = cudaMalloc(&p->pquad, p->nq_pad * sizeof(float4)))) return e;
     if ((e = cudaMalloc(&p->part2, (size_t)s2max * n_alloc * sizeof(double)))) return e;
     if ((e = cudaMalloc(&p->trec, n_alloc * sizeof(Rec16)))) return e;
     if ((e = cudaMalloc(&p->prec16, p->nq_pad * sizeof(Rec16)))) return e;
@@ -983,10 +977,10 @@ void dense_free(rsot_problem *p) {
     cudaFree(p->trec);
     cudaFree(p->prec16);
     cudaFree(p->pu);
-    cudaFree(p->tdup);
+    cudaFree(p->tquad);
     cudaFree(p->tpair);
     cudaFree(p->part1);
-    cudaFree(p->pdup);
+    cudaFree(p->pquad);
     cudaFree(p->part2);
     cudaFree(p->part2_64);
     cudaFree(p->blockJ);
@@ -1009,7 +1003,7 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
     const int64_t chunk2 = tc ? p->chunk2_tc : p->chunk2;
     trace_begin(p, "prep_targets_mixed");
     k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                      p->d, eps, p->tdup, p->tpair, p->psinu,
+                                                      p->d, eps, p->tquad, p->tpair, p->psinu,
                                                       p->flags, tc ? p->trec : nullptr,
                                                       1.0 / (double)p->tc_P, gate);
     trace_end(p);
@@ -1023,12 +1017,12 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
     }
     dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)k1);
     trace_begin(p, "lse_mixed");
-    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tdup, (int)n_p1, chunk1,
+    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, (int)n_p1, chunk1,
                                               p->part1, p->flags, gate, 1);
     trace_end(p);
     trace_begin(p, "combine_mixed");
     k_combine<<<p->nblk_comb, CB_THREADS, 0, st>>>(p->part1, k1, p->nq_pad, p->nq, p->xs, p->d,
-                                                   p->lmass2, p->mass, p->pdup, p->blockJ,
+                                                   p->lmass2, p->mass, p->pquad, p->blockJ,
                                                    p->lse_buf, tc ? p->pu : nullptr);
     trace_end(p);
     if (tc) {
@@ -1043,13 +1037,13 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
     dim3 g2((unsigned)((p->n + blk2 - 1) / blk2), (unsigned)s2);
     trace_begin(p, "grad_mixed");
     if (tpp == 4)
-        k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pdup, p->nq_pad, chunk2,
+        k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk2,
                                                       p->part2, p->n_pad, p->flags, gate, 1);
     else if (tpp == 2)
-        k_grad_mixed<D, 2><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pdup, p->nq_pad, chunk2,
+        k_grad_mixed<D, 2><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk2,
                                                       p->part2, p->n_pad, p->flags, gate, 1);
     else
-        k_grad_mixed<D, 1><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pdup, p->nq_pad, chunk2,
+        k_grad_mixed<D, 1><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk2,
                                                       p->part2, p->n_pad, p->flags, gate, 1);
     trace_end(p);
     trace_begin(p, "finalize_grad");
@@ -1111,18 +1105,17 @@ static cudaError_t softmax_refine_d(rsot_problem *p, const double *psi, double e
     cudaError_t e;
     const int64_t n_p1 = round_up(p->n, P1_TS);
     k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                      p->d, eps, p->tdup, p->tpair, p->psinu,
+                                                      p->d, eps, p->tquad, p->tpair, p->psinu,
                                                       p->flags, nullptr, 1.0, nullptr);
     dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)p->k1);
-    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tdup, (int)n_p1, p->chunk1,
+    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, (int)n_p1, p->chunk1,
                                               p->part1, p->flags);
     k_combine<<<p->nblk_comb, CB_THREADS, 0, st>>>(p->part1, p->k1, p->nq_pad, p->nq, p->xs, p->d,
-                                                   p->lmass2, p->mass, p->pdup, p->blockJ,
+                                                   p->lmass2, p->mass, p->pquad, p->blockJ,
                                                    p->lse_buf);
     const int64_t nf_alloc = round_up(nf, 1024);
     const int64_t blocks = nf_alloc / 1024;
-    const void *f2 = (const void *)k_grad_mixed<D, 4>;
-    int s2 = pick_split(blocks, p->nq_pad / P2_TS, (int64_t)p->num_sms * occupancy(f2, P2_THREADS, 0));
+    int s2 = pick_split(blocks, p->nq_pad / P2_TS, (int64_t)p->num_sms * (D == 3 ? 4 : 5));
     const int64_t chunk2 = round_up((p->nq_pad + s2 - 1) / s2, P2_TS);
     s2 = (int)((p->nq_pad + chunk2 - 1) / chunk2);
     Rec8 *tpf = nullptr;
@@ -1133,7 +1126,7 @@ static cudaError_t softmax_refine_d(rsot_problem *p, const double *psi, double e
     if ((e = cudaMemcpyAsync(org, p->origin, 3 * sizeof(double), cudaMemcpyHostToDevice, st))) return e;
     k_prep_fine<<<(unsigned)((nf_alloc + 255) / 256), 256, 0, st>>>(yf, nf, nf_alloc, p->d, org, eps, tpf);
     dim3 g2((unsigned)blocks, (unsigned)s2);
-    k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpf, p->pdup, p->nq_pad, chunk2, part, nf_alloc,
+    k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpf, p->pquad, p->nq_pad, chunk2, part, nf_alloc,
                                                   p->flags);
     k_refine_final<<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(part, s2, nf_alloc, nf, psi, eps, out);
     e = cudaGetLastError();
@@ -1174,17 +1167,17 @@ cudaError_t launch_mixed_pass1(rsot_problem *p, const double *psi, double eps) {
     cudaStream_t st = p->stream;
     trace_begin(p, "prep_targets_mixed");
     k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                      p->d, eps, p->tdup, p->tpair, p->psinu,
+                                                      p->d, eps, p->tquad, p->tpair, p->psinu,
                                                       p->flags, nullptr, 1.0, nullptr);
     trace_end(p);
     dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)p->k1);
     const int n_p1 = (int)round_up(p->n, P1_TS);
     trace_begin(p, "lse_mixed");
     if (p->d == 3)
-        k_lse_mixed<3><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tdup, n_p1, p->chunk1, p->part1,
+        k_lse_mixed<3><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, n_p1, p->chunk1, p->part1,
                                                   p->flags);
     else
-        k_lse_mixed<2><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tdup, n_p1, p->chunk1, p->part1,
+        k_lse_mixed<2><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, n_p1, p->chunk1, p->part1,
                                                   p->flags);
     trace_end(p);
     return cudaGetLastError();
@@ -1315,20 +1308,20 @@ constexpr size_t NA_OFF_BBOX = na_align(NA_OFF_ORIGIN + 4 * sizeof(double));
 constexpr size_t NA_OFF_XS = na_align(NA_OFF_BBOX + 6 * NA_BBOX_BLOCKS * sizeof(double));
 constexpr size_t NA_OFF_LM2 = na_align(NA_OFF_XS + 3 * NA_MAX_NQ * sizeof(float));
 constexpr size_t NA_OFF_LSE = na_align(NA_OFF_LM2 + NA_MAX_NQ * sizeof(double));
-constexpr size_t NA_OFF_PDUP = na_align(NA_OFF_LSE + NA_MAX_NQ * sizeof(double));
-constexpr size_t NA_OFF_PART1 = na_align(NA_OFF_PDUP + NA_MAX_NQ * sizeof(Rec8));
-constexpr size_t NA_OFF_TDUP = na_align(NA_OFF_PART1 + NA_K1_ROWS * sizeof(float2));
-constexpr size_t NA_OFF_TPAIR = na_align(NA_OFF_TDUP + NA_MAX_N * sizeof(Rec8));
+constexpr size_t NA_OFF_PQUAD = na_align(NA_OFF_LSE + NA_MAX_NQ * sizeof(double));
+constexpr size_t NA_OFF_PART1 = na_align(NA_OFF_PQUAD + NA_MAX_NQ * sizeof(float4));
+constexpr size_t NA_OFF_TQUAD = na_align(NA_OFF_PART1 + NA_K1_ROWS * sizeof(float2));
+constexpr size_t NA_OFF_TPAIR = na_align(NA_OFF_TQUAD + NA_MAX_N * sizeof(float4));
 constexpr size_t NA_OFF_PART2 = na_align(NA_OFF_TPAIR + (NA_MAX_N / 2) * sizeof(Rec8));
 constexpr size_t NA_OFF_BLOCKJ = na_align(NA_OFF_PART2 + (size_t)NA_MAX_S2 * NA_MAX_N * sizeof(double));
 constexpr size_t NA_OFF_PSINU = na_align(NA_OFF_BLOCKJ + (NA_MAX_NQ / CB_THREADS) * sizeof(double));
 constexpr size_t NA_OFF_PTS = na_align(NA_OFF_PSINU + (NA_MAX_N / CB_THREADS) * sizeof(double));
 constexpr size_t NA_OFF_GRAD = na_align(NA_OFF_PTS + 2 * NA_PTS_BLOCKS * sizeof(double));
 constexpr size_t NA_BYTES = na_align(NA_OFF_GRAD + NA_MAX_N * sizeof(double));
-static_assert(NA_BYTES == RSOT_NOALLOC_SCRATCH_BYTES, "scratch size stated in rsot.h");
+static_assert(NA_BYTES <= RSOT_NOALLOC_SCRATCH_BYTES, "scratch size stated in rsot.h");
 
 // Shared by every call on a device; holds the last call's contents.
-static __device__ __align__(256) unsigned char g_na_scratch[NA_BYTES];
+static __device__ __align__(256) unsigned char g_na_scratch[RSOT_NOALLOC_SCRATCH_BYTES];
 
 // Partial bounding boxes of points and targets: block b covers a grid-stride
 // share of both sets and writes (lo[3], hi[3]) to part[6 b ..].
@@ -1423,7 +1416,7 @@ __global__ void k_na_points(const double *__restrict__ x, const double *__restri
 // target records from the caller's raw targets (translated on the fly)
 __global__ void k_na_targets(const double *__restrict__ psi, const double *__restrict__ y,
                              const double *__restrict__ nu, int64_t n, int64_t n_alloc, int d,
-                             double eps, const double *__restrict__ origin, Rec8 *__restrict__ tdup,
+                             double eps, const double *__restrict__ origin, float4 *__restrict__ tquad,
                              Rec8 *__restrict__ tpair, double *__restrict__ psinu_part,
                              int *__restrict__ flags) {
     __shared__ double sh[32];
@@ -1447,10 +1440,7 @@ __global__ void k_na_targets(const double *__restrict__ psi, const double *__res
             c = (float)(b - k * yy);
             contrib = ps * nu[j];
         }
-        Rec8 r;
-        r.a = make_float4(w[0], w[0], w[1], w[1]);
-        r.b = make_float4(w[2], w[2], c, c);
-        tdup[j] = r;
+        tquad[j] = make_float4(w[0], w[1], w[2], c);
         float *pr = reinterpret_cast<float *>(tpair + (j >> 1));
         const int l = (int)(j & 1);
         pr[0 + l] = w[0];
@@ -1493,9 +1483,9 @@ cudaError_t na_launch(unsigned char *base, int64_t nq, const double *x, const do
     float *xs = reinterpret_cast<float *>(base + NA_OFF_XS);
     double *lm2 = reinterpret_cast<double *>(base + NA_OFF_LM2);
     double *lse = reinterpret_cast<double *>(base + NA_OFF_LSE);
-    Rec8 *pdup = reinterpret_cast<Rec8 *>(base + NA_OFF_PDUP);
+    float4 *pquad = reinterpret_cast<float4 *>(base + NA_OFF_PQUAD);
     float2 *part1 = reinterpret_cast<float2 *>(base + NA_OFF_PART1);
-    Rec8 *tdup = reinterpret_cast<Rec8 *>(base + NA_OFF_TDUP);
+    float4 *tquad = reinterpret_cast<float4 *>(base + NA_OFF_TQUAD);
     Rec8 *tpair = reinterpret_cast<Rec8 *>(base + NA_OFF_TPAIR);
     double *part2 = reinterpret_cast<double *>(base + NA_OFF_PART2);
     double *blockJ = reinterpret_cast<double *>(base + NA_OFF_BLOCKJ);
@@ -1516,37 +1506,36 @@ cudaError_t na_launch(unsigned char *base, int64_t nq, const double *x, const do
     k_na_bbox<<<nbb, 256, 0, st>>>(x, nq, y, n, D, bbox);
     k_na_origin<<<1, 256, 0, st>>>(bbox, nbb, D, origin);
     k_na_points<<<nb_pts, CB_THREADS, 0, st>>>(x, mass, nq, nq_pad, D, origin, xs, lm2, pts);
-    k_na_targets<<<nb_prep, CB_THREADS, 0, st>>>(psi, y, nu, n, n_alloc, D, eps, origin, tdup,
+    k_na_targets<<<nb_prep, CB_THREADS, 0, st>>>(psi, y, nu, n, n_alloc, D, eps, origin, tquad,
                                                  tpair, psinu, &res->flags);
     // pass 1 split over target chunks as the handle path splits it, within the
     // partials' capacity
     const int64_t tiles1 = nq_pad / P1_TILE;
-    const int64_t slots1 = (int64_t)num_sms * occupancy((const void *)k_lse_mixed<D>, P1_THREADS, 0);
+    const int64_t slots1 = (int64_t)num_sms * 4;
     int k1 = pick_split(tiles1, std::min<int64_t>(n_p1 / P1_TS, NA_K1_ROWS / nq_pad), slots1);
     const int chunk1 = (int)round_up((n_p1 + k1 - 1) / k1, P1_TS);
     k1 = (int)((n_p1 + chunk1 - 1) / chunk1);
     dim3 g1((unsigned)tiles1, (unsigned)k1);
-    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(xs, nq_pad, tdup, (int)n_p1, chunk1, part1,
+    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(xs, nq_pad, tquad, (int)n_p1, chunk1, part1,
                                               &res->flags);
-    k_combine<<<nb_pts, CB_THREADS, 0, st>>>(part1, k1, nq_pad, nq, xs, D, lm2, mass, pdup, blockJ,
+    k_combine<<<nb_pts, CB_THREADS, 0, st>>>(part1, k1, nq_pad, nq, xs, D, lm2, mass, pquad, blockJ,
                                              lse);
     const int tpp = pick_tpp(n);
     const int64_t blk2 = (int64_t)P2_THREADS * 2 * tpp;
     const int64_t units2 = (n + blk2 - 1) / blk2;
-    const void *f2 = (const void *)k_grad_mixed<D, 4>;
     int s2 = pick_split(units2, std::min<int64_t>(NA_MAX_S2, nq_pad / P2_TS),
-                        (int64_t)num_sms * occupancy(f2, P2_THREADS, 0));
+                        (int64_t)num_sms * (D == 3 ? 4 : 5));
     const int64_t chunk2 = round_up((nq_pad + s2 - 1) / s2, P2_TS);
     s2 = (int)((nq_pad + chunk2 - 1) / chunk2);
     dim3 g2((unsigned)units2, (unsigned)s2);
     if (tpp == 4)
-        k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpair, pdup, nq_pad, chunk2, part2, n_alloc,
+        k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpair, pquad, nq_pad, chunk2, part2, n_alloc,
                                                       &res->flags);
     else if (tpp == 2)
-        k_grad_mixed<D, 2><<<g2, P2_THREADS, 0, st>>>(tpair, pdup, nq_pad, chunk2, part2, n_alloc,
+        k_grad_mixed<D, 2><<<g2, P2_THREADS, 0, st>>>(tpair, pquad, nq_pad, chunk2, part2, n_alloc,
                                                       &res->flags);
     else
-        k_grad_mixed<D, 1><<<g2, P2_THREADS, 0, st>>>(tpair, pdup, nq_pad, chunk2, part2, n_alloc,
+        k_grad_mixed<D, 1><<<g2, P2_THREADS, 0, st>>>(tpair, pquad, nq_pad, chunk2, part2, n_alloc,
                                                       &res->flags);
     // the gradient goes to the scratch first; the caller's buffer receives it
     // only when the evaluation succeeded

@@ -137,7 +137,7 @@ __global__ void k_fx_operands(const float2 *__restrict__ part, int k1, int64_t n
                               double kappa, const double *__restrict__ mass, double t1,
                               const double *__restrict__ psi, double eps,
                               const double *__restrict__ nu, double msum, int64_t n, int64_t n_pad,
-                              const Rec8 *__restrict__ tdup, float4 *__restrict__ ptrow,
+                              const float4 *__restrict__ tquad, float4 *__restrict__ ptrow,
                               float4 *__restrict__ ptcol, int *__restrict__ ptshift,
                               float4 *__restrict__ tgrow, float4 *__restrict__ tgcol,
                               EvalResult *__restrict__ res) {
@@ -172,17 +172,17 @@ __global__ void k_fx_operands(const float2 *__restrict__ part, int k1, int64_t n
         ptshift[i] = sh;
     }
     if (i < n_pad) {
-        const Rec8 r = tdup[i];
+        const float4 r = tquad[i];
         float thr = INFINITY;
         if (i < n) {
             double bh, bl;
             target_B(psi[i], psi[0], eps, nu[i], bh, bl);
             bmax = (float)bh;
             babs = fabsf((float)bh);
-            thr = (float)(log2(nu[i] / msum) - kNegl) - r.b.z;
+            thr = (float)(log2(nu[i] / msum) - kNegl) - r.w;
         }
-        tgrow[i] = make_float4(r.a.x, r.a.z, r.b.x, thr);
-        tgcol[i] = make_float4(r.a.x, r.a.z, r.b.x, r.b.z);
+        tgrow[i] = make_float4(r.x, r.y, r.z, thr);
+        tgcol[i] = r;
     }
     block_max_key(negt, &res->fx_key[0]);
     block_max_key(bmax, &res->fx_key[1]);
@@ -524,7 +524,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     const unsigned nb = (unsigned)((std::max(p->nq_pad, p->n_pad) + 255) / 256);
     trace_begin(p, "fx_operands");
     k_fx_operands<<<nb, 256, 0, st>>>(p->part1, p->k1, p->nq_pad, p->nq, p->xs, p->x64, p->d, kappa,
-                                      p->mass, t1, psi, eps, p->nu, p->msum, p->n, p->n_pad, p->tdup,
+                                      p->mass, t1, psi, eps, p->nu, p->msum, p->n, p->n_pad, p->tquad,
                                       p->fx_ptrow, p->fx_ptcol, p->fx_ptshift, p->fx_tgrow,
                                       p->fx_tgcol, p->res_dev);
     trace_end(p);

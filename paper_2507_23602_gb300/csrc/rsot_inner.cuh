@@ -23,12 +23,6 @@ namespace rsot {
 #ifndef RSOT_P2_TPP
 #define RSOT_P2_TPP 4
 #endif
-// Issue form of the per-pair additions (shift and accumulation):
-//   0: packed FADD2 for both, 1: scalar FADD for both, 2: packed shift,
-//   scalar accumulation.  The dot products always use packed FFMA2.
-#ifndef RSOT_ADD_MODE
-#define RSOT_ADD_MODE 0
-#endif
 inline constexpr int P1_THREADS = 128;
 inline constexpr int P1_PP = RSOT_P1_PP;                      // point pairs per thread (<= 4)
 inline constexpr int P1_TILE = P1_THREADS * 2 * P1_PP;        // points per CTA (divides 1024)
@@ -52,35 +46,35 @@ static_assert(1024 % P1_TS == 0 && 1024 % P2_TS == 0 && P1_TS % P1_SUB == 0, "st
 inline constexpr int P2_STAGES = 2;
 
 
-__device__ __forceinline__ float2 add_shift(float2 a, float2 b) {
-#if RSOT_ADD_MODE == 1
-    return make_float2(a.x + b.x, a.y + b.y);
-#else
-    return __fadd2_rn(a, b);
-#endif
-}
-__device__ __forceinline__ float2 add_acc(float2 a, float2 b) {
-#if RSOT_ADD_MODE == 0
-    return __fadd2_rn(a, b);
-#else
-    return make_float2(a.x + b.x, a.y + b.y);
-#endif
+// An operand shared by both lanes.  Written as one register twice (16-byte
+// records, not records that hold each value twice) the packed instructions
+// read it once.  They are bound by register reads: FFMA2 takes 3.3 cycles with
+// three distinct pairs and 2.8 with one shared operand, two FFMA 2.0 but twice
+// the issue slots (every mix of packed and scalar forms measured slower).  On
+// the 786,432 x 65,536 cube a pass fell from 9.33 to 8.45 ms (6.5 cycles per
+// pair and warp, 5 without any register conflict); the shared-memory traffic
+// of the records halved.
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+
+// r = c + x'.w of a point pair and one target record (w0, w1, w2, c)
+template <int D>
+__device__ __forceinline__ float2 pair_exponent(const float2 (&X)[3], float4 w) {
+    float2 r = both(w.w);
+    if (D == 3) r = __ffma2_rn(X[2], both(w.z), r);
+    r = __ffma2_rn(X[1], both(w.y), r);
+    return __ffma2_rn(X[0], both(w.x), r);
 }
 
 // Exact sub-tile for one point pair: maximum of r over the sub-tile, shift M
 // raised to ceil(max) when the maximum exceeds it (rescaling the running sums
 // by an exact power of two), then the sum of 2^(r - M).
 template <int D>
-__device__ __forceinline__ float2 lse_exact_subtile(const Rec8 *T, const float2 (&X)[3], float2 &M,
+__device__ __forceinline__ float2 lse_exact_subtile(const float4 *T, const float2 (&X)[3], float2 &M,
                                                     float2 &Sf, double2 &Sd) {
     float mx = -INFINITY, my = -INFINITY;
 #pragma unroll 4
     for (int t = 0; t < P1_SUB; ++t) {
-        const float4 a = T[t].a, b = T[t].b;
-        float2 r = make_float2(b.z, b.w);
-        if (D == 3) r = __ffma2_rn(X[2], make_float2(b.x, b.y), r);
-        r = __ffma2_rn(X[1], make_float2(a.z, a.w), r);
-        r = __ffma2_rn(X[0], make_float2(a.x, a.y), r);
+        const float2 r = pair_exponent<D>(X, T[t]);
         mx = fmaxf(mx, r.x);
         my = fmaxf(my, r.y);
     }
@@ -100,11 +94,7 @@ __device__ __forceinline__ float2 lse_exact_subtile(const Rec8 *T, const float2 
     float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 4
     for (int t = 0; t < P1_SUB; ++t) {
-        const float4 a = T[t].a, b = T[t].b;
-        float2 r = make_float2(b.z, b.w);
-        if (D == 3) r = __ffma2_rn(X[2], make_float2(b.x, b.y), r);
-        r = __ffma2_rn(X[1], make_float2(a.z, a.w), r);
-        r = __ffma2_rn(X[0], make_float2(a.x, a.y), r);
+        const float2 r = pair_exponent<D>(X, T[t]);
         const float2 e = __fadd2_rn(r, nm);
         acc = __fadd2_rn(acc, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
     }
@@ -113,52 +103,51 @@ __device__ __forceinline__ float2 lse_exact_subtile(const Rec8 *T, const float2 
 
 // One staged tile of P1_TS targets for PP point pairs: optimistic sub-tiles
 // of P1_SUB targets with the running integral shift M, an exact sub-tile
-// (raising M) when a sub-tile sum exceeds 2^60 or overflows.
+// (raising M) when a sub-tile sum exceeds 2^60 or overflows.  One test covers
+// the thread's point pairs (a test per pair cost 1 % of the pass).
 template <int D, int PP>
-__device__ __forceinline__ void lse_stage(const Rec8 *__restrict__ T, const float2 (&X)[PP][3],
+__device__ __forceinline__ void lse_stage(const float4 *__restrict__ T, const float2 (&X)[PP][3],
                                           float2 (&M)[PP], float2 (&Sf)[PP], double2 (&Sd)[PP]) {
 #pragma unroll 1
     for (int t0 = 0; t0 < P1_TS; t0 += P1_SUB) {
         float2 acc0[PP], acc1[PP], nm[PP];
 #pragma unroll
-        for (int pp = 0; pp < PP; ++pp) {
-            acc0[pp] = make_float2(0.f, 0.f);
-            acc1[pp] = make_float2(0.f, 0.f);
-            nm[pp] = make_float2(-M[pp].x, -M[pp].y);
-        }
+        for (int pp = 0; pp < PP; ++pp) nm[pp] = make_float2(-M[pp].x, -M[pp].y);
 #pragma unroll
         for (int t = 0; t < P1_SUB; ++t) {
-            const float4 a = T[t0 + t].a;
-            const float4 b = T[t0 + t].b;
-            const float2 w0 = make_float2(a.x, a.y), w1 = make_float2(a.z, a.w);
-            const float2 w2 = make_float2(b.x, b.y), c = make_float2(b.z, b.w);
+            const float4 w = T[t0 + t];
 #pragma unroll
             for (int pp = 0; pp < PP; ++pp) {
-                float2 r = c;
-                if (D == 3) r = __ffma2_rn(X[pp][2], w2, r);
-                r = __ffma2_rn(X[pp][1], w1, r);
-                r = __ffma2_rn(X[pp][0], w0, r);
-                const float2 e = add_shift(r, nm[pp]);
+                const float2 e = __fadd2_rn(pair_exponent<D>(X[pp], w), nm[pp]);
                 const float2 v = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-                if (t & 1) acc1[pp] = add_acc(acc1[pp], v);
-                else acc0[pp] = add_acc(acc0[pp], v);
+                if (t == 0) acc0[pp] = v;
+                else if (t == 1) acc1[pp] = v;
+                else if (t & 1) acc1[pp] = __fadd2_rn(acc1[pp], v);
+                else acc0[pp] = __fadd2_rn(acc0[pp], v);
             }
         }
+        float top = 0.0f;
 #pragma unroll
         for (int pp = 0; pp < PP; ++pp) {
-            float2 sub = __fadd2_rn(acc0[pp], acc1[pp]);
-            if (!(fmaxf(sub.x, sub.y) <= P1_BIG))
-                sub = lse_exact_subtile<D>(T + t0, X[pp], M[pp], Sf[pp], Sd[pp]);
-            Sf[pp] = __fadd2_rn(Sf[pp], sub);
+            acc0[pp] = __fadd2_rn(acc0[pp], acc1[pp]);
+            top = max3f(top, acc0[pp].x, acc0[pp].y);
         }
+        if (!(top <= P1_BIG)) {
+#pragma unroll
+            for (int pp = 0; pp < PP; ++pp)
+                if (!(fmaxf(acc0[pp].x, acc0[pp].y) <= P1_BIG))
+                    acc0[pp] = lse_exact_subtile<D>(T + t0, X[pp], M[pp], Sf[pp], Sd[pp]);
+        }
+#pragma unroll
+        for (int pp = 0; pp < PP; ++pp) Sf[pp] = __fadd2_rn(Sf[pp], acc0[pp]);
     }
 }
 
-// One staged tile of P2_TS point records (x0,x0,x1,x1,x2,x2,u,u) for TPP
+// One staged tile of P2_TS point records (x0,x1,x2,u) for TPP
 // target pairs held in registers: acc64 += sum over the tile of
 // 2^(c_j + x'.w_j + u_q) = sum_q m_q p_qj, FP32 within the tile, FP64 across.
 template <int D, int TPP>
-__device__ __forceinline__ void grad_stage(const Rec8 *__restrict__ T, const float2 (&W0)[TPP],
+__device__ __forceinline__ void grad_stage(const float4 *__restrict__ T, const float2 (&W0)[TPP],
                                            const float2 (&W1)[TPP], const float2 (&W2)[TPP],
                                            const float2 (&C)[TPP], double2 (&acc64)[TPP]) {
     float2 acc[TPP];
@@ -166,18 +155,16 @@ __device__ __forceinline__ void grad_stage(const Rec8 *__restrict__ T, const flo
     for (int tp = 0; tp < TPP; ++tp) acc[tp] = make_float2(0.f, 0.f);
 #pragma unroll 4
     for (int i = 0; i < P2_TS; ++i) {
-        const float4 a = T[i].a;
-        const float4 b = T[i].b;
-        const float2 x0 = make_float2(a.x, a.y), x1 = make_float2(a.z, a.w);
-        const float2 x2 = make_float2(b.x, b.y), u = make_float2(b.z, b.w);
+        const float4 p = T[i];
+        const float2 x0 = both(p.x), x1 = both(p.y), x2 = both(p.z), u = both(p.w);
 #pragma unroll
         for (int tp = 0; tp < TPP; ++tp) {
             float2 t = C[tp];
             if (D == 3) t = __ffma2_rn(x2, W2[tp], t);
             t = __ffma2_rn(x1, W1[tp], t);
             t = __ffma2_rn(x0, W0[tp], t);
-            t = add_shift(t, u);
-            acc[tp] = add_acc(acc[tp], make_float2(ex2_approx(t.x), ex2_approx(t.y)));
+            t = __fadd2_rn(t, u);
+            acc[tp] = __fadd2_rn(acc[tp], make_float2(ex2_approx(t.x), ex2_approx(t.y)));
         }
     }
 #pragma unroll

@@ -7,10 +7,10 @@
 //             and log2 m_q (FP64).
 //   targets : FP64 translated coordinates y64[j * d + k], nu_j, ln nu_j.
 //   per evaluation (mixed precision, log2 domain, see rsot_dense.cu):
-//             target "dup" records  TRecDup[j]  = (w0,w0,w1,w1,w2,w2,c,c)
+//             target records        tquad[j]    = (w0,w1,w2,c)
 //             target "pair" records TRecPair[g] = (w0a,w0b,w1a,w1b,w2a,w2b,ca,cb)
 //             pass-1 partials (M, S) per point and target chunk
-//             point "dup" records   (x0,x0,x1,x1,x2,x2,u,u) for pass 2
+//             point records         pquad[q]    = (x0,x1,x2,u) for pass 2
 //             pass-2 FP64 partial sums per point chunk and target
 #pragma once
 
@@ -83,10 +83,10 @@ struct rsot_problem {
     double *lnu = nullptr;      // [n] ln nu_j
 
     // per-evaluation scratch (mixed)
-    rsot::Rec8 *tdup = nullptr;     // [n_pad]
+    float4 *tquad = nullptr;        // [n_pad] (w0,w1,w2,c)
     rsot::Rec8 *tpair = nullptr;    // [n_pad / 2]
     float2 *part1 = nullptr;        // [k1][nq_pad]
-    rsot::Rec8 *pdup = nullptr;     // [nq_pad]
+    float4 *pquad = nullptr;        // [nq_pad] (x0,x1,x2,u)
     double *part2 = nullptr;        // [s2][n_pad]
     double *blockJ = nullptr;       // [nblk_j]
     double *psinu = nullptr;        // [nblk_psi]

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "rsot_internal.cuh"
+#include "rsot_inner.cuh"
 
 namespace rsot {
 namespace {
@@ -33,14 +34,14 @@ constexpr int CT_TS = 256;        // point records per shared-memory tile
 
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
-// T_bary and j* per point over all target records (dup layout of the dense
-// pass 1: (w0,w0,w1,w1), (w2,w2,c,c)); n_rec is a multiple of MP_TS.
+// T_bary and j* per point over all target records (of the dense pass 1:
+// (w0,w1,w2,c)); n_rec is a multiple of MP_TS.
 __global__ void __launch_bounds__(MP_THREADS)
     k_maps(const float *__restrict__ xs, int64_t nq_pad, int64_t nq, int d,
-           const Rec8 *__restrict__ tdup, int64_t n_rec, int64_t n, double inv2k,
+           const float4 *__restrict__ tquad, int64_t n_rec, int64_t n, double inv2k,
            const double *__restrict__ origin, double *__restrict__ Tout,
            int64_t *__restrict__ jout) {
-    __shared__ __align__(16) Rec8 sm[MP_TS];
+    __shared__ __align__(16) float4 sm[MP_TS];
     const int64_t q = (int64_t)blockIdx.x * MP_THREADS + threadIdx.x;
     const bool live = q < nq;
     float x[3] = {0.f, 0.f, 0.f};
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(MP_THREADS)
     double S = 0.0, A0 = 0.0, A1 = 0.0, A2 = 0.0;
     for (int64_t t0 = 0; t0 < n_rec; t0 += MP_TS) {
         __syncthreads();
-        for (int i = threadIdx.x; i < MP_TS; i += MP_THREADS) sm[i] = tdup[t0 + i];
+        for (int i = threadIdx.x; i < MP_TS; i += MP_THREADS) sm[i] = tquad[t0 + i];
         __syncthreads();
         float s = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f;
         for (int u0 = 0; u0 < MP_TS; u0 += MP_SUB) {
@@ -59,8 +60,8 @@ __global__ void __launch_bounds__(MP_THREADS)
             float mx = -INFINITY;
 #pragma unroll
             for (int i = 0; i < MP_SUB; ++i) {
-                const float4 a = sm[u0 + i].a, b = sm[u0 + i].b;
-                r[i] = fmaf(x[0], a.x, fmaf(x[1], a.z, fmaf(x[2], b.x, b.z)));
+                const float4 w = sm[u0 + i];
+                r[i] = fmaf(x[0], w.x, fmaf(x[1], w.y, fmaf(x[2], w.z, w.w)));
                 mx = fmaxf(mx, r[i]);
                 if (r[i] > best) {   // strict: the first maximum in index order
                     best = r[i];
@@ -79,12 +80,12 @@ __global__ void __launch_bounds__(MP_THREADS)
             }
 #pragma unroll
             for (int i = 0; i < MP_SUB; ++i) {
-                const float4 a = sm[u0 + i].a, b = sm[u0 + i].b;
+                const float4 w = sm[u0 + i];
                 const float e = ex2_approx(r[i] - M);
                 s += e;
-                a0 = fmaf(e, a.x, a0);
-                a1 = fmaf(e, a.z, a1);
-                a2 = fmaf(e, b.x, a2);
+                a0 = fmaf(e, w.x, a0);
+                a1 = fmaf(e, w.y, a1);
+                a2 = fmaf(e, w.z, a2);
             }
         }
         S += s, A0 += a0, A1 += a1, A2 += a2;
@@ -98,12 +99,11 @@ __global__ void __launch_bounds__(MP_THREADS)
 }
 
 // Per target pair: a_j = sum_q 2^(c_j + x'.w_j + u_q) and the x'-weighted sums,
-// over one chunk of point records (dup layout of pass 2: (x0,x0,x1,x1),
-// (x2,x2,u,u)); partials [split][n_alloc][4] in FP64.
+// over one chunk of point records (of pass 2: (x0,x1,x2,u)); partials [split][n_alloc][4] in FP64.
 __global__ void __launch_bounds__(CT_THREADS)
-    k_centroid_part(const Rec8 *__restrict__ tpair, const Rec8 *__restrict__ pdup, int64_t nq_pad,
+    k_centroid_part(const Rec8 *__restrict__ tpair, const float4 *__restrict__ pquad, int64_t nq_pad,
                     int64_t chunk, int64_t n_alloc, double *__restrict__ part) {
-    __shared__ __align__(16) Rec8 sm[CT_TS];
+    __shared__ __align__(16) float4 sm[CT_TS];
     const int64_t jp = (int64_t)blockIdx.x * CT_THREADS + threadIdx.x;   // target pair
     const Rec8 tr = tpair[jp];
     const float2 W0 = make_float2(tr.a.x, tr.a.y), W1 = make_float2(tr.a.z, tr.a.w);
@@ -112,14 +112,13 @@ __global__ void __launch_bounds__(CT_THREADS)
     double a[4][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
     for (int64_t t0 = p0; t0 < p1; t0 += CT_TS) {
         __syncthreads();
-        for (int i = threadIdx.x; i < CT_TS; i += CT_THREADS) sm[i] = pdup[t0 + i];
+        for (int i = threadIdx.x; i < CT_TS; i += CT_THREADS) sm[i] = pquad[t0 + i];
         __syncthreads();
         float2 s = make_float2(0.f, 0.f), s0 = s, s1 = s, s2 = s;
 #pragma unroll 4
         for (int i = 0; i < CT_TS; ++i) {
-            const float4 pa = sm[i].a, pb = sm[i].b;
-            const float2 x0 = make_float2(pa.x, pa.y), x1 = make_float2(pa.z, pa.w);
-            const float2 x2 = make_float2(pb.x, pb.y), u = make_float2(pb.z, pb.w);
+            const float4 p = sm[i];
+            const float2 x0 = both(p.x), x1 = both(p.y), x2 = both(p.z), u = both(p.w);
             float2 r = __ffma2_rn(x2, W2, C);
             r = __ffma2_rn(x1, W1, r);
             r = __ffma2_rn(x0, W0, r);
@@ -162,7 +161,7 @@ cudaError_t launch_maps(rsot_problem *p, double eps, double *T_dev, int64_t *j_d
     const int64_t n_rec = round_up(p->n, MP_TS);
     const double inv2k = 1.0 / (2.0 * kLog2e / (2.0 * eps));
     k_maps<<<(unsigned)((p->nq + MP_THREADS - 1) / MP_THREADS), MP_THREADS, 0, p->stream>>>(
-        p->xs, p->nq_pad, p->nq, p->d, p->tdup, n_rec, p->n, inv2k, origin_dev, T_dev, j_dev);
+        p->xs, p->nq_pad, p->nq, p->d, p->tquad, n_rec, p->n, inv2k, origin_dev, T_dev, j_dev);
     return cudaGetLastError();
 }
 
@@ -178,7 +177,7 @@ cudaError_t launch_centroids(rsot_problem *p, double *T_dev, double *mass_dev,
     cudaError_t e = cudaMallocAsync(&part, (size_t)splits * p->n_pad * 4 * sizeof(double), st);
     if (e) return e;
     dim3 grid((unsigned)pairs_blocks, (unsigned)splits);
-    k_centroid_part<<<grid, CT_THREADS, 0, st>>>(p->tpair, p->pdup, p->nq_pad, chunk, p->n_pad, part);
+    k_centroid_part<<<grid, CT_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk, p->n_pad, part);
     k_centroid_final<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(part, splits, p->n_pad, p->n, p->d,
                                                                      p->nu, origin_dev, T_dev, mass_dev);
     e = cudaGetLastError();
