@@ -33,6 +33,7 @@
 #include <algorithm>
 
 #include "rsot_internal.cuh"
+#include "rsot_inner.cuh"
 #include "rsot_tc.cuh"
 
 namespace rsot {
@@ -83,7 +84,8 @@ struct Grid {
     float *pa512 = nullptr, *tb512 = nullptr, *tb1024 = nullptr;
     float2 *part1b = nullptr;
     double *part2b = nullptr;
-    Rec8 *pdup_s = nullptr;   // FP32 block-skip pass 2: sorted point records (per evaluation)
+    float4 *tquad_s = nullptr, *pquad_s = nullptr;   // block-skip passes: sorted records (per evaluation)
+    float *nb_s = nullptr;                           // and the targets' test operand
     float *nAq_s = nullptr;   // FP32 block-skip pass 2: -A_q 2^64 of the sorted points (per evaluation)
     int *off1b = nullptr, *off2b = nullptr;
     int k1b = 0, k2b = 0;
@@ -401,10 +403,13 @@ __global__ void k_item_offsets(const int *__restrict__ cnt1, int ptiles, int ch1
     }
 }
 
-// target records in sorted order: (w0,w0,w1,w1) (w2,w2,c,c) (-b,-b,0,0)
+// target records in sorted order: (w0,w1,w2,c) and -b_j + 2k beta_j (block-skip
+// passes, always), (w0,w0,w1,w1) (w2,w2,c,c) (-b,-b,0,0) (queue passes, tdup
+// non-null)
 __global__ void k_prep_trunc(const double *__restrict__ psi, const int *__restrict__ perm_t,
                              const double *__restrict__ y64s, const double *__restrict__ lnu_s,
-                             int64_t n, int64_t nt, int d, double eps, Rec12 *__restrict__ tdup,
+                             int64_t n, int64_t nt, int d, double eps, float4 *__restrict__ tquad,
+                             float *__restrict__ nb_s, Rec12 *__restrict__ tdup,
                              double *__restrict__ psinu_part, const double *__restrict__ nu_s,
                              int *__restrict__ flags, Rec16 *__restrict__ trec, float *__restrict__ bs,
                              double inv_P, int *__restrict__ gate, const double *__restrict__ beta) {
@@ -431,11 +436,15 @@ __global__ void k_prep_trunc(const double *__restrict__ psi, const int *__restri
             nb = (float)(2.0 * k * beta[perm_t[s]] - b);
             contrib = ps * nu_s[s];
         }
-        Rec12 r;
-        r.a = make_float4(w[0], w[0], w[1], w[1]);
-        r.b = make_float4(w[2], w[2], c, c);
-        r.c = make_float4(nb, nb, 0.f, 0.f);
-        tdup[s] = r;
+        tquad[s] = make_float4(w[0], w[1], w[2], c);
+        nb_s[s] = nb;
+        if (tdup) {
+            Rec12 r;
+            r.a = make_float4(w[0], w[0], w[1], w[1]);
+            r.b = make_float4(w[2], w[2], c, c);
+            r.c = make_float4(nb, nb, 0.f, 0.f);
+            tdup[s] = r;
+        }
         if (trec) {
             // tensor-core operands (rsot_tc.cuh) and b_j (+inf for padding: the
             // truncation test r - b_j > A_q then fails)
@@ -1251,35 +1260,37 @@ constexpr int FB_TS = TC_TS;                // records per stage (1,024 columns)
 constexpr int FB_NBS = FB_TS / 8;           // n-blocks per stage
 constexpr int FB_STAGES = 2;
 constexpr int FB_GROUP = 8;                 // n-blocks per optimistic group (pass 1)
-constexpr size_t FB_SMEM1 = (size_t)FB_STAGES * (FB_TS * sizeof(Rec12) + FB_NBS * (sizeof(float4) + sizeof(float2)));
-constexpr size_t FB_SMEM2 =
-    (size_t)FB_STAGES * (FB_TS * (sizeof(Rec8) + sizeof(float)) + FB_NBS * (sizeof(float4) + sizeof(float2)));
+// a stage: a record and the test's operand per column, a ball and a range per n-block
+constexpr unsigned FB_STAGE = FB_TS * (sizeof(float4) + sizeof(float)) + FB_NBS * (sizeof(float4) + sizeof(float2));
+constexpr size_t FB_SMEM = (size_t)FB_STAGES * FB_STAGE;
 static_assert(FB_ROWS == PT && FB_TS == 1024 && FB_ROWS % TT == 0, "FB layout: a CTA is a point tile / four target tiles");
 
 // pass-1 exponents of one target for the lane's row pair of half h: returns r
 template <int D>
-__device__ __forceinline__ float2 fb_r(const float2 (&X)[3], float2 w0, float2 w1, float2 w2, float2 c) {
-    float2 r = c;
-    if (D == 3) r = __ffma2_rn(X[2], w2, r);
-    r = __ffma2_rn(X[1], w1, r);
-    r = __ffma2_rn(X[0], w0, r);
-    return r;
+__device__ __forceinline__ float2 fb_r(const float2 (&X)[3], float4 w) {
+    return pair_exponent<D>(X, w);
+}
+// pass-2 exponents of one point for the lane's target pair
+template <int D>
+__device__ __forceinline__ float2 fb_r2(const float2 (&W)[3], float2 C, float4 p) {
+    float2 r = C;
+    if (D == 3) r = __ffma2_rn(both(p.z), W[2], r);
+    r = __ffma2_rn(both(p.y), W[1], r);
+    return __ffma2_rn(both(p.x), W[0], r);
 }
 
 // pass 1, one half of the warp live in an n-block: the eight targets of the
 // half's row pair, tested (boundary) or not (inside)
 template <int D>
-__device__ __forceinline__ void fb1_half(const Rec12 *T, const float2 (&X)[3], float2 ng, float2 a, bool bnd,
+__device__ __forceinline__ void fb1_half(const float4 *T, const float *Nb, const float2 (&X)[3], float2 ng, float2 a, bool bnd,
                                          float2 &acc, float2 &cntf) {
     if (bnd) {
 #pragma unroll
         for (int tt = 0; tt < 8; ++tt) {
-            const float4 a4 = T[tt].a, b4 = T[tt].b;
-            const float2 r = fb_r<D>(X, make_float2(a4.x, a4.y), make_float2(a4.z, a4.w),
-                                     make_float2(b4.x, b4.y), make_float2(b4.z, b4.w));
+            const float2 r = fb_r<D>(X, T[tt]);
             const float2 e = __fadd2_rn(r, ng);
             const float2 p = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-            const float2 v = __fadd2_rn(r, make_float2(T[tt].c.x, T[tt].c.y));
+            const float2 v = __fadd2_rn(r, both(Nb[tt]));
             const float2 y = make_float2(tp_incl(v.x, a.x), tp_incl(v.y, a.y));
             acc = __ffma2_rn(p, y, acc);
             cntf = __fadd2_rn(cntf, y);
@@ -1287,9 +1298,7 @@ __device__ __forceinline__ void fb1_half(const Rec12 *T, const float2 (&X)[3], f
     } else {
 #pragma unroll
         for (int tt = 0; tt < 8; ++tt) {
-            const float4 a4 = T[tt].a, b4 = T[tt].b;
-            const float2 r = fb_r<D>(X, make_float2(a4.x, a4.y), make_float2(a4.z, a4.w),
-                                     make_float2(b4.x, b4.y), make_float2(b4.z, b4.w));
+            const float2 r = fb_r<D>(X, T[tt]);
             const float2 e = __fadd2_rn(r, ng);
             acc = __fadd2_rn(acc, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
         }
@@ -1301,22 +1310,24 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
     k_lse_fb(const float *__restrict__ xs, int64_t nqt, const float *__restrict__ Aq,
              const float *__restrict__ M0, const float4 *__restrict__ pball64,
              const float2 *__restrict__ pal64, const float *__restrict__ pbox1024,
-             const float *__restrict__ pa1024, const Rec12 *__restrict__ tdup, int64_t n,
+             const float *__restrict__ pa1024, const float4 *__restrict__ tquad,
+             const float *__restrict__ nb_s, int64_t n,
              const float4 *__restrict__ tball8, const float2 *__restrict__ tbe8,
              const float *__restrict__ tbox1024, const float *__restrict__ tb1024, int nstages,
              int k1, float2 *__restrict__ part1, unsigned long long *__restrict__ pairs,
              int *__restrict__ flags) {
     extern __shared__ __align__(128) unsigned char fb_smem[];
-    constexpr size_t oBall = (size_t)FB_STAGES * FB_TS * sizeof(Rec12);
+    constexpr size_t oNb = (size_t)FB_STAGES * FB_TS * sizeof(float4);
+    constexpr size_t oBall = oNb + (size_t)FB_STAGES * FB_TS * sizeof(float);
     constexpr size_t oBe = oBall + (size_t)FB_STAGES * FB_NBS * sizeof(float4);
-    Rec12 (*s_rec)[FB_TS] = reinterpret_cast<Rec12 (*)[FB_TS]>(fb_smem);
+    float4 (*s_rec)[FB_TS] = reinterpret_cast<float4 (*)[FB_TS]>(fb_smem);
+    float (*s_nb)[FB_TS] = reinterpret_cast<float (*)[FB_TS]>(fb_smem + oNb);
     float4 (*s_ball)[FB_NBS] = reinterpret_cast<float4 (*)[FB_NBS]>(fb_smem + oBall);
     float2 (*s_be)[FB_NBS] = reinterpret_cast<float2 (*)[FB_NBS]>(fb_smem + oBe);
     __shared__ __align__(8) uint64_t full[FB_STAGES], empty[FB_STAGES];
     __shared__ int s_list[BS_CHUNK], s_cnt, s_ab;
     __shared__ unsigned long long s_pairs;
     __shared__ double2 s_Sd[FB_WARPS][32][2];
-    constexpr unsigned kStage = FB_TS * sizeof(Rec12) + FB_NBS * (sizeof(float4) + sizeof(float2));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int kc = blockIdx.y;
     if (tid == 0) {
@@ -1336,8 +1347,9 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
     do {                                                                                             \
         const int sl_ = (it_) % FB_STAGES;                                                           \
         const int64_t j_ = (int64_t)s_list[it_] * FB_TS;                                             \
-        mbar_expect_tx(&full[sl_], kStage);                                                          \
-        bulk_g2s(s_rec[sl_], tdup + j_, FB_TS * sizeof(Rec12), &full[sl_]);                          \
+        mbar_expect_tx(&full[sl_], FB_STAGE);                                                        \
+        bulk_g2s(s_rec[sl_], tquad + j_, FB_TS * sizeof(float4), &full[sl_]);                        \
+        bulk_g2s(s_nb[sl_], nb_s + j_, FB_TS * sizeof(float), &full[sl_]);                           \
         bulk_g2s(s_ball[sl_], tball8 + j_ / 8, FB_NBS * sizeof(float4), &full[sl_]);                 \
         bulk_g2s(s_be[sl_], tbe8 + j_ / 8, FB_NBS * sizeof(float2), &full[sl_]);                     \
     } while (0)
@@ -1411,23 +1423,22 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                     const unsigned jreal = (unsigned)max(0, min(8, sreal - 8 * nb));
                     if (l0 && !x0) icnt += rvs[0] * jreal;
                     if (l1 && !x1) icnt += rvs[1] * jreal;
-                    const Rec12 *T = &s_rec[slot][8 * nb];
+                    const float4 *T = &s_rec[slot][8 * nb];
+                    const float *Nb = &s_nb[slot][8 * nb];
                     if (l0 != l1) {
                         // one half live: its chain alone (eight targets in flight)
-                        if (l0) fb1_half<D>(T, X[0], ng[0], nAS[0], x0, acc[0], cntf);
-                        else fb1_half<D>(T, X[1], ng[1], nAS[1], x1, acc[1], cntf);
+                        if (l0) fb1_half<D>(T, Nb, X[0], ng[0], nAS[0], x0, acc[0], cntf);
+                        else fb1_half<D>(T, Nb, X[1], ng[1], nAS[1], x1, acc[1], cntf);
                         continue;
                     }
                     if (l0 && l1 && !x0 && !x1) {
                         // both halves inside: no test, both chains interleaved
 #pragma unroll
                         for (int tt = 0; tt < 8; ++tt) {
-                            const float4 a4 = T[tt].a, b4 = T[tt].b;
-                            const float2 w0 = make_float2(a4.x, a4.y), w1 = make_float2(a4.z, a4.w);
-                            const float2 w2 = make_float2(b4.x, b4.y), c = make_float2(b4.z, b4.w);
+                            const float4 w = T[tt];
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                const float2 r = fb_r<D>(X[h], w0, w1, w2, c);
+                                const float2 r = fb_r<D>(X[h], w);
                                 const float2 e = __fadd2_rn(r, ng[h]);
                                 acc[h] = __fadd2_rn(acc[h], make_float2(ex2_approx(e.x), ex2_approx(e.y)));
                             }
@@ -1448,13 +1459,11 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                         }
 #pragma unroll
                         for (int tt = 0; tt < 8; ++tt) {
-                            const float4 a4 = T[tt].a, b4 = T[tt].b;
-                            const float2 w0 = make_float2(a4.x, a4.y), w1 = make_float2(a4.z, a4.w);
-                            const float2 w2 = make_float2(b4.x, b4.y), c = make_float2(b4.z, b4.w);
-                            const float2 nbv = make_float2(T[tt].c.x, T[tt].c.y);
+                            const float4 w = T[tt];
+                            const float2 nbv = both(Nb[tt]);
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                const float2 r = fb_r<D>(X[h], w0, w1, w2, c);
+                                const float2 r = fb_r<D>(X[h], w);
                                 const float2 e = __fadd2_rn(r, ng[h]);
                                 const float2 p = make_float2(ex2_approx(e.x), ex2_approx(e.y));
                                 const float2 v = __fadd2_rn(r, nbv);
@@ -1481,14 +1490,13 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                         for (unsigned gm = gh; gm; gm &= gm - 1) {
                             const int b = __ffs(gm) - 1, nb = grp * FB_GROUP + b;
                             const bool bnd = (bh >> b) & 1u;
-                            const Rec12 *T = &s_rec[slot][8 * nb];
+                            const float4 *T = &s_rec[slot][8 * nb];
+                            const float *Nb = &s_nb[slot][8 * nb];
                             for (int tt = 0; tt < 8; ++tt) {
-                                const float4 a4 = T[tt].a, b4 = T[tt].b;
-                                const float2 r = fb_r<D>(X[h], make_float2(a4.x, a4.y), make_float2(a4.z, a4.w),
-                                                         make_float2(b4.x, b4.y), make_float2(b4.z, b4.w));
+                                const float2 r = fb_r<D>(X[h], T[tt]);
                                 float2 y = make_float2(1.f, 1.f);
                                 if (bnd) {
-                                    const float2 v = __fadd2_rn(r, make_float2(T[tt].c.x, T[tt].c.y));
+                                    const float2 v = __fadd2_rn(r, both(Nb[tt]));
                                     y = make_float2(tp_incl(v.x, nAS[h].x), tp_incl(v.y, nAS[h].y));
                                 }
                                 mx = fmaxf(mx, y.x > 0.f ? r.x : -INFINITY);
@@ -1502,14 +1510,13 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                         for (unsigned gm = gh; gm; gm &= gm - 1) {
                             const int b = __ffs(gm) - 1, nb = grp * FB_GROUP + b;
                             const bool bnd = (bh >> b) & 1u;
-                            const Rec12 *T = &s_rec[slot][8 * nb];
+                            const float4 *T = &s_rec[slot][8 * nb];
+                            const float *Nb = &s_nb[slot][8 * nb];
                             for (int tt = 0; tt < 8; ++tt) {
-                                const float4 a4 = T[tt].a, b4 = T[tt].b;
-                                const float2 r = fb_r<D>(X[h], make_float2(a4.x, a4.y), make_float2(a4.z, a4.w),
-                                                         make_float2(b4.x, b4.y), make_float2(b4.z, b4.w));
+                                const float2 r = fb_r<D>(X[h], T[tt]);
                                 float2 y = make_float2(1.f, 1.f);
                                 if (bnd) {
-                                    const float2 v = __fadd2_rn(r, make_float2(T[tt].c.x, T[tt].c.y));
+                                    const float2 v = __fadd2_rn(r, both(Nb[tt]));
                                     y = make_float2(tp_incl(v.x, nAS[h].x), tp_incl(v.y, nAS[h].y));
                                 }
                                 const float2 e = __fadd2_rn(r, nm);
@@ -1569,20 +1576,16 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
     }
 }
 
-// sorted point records of the FP32 block-skip pass 2: (x0,x0,x1,x1) (x2,x2,u,u),
+// sorted point records of the FP32 block-skip pass 2: (x0,x1,x2,u),
 // and the points' -A_q 2^64 (the tests' operand, formed once per evaluation)
-__global__ void k_pdup_s(const float *__restrict__ xs, const float *__restrict__ u_s,
-                         const float *__restrict__ Aq, int64_t nqt, int d, Rec8 *__restrict__ pdup,
+__global__ void k_pquad_s(const float *__restrict__ xs, const float *__restrict__ u_s,
+                         const float *__restrict__ Aq, int64_t nqt, int d, float4 *__restrict__ pquad,
                          float *__restrict__ nAq) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= nqt) return;
     float x[3] = {0.f, 0.f, 0.f};
     for (int t = 0; t < d; ++t) x[t] = xs[t * nqt + q];
-    const float u = u_s[q];
-    Rec8 r;
-    r.a = make_float4(x[0], x[0], x[1], x[1]);
-    r.b = make_float4(x[2], x[2], u, u);
-    pdup[q] = r;
+    pquad[q] = make_float4(x[0], x[1], x[2], u_s[q]);
     nAq[q] = Aq[q] * -TP_S;   // the operand of tp_incl, bitwise as pass 1 forms it
 }
 
@@ -1594,17 +1597,14 @@ __global__ void k_pdup_s(const float *__restrict__ xs, const float *__restrict__
 // the half's target pair, tested (boundary) or not (inside); Ab holds the
 // points' -A_q 2^64
 template <int D>
-__device__ __forceinline__ void fb2_half(const Rec8 *T, const float *Ab, const float2 (&W)[3], float2 C,
+__device__ __forceinline__ void fb2_half(const float4 *T, const float *Ab, const float2 (&W)[3], float2 C,
                                          float2 NB, bool bnd, float2 &acc) {
     if (bnd) {
 #pragma unroll
         for (int tt = 0; tt < 8; ++tt) {
-            const float4 a4 = T[tt].a, b4 = T[tt].b;
-            float2 r = C;
-            if (D == 3) r = __ffma2_rn(make_float2(b4.x, b4.y), W[2], r);
-            r = __ffma2_rn(make_float2(a4.z, a4.w), W[1], r);
-            r = __ffma2_rn(make_float2(a4.x, a4.y), W[0], r);
-            const float2 e = __fadd2_rn(r, make_float2(b4.z, b4.w));
+            const float4 p4 = T[tt];
+            const float2 r = fb_r2<D>(W, C, p4);
+            const float2 e = __fadd2_rn(r, both(p4.w));
             const float2 p = make_float2(ex2_approx(e.x), ex2_approx(e.y));
             const float2 v = __fadd2_rn(r, NB);
             const float a = Ab[tt];
@@ -1613,12 +1613,9 @@ __device__ __forceinline__ void fb2_half(const Rec8 *T, const float *Ab, const f
     } else {
 #pragma unroll
         for (int tt = 0; tt < 8; ++tt) {
-            const float4 a4 = T[tt].a, b4 = T[tt].b;
-            float2 r = C;
-            if (D == 3) r = __ffma2_rn(make_float2(b4.x, b4.y), W[2], r);
-            r = __ffma2_rn(make_float2(a4.z, a4.w), W[1], r);
-            r = __ffma2_rn(make_float2(a4.x, a4.y), W[0], r);
-            const float2 e = __fadd2_rn(r, make_float2(b4.z, b4.w));
+            const float4 p4 = T[tt];
+            const float2 r = fb_r2<D>(W, C, p4);
+            const float2 e = __fadd2_rn(r, both(p4.w));
             acc = __fadd2_rn(acc, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
         }
     }
@@ -1626,24 +1623,24 @@ __device__ __forceinline__ void fb2_half(const Rec8 *T, const float *Ab, const f
 
 template <int D>
 __global__ void __launch_bounds__(FB_THREADS, 2)
-    k_grad_fb(const Rec12 *__restrict__ tdup, const float4 *__restrict__ tball64,
+    k_grad_fb(const float4 *__restrict__ tquad, const float *__restrict__ nb_s,
+              const float4 *__restrict__ tball64,
               const float2 *__restrict__ tbe64, const float *__restrict__ tbox1024,
-              const float *__restrict__ tb1024, const Rec8 *__restrict__ pdup,
+              const float *__restrict__ tb1024, const float4 *__restrict__ pquad,
               const float *__restrict__ nAq, const float4 *__restrict__ pball8,
               const float2 *__restrict__ pal8, const float *__restrict__ pbox1024,
               const float *__restrict__ pa1024, int nstages, int k2, double *__restrict__ part2,
               int *__restrict__ flags) {
     extern __shared__ __align__(128) unsigned char fb_smem[];
-    constexpr size_t oA = (size_t)FB_STAGES * FB_TS * sizeof(Rec8);
+    constexpr size_t oA = (size_t)FB_STAGES * FB_TS * sizeof(float4);
     constexpr size_t oBall = oA + (size_t)FB_STAGES * FB_TS * sizeof(float);
     constexpr size_t oAl = oBall + (size_t)FB_STAGES * FB_NBS * sizeof(float4);
-    Rec8 (*s_rec)[FB_TS] = reinterpret_cast<Rec8 (*)[FB_TS]>(fb_smem);
+    float4 (*s_rec)[FB_TS] = reinterpret_cast<float4 (*)[FB_TS]>(fb_smem);
     float (*s_A)[FB_TS] = reinterpret_cast<float (*)[FB_TS]>(fb_smem + oA);
     float4 (*s_ball)[FB_NBS] = reinterpret_cast<float4 (*)[FB_NBS]>(fb_smem + oBall);
     float2 (*s_al)[FB_NBS] = reinterpret_cast<float2 (*)[FB_NBS]>(fb_smem + oAl);
     __shared__ __align__(8) uint64_t full[FB_STAGES], empty[FB_STAGES];
     __shared__ int s_list[BS_CHUNK], s_cnt;
-    constexpr unsigned kStage = FB_TS * (sizeof(Rec8) + sizeof(float)) + FB_NBS * (sizeof(float4) + sizeof(float2));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int kc = blockIdx.y;
     if (tid == 0) {
@@ -1661,8 +1658,8 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
     do {                                                                                             \
         const int sl_ = (it_) % FB_STAGES;                                                           \
         const int64_t q_ = (int64_t)s_list[it_] * FB_TS;                                             \
-        mbar_expect_tx(&full[sl_], kStage);                                                          \
-        bulk_g2s(s_rec[sl_], pdup + q_, FB_TS * sizeof(Rec8), &full[sl_]);                           \
+        mbar_expect_tx(&full[sl_], FB_STAGE);                                                        \
+        bulk_g2s(s_rec[sl_], pquad + q_, FB_TS * sizeof(float4), &full[sl_]);                        \
         bulk_g2s(s_A[sl_], nAq + q_, FB_TS * sizeof(float), &full[sl_]);                              \
         bulk_g2s(s_ball[sl_], pball8 + q_ / 8, FB_NBS * sizeof(float4), &full[sl_]);                 \
         bulk_g2s(s_al[sl_], pal8 + q_ / 8, FB_NBS * sizeof(float2), &full[sl_]);                     \
@@ -1678,12 +1675,12 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int64_t ja = j0 + 64 * h + 2 * lane;
-        const Rec12 ra = tdup[ja], rb = tdup[ja + 1];
-        W[h][0] = make_float2(ra.a.x, rb.a.x);
-        W[h][1] = make_float2(ra.a.z, rb.a.z);
-        W[h][2] = make_float2(ra.b.x, rb.b.x);
-        C[h] = make_float2(ra.b.z, rb.b.z);
-        NB[h] = make_float2(ra.c.x, rb.c.x);
+        const float4 ra = tquad[ja], rb = tquad[ja + 1];
+        W[h][0] = make_float2(ra.x, rb.x);
+        W[h][1] = make_float2(ra.y, rb.y);
+        W[h][2] = make_float2(ra.z, rb.z);
+        C[h] = make_float2(ra.w, rb.w);
+        NB[h] = make_float2(nb_s[ja], nb_s[ja + 1]);
         acc64[h] = make_double2(0.0, 0.0);
         wball[h] = tball64[(j0 + 64 * h) / 64];
         wbe[h] = tbe64[(j0 + 64 * h) / 64];
@@ -1716,7 +1713,7 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                 const int b = __ffs(live) - 1, nb = 32 * i + b;
                 const bool l0 = (lv0 >> b) & 1u, l1 = (lv1 >> b) & 1u;
                 const bool x0 = (bd0 >> b) & 1u, x1 = (bd1 >> b) & 1u;
-                const Rec8 *T = &s_rec[slot][8 * nb];
+                const float4 *T = &s_rec[slot][8 * nb];
                 const float *Ab = &s_A[slot][8 * nb];
                 if (l0 != l1) {
                     // one half live: its chain alone (eight points in flight)
@@ -1728,16 +1725,11 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                     // both halves inside: no test, both chains interleaved
 #pragma unroll
                     for (int tt = 0; tt < 8; ++tt) {
-                        const float4 a4 = T[tt].a, b4 = T[tt].b;
-                        const float2 x0v = make_float2(a4.x, a4.y), x1v = make_float2(a4.z, a4.w);
-                        const float2 x2v = make_float2(b4.x, b4.y), u = make_float2(b4.z, b4.w);
+                        const float4 p4 = T[tt];
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            float2 r = C[h];
-                            if (D == 3) r = __ffma2_rn(x2v, W[h][2], r);
-                            r = __ffma2_rn(x1v, W[h][1], r);
-                            r = __ffma2_rn(x0v, W[h][0], r);
-                            const float2 e = __fadd2_rn(r, u);
+                            const float2 r = fb_r2<D>(W[h], C[h], p4);
+                            const float2 e = __fadd2_rn(r, both(p4.w));
                             acc[h] = __fadd2_rn(acc[h], make_float2(ex2_approx(e.x), ex2_approx(e.y)));
                         }
                     }
@@ -1755,17 +1747,12 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                     }
 #pragma unroll
                     for (int tt = 0; tt < 8; ++tt) {
-                        const float4 a4 = T[tt].a, b4 = T[tt].b;
-                        const float2 x0v = make_float2(a4.x, a4.y), x1v = make_float2(a4.z, a4.w);
-                        const float2 x2v = make_float2(b4.x, b4.y), u = make_float2(b4.z, b4.w);
+                        const float4 p4 = T[tt];
                         const float nA = Ab[tt];
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            float2 r = C[h];
-                            if (D == 3) r = __ffma2_rn(x2v, W[h][2], r);
-                            r = __ffma2_rn(x1v, W[h][1], r);
-                            r = __ffma2_rn(x0v, W[h][0], r);
-                            const float2 e = __fadd2_rn(r, u);
+                            const float2 r = fb_r2<D>(W[h], C[h], p4);
+                            const float2 e = __fadd2_rn(r, both(p4.w));
                             const float2 p = make_float2(ex2_approx(e.x), ex2_approx(e.y));
                             const float2 v = __fadd2_rn(r, NBc[h]);
                             const float2 y = make_float2(tp_incl(v.x, nA), tp_incl(v.y, nA));
@@ -1790,19 +1777,16 @@ __global__ void __launch_bounds__(FB_THREADS, 2)
                 const unsigned bd1 = __ballot_sync(0xffffffffu, ((cls1 >> (2 * i)) & 3u) == 2u);
                 for (unsigned live = lv0 | lv1; live; live &= live - 1) {
                     const int b = __ffs(live) - 1, nb = 32 * i + b;
-                    const Rec8 *T = &s_rec[slot][8 * nb];
+                    const float4 *T = &s_rec[slot][8 * nb];
                     const float *Ab = &s_A[slot][8 * nb];
                     for (int tt = 0; tt < 8; ++tt) {
-                        const float4 a4 = T[tt].a, b4 = T[tt].b;
+                        const float4 p4 = T[tt];
                         const float nA = Ab[tt];
                         for (int h = 0; h < 2; ++h) {
                             if (!(((h ? lv1 : lv0) >> b) & 1u)) continue;
                             const bool bnd = ((h ? bd1 : bd0) >> b) & 1u;
-                            float2 r = C[h];
-                            if (D == 3) r = __ffma2_rn(make_float2(b4.x, b4.y), W[h][2], r);
-                            r = __ffma2_rn(make_float2(a4.z, a4.w), W[h][1], r);
-                            r = __ffma2_rn(make_float2(a4.x, a4.y), W[h][0], r);
-                            const float2 e = __fadd2_rn(r, make_float2(b4.z, b4.w));
+                            const float2 r = fb_r2<D>(W[h], C[h], p4);
+                            const float2 e = __fadd2_rn(r, both(p4.w));
                             float2 y = make_float2(1.f, 1.f);
                             if (bnd) {
                                 const float2 v = __fadd2_rn(r, NB[h]);
@@ -2214,7 +2198,9 @@ static cudaError_t grid_build(rsot_problem *p) {
     ALLOC(g->part2b, (int64_t)g->ttiles * g->k2b * TT);
     ALLOC(g->off1b, g->ptiles + 1);
     ALLOC(g->off2b, g->ttiles + 1);
-    ALLOC(g->pdup_s, g->nqt);
+    ALLOC(g->tquad_s, g->nt);
+    ALLOC(g->nb_s, g->nt);
+    ALLOC(g->pquad_s, g->nqt);
     ALLOC(g->nAq_s, g->nqt);
 #undef ALLOC
     k_gather_points<<<(unsigned)((g->nqt + 255) / 256), 256, 0, st>>>(
@@ -2238,9 +2224,9 @@ static cudaError_t grid_build(rsot_problem *p) {
             return e;
         const void *fb1 = d == 3 ? (const void *)k_lse_fb<3> : (const void *)k_lse_fb<2>;
         const void *fb2 = d == 3 ? (const void *)k_grad_fb<3> : (const void *)k_grad_fb<2>;
-        if ((e = cudaFuncSetAttribute(fb1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FB_SMEM1)))
+        if ((e = cudaFuncSetAttribute(fb1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FB_SMEM)))
             return e;
-        if ((e = cudaFuncSetAttribute(fb2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FB_SMEM2)))
+        if ((e = cudaFuncSetAttribute(fb2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FB_SMEM)))
             return e;
     }
     k_block_balls<<<(unsigned)((g->nqt / 64 + 127) / 128), 128, 0, st>>>(g->x64, p->nq, d, 64, g->nqt / 64, g->pball64);
@@ -2276,27 +2262,31 @@ static cudaError_t trunc_mixed(rsot_problem *p, const double *psi, double eps, d
                                                     g->ptiles);
     k_ranges8<<<nb_of(g->nt / 8), 256, 0, st>>>(p->beta, g->perm_t, p->n, g->nt / 8, g->tbe8);
     k_ranges_merge<<<nb_of(g->nt / 64), 256, 0, st>>>(g->tbe8, g->nt / 8, 8, g->tbe64, nullptr, g->nt / 64);
-    k_ranges_merge<<<nb_of(g->ttiles), 256, 0, st>>>(g->tbe64, g->nt / 64, TT / 64, nullptr, g->ttmax,
-                                                    g->ttiles);
-    k_ranges_merge<<<nb_of(g->nqt / TC_ROWS), 256, 0, st>>>(g->pal64, g->nqt / 64, TC_ROWS / 64, nullptr,
-                                                           g->pa512, g->nqt / TC_ROWS);
-    k_ranges_merge<<<nb_of(g->nt / TC_ROWS), 256, 0, st>>>(g->tbe64, g->nt / 64, TC_ROWS / 64, nullptr,
-                                                          g->tb512, g->nt / TC_ROWS);
     k_ranges_merge<<<nb_of(g->nt / TC_TS), 256, 0, st>>>(g->tbe64, g->nt / 64, TC_TS / 64, nullptr,
                                                         g->tb1024, g->nt / TC_TS);
-    cudaMemsetAsync(g->bits_tp, 0, (size_t)g->ttiles * g->pw * 4, st);
-    cudaMemsetAsync(g->cnt2, 0, (size_t)g->ttiles * 4, st);
-    k_tile_pairs<<<g->ptiles, 256, 0, st>>>(g->pbox, g->tbox, g->ptiles, g->ttiles, g->tw, g->pw,
-                                            g->ptmax, g->ttmax, g->bits_pt, g->bits_tp, g->cnt1, g->cnt2);
-    k_item_offsets<<<1, 64, 0, st>>>(g->cnt1, g->ptiles, g->ch1, g->cnt2, g->ttiles, g->ch2, g->off1,
-                                     g->off2, g->counters);
     const int nbp = (int)((g->nt + 255) / 256);
     // tensor-core passes (the automatic choice of the dense path), FP32 passes as
     // their fallback when an operand leaves the f16 range (gate)
     const bool tc = use_tensor_pairs(p);
+    if (tc) {
+        // ranges of the tensor-core row tiles; tile pairs and items of the queue kernels
+        k_ranges_merge<<<nb_of(g->ttiles), 256, 0, st>>>(g->tbe64, g->nt / 64, TT / 64, nullptr, g->ttmax,
+                                                        g->ttiles);
+        k_ranges_merge<<<nb_of(g->nqt / TC_ROWS), 256, 0, st>>>(g->pal64, g->nqt / 64, TC_ROWS / 64, nullptr,
+                                                               g->pa512, g->nqt / TC_ROWS);
+        k_ranges_merge<<<nb_of(g->nt / TC_ROWS), 256, 0, st>>>(g->tbe64, g->nt / 64, TC_ROWS / 64, nullptr,
+                                                              g->tb512, g->nt / TC_ROWS);
+        cudaMemsetAsync(g->bits_tp, 0, (size_t)g->ttiles * g->pw * 4, st);
+        cudaMemsetAsync(g->cnt2, 0, (size_t)g->ttiles * 4, st);
+        k_tile_pairs<<<g->ptiles, 256, 0, st>>>(g->pbox, g->tbox, g->ptiles, g->ttiles, g->tw, g->pw,
+                                                g->ptmax, g->ttmax, g->bits_pt, g->bits_tp, g->cnt1,
+                                                g->cnt2);
+        k_item_offsets<<<1, 64, 0, st>>>(g->cnt1, g->ptiles, g->ch1, g->cnt2, g->ttiles, g->ch2, g->off1,
+                                         g->off2, g->counters);
+    }
     int *gate = tc ? &p->res_dev->gate : nullptr;
-    k_prep_trunc<<<nbp, 256, 0, st>>>(psi, g->perm_t, g->y64, g->lnu, p->n, g->nt, D, eps, g->tdup,
-                                      p->psinu, g->nu, p->flags, tc ? g->trec_s : nullptr, g->b_s,
+    k_prep_trunc<<<nbp, 256, 0, st>>>(psi, g->perm_t, g->y64, g->lnu, p->n, g->nt, D, eps, g->tquad_s,
+                                      g->nb_s, tc ? g->tdup : nullptr, p->psinu, g->nu, p->flags, tc ? g->trec_s : nullptr, g->b_s,
                                       1.0 / (double)p->tc_P, gate, p->beta);
     trace_end(p);
     unsigned long long *pairs = reinterpret_cast<unsigned long long *>(&p->res_dev->pairs);
@@ -2305,8 +2295,8 @@ static cudaError_t trunc_mixed(rsot_problem *p, const double *psi, double eps, d
     if (!tc) {
         // FP32 pair arithmetic on the block-skip pipeline
         trace_begin(p, "lse_trunc_fb");
-        k_lse_fb<D><<<dim3((unsigned)(g->nqt / FB_ROWS), (unsigned)g->k1b), FB_THREADS, FB_SMEM1, st>>>(
-            g->xs, g->nqt, g->Aq, g->m0_s, g->pball64, g->pal64, g->pbox, g->ptmax, g->tdup, p->n,
+        k_lse_fb<D><<<dim3((unsigned)(g->nqt / FB_ROWS), (unsigned)g->k1b), FB_THREADS, FB_SMEM, st>>>(
+            g->xs, g->nqt, g->Aq, g->m0_s, g->pball64, g->pal64, g->pbox, g->ptmax, g->tquad_s, g->nb_s, p->n,
             g->tball8, g->tbe8, g->tbox1024, g->tb1024, (int)(g->nt / FB_TS), g->k1b, g->part1b, pairs,
             p->flags);
         trace_end(p);
@@ -2314,11 +2304,11 @@ static cudaError_t trunc_mixed(rsot_problem *p, const double *psi, double eps, d
         k_combine_trunc<<<g->nblk_comb, 256, 0, st>>>(g->part1b, g->off1b, p->nq, g->nqt, g->xs, g->x64,
                                                       g->mass, g->lm2, g->Aq, psi, eps, D, g->ppair,
                                                       g->lse_s, g->blockJ, p->res_dev, g->u_s, nullptr, 0);
-        k_pdup_s<<<nb_of(g->nqt), 256, 0, st>>>(g->xs, g->u_s, g->Aq, g->nqt, D, g->pdup_s, g->nAq_s);
+        k_pquad_s<<<nb_of(g->nqt), 256, 0, st>>>(g->xs, g->u_s, g->Aq, g->nqt, D, g->pquad_s, g->nAq_s);
         trace_end(p);
         trace_begin(p, "grad_trunc_fb");
-        k_grad_fb<D><<<dim3((unsigned)(g->nt / FB_ROWS), (unsigned)g->k2b), FB_THREADS, FB_SMEM2, st>>>(
-            g->tdup, g->tball64, g->tbe64, g->tbox1024, g->tb1024, g->pdup_s, g->nAq_s, g->pball8, g->pal8,
+        k_grad_fb<D><<<dim3((unsigned)(g->nt / FB_ROWS), (unsigned)g->k2b), FB_THREADS, FB_SMEM, st>>>(
+            g->tquad_s, g->nb_s, g->tball64, g->tbe64, g->tbox1024, g->tb1024, g->pquad_s, g->nAq_s, g->pball8, g->pal8,
             g->pbox, g->ptmax, (int)(g->nqt / FB_TS), g->k2b, g->part2b, p->flags);
         trace_end(p);
         trace_begin(p, "finalize_trunc");
@@ -2416,7 +2406,7 @@ void trunc_free(rsot_problem *p) {
                     g->pball64, g->pball8, g->tball64, g->tball8, g->prec_s, g->trec_s, g->b_s,
                     g->u_s, g->pal8, g->pal64, g->ptmax, g->tbe8, g->tbe64, g->ttmax, g->m0_s,
                     g->pbox512, g->tbox512, g->tbox1024, g->pa512, g->tb512, g->tb1024, g->part1b,
-                    g->part2b, g->off1b, g->off2b, g->pdup_s, g->nAq_s};
+                    g->part2b, g->off1b, g->off2b, g->pquad_s, g->nAq_s, g->tquad_s, g->nb_s};
     for (void *q : ptrs) cudaFree(q);
     delete g;
     p->grid = nullptr;
