@@ -227,6 +227,7 @@ rsot_status rsot_create(int d, int64_t nq, const double *x, const double *mass, 
     for (int k = 0; k < d; ++k) p->origin[k] = 0.5 * (lo[k] + hi[k]);
     p->diam2 = 0.0;
     for (int k = 0; k < d; ++k) p->diam2 += (hi[k] - lo[k]) * (hi[k] - lo[k]);
+    for (int k = 0; k < d; ++k) p->half_ext = std::max(p->half_ext, 0.5 * (hi[k] - lo[k]));
     p->nq_pad = round_up(nq, 1024);
 
     // translated coordinates (cost is translation invariant)

@@ -40,6 +40,7 @@
 #include <algorithm>
 
 #include "rsot_internal.cuh"
+#include "rsot_inner.cuh"
 
 namespace rsot {
 
@@ -54,21 +55,22 @@ constexpr int D_TS = 128;                 // records per shared-memory tile
 constexpr int D_SUB = 8;                  // targets per max sub-tile (pass 1)
 constexpr float kExcl = -1.0e30f;
 
-// 64-byte record, every value twice: (v0h, v0h, v0t, v0t), (v1h, ...), (v2h, ...),
-// (sh, sh, st, st) -- v = w (targets) or x' (points), s = c (targets) or u (points)
+// 32-byte record (v0h, v0t, v1h, v1t), (v2h, v2t, sh, st) -- v = w (targets) or
+// x' (points), s = c (targets) or u (points)
 struct __align__(16) DRec {
-    float4 a, b, c, d;
+    float4 a, b;
 };
 
 
 typedef float2 f2;
-__device__ __forceinline__ f2 add2(f2 a, f2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
+#ifndef DFV
+#define DFV 0
+#endif
+__device__ __forceinline__ f2 add2(f2 a, f2 b) { if (DFV & 1) return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)); return __fadd2_rn(a, b); }
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) { if (DFV & 2) return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)); return __fmul2_rn(a, b); }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { if (DFV & 4) return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y)); return __ffma2_rn(a, b, c); }
 // a - b rounded once: the product b * -1 is exact
-__device__ __forceinline__ f2 sub2(f2 a, f2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ f2 lo2(float4 v) { return make_float2(v.x, v.y); }   // heads
-__device__ __forceinline__ f2 hi2(float4 v) { return make_float2(v.z, v.w); }   // tails
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) { if (DFV & 8) return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y)); return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
 // s + e = a + b exactly in each lane (Knuth's TwoSum)
 __device__ __forceinline__ void two_sum2(f2 a, f2 b, f2 &s, f2 &e) {
@@ -111,9 +113,9 @@ template <int D>
 __device__ __forceinline__ void df_exponent2(const Op2 *R, const DRec &B, f2 sh, f2 st, f2 &rh,
                                              f2 &rt) {
     f2 s = sh, lo = st;
-    df_term2(R[0], lo2(B.a), hi2(B.a), s, lo);
-    df_term2(R[1], lo2(B.b), hi2(B.b), s, lo);
-    if (D == 3) df_term2(R[2], lo2(B.c), hi2(B.c), s, lo);
+    df_term2(R[0], both(B.a.x), both(B.a.y), s, lo);
+    df_term2(R[1], both(B.a.z), both(B.a.w), s, lo);
+    if (D == 3) df_term2(R[2], both(B.b.x), both(B.b.y), s, lo);
     rh = add2(s, lo);                // |lo| << |s|: Fast2Sum renormalisation
     rt = sub2(lo, sub2(rh, s));
 }
@@ -125,23 +127,22 @@ __device__ __forceinline__ void split_f(double v, float &h, float &t) {
 
 __device__ __forceinline__ DRec make_drec(const float *v /* 8: h,t pairs */) {
     DRec r;
-    r.a = make_float4(v[0], v[0], v[1], v[1]);
-    r.b = make_float4(v[2], v[2], v[3], v[3]);
-    r.c = make_float4(v[4], v[4], v[5], v[5]);
-    r.d = make_float4(v[6], v[6], v[7], v[7]);
+    r.a = make_float4(v[0], v[1], v[2], v[3]);
+    r.b = make_float4(v[4], v[5], v[6], v[7]);
     return r;
 }
 
 // the two lanes' operands from two records (lane 0 from r0, lane 1 from r1)
 __device__ __forceinline__ void load_ops(const DRec &r0, const DRec &r1, Op2 *R, f2 &sh, f2 &st) {
-    const float4 *a0 = &r0.a, *a1 = &r1.a;
+    const float v0[6] = {r0.a.x, r0.a.y, r0.a.z, r0.a.w, r0.b.x, r0.b.y};
+    const float v1[6] = {r1.a.x, r1.a.y, r1.a.z, r1.a.w, r1.b.x, r1.b.y};
     for (int t = 0; t < 3; ++t) {
-        R[t].h = make_float2(a0[t].x, a1[t].x);
-        R[t].t = make_float2(a0[t].z, a1[t].z);
-        R[t].nh = make_float2(-a0[t].x, -a1[t].x);
+        R[t].h = make_float2(v0[2 * t], v1[2 * t]);
+        R[t].t = make_float2(v0[2 * t + 1], v1[2 * t + 1]);
+        R[t].nh = make_float2(-v0[2 * t], -v1[2 * t]);
     }
-    sh = make_float2(r0.d.x, r1.d.x);
-    st = make_float2(r0.d.z, r1.d.z);
+    sh = make_float2(r0.b.z, r1.b.z);
+    st = make_float2(r0.b.w, r1.b.w);
 }
 
 // FP32 test c(x, y) < alpha + beta outside a margin that bounds the FP32
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(D_THREADS, TRUNC ? 5 : 1)
     #pragma unroll
                 for (int i = 0; i < D_SUB; ++i) {
                     const DRec &B = sm[u0 + i];
-                    df_exponent2<D>(X, B, lo2(B.d), hi2(B.d), rh[i], rt[i]);
+                    df_exponent2<D>(X, B, both(B.b.z), both(B.b.w), rh[i], rt[i]);
                     mx0 = fmaxf(mx0, rh[i].x);
                     mx1 = fmaxf(mx1, rh[i].y);
                 }
@@ -428,7 +429,7 @@ __global__ void __launch_bounds__(D_THREADS, TRUNC ? 5 : 1)
                 for (int i = 0; i < D_SUB; ++i) {
                     const int64_t j = t0 + u0 + i;
                     const DRec &B = sm[u0 + i];
-                    df_exponent2<D>(X, B, lo2(B.d), hi2(B.d), rh[i], rt[i]);
+                    df_exponent2<D>(X, B, both(B.b.z), both(B.b.w), rh[i], rt[i]);
                     for (int l = 0; l < 2; ++l) {
                         bool k = j < n && q[l] < nq;
                         if (k && test) {
@@ -506,7 +507,8 @@ __global__ void __launch_bounds__(D_THREADS, TRUNC ? 5 : 1)
                 }
             }
         }
-        prec[qq].d = make_float4(uh, uh, ut, ut);
+        prec[qq].b.z = uh;
+        prec[qq].b.w = ut;
     }
     if (TRUNC && npair) atomicAdd(&s_cnt, npair);
     if (empties) atomicAdd(&s_empty, (unsigned long long)empties);
@@ -564,10 +566,10 @@ __global__ void __launch_bounds__(D_THREADS)
                 f2 rh, rt;
                 df_exponent2<D>(W, B, Ch, Ct, rh, rt);
                 f2 th, te;
-                two_sum2(rh, lo2(B.d), th, te);
+                two_sum2(rh, both(B.b.z), th, te);
                 const f2 e = make_float2(ex2_approx(th.x), ex2_approx(th.y));
                 kahan2(s, comp, e);
-                cs = fma2(e, add2(add2(te, rt), hi2(B.d)), cs);
+                cs = fma2(e, add2(add2(te, rt), both(B.b.w)), cs);
             }
             acc0 += ((double)s.x - (double)comp.x) + kLn2 * (double)cs.x;
             acc1 += ((double)s.y - (double)comp.y) + kLn2 * (double)cs.y;
@@ -609,7 +611,7 @@ __global__ void __launch_bounds__(D_THREADS)
                     f2 rh, rt;
                     df_exponent2<D>(W, B, Ch, Ct, rh, rt);
                     f2 th, te;
-                    two_sum2(rh, lo2(B.d), th, te);
+                    two_sum2(rh, both(B.b.z), th, te);
                     f2 e = make_float2(ex2_approx(th.x), ex2_approx(th.y));
                     if (test) {
                         const float Ai = sA[i];
@@ -627,7 +629,7 @@ __global__ void __launch_bounds__(D_THREADS)
                         }
                     }
                     kahan2(s, comp, e);
-                    cs = fma2(e, add2(add2(te, rt), hi2(B.d)), cs);
+                    cs = fma2(e, add2(add2(te, rt), both(B.b.w)), cs);
                 }
             }
             acc0 += ((double)s.x - (double)comp.x) + kLn2 * (double)cs.x;

@@ -128,6 +128,57 @@ __device__ __forceinline__ int2 fx_coord(double x, double c0, double c1, int s) 
 }  // namespace
 
 // ----------------------------------------------------------------------------
+// Order of the target rows of pass 2: by cells of a 2^b grid in Morton order
+// (counting sort, once per problem), so that a warp's targets are near each
+// other and most of a far point's pairs are skipped by whole warps: at eps 1e-3
+// (98,304 x 16,384) pass 2 takes 1.6 ms, 3.7 in the caller's order.  The order inside
+// a cell is whatever the atomics give; a row's sum does not depend on it.
+// ----------------------------------------------------------------------------
+constexpr int SORT_CELLS = 4096;
+
+__global__ void k_cell_count(const double *__restrict__ y64, int64_t n, int d, double half,
+                             int *__restrict__ cell, int *__restrict__ count) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const int bits = d == 3 ? 4 : 6;
+    int id = 0;
+    for (int t = 0; t < d; ++t) {
+        const double u = half > 0.0 ? (y64[j * d + t] / half + 1.0) * 0.5 : 0.0;
+        const int c = min(max((int)(u * (1 << bits)), 0), (1 << bits) - 1);
+        for (int b = 0; b < bits; ++b) id |= ((c >> b) & 1) << (d * b + t);
+    }
+    cell[j] = id;
+    atomicAdd(&count[id], 1);
+}
+
+// exclusive scan of the 4,096 counts (one block of 1,024 threads)
+__global__ void k_cell_scan(int *__restrict__ count) {
+    __shared__ int sh[1024];
+    int v[4], sum = 0;
+    for (int k = 0; k < 4; ++k) {
+        v[k] = sum;
+        sum += count[threadIdx.x * 4 + k];
+    }
+    sh[threadIdx.x] = sum;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+        const int t = threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
+        __syncthreads();
+        sh[threadIdx.x] += t;
+        __syncthreads();
+    }
+    const int base = threadIdx.x ? sh[threadIdx.x - 1] : 0;
+    for (int k = 0; k < 4; ++k) count[threadIdx.x * 4 + k] = base + v[k];
+}
+
+__global__ void k_cell_scatter(const int *__restrict__ cell, int64_t n, int64_t n_pad,
+                               int *__restrict__ offset, int *__restrict__ perm) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) perm[atomicAdd(&offset[cell[j]], 1)] = (int)j;
+    else if (j < n_pad) perm[j] = (int)j;
+}
+
+// ----------------------------------------------------------------------------
 // Per point: R_q from the FP32 pass 1 (log2 sum_j 2^(t_qj + kappa |x'_q|^2)),
 // the float operands of both passes and the integral shift of pass 1; per
 // target: the float operands.  The ranges that fix F go into the result block.
@@ -266,12 +317,13 @@ __global__ void k_fx_records(const double *__restrict__ x64, int64_t nq, int64_t
 // ----------------------------------------------------------------------------
 // One pass: out[chunk][row] = sum over the chunk's columns of
 // 2^(C_col - kappa d^2 - shift_row).  Pass 1: rows = points, columns = targets;
-// pass 2: rows = targets, columns = points.
+// pass 2: rows = targets (in the order of perm), columns = points.
 // ----------------------------------------------------------------------------
 template <int D, int R>
 __global__ void __launch_bounds__(FX_THREADS)
     k_fx_pass(const FxRec *__restrict__ rowrec, const float4 *__restrict__ rowf,
-              const int *__restrict__ rowshift, int neg_shift, int64_t rows_pad,
+              const int *__restrict__ rowshift, int neg_shift, const int *__restrict__ perm,
+              int64_t rows_pad,
               const FxRec *__restrict__ colrec, const float4 *__restrict__ colf, int64_t cols,
               int64_t chunk, const double *__restrict__ tab, double *__restrict__ out,
               const EvalResult *__restrict__ res) {
@@ -285,7 +337,7 @@ __global__ void __launch_bounds__(FX_THREADS)
     const int F = res->fx_F;
     const float E = res->fx_E;
     const int shE = F - 32, shI = F - 46, shG = 75 - F;
-    int H[R][3], Lo[R][3], rs[R];
+    int H[R][3], Lo[R][3], rs[R], at[R];
     float4 xf[R];
     double acc[R];
 #pragma unroll
@@ -296,11 +348,13 @@ __global__ void __launch_bounds__(FX_THREADS)
         rs[k] = 0;
         FxRec r;
         r.a = r.b = make_int4(0, 0, 0, 0);
+        at[k] = -1;
         if (i < rows_pad) {
-            r = rowrec[i];
-            xf[k] = rowf[i];
+            at[k] = perm ? perm[i] : (int)i;
+            r = rowrec[at[k]];
+            xf[k] = rowf[at[k]];
             xf[k].w -= 2.0f * E;
-            rs[k] = rowshift[i];
+            rs[k] = rowshift[at[k]];
             if (neg_shift) rs[k] = -rs[k];
             rs[k] = (int)((unsigned)rs[k] << shE);
         }
@@ -365,10 +419,8 @@ __global__ void __launch_bounds__(FX_THREADS)
         }
     }
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-        const int64_t i = (int64_t)blockIdx.x * (FX_THREADS * R) + k * FX_THREADS + tid;
-        if (i < rows_pad) out[(int64_t)blockIdx.y * rows_pad + i] = acc[k];
-    }
+    for (int k = 0; k < R; ++k)
+        if (at[k] >= 0) out[(int64_t)blockIdx.y * rows_pad + at[k]] = acc[k];
 }
 
 // Per point: L_q, the mass's J term, and the column constant of pass 2,
@@ -434,16 +486,16 @@ inline int fx_rows(const rsot_problem *p, int64_t rows, int64_t cols) {
 }
 
 template <int D>
-void fx_launch(rsot_problem *p, int R, const FxRec *rr, const float4 *rf, const int *rsh, int neg,
+void fx_launch(rsot_problem *p, int R, const FxRec *rr, const float4 *rf, const int *rsh, int neg, const int *perm,
                int64_t rows, int64_t rows_pad, const FxRec *cr, const float4 *cf, int64_t cols, int64_t chunk, int splits,
                double *out) {
     // rows_pad is the stride of out; blocks of padding rows alone are not launched
     dim3 g((unsigned)((rows + FX_THREADS * R - 1) / (FX_THREADS * R)), (unsigned)splits);
     if (R == 2)
-        k_fx_pass<D, 2><<<g, FX_THREADS, 0, p->stream>>>(rr, rf, rsh, neg, rows_pad, cr, cf, cols, chunk,
+        k_fx_pass<D, 2><<<g, FX_THREADS, 0, p->stream>>>(rr, rf, rsh, neg, perm, rows_pad, cr, cf, cols, chunk,
                                                          p->fx_tab, out, p->res_dev);
     else
-        k_fx_pass<D, 1><<<g, FX_THREADS, 0, p->stream>>>(rr, rf, rsh, neg, rows_pad, cr, cf, cols, chunk,
+        k_fx_pass<D, 1><<<g, FX_THREADS, 0, p->stream>>>(rr, rf, rsh, neg, perm, rows_pad, cr, cf, cols, chunk,
                                                          p->fx_tab, out, p->res_dev);
 }
 
@@ -479,6 +531,7 @@ static bool fx_alloc(rsot_problem *p) {
     const size_t o_prow = take(np * 16), o_pcol = take(np * 16), o_psh = take(np * 4);
     const size_t o_trow = take(nt * 16), o_tcol = take(nt * 16), o_tsh = take(nt * 4);
     const size_t o_tsc = take(nt * 8), o_tab = take(FX_TAB * 8);
+    const size_t o_perm = take(nt * 4), o_cell = take(nt * 4 + SORT_CELLS * 4);
     const size_t o_p1 = take(np * 8 * p->fx_k1), o_p2 = take(nt * 8 * p->fx_s2);
     char *b = nullptr;
     if (cudaMalloc(&b, at) != cudaSuccess) {
@@ -498,6 +551,19 @@ static bool fx_alloc(rsot_problem *p) {
     p->fx_tab = reinterpret_cast<double *>(b + o_tab);
     p->fx_part1 = reinterpret_cast<double *>(b + o_p1);
     p->fx_part2 = reinterpret_cast<double *>(b + o_p2);
+    p->fx_perm = reinterpret_cast<int *>(b + o_perm);
+    int *cell = reinterpret_cast<int *>(b + o_cell), *count = cell + nt;
+    cudaMemsetAsync(count, 0, SORT_CELLS * 4, p->stream);
+    const unsigned nb = (unsigned)((p->n_pad + 255) / 256);
+    k_cell_count<<<nb, 256, 0, p->stream>>>(p->y64, p->n, p->d, p->half_ext, cell, count);
+    k_cell_scan<<<1, 1024, 0, p->stream>>>(count);
+    k_cell_scatter<<<nb, 256, 0, p->stream>>>(cell, p->n, p->n_pad, count, p->fx_perm);
+    // once per problem: a later evaluation may run on another stream
+    if (cudaStreamSynchronize(p->stream) != cudaSuccess) {
+        cudaGetLastError();
+        fx64_free(p);
+        return false;
+    }
     return true;
 }
 
@@ -506,6 +572,23 @@ bool fx64_ready(rsot_problem *p, double eps) {
     // the estimate's error bound must allow a decision (see k_fx_records)
     if (!(kappa * p->diam2 <= 0x1p23) || !(p->msum > 0.0)) return false;
     return fx_alloc(p);
+}
+
+// the FP32 estimate of R_q and of the exponents' ranges: terms below 2^-t1 of a
+// point's sum (pass 1) and below 2^-60 nu_j / sum m (pass 2) are told apart
+cudaError_t launch_estimate(rsot_problem *p, const double *psi, double eps, double t1) {
+    cudaStream_t st = p->stream;
+    const double kappa = kLog2e / (2.0 * eps);
+    cudaError_t e = launch_mixed_pass1(p, psi, eps);
+    if (e) return e;
+    const unsigned nb = (unsigned)((std::max(p->nq_pad, p->n_pad) + 255) / 256);
+    trace_begin(p, "fx_operands");
+    k_fx_operands<<<nb, 256, 0, st>>>(p->part1, p->k1, p->nq_pad, p->nq, p->xs, p->x64, p->d, kappa,
+                                      p->mass, t1, psi, eps, p->nu, p->msum, p->n, p->n_pad, p->tquad,
+                                      p->fx_ptrow, p->fx_ptcol, p->fx_ptshift, p->fx_tgrow,
+                                      p->fx_tgcol, p->res_dev);
+    trace_end(p);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, double *grad) {
@@ -519,15 +602,9 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     const double c0 = sqrt(kh), c1 = (-fma(c0, c0, -kh) + kl) / (2.0 * c0);
     const double t1 = kNegl + log2((double)p->n) + 1.0;
     const double tmax = std::max(t1, kNegl + log2(p->msum / p->nu_min));
-    cudaError_t e = launch_mixed_pass1(p, psi, eps);
+    cudaError_t e = launch_estimate(p, psi, eps, t1);
     if (e) return e;
     const unsigned nb = (unsigned)((std::max(p->nq_pad, p->n_pad) + 255) / 256);
-    trace_begin(p, "fx_operands");
-    k_fx_operands<<<nb, 256, 0, st>>>(p->part1, p->k1, p->nq_pad, p->nq, p->xs, p->x64, p->d, kappa,
-                                      p->mass, t1, psi, eps, p->nu, p->msum, p->n, p->n_pad, p->tquad,
-                                      p->fx_ptrow, p->fx_ptcol, p->fx_ptshift, p->fx_tgrow,
-                                      p->fx_tgcol, p->res_dev);
-    trace_end(p);
     trace_begin(p, "fx_records");
     k_fx_records<<<std::max(nb, (unsigned)(FX_TAB / 256)), 256, 0, st>>>(
         p->x64, p->nq, p->nq_pad, p->y64, p->n, p->n_pad, p->d, c0, c1, kappa * p->diam2, tmax, psi,
@@ -535,7 +612,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     trace_end(p);
     trace_begin(p, "fx_lse");
     const int r1 = fx_rows(p, p->nq, p->n), r2 = fx_rows(p, p->n, p->nq);
-    (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, r1, p->fx_prec, p->fx_ptrow, p->fx_ptshift, 0, p->nq, p->nq_pad,
+    (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, r1, p->fx_prec, p->fx_ptrow, p->fx_ptshift, 0, nullptr, p->nq, p->nq_pad,
                                               p->fx_trec, p->fx_tgcol, p->n, p->fx_chunk1, p->fx_k1,
                                               p->fx_part1);
     trace_end(p);
@@ -545,7 +622,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
                                       psi, eps, p->fx_prec, p->lse_buf, p->blockJ, p->res_dev);
     trace_end(p);
     trace_begin(p, "fx_grad");
-    (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, r2, p->fx_trec, p->fx_tgrow, p->fx_tgshift, 1, p->n, p->n_pad,
+    (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, r2, p->fx_trec, p->fx_tgrow, p->fx_tgshift, 1, p->fx_perm, p->n, p->n_pad,
                                               p->fx_prec, p->fx_ptcol, p->nq, p->fx_chunk2, p->fx_s2,
                                               p->fx_part2);
     trace_end(p);

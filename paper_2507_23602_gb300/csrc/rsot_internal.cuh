@@ -70,6 +70,7 @@ struct rsot_problem {
     double msum = 0.0;          // sum_q m_q
     double hx = 0.0;            // sum_q m_q |x'_q|^2 / 2 (translated coordinates)
     double nu_min = 0.0, nu_max = 0.0;
+    double half_ext = 0.0;      // largest half extent of that box along an axis
     double diam2 = 0.0;         // squared diameter of the bounding box of points and targets
     int num_sms = 0;
 
@@ -126,6 +127,7 @@ struct rsot_problem {
     double *fx_tgscale = nullptr;                         // 2^(fraction of B_j)
     double *fx_tab = nullptr;                             // 2^(-i/2048)
     double *fx_part1 = nullptr, *fx_part2 = nullptr;      // row sums per column chunk
+    int *fx_perm = nullptr;                               // order of the target rows
     int fx_k1 = 0, fx_s2 = 0;
     int64_t fx_chunk1 = 0, fx_chunk2 = 0;
     // compensated path scratch (rsot_df.cu), allocated on first use
@@ -225,6 +227,7 @@ cudaError_t launch_finalize_J64(rsot_problem *p, const double *psi_dev, double e
 // dense FP64 evaluation with fixed-point exponents (rsot_fx64.cu); fx64_ready:
 // its buffers exist and the sizes of the exponents allow it
 bool fx64_ready(rsot_problem *p, double eps);
+cudaError_t launch_estimate(rsot_problem *p, const double *psi_dev, double eps, double t1);
 cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
 void fx64_free(rsot_problem *p);
 cudaError_t launch_trunc_fp64(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
