@@ -161,7 +161,9 @@ void rsot_destroy(rsot_problem *p) {
     trunc_free(p);
     compensated_free(p);
     cutoff_free(p);
+    skip_free(p);
     fx64_free(p);
+    cx_free(p);
     dense_free(p);
     cudaFree(p->xs);
     cudaFree(p->x64);
@@ -351,13 +353,18 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     if (!e && !dense) e = mode == 1 ? cutoffs_uniform(p, 0.5 * arg * arg) : cutoffs_separable(p, psid, eps, arg);
     // dense FP64: fixed-point exponents where they can hold the range, the FP64
     // passes otherwise (or when the device finds that they cannot, kErrRange64)
-    bool fx = prec == RSOT_FP64 && dense && !e && fx64_ready(p, eps);
+    // (likewise the compensated evaluation's faster form)
+    const bool alt = !e && dense && ((prec == RSOT_FP64 && fx64_ready(p, eps)) ||
+                                     (prec == RSOT_COMPENSATED && cx_ready(p, eps)));
+    bool retry = alt;
     if (!e) {
-        if (prec == RSOT_COMPENSATED)
+        if (alt)
+            e = prec == RSOT_FP64 ? launch_dense_fx64(p, psid, eps, gd)
+                                  : launch_compensated_cx(p, psid, eps, gd);
+        else if (prec == RSOT_COMPENSATED)
             e = launch_compensated(p, psid, eps, !dense, gd);
         else if (dense)
             e = (prec == RSOT_MIXED) ? launch_dense_mixed(p, psid, eps, gd)
-                : fx                 ? launch_dense_fx64(p, psid, eps, gd)
                                      : launch_dense_fp64(p, psid, eps, gd);
         else
             e = trunc_eval(p, psid, eps, prec == RSOT_MIXED, gd);
@@ -368,10 +375,12 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
         if (!e && !gdev) e = cudaMemcpyAsync(p->grad_host, gd, nb, cudaMemcpyDeviceToHost, st);
         if (!e) e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(EvalResult), cudaMemcpyDeviceToHost, st);
         if (!e) e = cudaStreamSynchronize(st);
-        if (e || !fx || !(p->res_host->flags & kErrRange64)) break;
-        fx = false;
+        if (e || !retry || !(p->res_host->flags & kErrRange64)) break;
+        retry = false;
         e = cudaMemsetAsync(p->res_dev, 0, sizeof(EvalResult), st);
-        if (!e) e = launch_dense_fp64(p, psid, eps, gd);
+        if (!e)
+            e = prec == RSOT_FP64 ? launch_dense_fp64(p, psid, eps, gd)
+                                  : launch_compensated(p, psid, eps, false, gd);
     }
     if (e) {
         cudaGetLastError();

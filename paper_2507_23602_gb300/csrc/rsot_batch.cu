@@ -1029,7 +1029,8 @@ rsot_status rsot_batch_create(int count, const rsot_problem_desc *probs, rsot_ba
         return to_status(e);
     }
     b->slots1 = b->num_sms * occ((const void *)k_blse, P1_THREADS);
-    b->slots2 = b->num_sms * occ((const void *)k_bgrad, P2_THREADS);
+    // five CTAs per SM at most: six run each item slower and leave a longer tail
+    b->slots2 = b->num_sms * std::min(occ((const void *)k_bgrad, P2_THREADS), 5);
     b->slots1_tc = b->num_sms * occ((const void *)k_blse_tc, BT_THREADS);
     b->slots2_tc = b->num_sms * occ((const void *)k_bgrad_tc, BT_THREADS);
     plan_items(b, b->item_exp);

@@ -1144,15 +1144,15 @@ cudaError_t launch_softmax_refine(rsot_problem *p, const double *psi_dev, double
 
 // gradient and log2-domain J from pass-2 partials [s2][n_pad] and nbj pass-1
 // block partials of sum_q m_q R_q (the compensated path's finalisation)
-cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps,
-                                 const double *part2, int s2, int nbj, double *grad) {
+cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps, const double *blockJ,
+                                 int nbj, const double *part2, int s2, double *grad) {
     cudaStream_t st = p->stream;
     trace_begin(p, "finalize_grad");
     k_finalize_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(part2, s2, p->n_pad, p->nu,
                                                                     p->n, grad);
     trace_end(p);
     trace_begin(p, "finalize_J");
-    k_finalize_J<<<1, 256, 0, st>>>(p->blockJ, nbj, p->psinu, p->nblk_prep, psi, eps, p->msum,
+    k_finalize_J<<<1, 256, 0, st>>>(blockJ, nbj, p->psinu, p->nblk_prep, psi, eps, p->msum,
                                     p->hx, 1, p->res_dev);
     trace_end(p);
     return cudaGetLastError();
@@ -1162,23 +1162,12 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi, double eps, d
     return p->d == 3 ? launch_mixed_d<3>(p, psi, eps, grad) : launch_mixed_d<2>(p, psi, eps, grad);
 }
 
-// the FP32 pass 1 alone (records and per-chunk partials), for the fixed-point passes
-cudaError_t launch_mixed_pass1(rsot_problem *p, const double *psi, double eps) {
-    cudaStream_t st = p->stream;
+// the target records of the mixed passes alone, for the pair skipping
+cudaError_t launch_prep_mixed(rsot_problem *p, const double *psi, double eps) {
     trace_begin(p, "prep_targets_mixed");
-    k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                      p->d, eps, p->tquad, p->tpair, p->psinu,
-                                                      p->flags, nullptr, 1.0, nullptr);
-    trace_end(p);
-    dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)p->k1);
-    const int n_p1 = (int)round_up(p->n, P1_TS);
-    trace_begin(p, "lse_mixed");
-    if (p->d == 3)
-        k_lse_mixed<3><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, n_p1, p->chunk1, p->part1,
-                                                  p->flags);
-    else
-        k_lse_mixed<2><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, n_p1, p->chunk1, p->part1,
-                                                  p->flags);
+    k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, p->stream>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
+                                                             p->d, eps, p->tquad, p->tpair, p->psinu,
+                                                             p->flags, nullptr, 1.0, nullptr);
     trace_end(p);
     return cudaGetLastError();
 }

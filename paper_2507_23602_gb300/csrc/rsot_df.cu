@@ -16,8 +16,8 @@
 // Every step is an explicitly rounded add / mul / fma (no contraction), and
 // each thread carries two pairs in the two lanes of the packed FP32x2
 // instructions (add/sub/mul/fma .f32x2): two points per thread in pass 1, two
-// targets in pass 2; the shared-memory records of the other side hold each
-// value twice so that one 16-byte load gives both lanes' operand.
+// targets in pass 2; an operand of the other side goes to both lanes as one
+// register (rsot_inner.cuh, both()).
 //
 // Error budget, relative to each term (ex2.approx: measured <= 2^-22.71 over
 // 3 x 2^30 arguments; the budget takes 2^-22.5):
@@ -44,8 +44,8 @@
 
 namespace rsot {
 
-cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps,
-                                 const double *part2, int s2, int nbj, double *grad);
+cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps, const double *blockJ,
+                                 int nbj, const double *part2, int s2, double *grad);
 
 namespace {
 
@@ -63,14 +63,11 @@ struct __align__(16) DRec {
 
 
 typedef float2 f2;
-#ifndef DFV
-#define DFV 0
-#endif
-__device__ __forceinline__ f2 add2(f2 a, f2 b) { if (DFV & 1) return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)); return __fadd2_rn(a, b); }
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) { if (DFV & 2) return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)); return __fmul2_rn(a, b); }
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { if (DFV & 4) return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y)); return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
 // a - b rounded once: the product b * -1 is exact
-__device__ __forceinline__ f2 sub2(f2 a, f2 b) { if (DFV & 8) return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y)); return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
 // s + e = a + b exactly in each lane (Knuth's TwoSum)
 __device__ __forceinline__ void two_sum2(f2 a, f2 b, f2 &s, f2 &e) {
@@ -719,7 +716,7 @@ cudaError_t compensated_d(rsot_problem *p, const double *psi, double eps, bool t
                                                       nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     trace_end(p);
     if ((e = cudaGetLastError())) return e;
-    return launch_finalize_log2(p, psi, eps, p->df_part2, (int)s2, (int)nb1, grad);
+    return launch_finalize_log2(p, psi, eps, p->blockJ, (int)nb1, p->df_part2, (int)s2, grad);
 }
 
 }  // namespace

@@ -49,9 +49,8 @@ struct EvalResult {
     long long empty;
     int flags;
     int gate;           // bit 0: an f16 operand is out of range (both passes take the FP32 kernels)
-    unsigned fx_key[3]; // fixed-point passes (rsot_fx64.cu): largest -t*_q, B_j, |B_j| as ordered keys
-    int fx_F;           // their fraction bits
-    float fx_E;         // error bound of their FP32 exponent estimate
+    unsigned fx_key[3]; // pair skipping (rsot_skip.cuh): largest A_q, B_j, |B_j| as ordered keys
+    int fx_F;           // fraction bits of the fixed-point passes (rsot_fx64.cu)
 };
 
 struct Grid;  // truncated-path cell grid (rsot_trunc.cu)
@@ -118,18 +117,30 @@ struct rsot_problem {
     int s2_64 = 0;
     int64_t chunk2_64 = 0;
     double *part2_64 = nullptr;     // [s2_64][n_pad]
+    // pair skipping of the dense FP64 and compensated passes (rsot_skip.cu): one
+    // allocation on first use
+    void *sk_buf = nullptr;
+    float *sk_part = nullptr;                              // largest exponents per target chunk
+    float4 *sk_ptrow = nullptr, *sk_ptcol = nullptr, *sk_tgrow = nullptr;   // FP32 records
+    float *sk_ptA = nullptr, *sk_tgB = nullptr;            // values of the ball test
+    int *sk_perm = nullptr;                                // order of the target rows
+    int sk_pp = 0, sk_k = 0;
+    int64_t sk_chunk = 0;
     // fixed-point passes of the dense FP64 path (rsot_fx64.cu): one allocation on first use
     void *fx_buf = nullptr;
     rsot::FxRec *fx_prec = nullptr, *fx_trec = nullptr;   // integer operands of points, targets
-    float4 *fx_ptrow = nullptr, *fx_ptcol = nullptr;      // FP32 operands of the estimate
-    float4 *fx_tgrow = nullptr, *fx_tgcol = nullptr;
     int *fx_ptshift = nullptr, *fx_tgshift = nullptr;     // integral row shifts
     double *fx_tgscale = nullptr;                         // 2^(fraction of B_j)
     double *fx_tab = nullptr;                             // 2^(-i/2048)
     double *fx_part1 = nullptr, *fx_part2 = nullptr;      // row sums per column chunk
-    int *fx_perm = nullptr;                               // order of the target rows
     int fx_k1 = 0, fx_s2 = 0;
     int64_t fx_chunk1 = 0, fx_chunk2 = 0;
+    // compensated dense evaluation outside the solver (rsot_cx.cu): one allocation on first use
+    void *cx_buf = nullptr, *cx_prec = nullptr, *cx_trec = nullptr;
+    double *cx_part1 = nullptr, *cx_part2 = nullptr;
+    float *cx_shift = nullptr;
+    int cx_s2 = 0;
+    int64_t cx_chunk2 = 0;
     // compensated path scratch (rsot_df.cu), allocated on first use
     void *df_prec = nullptr;        // [nq_pad] point head/tail records (64 B)
     void *df_trec = nullptr;        // [n_pad] target head/tail records (64 B)
@@ -222,14 +233,24 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi_dev, double ep
                                double *grad_dev);
 cudaError_t launch_dense_fp64(rsot_problem *p, const double *psi_dev, double eps,
                               double *grad_dev);
-cudaError_t launch_mixed_pass1(rsot_problem *p, const double *psi_dev, double eps);
+cudaError_t launch_prep_mixed(rsot_problem *p, const double *psi_dev, double eps);
 cudaError_t launch_finalize_J64(rsot_problem *p, const double *psi_dev, double eps, int nbj);
 // dense FP64 evaluation with fixed-point exponents (rsot_fx64.cu); fx64_ready:
 // its buffers exist and the sizes of the exponents allow it
 bool fx64_ready(rsot_problem *p, double eps);
-cudaError_t launch_estimate(rsot_problem *p, const double *psi_dev, double eps, double t1);
+// pair skipping (rsot_skip.cu)
+bool skip_ready(rsot_problem *p, double eps);
+double skip_t1(const rsot_problem *p);
+cudaError_t launch_skip(rsot_problem *p, const double *psi_dev, double eps);
+void skip_free(rsot_problem *p);
 cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
 void fx64_free(rsot_problem *p);
+// the smallest column split whose CTAs fill the resident slots
+int split_for_slots(int64_t units, int64_t tiles, int64_t slots);
+// compensated dense evaluation outside the solver (rsot_cx.cu)
+bool cx_ready(rsot_problem *p, double eps);
+cudaError_t launch_compensated_cx(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
+void cx_free(rsot_problem *p);
 cudaError_t launch_trunc_fp64(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);
 cudaError_t launch_covering_cost(rsot_problem *p, double *C0_dev);
 cudaError_t launch_psi_stats(rsot_problem *p, const double *psi_dev, double *out3_dev);
@@ -300,6 +321,15 @@ __device__ __forceinline__ float pow2_int_f(float k) {
 }
 __device__ __forceinline__ double pow2_int_d(float k) {
     return k < -1022.0f ? 0.0 : __longlong_as_double((long long)((int)k + 1023) << 52);
+}
+
+// floats as unsigned keys in the same order (for atomicMax); 0 is below every float
+__device__ __forceinline__ unsigned ordered_key(float f) {
+    const unsigned b = __float_as_uint(f);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float from_key(unsigned k) {
+    return __uint_as_float(k & 0x80000000u ? k & 0x7fffffffu : ~k);
 }
 
 // ---- mbarrier + bulk-copy (TMA) wrappers ------------------------------------

@@ -1,0 +1,270 @@
+// Operands of the pair skipping (rsot_skip.cuh): the largest FP32 exponent of
+// every point, the records and thresholds of the tests, and the order of the
+// target rows.
+#include <math.h>
+
+#include <algorithm>
+
+#include "rsot_internal.cuh"
+#include "rsot_inner.cuh"
+#include "rsot_skip.cuh"
+
+namespace rsot {
+namespace {
+
+constexpr int RM_THREADS = 128;
+constexpr int RM_TS = 256;   // targets per shared-memory tile
+constexpr int SORT_CELLS = 4096;
+
+// max_j r_qj over a chunk of targets, two points per lane pair and PP pairs a
+// thread (4 share a target's load; 1 where that leaves SMs idle)
+template <int D, int PP>
+__global__ void __launch_bounds__(RM_THREADS)
+    k_row_max(const float *__restrict__ xs, int64_t nq_pad, const float4 *__restrict__ tquad, int64_t n,
+              int64_t chunk, float *__restrict__ out) {
+    __shared__ __align__(16) float4 sm[RM_TS];
+    const int64_t q0 = (int64_t)blockIdx.x * (2 * PP * RM_THREADS);
+    float2 X[PP][3], m[PP];
+#pragma unroll
+    for (int pp = 0; pp < PP; ++pp) {
+        const int64_t q = q0 + 2 * (pp * RM_THREADS + threadIdx.x);
+        for (int t = 0; t < 3; ++t)
+            X[pp][t] = t < D ? *reinterpret_cast<const float2 *>(xs + t * nq_pad + q) : make_float2(0.f, 0.f);
+        m[pp] = make_float2(-INFINITY, -INFINITY);
+    }
+    const int64_t c_begin = (int64_t)blockIdx.y * chunk, c_end = min(n, c_begin + chunk);
+    for (int64_t t0 = c_begin; t0 < c_end; t0 += RM_TS) {
+        const int cnt = (int)min((int64_t)RM_TS, c_end - t0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < cnt; i += RM_THREADS) sm[i] = tquad[t0 + i];
+        if ((cnt & 1) && threadIdx.x == 0) sm[cnt] = tquad[t0 + cnt - 1];   // cnt < RM_TS: in range
+        __syncthreads();
+#pragma unroll 4
+        for (int i = 0; i < cnt; i += 2) {
+            const float4 w0 = sm[i], w1 = sm[i + 1];
+#pragma unroll
+            for (int pp = 0; pp < PP; ++pp) {
+                const float2 a = pair_exponent<D>(X[pp], w0), b = pair_exponent<D>(X[pp], w1);
+                m[pp].x = max3f(m[pp].x, a.x, b.x);
+                m[pp].y = max3f(m[pp].y, a.y, b.y);
+            }
+        }
+    }
+#pragma unroll
+    for (int pp = 0; pp < PP; ++pp) {
+        const int64_t q = q0 + 2 * (pp * RM_THREADS + threadIdx.x);
+        *reinterpret_cast<float2 *>(out + (int64_t)blockIdx.y * nq_pad + q) = m[pp];
+    }
+}
+
+__device__ __forceinline__ void block_max_key(float v, unsigned *key) {
+    __shared__ float sh[32];
+    v = warp_max_f(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = fmaxf(v, sh[w]);
+        if (v > -INFINITY) atomicMax(key, ordered_key(v));
+    }
+}
+
+// Per point: max_j r_qj, the row record (x', max - t1), A_q = k |x'|^2 - max;
+// per target: the row record (w, log2(nu / sum m) - 60 - c) and B_j.  The
+// largest A_q, B_j and |B_j| go into the result block.
+__global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t nq_pad, int64_t nq,
+                                const float *__restrict__ xs, const double *__restrict__ x64, int d,
+                                double kappa, float t1, const double *__restrict__ psi, double eps,
+                                const double *__restrict__ nu, double msum, int64_t n, int64_t n_pad,
+                                const float4 *__restrict__ tquad, float4 *__restrict__ ptrow,
+                                float *__restrict__ ptA, float4 *__restrict__ tgrow,
+                                float *__restrict__ tgB, EvalResult *__restrict__ res) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    float amax = -INFINITY, bmax = -INFINITY, babs = -INFINITY;
+    if (i < nq_pad) {
+        float4 row = make_float4(0.f, 0.f, 0.f, INFINITY);
+        float A = -INFINITY;
+        if (i < nq) {
+            float mx = -INFINITY;
+            for (int k = 0; k < k1; ++k) mx = fmaxf(mx, part[(int64_t)k * nq_pad + i]);
+            float x[3] = {0.f, 0.f, 0.f};
+            double r2 = 0.0;
+            for (int t = 0; t < d; ++t) {
+                x[t] = xs[t * nq_pad + i];
+                r2 = fma(x64[i * d + t], x64[i * d + t], r2);
+            }
+            A = amax = (float)(kappa * r2 - (double)mx);
+            row = make_float4(x[0], x[1], x[2], mx - t1);
+        }
+        ptrow[i] = row;
+        ptA[i] = A;
+    }
+    if (i < n_pad) {
+        float4 r = tquad[i];
+        float B = -INFINITY;
+        r.w = INFINITY;
+        if (i < n) {
+            double bh, bl;
+            target_B(psi[i], psi[0], eps, nu[i], bh, bl);
+            B = bmax = (float)bh;
+            babs = fabsf(B);
+            r.w = (float)(log2(nu[i] / msum) - 60.0) - tquad[i].w;
+        }
+        tgrow[i] = r;
+        tgB[i] = B;
+    }
+    block_max_key(amax, &res->fx_key[0]);
+    block_max_key(bmax, &res->fx_key[1]);
+    block_max_key(babs, &res->fx_key[2]);
+}
+
+// Order of the target rows of pass 2: by cells of a 2^b grid in Morton order
+// (counting sort, once per problem), so that a warp's targets are near each
+// other and most of a far point's pairs are skipped by whole warps: at eps 1e-3
+// (98,304 x 16,384) the FP64 pass 2 takes 1.6 ms, 3.7 in the caller's order.
+// The order inside a cell is whatever the atomics give; a row's sum does not
+// depend on it.
+__global__ void k_cell_count(const double *__restrict__ y64, int64_t n, int d, double half,
+                             int *__restrict__ cell, int *__restrict__ count) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const int bits = d == 3 ? 4 : 6;
+    int id = 0;
+    for (int t = 0; t < d; ++t) {
+        const double u = half > 0.0 ? (y64[j * d + t] / half + 1.0) * 0.5 : 0.0;
+        const int c = min(max((int)(u * (1 << bits)), 0), (1 << bits) - 1);
+        for (int b = 0; b < bits; ++b) id |= ((c >> b) & 1) << (d * b + t);
+    }
+    cell[j] = id;
+    atomicAdd(&count[id], 1);
+}
+
+// exclusive scan of the 4,096 counts (one block of 1,024 threads)
+__global__ void k_cell_scan(int *__restrict__ count) {
+    __shared__ int sh[1024];
+    int v[4], sum = 0;
+    for (int k = 0; k < 4; ++k) {
+        v[k] = sum;
+        sum += count[threadIdx.x * 4 + k];
+    }
+    sh[threadIdx.x] = sum;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+        const int t = threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
+        __syncthreads();
+        sh[threadIdx.x] += t;
+        __syncthreads();
+    }
+    const int base = threadIdx.x ? sh[threadIdx.x - 1] : 0;
+    for (int k = 0; k < 4; ++k) count[threadIdx.x * 4 + k] = base + v[k];
+}
+
+__global__ void k_cell_scatter(const int *__restrict__ cell, int64_t n, int64_t n_pad,
+                               int *__restrict__ offset, int *__restrict__ perm) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) perm[atomicAdd(&offset[cell[j]], 1)] = (int)j;
+    else if (j < n_pad) perm[j] = (int)j;
+}
+
+template <int D>
+void row_max(rsot_problem *p) {
+    dim3 g((unsigned)(p->nq_pad / (2 * p->sk_pp * RM_THREADS)), (unsigned)p->sk_k);
+    if (p->sk_pp == 4)
+        k_row_max<D, 4><<<g, RM_THREADS, 0, p->stream>>>(p->xs, p->nq_pad, p->tquad, p->n, p->sk_chunk,
+                                                        p->sk_part);
+    else
+        k_row_max<D, 1><<<g, RM_THREADS, 0, p->stream>>>(p->xs, p->nq_pad, p->tquad, p->n, p->sk_chunk,
+                                                        p->sk_part);
+}
+
+}  // namespace
+
+// the smallest column split whose CTAs fill the resident slots (at most 5 % idle
+// in the last wave)
+int split_for_slots(int64_t units, int64_t tiles, int64_t slots) {
+    int best = 1;
+    double best_eff = 0.0;
+    for (int64_t s = 1; s <= std::min<int64_t>(tiles, 256); ++s) {
+        const int64_t items = units * s, waves = (items + slots - 1) / slots;
+        const double eff = (double)items / (double)(waves * slots);
+        if (eff > best_eff + 0.01) best_eff = eff, best = (int)s;
+        if (items >= slots && eff >= 0.95) return (int)s;
+    }
+    return best;
+}
+
+void skip_free(rsot_problem *p) {
+    cudaFree(p->sk_buf);
+    p->sk_buf = nullptr;
+}
+
+// buffers and the target order, once per problem; false: not for these sizes,
+// or no memory (the callers have passes that need none of it)
+bool skip_ready(rsot_problem *p, double eps) {
+    const double kappa = kLog2e / (2.0 * eps);
+    // the estimate's error bound must allow a decision
+    if (!(kappa * p->diam2 <= 0x1p23) || !(p->msum > 0.0)) return false;
+    if (p->sk_buf) return true;
+    const int64_t tiles = (p->n + RM_TS - 1) / RM_TS;
+    p->sk_pp = p->nq_pad / 1024 * tiles >= 4 * p->num_sms ? 4 : 1;
+    p->sk_k = split_for_slots(p->nq_pad / (2 * p->sk_pp * RM_THREADS), tiles, (int64_t)p->num_sms * 6);
+    p->sk_chunk = (tiles + p->sk_k - 1) / p->sk_k * RM_TS;
+    p->sk_k = (int)((p->n + p->sk_chunk - 1) / p->sk_chunk);
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 255) / 256 * 256;
+        return o;
+    };
+    const size_t np = (size_t)p->nq_pad, nt = (size_t)p->n_pad;
+    const size_t o_part = take(np * 4 * p->sk_k), o_prow = take(np * 16), o_pcol = take(np * 16);
+    const size_t o_pA = take(np * 4), o_trow = take(nt * 16), o_tB = take(nt * 4), o_perm = take(nt * 4);
+    const size_t o_cell = take(nt * 4 + SORT_CELLS * 4);
+    char *b = nullptr;
+    if (cudaMalloc(&b, at) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    p->sk_buf = b;
+    p->sk_part = reinterpret_cast<float *>(b + o_part);
+    p->sk_ptrow = reinterpret_cast<float4 *>(b + o_prow);
+    p->sk_ptcol = reinterpret_cast<float4 *>(b + o_pcol);
+    p->sk_ptA = reinterpret_cast<float *>(b + o_pA);
+    p->sk_tgrow = reinterpret_cast<float4 *>(b + o_trow);
+    p->sk_tgB = reinterpret_cast<float *>(b + o_tB);
+    p->sk_perm = reinterpret_cast<int *>(b + o_perm);
+    int *cell = reinterpret_cast<int *>(b + o_cell), *count = cell + nt;
+    cudaMemsetAsync(count, 0, SORT_CELLS * 4, p->stream);
+    const unsigned nb = (unsigned)((p->n_pad + 255) / 256);
+    k_cell_count<<<nb, 256, 0, p->stream>>>(p->y64, p->n, p->d, p->half_ext, cell, count);
+    k_cell_scan<<<1, 1024, 0, p->stream>>>(count);
+    k_cell_scatter<<<nb, 256, 0, p->stream>>>(cell, p->n, p->n_pad, count, p->sk_perm);
+    // once per problem: a later evaluation may run on another stream
+    if (cudaStreamSynchronize(p->stream) != cudaSuccess) {
+        cudaGetLastError();
+        skip_free(p);
+        return false;
+    }
+    return true;
+}
+
+double skip_t1(const rsot_problem *p) { return 60.0 + log2((double)p->n) + 1.0; }
+
+cudaError_t launch_skip(rsot_problem *p, const double *psi, double eps) {
+    cudaStream_t st = p->stream;
+    cudaError_t e = launch_prep_mixed(p, psi, eps);
+    if (e) return e;
+    trace_begin(p, "row_max");
+    (p->d == 3 ? row_max<3> : row_max<2>)(p);
+    trace_end(p);
+    const unsigned nb = (unsigned)((std::max(p->nq_pad, p->n_pad) + 255) / 256);
+    trace_begin(p, "skip_operands");
+    k_skip_operands<<<nb, 256, 0, st>>>(p->sk_part, p->sk_k, p->nq_pad, p->nq, p->xs, p->x64, p->d,
+                                        kLog2e / (2.0 * eps), (float)skip_t1(p), psi, eps, p->nu, p->msum,
+                                        p->n, p->n_pad, p->tquad, p->sk_ptrow, p->sk_ptA, p->sk_tgrow,
+                                        p->sk_tgB, p->res_dev);
+    trace_end(p);
+    return cudaGetLastError();
+}
+
+}  // namespace rsot
