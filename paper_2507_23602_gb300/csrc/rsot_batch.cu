@@ -58,6 +58,7 @@ struct rsot_batch {
     int64_t items1 = 0, items2 = 0, items1_cap = 0, items2_cap = 0;
     int nblk_p = 0, nblk_t = 0;
     int slots1 = 0, slots2 = 0;
+    int pp = 4, tpp = 4;       // point / target pairs per thread of the FP32 passes (plan_items)
     int *blk2prob_p = nullptr, *blk2prob_t = nullptr;
     int64_t *item1_base = nullptr, *item2_base = nullptr;   // count + 1
     float *xs = nullptr;
@@ -158,8 +159,12 @@ __global__ void k_bprep(const BProb *__restrict__ probs, const int *__restrict__
     if (threadIdx.x == 0) psinu[b] = s;
 }
 
-// pass 1 over all problems (3-D arithmetic; 2-D problems carry x2 = y2 = 0)
-__global__ void __launch_bounds__(P1_THREADS, 4)
+// pass 1 over all problems (2-D problems carry x2 = y2 = 0).  A CTA takes an item
+// (PP = P1_PP), or a half or quarter of its point tile where the items are few:
+// an item of 2^22 pairs keeps one CTA busy for 0.1 to 0.4 ms, so a batch of fewer
+// items than resident CTAs took as long as one of them.
+template <int PP>
+__global__ void __launch_bounds__(P1_THREADS, p1_minb(PP))
     k_blse(const BProb *__restrict__ probs, int count, const int64_t *__restrict__ item1_base,
            const unsigned char *__restrict__ active, const float *__restrict__ xs,
            const float4 *__restrict__ tquad, float2 *__restrict__ part1, int *__restrict__ counter,
@@ -178,6 +183,7 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
         fence_barrier_init();
     }
     __syncthreads();
+    constexpr int NSUB = P1_PP / PP;
     const int64_t total = item1_base[count];
     unsigned git = 0;
     bool aborted = false;
@@ -185,11 +191,12 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
         if (tid == 0) {
             const long long it = atomicAdd(counter, 1);
             s_item = it;
-            if (it < total) s_p = find_prob(item1_base, count, it);
+            if (it < total * NSUB) s_p = find_prob(item1_base, count, it / NSUB);
         }
         __syncthreads();
-        const int64_t item = s_item;
-        if (item >= total) break;
+        if (s_item >= total * NSUB) break;
+        const int64_t item = s_item / NSUB;
+        const int l0 = (int)(s_item % NSUB) * (2 * PP * P1_THREADS);   // first point in the tile
         const int p = s_p;
         if (active[p]) {
             const BProb P = probs[p];
@@ -197,7 +204,8 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
             const int64_t tile = local / P.nck1;
             const int c = (int)(local % P.nck1);
             const int64_t t_begin = P.t_base + (int64_t)c * P.chunk1;
-            const int ntile = (int)(min((int64_t)P.chunk1, P.n_p1 - (int64_t)c * P.chunk1) / P1_TS);
+            const int t_count = (int)min((int64_t)P.chunk1, P.n - (int64_t)c * P.chunk1);
+            const int ntile = (t_count + P1_TS - 1) / P1_TS;
             if (tid == 0)
                 for (int s = 0; s < 2 && s < ntile; ++s) {
                     const unsigned slot = (git + s) & 1u;
@@ -206,18 +214,18 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
                              &full[slot]);
                 }
             const float *xb = xs + 3 * P.pt_base;
-            float2 X[P1_PP][3];
+            float2 X[PP][3];
 #pragma unroll
-            for (int pp = 0; pp < P1_PP; ++pp) {
-                const int64_t q = tile * P1_TILE + 2 * (pp * P1_THREADS + tid);
+            for (int pp = 0; pp < PP; ++pp) {
+                const int64_t q = tile * P1_TILE + l0 + 2 * (pp * P1_THREADS + tid);
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
                     X[pp][k] = *reinterpret_cast<const float2 *>(xb + k * P.nq_pad + q);
             }
-            float2 M[P1_PP], Sf[P1_PP];
-            double2 Sd[P1_PP];
+            float2 M[PP], Sf[PP];
+            double2 Sd[PP];
 #pragma unroll
-            for (int pp = 0; pp < P1_PP; ++pp) {
+            for (int pp = 0; pp < PP; ++pp) {
                 M[pp] = make_float2(kPadC, kPadC);
                 Sf[pp] = make_float2(0.f, 0.f);
                 Sd[pp] = make_double2(0.0, 0.0);
@@ -228,7 +236,9 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
                     s_abort[it & 1] = 1;
                     atomicOr(flags, kErrTimeout);
                 } else {
-                    lse_stage<3, P1_PP>(sm[slot], X, M, Sf, Sd);
+                    const int cnt = min(P1_TS, t_count - it * P1_TS);
+                    if (P.d == 3) lse_stage<3, PP>(sm[slot], cnt, X, M, Sf, Sd);
+                    else lse_stage<2, PP>(sm[slot], cnt, X, M, Sf, Sd);
                 }
                 __syncthreads();
                 aborted = s_abort[it & 1] != 0;
@@ -239,7 +249,7 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
                              P1_TS * sizeof(float4), &full[slot]);
                 }
 #pragma unroll
-                for (int pp = 0; pp < P1_PP; ++pp) {
+                for (int pp = 0; pp < PP; ++pp) {
                     Sd[pp].x += (double)Sf[pp].x;
                     Sd[pp].y += (double)Sf[pp].y;
                     Sf[pp] = make_float2(0.f, 0.f);
@@ -248,8 +258,8 @@ __global__ void __launch_bounds__(P1_THREADS, 4)
             if (aborted) break;
             git += ntile;
 #pragma unroll
-            for (int pp = 0; pp < P1_PP; ++pp) {
-                const int l = 2 * (pp * P1_THREADS + tid);
+            for (int pp = 0; pp < PP; ++pp) {
+                const int l = l0 + 2 * (pp * P1_THREADS + tid);
                 *reinterpret_cast<float4 *>(part1 + item * P1_TILE + l) =
                     make_float4(M[pp].x, (float)Sd[pp].x, M[pp].y, (float)Sd[pp].y);
             }
@@ -569,6 +579,8 @@ __global__ void __launch_bounds__(BT_THREADS, 1)
 
 constexpr int B_TPP = 4;   // pass 2: 1024 targets per block
 
+// pass 2: a CTA takes an item (TPP = B_TPP) or a half or quarter of its targets
+template <int TPP>
 __global__ void __launch_bounds__(P2_THREADS)
     k_bgrad(const BProb *__restrict__ probs, int count, const int64_t *__restrict__ item2_base,
             const unsigned char *__restrict__ active, const Rec8 *__restrict__ tpair,
@@ -587,6 +599,7 @@ __global__ void __launch_bounds__(P2_THREADS)
         fence_barrier_init();
     }
     __syncthreads();
+    constexpr int NSUB = B_TPP / TPP;
     const int64_t total = item2_base[count];
     unsigned git = 0;
     bool aborted = false;
@@ -594,11 +607,12 @@ __global__ void __launch_bounds__(P2_THREADS)
         if (tid == 0) {
             const long long it = atomicAdd(counter, 1);
             s_item = it;
-            if (it < total) s_p = find_prob(item2_base, count, it);
+            if (it < total * NSUB) s_p = find_prob(item2_base, count, it / NSUB);
         }
         __syncthreads();
-        const int64_t item = s_item;
-        if (item >= total) break;
+        if (s_item >= total * NSUB) break;
+        const int64_t item = s_item / NSUB;
+        const int l0 = (int)(s_item % NSUB) * (2 * TPP * P2_THREADS);   // first target in the block
         const int p = s_p;
         if (active[p]) {
             const BProb P = probs[p];
@@ -606,7 +620,8 @@ __global__ void __launch_bounds__(P2_THREADS)
             const int64_t blk = local / P.nsp2;
             const int s = (int)(local % P.nsp2);
             const int64_t p_begin = P.pt_base + (int64_t)s * P.chunk2;
-            const int ntile = (int)(min(P.chunk2, P.nq_pad - (int64_t)s * P.chunk2) / P2_TS);
+            const int64_t p_count = min(P.chunk2, P.nq - (int64_t)s * P.chunk2);   // < 0: padding alone
+            const int ntile = p_count > 0 ? (int)((p_count + P2_TS - 1) / P2_TS) : 0;
             if (tid == 0)
                 for (int st = 0; st < 2 && st < ntile; ++st) {
                     const unsigned slot = (git + st) & 1u;
@@ -614,11 +629,11 @@ __global__ void __launch_bounds__(P2_THREADS)
                     bulk_g2s(sm[slot], pquad + p_begin + (int64_t)st * P2_TS, P2_TS * sizeof(float4),
                              &full[slot]);
                 }
-            const int64_t g0 = P.t_base / 2 + blk * (P2_THREADS * B_TPP);
-            float2 W0[B_TPP], W1[B_TPP], W2[B_TPP], C[B_TPP];
-            double2 acc64[B_TPP];
+            const int64_t g0 = P.t_base / 2 + blk * (P2_THREADS * B_TPP) + l0 / 2;
+            float2 W0[TPP], W1[TPP], W2[TPP], C[TPP];
+            double2 acc64[TPP];
 #pragma unroll
-            for (int tp = 0; tp < B_TPP; ++tp) {
+            for (int tp = 0; tp < TPP; ++tp) {
                 const Rec8 r = tpair[g0 + tp * P2_THREADS + tid];
                 W0[tp] = make_float2(r.a.x, r.a.y);
                 W1[tp] = make_float2(r.a.z, r.a.w);
@@ -632,7 +647,9 @@ __global__ void __launch_bounds__(P2_THREADS)
                     s_abort[it & 1] = 1;
                     atomicOr(flags, kErrTimeout);
                 } else {
-                    grad_stage<3, B_TPP>(sm[slot], W0, W1, W2, C, acc64);
+                    const int cnt = (int)min((int64_t)P2_TS, p_count - (int64_t)it * P2_TS);
+                    if (P.d == 3) grad_stage<3, TPP>(sm[slot], cnt, W0, W1, W2, C, acc64);
+                    else grad_stage<2, TPP>(sm[slot], cnt, W0, W1, W2, C, acc64);
                 }
                 __syncthreads();
                 aborted = s_abort[it & 1] != 0;
@@ -646,8 +663,8 @@ __global__ void __launch_bounds__(P2_THREADS)
             if (aborted) break;
             git += ntile;
 #pragma unroll
-            for (int tp = 0; tp < B_TPP; ++tp) {
-                const int64_t j = 2 * (tp * P2_THREADS + tid);
+            for (int tp = 0; tp < TPP; ++tp) {
+                const int64_t j = l0 + 2 * (tp * P2_THREADS + tid);
                 *reinterpret_cast<double2 *>(part2 + item * (2 * P2_THREADS * B_TPP) + j) = acc64[tp];
             }
         }
@@ -727,6 +744,19 @@ void plan_items(rsot_batch *b, int e) {
     }
     b->items1 = i1;
     b->items2 = i2;
+    // smaller CTAs while the items would not fill the resident slots `kFill` times
+    // (a batch of 2 problems 812 -> 378 us, of 16 3,529 -> 3,518; 1 or 4: within 5 %)
+    constexpr int kFill = 2;
+    const void *f1[] = {(const void *)k_blse<4>, (const void *)k_blse<2>, (const void *)k_blse<1>};
+    const void *f2[] = {(const void *)k_bgrad<4>, (const void *)k_bgrad<2>, (const void *)k_bgrad<1>};
+    int k = 0;
+    for (b->pp = 4; (b->slots1 = b->num_sms * occ(f1[k], P1_THREADS), k < 2) &&
+                    (i1 << k) < (int64_t)kFill * b->slots1; ++k)
+        b->pp /= 2;
+    k = 0;
+    for (b->tpp = 4; (b->slots2 = b->num_sms * std::min(occ(f2[k], P2_THREADS), 5 << k), k < 2) &&
+                     (i2 << k) < (int64_t)kFill * b->slots2; ++k)
+        b->tpp /= 2;
 }
 
 cudaError_t upload_plan(rsot_batch *b) {
@@ -773,8 +803,9 @@ cudaError_t enqueue_round(rsot_batch *b, bool force_fp32 = false) {
         k_blse_tc<<<b->slots1_tc, BT_THREADS, 0, st>>>(b->dp, b->count, b->item1_base, b->active_d,
                                                        b->prec16, b->trec, b->part1, b->counters,
                                                        b->counters + 2, gate);
-    k_blse<<<b->slots1, P1_THREADS, 0, st>>>(b->dp, b->count, b->item1_base, b->active_d, b->xs,
-                                             b->tquad, b->part1, b->counters, b->counters + 2, gate);
+    auto lse = b->pp == 4 ? k_blse<4> : b->pp == 2 ? k_blse<2> : k_blse<1>;
+    lse<<<b->slots1, P1_THREADS, 0, st>>>(b->dp, b->count, b->item1_base, b->active_d, b->xs, b->tquad,
+                                          b->part1, b->counters, b->counters + 2, gate);
     k_bcombine<<<b->nblk_p, B_T, 0, st>>>(b->dp, b->blk2prob_p, b->active_d, b->part1, b->xs,
                                          b->mass, b->lm2, b->pquad, b->blockJ,
                                          tc ? b->pu : nullptr);
@@ -782,9 +813,9 @@ cudaError_t enqueue_round(rsot_batch *b, bool force_fp32 = false) {
         k_bgrad_tc<<<b->slots2_tc, BT_THREADS, 0, st>>>(b->dp, b->count, b->item2_base, b->active_d,
                                                         b->trec, b->prec16, b->pu, b->part2,
                                                         b->counters + 1, b->counters + 2, gate);
-    k_bgrad<<<b->slots2, P2_THREADS, 0, st>>>(b->dp, b->count, b->item2_base, b->active_d,
-                                              b->tpair, b->pquad, b->part2, b->counters + 1,
-                                              b->counters + 2, gate);
+    auto grad = b->tpp == 4 ? k_bgrad<4> : b->tpp == 2 ? k_bgrad<2> : k_bgrad<1>;
+    grad<<<b->slots2, P2_THREADS, 0, st>>>(b->dp, b->count, b->item2_base, b->active_d, b->tpair,
+                                           b->pquad, b->part2, b->counters + 1, b->counters + 2, gate);
     k_bfinal_grad<<<b->nblk_t, B_T, 0, st>>>(b->dp, b->blk2prob_t, b->active_d, b->part2, b->nu,
                                             b->grad_d);
     k_bfinal_J<<<b->count, B_T, 0, st>>>(b->dp, b->active_d, b->blockJ, b->psinu, b->psi_d,
@@ -1028,9 +1059,6 @@ rsot_status rsot_batch_create(int count, const rsot_problem_desc *probs, rsot_ba
         rsot_batch_destroy(b);
         return to_status(e);
     }
-    b->slots1 = b->num_sms * occ((const void *)k_blse, P1_THREADS);
-    // five CTAs per SM at most: six run each item slower and leave a longer tail
-    b->slots2 = b->num_sms * std::min(occ((const void *)k_bgrad, P2_THREADS), 5);
     b->slots1_tc = b->num_sms * occ((const void *)k_blse_tc, BT_THREADS);
     b->slots2_tc = b->num_sms * occ((const void *)k_bgrad_tc, BT_THREADS);
     plan_items(b, b->item_exp);

@@ -106,10 +106,12 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
 // ----------------------------------------------------------------------------
 // Pass 1: per-point log-sum-exp over one target chunk (step a2).
 // ----------------------------------------------------------------------------
-template <int D>
-__global__ void __launch_bounds__(P1_THREADS, P1_MINB)
+// PP point pairs per thread: P1_PP, or fewer where that leaves SMs without a CTA
+// (a point's sums do not depend on it).
+template <int D, int PP>
+__global__ void __launch_bounds__(P1_THREADS, p1_minb(PP))
     k_lse_mixed(const float *__restrict__ xs, int64_t nq_pad, const float4 *__restrict__ tquad,
-                int n_p1, int chunk, float2 *__restrict__ part, int *__restrict__ flags,
+                int n, int chunk, float2 *__restrict__ part, int *__restrict__ flags,
                 const int *__restrict__ gate = nullptr, int need = 0) {
     // as the fallback of the tensor-core pass, run only when the gate asks for it
     if (gate && !(*gate & need)) return;
@@ -118,25 +120,25 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
     __shared__ int s_abort[2];   // indexed by iteration parity
 
     const int tid = threadIdx.x;
-    const int64_t q0 = (int64_t)blockIdx.x * P1_TILE;
+    const int64_t q0 = (int64_t)blockIdx.x * (2 * PP * P1_THREADS);
     const int kc = blockIdx.y;
     const int t_begin = kc * chunk;
-    const int t_count = min(chunk, n_p1 - t_begin);
-    const int ntile = t_count / P1_TS;
+    const int t_count = min(chunk, n - t_begin);
+    const int ntile = (t_count + P1_TS - 1) / P1_TS;
 
-    float2 X[P1_PP][3];
+    float2 X[PP][3];
 #pragma unroll
-    for (int pp = 0; pp < P1_PP; ++pp) {
+    for (int pp = 0; pp < PP; ++pp) {
         const int64_t q = q0 + 2 * (pp * P1_THREADS + tid);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             X[pp][k] = (k < D) ? *reinterpret_cast<const float2 *>(xs + k * nq_pad + q)
                                : make_float2(0.f, 0.f);
     }
-    float2 M[P1_PP], Sf[P1_PP];
-    double2 Sd[P1_PP];
+    float2 M[PP], Sf[PP];
+    double2 Sd[PP];
 #pragma unroll
-    for (int pp = 0; pp < P1_PP; ++pp) {
+    for (int pp = 0; pp < PP; ++pp) {
         M[pp] = make_float2(kPadC, kPadC);
         Sf[pp] = make_float2(0.f, 0.f);
         Sd[pp] = make_double2(0.0, 0.0);
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
             s_abort[it & 1] = 1;
             atomicOr(flags, kErrTimeout);
         } else {
-            lse_stage<D, P1_PP>(sm[s], X, M, Sf, Sd);
+            lse_stage<D, PP>(sm[s], min(P1_TS, t_count - it * P1_TS), X, M, Sf, Sd);
         }
         __syncthreads();
         aborted = s_abort[it & 1] != 0;
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
             ++issued;
         }
 #pragma unroll
-        for (int pp = 0; pp < P1_PP; ++pp) {
+        for (int pp = 0; pp < PP; ++pp) {
             Sd[pp].x += (double)Sf[pp].x;
             Sd[pp].y += (double)Sf[pp].y;
             Sf[pp] = make_float2(0.f, 0.f);
@@ -194,7 +196,7 @@ __global__ void __launch_bounds__(P1_THREADS, P1_MINB)
         return;
     }
 #pragma unroll
-    for (int pp = 0; pp < P1_PP; ++pp) {
+    for (int pp = 0; pp < PP; ++pp) {
         const int64_t q = q0 + 2 * (pp * P1_THREADS + tid);
         *reinterpret_cast<float4 *>(part + (int64_t)kc * nq_pad + q) =
             make_float4(M[pp].x, (float)Sd[pp].x, M[pp].y, (float)Sd[pp].y);
@@ -245,7 +247,7 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
 // ----------------------------------------------------------------------------
 template <int D, int TPP>
 __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
-    k_grad_mixed(const Rec8 *__restrict__ tpair, const float4 *__restrict__ pquad, int64_t nq_pad,
+    k_grad_mixed(const Rec8 *__restrict__ tpair, const float4 *__restrict__ pquad, int64_t nq,
                  int64_t chunk, double *__restrict__ part2, int64_t stride,
                  int *__restrict__ flags, const int *__restrict__ gate = nullptr, int need = 0) {
     if (gate && !(*gate & need)) return;
@@ -265,8 +267,8 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
         C[tp] = make_float2(r.b.z, r.b.w);
     }
     const int64_t p_begin = (int64_t)blockIdx.y * chunk;
-    const int64_t p_count = min(chunk, nq_pad - p_begin);
-    const int ntile = (int)(p_count / P2_TS);
+    const int64_t p_count = min(chunk, nq - p_begin);   // < 0 in a chunk of padding alone
+    const int ntile = p_count > 0 ? (int)((p_count + P2_TS - 1) / P2_TS) : 0;
 
     double2 acc64[TPP];
 #pragma unroll
@@ -294,7 +296,8 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
             s_abort[it & 1] = 1;
             atomicOr(flags, kErrTimeout);
         } else {
-            grad_stage<D, TPP>(sm[s], W0, W1, W2, C, acc64);
+            grad_stage<D, TPP>(sm[s], (int)min((int64_t)P2_TS, p_count - (int64_t)it * P2_TS), W0, W1, W2, C,
+                               acc64);
         }
         __syncthreads();
         aborted = s_abort[it & 1] != 0;
@@ -990,6 +993,42 @@ void dense_free(rsot_problem *p) {
     cudaFree(p->lse_buf);
 }
 
+// Point pairs (pass 1) or target pairs (pass 2) per thread: `most` where the grid
+// of `items` such CTAs fills three quarters of the resident slots, else half or a quarter of
+// it: smaller CTAs in the same order, whose sums are the same (24,576 x 4,096:
+// passes of 31 + 31 -> 27 + 25 us, 5,184 x 1,500: 40 + 16 -> 27 + 12).
+static int pairs_per_thread(int most, int64_t items, int64_t slots) {
+    int pp = most;
+    while (pp > 1 && 4 * items < 3 * slots) {
+        pp /= 2;
+        items *= 2;
+        slots *= 2;
+    }
+    return pp;
+}
+
+template <int D>
+static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tquad, int64_t n, int chunk,
+                             int k1, float2 *part, int *flags, const int *gate, int num_sms,
+                             cudaStream_t st) {
+    const int pp = pairs_per_thread(P1_PP, nq_pad / P1_TILE * k1, (int64_t)num_sms * P1_MINB);
+    dim3 g((unsigned)(nq_pad / (2 * pp * P1_THREADS)), (unsigned)k1);
+    auto f = pp == 4 ? k_lse_mixed<D, 4> : pp == 2 ? k_lse_mixed<D, 2> : k_lse_mixed<D, 1>;
+    f<<<g, P1_THREADS, 0, st>>>(xs, nq_pad, tquad, (int)n, chunk, part, flags, gate, 1);
+}
+
+template <int D>
+static void launch_grad_mixed(const Rec8 *tpair, int64_t n, const float4 *pquad, int64_t nq,
+                              int64_t chunk, int s2, double *part2, int64_t stride, int *flags,
+                              const int *gate, int num_sms, cudaStream_t st) {
+    const int most = pick_tpp(n);
+    const int64_t blk = (int64_t)P2_THREADS * 2 * most;
+    const int tpp = pairs_per_thread(most, (n + blk - 1) / blk * s2, (int64_t)num_sms * 16 / most);
+    dim3 g((unsigned)((n + 2 * P2_THREADS * tpp - 1) / (2 * P2_THREADS * tpp)), (unsigned)s2);
+    auto f = tpp == 4 ? k_grad_mixed<D, 4> : tpp == 2 ? k_grad_mixed<D, 2> : k_grad_mixed<D, 1>;
+    f<<<g, P2_THREADS, 0, st>>>(tpair, pquad, nq, chunk, part2, stride, flags, gate, 1);
+}
+
 template <int D>
 static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps, double *grad) {
     cudaStream_t st = p->stream;
@@ -1015,10 +1054,9 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
                                             p->flags, gate);
         trace_end(p);
     }
-    dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)k1);
     trace_begin(p, "lse_mixed");
-    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, (int)n_p1, chunk1,
-                                              p->part1, p->flags, gate, 1);
+    launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, chunk1, k1, p->part1, p->flags, gate,
+                        p->num_sms, st);
     trace_end(p);
     trace_begin(p, "combine_mixed");
     k_combine<<<p->nblk_comb, CB_THREADS, 0, st>>>(p->part1, k1, p->nq_pad, p->nq, p->xs, p->d,
@@ -1032,19 +1070,9 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
                                              p->part2, p->n_pad, p->flags, gate);
         trace_end(p);
     }
-    const int tpp = pick_tpp(p->n);
-    const int64_t blk2 = (int64_t)P2_THREADS * 2 * tpp;
-    dim3 g2((unsigned)((p->n + blk2 - 1) / blk2), (unsigned)s2);
     trace_begin(p, "grad_mixed");
-    if (tpp == 4)
-        k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk2,
-                                                      p->part2, p->n_pad, p->flags, gate, 1);
-    else if (tpp == 2)
-        k_grad_mixed<D, 2><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk2,
-                                                      p->part2, p->n_pad, p->flags, gate, 1);
-    else
-        k_grad_mixed<D, 1><<<g2, P2_THREADS, 0, st>>>(p->tpair, p->pquad, p->nq_pad, chunk2,
-                                                      p->part2, p->n_pad, p->flags, gate, 1);
+    launch_grad_mixed<D>(p->tpair, p->n, p->pquad, p->nq, chunk2, s2, p->part2, p->n_pad, p->flags,
+                         gate, p->num_sms, st);
     trace_end(p);
     trace_begin(p, "finalize_grad");
     k_finalize_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(p->part2, s2, p->n_pad,
@@ -1107,9 +1135,8 @@ static cudaError_t softmax_refine_d(rsot_problem *p, const double *psi, double e
     k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
                                                       p->d, eps, p->tquad, p->tpair, p->psinu,
                                                       p->flags, nullptr, 1.0, nullptr);
-    dim3 g1((unsigned)(p->nq_pad / P1_TILE), (unsigned)p->k1);
-    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(p->xs, p->nq_pad, p->tquad, (int)n_p1, p->chunk1,
-                                              p->part1, p->flags);
+    launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, p->chunk1, p->k1, p->part1, p->flags, nullptr,
+                        p->num_sms, st);
     k_combine<<<p->nblk_comb, CB_THREADS, 0, st>>>(p->part1, p->k1, p->nq_pad, p->nq, p->xs, p->d,
                                                    p->lmass2, p->mass, p->pquad, p->blockJ,
                                                    p->lse_buf);
@@ -1126,8 +1153,7 @@ static cudaError_t softmax_refine_d(rsot_problem *p, const double *psi, double e
     if ((e = cudaMemcpyAsync(org, p->origin, 3 * sizeof(double), cudaMemcpyHostToDevice, st))) return e;
     k_prep_fine<<<(unsigned)((nf_alloc + 255) / 256), 256, 0, st>>>(yf, nf, nf_alloc, p->d, org, eps, tpf);
     dim3 g2((unsigned)blocks, (unsigned)s2);
-    k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpf, p->pquad, p->nq_pad, chunk2, part, nf_alloc,
-                                                  p->flags);
+    k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpf, p->pquad, p->nq, chunk2, part, nf_alloc, p->flags);
     k_refine_final<<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(part, s2, nf_alloc, nf, psi, eps, out);
     e = cudaGetLastError();
     cudaFreeAsync(tpf, st);
@@ -1504,9 +1530,7 @@ cudaError_t na_launch(unsigned char *base, int64_t nq, const double *x, const do
     int k1 = pick_split(tiles1, std::min<int64_t>(n_p1 / P1_TS, NA_K1_ROWS / nq_pad), slots1);
     const int chunk1 = (int)round_up((n_p1 + k1 - 1) / k1, P1_TS);
     k1 = (int)((n_p1 + chunk1 - 1) / chunk1);
-    dim3 g1((unsigned)tiles1, (unsigned)k1);
-    k_lse_mixed<D><<<g1, P1_THREADS, 0, st>>>(xs, nq_pad, tquad, (int)n_p1, chunk1, part1,
-                                              &res->flags);
+    launch_lse_mixed<D>(xs, nq_pad, tquad, n, chunk1, k1, part1, &res->flags, nullptr, num_sms, st);
     k_combine<<<nb_pts, CB_THREADS, 0, st>>>(part1, k1, nq_pad, nq, xs, D, lm2, mass, pquad, blockJ,
                                              lse);
     const int tpp = pick_tpp(n);
@@ -1516,16 +1540,7 @@ cudaError_t na_launch(unsigned char *base, int64_t nq, const double *x, const do
                         (int64_t)num_sms * (D == 3 ? 4 : 5));
     const int64_t chunk2 = round_up((nq_pad + s2 - 1) / s2, P2_TS);
     s2 = (int)((nq_pad + chunk2 - 1) / chunk2);
-    dim3 g2((unsigned)units2, (unsigned)s2);
-    if (tpp == 4)
-        k_grad_mixed<D, 4><<<g2, P2_THREADS, 0, st>>>(tpair, pquad, nq_pad, chunk2, part2, n_alloc,
-                                                      &res->flags);
-    else if (tpp == 2)
-        k_grad_mixed<D, 2><<<g2, P2_THREADS, 0, st>>>(tpair, pquad, nq_pad, chunk2, part2, n_alloc,
-                                                      &res->flags);
-    else
-        k_grad_mixed<D, 1><<<g2, P2_THREADS, 0, st>>>(tpair, pquad, nq_pad, chunk2, part2, n_alloc,
-                                                      &res->flags);
+    launch_grad_mixed<D>(tpair, n, pquad, nq, chunk2, s2, part2, n_alloc, &res->flags, nullptr, num_sms, st);
     // the gradient goes to the scratch first; the caller's buffer receives it
     // only when the evaluation succeeded
     k_finalize_grad<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part2, s2, n_alloc, nu, n, gscr);

@@ -27,6 +27,7 @@ inline constexpr int P1_THREADS = 128;
 inline constexpr int P1_PP = RSOT_P1_PP;                      // point pairs per thread (<= 4)
 inline constexpr int P1_TILE = P1_THREADS * 2 * P1_PP;        // points per CTA (divides 1024)
 inline constexpr int P1_MINB = RSOT_P1_MINB;                  // resident CTAs per SM asked of ptxas
+__host__ __device__ constexpr int p1_minb(int pp) { return pp == 4 ? P1_MINB : pp == 2 ? 2 * P1_MINB : 12; }
 #ifndef RSOT_P1_TS
 #define RSOT_P1_TS 512
 #endif
@@ -101,15 +102,16 @@ __device__ __forceinline__ float2 lse_exact_subtile(const float4 *T, const float
     return acc;
 }
 
-// One staged tile of P1_TS targets for PP point pairs: optimistic sub-tiles
+// One staged tile of cnt <= P1_TS targets (the sub-tiles beyond hold padding, whose
+// exponentials are 0) for PP point pairs: optimistic sub-tiles
 // of P1_SUB targets with the running integral shift M, an exact sub-tile
 // (raising M) when a sub-tile sum exceeds 2^60 or overflows.  One test covers
 // the thread's point pairs (a test per pair cost 1 % of the pass).
 template <int D, int PP>
-__device__ __forceinline__ void lse_stage(const float4 *__restrict__ T, const float2 (&X)[PP][3],
+__device__ __forceinline__ void lse_stage(const float4 *__restrict__ T, int cnt, const float2 (&X)[PP][3],
                                           float2 (&M)[PP], float2 (&Sf)[PP], double2 (&Sd)[PP]) {
 #pragma unroll 1
-    for (int t0 = 0; t0 < P1_TS; t0 += P1_SUB) {
+    for (int t0 = 0; t0 < cnt; t0 += P1_SUB) {
         float2 acc0[PP], acc1[PP], nm[PP];
 #pragma unroll
         for (int pp = 0; pp < PP; ++pp) nm[pp] = make_float2(-M[pp].x, -M[pp].y);
@@ -143,18 +145,18 @@ __device__ __forceinline__ void lse_stage(const float4 *__restrict__ T, const fl
     }
 }
 
-// One staged tile of P2_TS point records (x0,x1,x2,u) for TPP
+// One staged tile of cnt <= P2_TS point records (x0,x1,x2,u) for TPP
 // target pairs held in registers: acc64 += sum over the tile of
 // 2^(c_j + x'.w_j + u_q) = sum_q m_q p_qj, FP32 within the tile, FP64 across.
 template <int D, int TPP>
-__device__ __forceinline__ void grad_stage(const float4 *__restrict__ T, const float2 (&W0)[TPP],
+__device__ __forceinline__ void grad_stage(const float4 *__restrict__ T, int cnt, const float2 (&W0)[TPP],
                                            const float2 (&W1)[TPP], const float2 (&W2)[TPP],
                                            const float2 (&C)[TPP], double2 (&acc64)[TPP]) {
     float2 acc[TPP];
 #pragma unroll
     for (int tp = 0; tp < TPP; ++tp) acc[tp] = make_float2(0.f, 0.f);
 #pragma unroll 4
-    for (int i = 0; i < P2_TS; ++i) {
+    for (int i = 0; i < cnt; ++i) {
         const float4 p = T[i];
         const float2 x0 = both(p.x), x1 = both(p.y), x2 = both(p.z), u = both(p.w);
 #pragma unroll
