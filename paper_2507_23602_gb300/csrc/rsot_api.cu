@@ -337,16 +337,23 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     const size_t nb = (size_t)p->n * sizeof(double);
     const double *psid = psi;
     cudaError_t e = cudaSuccess;
-    if (wpsi == 0) {
-        e = cudaMemcpyAsync(p->psi_dev, psi, nb, cudaMemcpyHostToDevice, st);
-        psid = p->psi_dev;
-    }
-    // the passes write the handle's gradient; the caller's buffer receives it
-    // only when the evaluation succeeds (a device-side conditional copy, or a
-    // pinned staging copy for host memory)
+    // the handle's copy of psi: from host memory (through the pinned buffer), and
+    // where the caller's gradient overlaps it (the final kernel reads psi[0])
     const bool gdev = wgrad == 1;
+    if (wpsi == 0) {
+        memcpy(p->grad_host, psi, nb);
+        psid = p->psi_dev;
+        e = cudaMemcpyAsync(p->psi_dev, p->grad_host, nb, cudaMemcpyHostToDevice, st);
+    } else if (gdev && psi < grad_out + p->n && grad_out < psi + p->n) {
+        psid = p->psi_dev;
+        e = cudaMemcpyAsync(p->psi_dev, psi, nb, cudaMemcpyDeviceToDevice, st);
+    }
+    // the passes write the handle's gradient; the caller's buffer (or the pinned
+    // staging buffer of a host one) receives it only when the evaluation succeeds
     double *gd = p->grad_dev;
-    if (!e) e = cudaMemsetAsync(p->res_dev, 0, sizeof(EvalResult), st);
+    p->final_out = !gdev ? p->grad_host : grad_out != gd ? grad_out : nullptr;
+    if (!e && !p->res_clean) e = cudaMemsetAsync(p->res_dev, 0, sizeof(EvalResult), st);
+    p->res_clean = false;
     // a radius beyond the diameter of the data keeps every pair: dense
     const bool dense = mode == 0 || (mode == 1 && (!(arg > 0.0) || isinf(arg) ||
                                                     arg * arg > p->diam2 * (1.0 + 1e-12)));
@@ -354,9 +361,9 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     // dense FP64: fixed-point exponents where they can hold the range, the FP64
     // passes otherwise (or when the device finds that they cannot, kErrRange64)
     // (likewise the compensated evaluation's faster form)
+    p->final_nonempty = dense ? 0 : 1;
     const bool alt = !e && dense && ((prec == RSOT_FP64 && fx64_ready(p, eps)) ||
                                      (prec == RSOT_COMPENSATED && cx_ready(p, eps)));
-    bool retry = alt;
     if (!e) {
         if (alt)
             e = prec == RSOT_FP64 ? launch_dense_fx64(p, psid, eps, gd)
@@ -369,25 +376,28 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
         else
             e = trunc_eval(p, psid, eps, prec == RSOT_MIXED, gd);
     }
-    for (;;) {
-        if (!e && gdev && grad_out != gd)
-            e = launch_commit_grad(gd, grad_out, p->n, p->res_dev, dense ? 0 : 1, st);
+    // the truncated mixed passes have their own last kernels; every other path
+    // ends with launch_finalize()
+    const bool fused = dense || prec != RSOT_MIXED;
+    if (!fused) {
+        if (!e && gdev && grad_out != gd) e = launch_commit_grad(gd, grad_out, p->n, p->res_dev, 1, st);
         if (!e && !gdev) e = cudaMemcpyAsync(p->grad_host, gd, nb, cudaMemcpyDeviceToHost, st);
         if (!e) e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(EvalResult), cudaMemcpyDeviceToHost, st);
-        if (!e) e = cudaStreamSynchronize(st);
-        if (e || !retry || !(p->res_host->flags & kErrRange64)) break;
-        retry = false;
-        e = cudaMemsetAsync(p->res_dev, 0, sizeof(EvalResult), st);
-        if (!e)
-            e = prec == RSOT_FP64 ? launch_dense_fp64(p, psid, eps, gd)
-                                  : launch_compensated(p, psid, eps, false, gd);
     }
+    if (!e) e = cudaStreamSynchronize(st);
+    if (!e && alt && (p->res_host->flags & kErrRange64)) {
+        e = prec == RSOT_FP64 ? launch_dense_fp64(p, psid, eps, gd)
+                              : launch_compensated(p, psid, eps, false, gd);
+        if (!e) e = cudaStreamSynchronize(st);
+    }
+    p->final_out = nullptr;
     if (e) {
         cudaGetLastError();
         p->tr_open.clear();
         p->tr_used = 0;
         return from_cuda(e);
     }
+    p->res_clean = fused;
     trace_collect(p);
     const EvalResult r = *p->res_host;
     p->last_kind = -1;

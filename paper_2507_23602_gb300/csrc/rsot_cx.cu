@@ -40,9 +40,6 @@
 
 namespace rsot {
 
-cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps, const double *blockJ,
-                                 int nbj, const double *part2, int s2, double *grad);
-
 namespace {
 
 constexpr int CX_THREADS = 128;
@@ -426,7 +423,10 @@ cudaError_t launch_compensated_cx(rsot_problem *p, const double *psi, double eps
     trace_end(p);
     (p->d == 3 ? cx_passes<3> : cx_passes<2>)(p, eps, (float)skip_t1(p), (float)kd);
     if ((e = cudaGetLastError())) return e;
-    return launch_finalize_log2(p, psi, eps, p->blockJ, (int)(p->nq_pad / 256), p->cx_part2, p->cx_s2, grad);
+    return launch_finalize(p, psi, eps,
+                           {p->cx_part2, p->cx_s2, p->n_pad, nullptr, p->blockJ, (int)(p->nq_pad / 256), 1, 1,
+                            p->per_prep},
+                           grad);
 }
 
 }  // namespace rsot

@@ -48,6 +48,29 @@ constexpr int F_TS = 128;
 
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
+// Partial sums of v: one per block of 256 threads, or one per warp in smaller
+// blocks (kSmall), which final_term() adds in the order of block_sum_d -- the
+// same bits either way.  Smaller blocks spread the FP64 work of few targets or
+// points over more SMs: 16 blocks of 256 threads kept 16 SMs' two FP64 lanes busy
+// for 7 us.
+constexpr int kSmall = 64;
+__device__ __forceinline__ void store_partial(double v, double *__restrict__ out) {
+    if (blockDim.x == 256) {
+        __shared__ double sh[32];
+        const double s = block_sum_d(v, sh);
+        if (threadIdx.x == 0) out[blockIdx.x] = s;
+    } else {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) out[blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)] = v;
+    }
+}
+__device__ __forceinline__ double final_term(const double *__restrict__ p, int per, int i) {
+    if (per == 1) return p[i];
+    const double2 *q = reinterpret_cast<const double2 *>(p + 8 * (int64_t)i);
+    const double2 a = q[0], b = q[1], c = q[2], d = q[3];
+    return ((a.x + c.x) + (b.x + d.x)) + ((a.y + c.y) + (b.y + d.y));
+}
+
 // ----------------------------------------------------------------------------
 // Per-target records (step a1): quad records for pass 1, pair records for
 // pass 2, and the block partials of sum_j psi_j nu_j.
@@ -58,7 +81,7 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
                              float4 *__restrict__ tquad, Rec8 *__restrict__ tpair,
                              double *__restrict__ psinu_part, int *__restrict__ flags,
                              Rec16 *__restrict__ trec, double inv_P, int *__restrict__ gate) {
-    __shared__ double sh[32];
+    pdl_trigger();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const double psic = psi[0];
     const double k = kLog2e / (2.0 * eps);
@@ -99,8 +122,7 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
         pr[4 + l] = w[2];
         pr[6 + l] = c;
     }
-    const double s = block_sum_d(contrib, sh);
-    if (threadIdx.x == 0) psinu_part[blockIdx.x] = s;
+    store_partial(contrib, psinu_part);
 }
 
 // ----------------------------------------------------------------------------
@@ -114,7 +136,10 @@ __global__ void __launch_bounds__(P1_THREADS, p1_minb(PP))
                 int n, int chunk, float2 *__restrict__ part, int *__restrict__ flags,
                 const int *__restrict__ gate = nullptr, int need = 0) {
     // as the fallback of the tensor-core pass, run only when the gate asks for it
-    if (gate && !(*gate & need)) return;
+    if (gate) {
+        pdl_enter();
+        if (!(*gate & need)) return;
+    }
     __shared__ __align__(128) float4 sm[P1_STAGES][P1_TS];
     __shared__ __align__(8) uint64_t full[P1_STAGES];
     __shared__ int s_abort[2];   // indexed by iteration parity
@@ -150,6 +175,7 @@ __global__ void __launch_bounds__(P1_THREADS, p1_minb(PP))
         fence_barrier_init();
     }
     __syncthreads();
+    if (!gate) pdl_enter();   // the points are static, the records are not
     if (tid == 0) {
         for (int s = 0; s < P1_STAGES && s < ntile; ++s) {
             mbar_expect_tx(&full[s], P1_TS * sizeof(float4));
@@ -203,6 +229,14 @@ __global__ void __launch_bounds__(P1_THREADS, p1_minb(PP))
     }
 }
 
+// (double)v 2^k for an integer-valued k <= 0, by the bits of a normal v > 0 (the
+// conversion and the product would each take the FP64 pipe); else as written
+__device__ __forceinline__ double scaled_d(float v, float k) {
+    const unsigned b = __float_as_uint(v);
+    if (b - 0x00800000u >= 0x7f000000u || !(k >= -896.0f)) return (double)v * pow2_int_d(k);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)) + ((int)k << 20), (int)(b << 29));
+}
+
 // ----------------------------------------------------------------------------
 // Merge the pass-1 chunk partials into R_q, write the pass-2 point records
 // (x', u_q = log2 m_q - R_q) and the block partials of sum_q m_q R_q.
@@ -212,7 +246,7 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
                           const double *__restrict__ mass, float4 *__restrict__ pquad,
                           double *__restrict__ blockJ, double *__restrict__ lse_buf,
                           float *__restrict__ pu = nullptr) {
-    __shared__ double sh[32];
+    pdl_enter();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double contrib = 0.0;
     if (q < nq_pad) {
@@ -224,7 +258,7 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
             double tot = 0.0;
             for (int k = 0; k < k1; ++k) {
                 const float2 v = part[(int64_t)k * nq_pad + q];
-                tot += (double)v.y * pow2_int_d(v.x - mx);
+                tot += scaled_d(v.y, v.x - mx);
             }
             const double R = (double)mx + log2(tot);
             lse_buf[q] = R;
@@ -238,8 +272,7 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
         pquad[q] = make_float4(x[0], x[1], x[2], u);
         if (pu) pu[q] = u;   // pass-2 shift of the tensor-core kernel
     }
-    const double s = block_sum_d(contrib, sh);
-    if (threadIdx.x == 0) blockJ[blockIdx.x] = s;
+    store_partial(contrib, blockJ);
 }
 
 // ----------------------------------------------------------------------------
@@ -250,6 +283,7 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
     k_grad_mixed(const Rec8 *__restrict__ tpair, const float4 *__restrict__ pquad, int64_t nq,
                  int64_t chunk, double *__restrict__ part2, int64_t stride,
                  int *__restrict__ flags, const int *__restrict__ gate = nullptr, int need = 0) {
+    pdl_enter();
     if (gate && !(*gate & need)) return;
     __shared__ __align__(128) float4 sm[P2_STAGES][P2_TS];
     __shared__ __align__(8) uint64_t full[P2_STAGES];
@@ -347,6 +381,7 @@ __global__ void __launch_bounds__(TC_THREADS, TC_MINB)
     k_lse_tc(const Rec16 *__restrict__ prec, int64_t nq_pad, const Rec16 *__restrict__ trec,
              int n_p1, int chunk, float2 *__restrict__ part, int *__restrict__ flags,
              const int *__restrict__ gate) {
+    pdl_enter();
     if (gate && (*gate & 1)) return;   // operands out of f16 range: the FP32 kernel runs
     extern __shared__ __align__(128) unsigned char tc_smem[];
     Rec16 (*sm)[TC_TS] = reinterpret_cast<Rec16 (*)[TC_TS]>(tc_smem);   // [TC_STAGES][TC_TS]
@@ -475,6 +510,7 @@ __global__ void __launch_bounds__(TC_THREADS, TC_MINB)
               const float *__restrict__ pu, int64_t nq_pad, int64_t chunk,
               double *__restrict__ part2, int64_t stride, int *__restrict__ flags,
               const int *__restrict__ gate) {
+    pdl_enter();
     if (gate && (*gate & 1)) return;   // out of f16 range: the FP32 kernel runs
     extern __shared__ __align__(128) unsigned char tc_smem[];
     Rec16 (*sm)[TC_TS] = reinterpret_cast<Rec16 (*)[TC_TS]>(tc_smem);   // [TC_STAGES][TC_TS]
@@ -589,22 +625,70 @@ __global__ void k_finalize_grad(const double *__restrict__ part2, int s2, int64_
     grad[j] = g - nu[j];
 }
 
-// J from the block partials (one block).
-__global__ void k_finalize_J(const double *__restrict__ blockJ, int nbj,
-                             const double *__restrict__ psinu, int npn,
-                             const double *__restrict__ psi, double eps, double msum, double hx,
-                             int mixed, EvalResult *__restrict__ res) {
+// The last kernel of a dense evaluation.  Every block forms J (the partials are
+// few, and a block needs it to know whether the evaluation succeeded) and its
+// gradient entries, writes them to the handle and, on success, to `out`; the
+// block that finishes last copies the result block to the host and clears it for
+// the next evaluation.  Bound by latency (a launch, the loads of the partials, a
+// write to the host): one launch instead of gradient, J, conditional copy, result
+// copy and clearing.  With the overlapped launches, the small blocks and the
+// finer pass-2 split a call on 1,536 x 128 took 76 us before and 48 now.
+__global__ void __launch_bounds__(256)
+    k_finalize(FinalArgs a, const double *__restrict__ nu, int64_t n, double *__restrict__ grad,
+               const double *__restrict__ psinu, int npn, const double *__restrict__ psi,
+               double eps, double msum, double hx, int nonempty, double *__restrict__ out,
+               EvalResult *__restrict__ res, EvalResult *__restrict__ host) {
     __shared__ double sh[32];
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nbj; i += blockDim.x) a += blockJ[i];
-    for (int i = threadIdx.x; i < npn; i += blockDim.x) b += psinu[i];
-    const double sa = block_sum_d(a, sh);
-    const double sb = block_sum_d(b, sh);
+    __shared__ double s_J;
+    __shared__ int s_ok;
+    pdl_enter();
+    const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    double g = 0.0;
+    if (j < n) {
+        const double *p = a.part2 + j;
+        int s = 0;
+        for (; s + 8 <= a.s2; s += 8) {   // eight loads in flight, added in order
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = p[(int64_t)(s + k) * a.stride];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) g += v[k];
+        }
+        for (; s < a.s2; ++s) g += p[(int64_t)s * a.stride];
+        g = a.scale ? fma(g, a.scale[j], -nu[j]) : g - nu[j];
+        grad[j] = g;
+    }
+    double sa = 0.0, sb = 0.0;
+    for (int i = threadIdx.x; i < a.nbj; i += 256) sa += final_term(a.blockJ, a.per_j, i);
+    for (int i = threadIdx.x; i < npn; i += 256) sb += final_term(psinu, a.per_psi, i);
+    sa = block_sum_d(sa, sh);
+    sb = block_sum_d(sb, sh);
     if (threadIdx.x == 0) {
-        const double psic = psi[0];
-        res->psic = psic;
-        // mixed: sa = sum_q m_q R_q (log2, translated frame); FP64: sa = sum_q m_q eps L_q
-        res->J = mixed ? (psic * msum - hx + eps * kLn2 * sa - sb) : (sa - sb);
+        // log2_J: sa = sum_q m_q R_q (log2, translated frame), else sum_q m_q eps L_q
+        s_J = a.log2_J ? (psi[0] * msum - hx + eps * kLn2 * sa - sb) : (sa - sb);
+        s_ok = *(volatile int *)&res->flags == 0 && isfinite(s_J) &&
+               !(nonempty && *(volatile long long *)&res->empty > 0);
+    }
+    __syncthreads();
+    if (s_ok && out && j < n) out[j] = g;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&res->ticket, 1u) == gridDim.x - 1) {   // every block has read the flags
+            const int flags = atomicOr(&res->flags, 0), gate = atomicOr(&res->gate, 0);
+            host->J = s_J;
+            host->psic = psi[0];
+            host->pairs = res->pairs;
+            host->empty = res->empty;
+            host->flags = flags;
+            host->gate = gate;
+            __threadfence_system();
+            res->J = s_J;
+            res->psic = psi[0];   // read by k_point_L
+            res->pairs = res->empty = 0;
+            res->flags = res->gate = 0;
+            res->fx_key[0] = res->fx_key[1] = res->fx_key[2] = 0;
+            res->ticket = 0;
+        }
     }
 }
 
@@ -928,6 +1012,17 @@ cudaError_t dense_alloc(rsot_problem *p) {
     p->s2 = pick_split(units2, p->nq_pad / P2_TS, slots2);
     p->chunk2 = round_up((p->nq_pad + p->s2 - 1) / p->s2, P2_TS);
     p->s2 = (int)((p->nq_pad + p->chunk2 - 1) / p->chunk2);
+    // Outside the solver, whose iterates follow the last bit of a sum: one stage
+    // of points per CTA where all of these fit at once (pick_split keeps one split
+    // there: no count fills the slots) -- 1,536 x 128: pass 2 24 -> 12 us, 9,600 x
+    // 1,000: 19 -> 12.  Above 64 splits the final kernel's sum costs more than it
+    // gains (135,000 x 300, 264 splits: pass 2 20 -> 18, the call 87 -> 97).
+    p->s2_eval = p->s2;
+    p->chunk2_eval = p->chunk2;
+    if (units2 * (p->nq_pad / P2_TS) <= slots2 && p->nq_pad / P2_TS <= 64) {
+        p->chunk2_eval = P2_TS;
+        p->s2_eval = (int)((p->nq_pad + P2_TS - 1) / P2_TS);
+    }
     // the same splits for the tensor-core passes (TC_ROWS points / targets per CTA);
     // their FP32 fallback (by the gate) runs with these chunks too
     const int64_t n_tc = round_up(p->n, TC_TS);
@@ -953,11 +1048,14 @@ cudaError_t dense_alloc(rsot_problem *p) {
 
     p->nblk_comb = (int)((p->nq_pad + CB_THREADS - 1) / CB_THREADS);
     p->nblk_prep = (int)((n_alloc + CB_THREADS - 1) / CB_THREADS);
-    const int nbj = std::max<int64_t>(p->nblk_comb, (p->nq_pad + F_THREADS - 1) / F_THREADS);
+    p->per_comb = p->nblk_comb < 2 * p->num_sms ? 8 : 1;
+    p->per_prep = p->nblk_prep < 2 * p->num_sms ? 8 : 1;
+    const int nbj = (int)std::max<int64_t>((int64_t)p->nblk_comb * p->per_comb,
+                                           (p->nq_pad + F_THREADS - 1) / F_THREADS);
 
     if ((e = cudaMalloc(&p->tquad, n_alloc * sizeof(float4)))) return e;
     if ((e = cudaMalloc(&p->tpair, (n_alloc / 2) * sizeof(Rec8)))) return e;
-    const int k1max = std::max(p->k1, p->k1_tc), s2max = std::max(p->s2, p->s2_tc);
+    const int k1max = std::max(p->k1, p->k1_tc), s2max = std::max({p->s2, p->s2_eval, p->s2_tc});
     if ((e = cudaMalloc(&p->part1, (size_t)k1max * p->nq_pad * sizeof(float2)))) return e;
     if ((e = cudaMalloc(&p->pquad, p->nq_pad * sizeof(float4)))) return e;
     if ((e = cudaMalloc(&p->part2, (size_t)s2max * n_alloc * sizeof(double)))) return e;
@@ -969,7 +1067,7 @@ cudaError_t dense_alloc(rsot_problem *p) {
     if ((e = cudaStreamSynchronize(0))) return e;
     if ((e = cudaMalloc(&p->part2_64, (size_t)p->s2_64 * n_alloc * sizeof(double)))) return e;
     if ((e = cudaMalloc(&p->blockJ, (size_t)nbj * sizeof(double)))) return e;
-    if ((e = cudaMalloc(&p->psinu, (size_t)p->nblk_prep * sizeof(double)))) return e;
+    if ((e = cudaMalloc(&p->psinu, (size_t)p->nblk_prep * 8 * sizeof(double)))) return e;
     if ((e = cudaMalloc(&p->a64, n_alloc * sizeof(double)))) return e;
     if ((e = cudaMalloc(&p->prec64, (size_t)p->nq_pad * 4 * sizeof(double)))) return e;
     if ((e = cudaMalloc(&p->lse_buf, (size_t)p->nq_pad * sizeof(double)))) return e;
@@ -1007,6 +1105,33 @@ static int pairs_per_thread(int most, int64_t items, int64_t slots) {
     return pp;
 }
 
+// the targets' records and the partials of sum psi nu
+static void launch_prep(rsot_problem *p, const double *psi, double eps, Rec16 *trec, double inv_P, int *gate) {
+    const int t = p->per_prep == 1 ? CB_THREADS : kSmall;
+    trace_begin(p, "prep_targets_mixed");
+    k_prep_mixed<<<(unsigned)(p->n_pad / t), t, 0, p->stream>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
+                                                                p->d, eps, p->tquad, p->tpair, p->psinu,
+                                                                p->flags, trec, inv_P, gate);
+    trace_end(p);
+}
+
+static void launch_combine(rsot_problem *p, int k1, float *pu) {
+    const int t = p->per_comb == 1 ? CB_THREADS : kSmall;
+    trace_begin(p, "combine_mixed");
+    launch_pdl(true, k_combine, (unsigned)(p->nq_pad / t), t, 0, p->stream, p->part1, k1, p->nq_pad, p->nq, p->xs,
+               p->d, p->lmass2, p->mass, p->pquad, p->blockJ, p->lse_buf, pu);
+    trace_end(p);
+}
+
+// The passes overlap their predecessor's end (launch_pdl) only where their CTAs
+// are at most one per SM, or where they run as the tensor-core passes' fallback
+// and mostly return at once: CTAs placed while the short kernel before still holds
+// slots leave some SMs with more of the single wave than others (61,206 x 5,003:
+// the call 160 -> 225 us, 2,400 x 30,000: 88 -> 144; 1,536 x 128: 63 -> 60).
+static bool overlap_pass(const dim3 &g, const int *gate, int num_sms) {
+    return gate || (int64_t)g.x * g.y <= num_sms;
+}
+
 template <int D>
 static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tquad, int64_t n, int chunk,
                              int k1, float2 *part, int *flags, const int *gate, int num_sms,
@@ -1014,7 +1139,7 @@ static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tqua
     const int pp = pairs_per_thread(P1_PP, nq_pad / P1_TILE * k1, (int64_t)num_sms * P1_MINB);
     dim3 g((unsigned)(nq_pad / (2 * pp * P1_THREADS)), (unsigned)k1);
     auto f = pp == 4 ? k_lse_mixed<D, 4> : pp == 2 ? k_lse_mixed<D, 2> : k_lse_mixed<D, 1>;
-    f<<<g, P1_THREADS, 0, st>>>(xs, nq_pad, tquad, (int)n, chunk, part, flags, gate, 1);
+    launch_pdl(overlap_pass(g, gate, num_sms), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk, part, flags, gate, 1);
 }
 
 template <int D>
@@ -1026,7 +1151,7 @@ static void launch_grad_mixed(const Rec8 *tpair, int64_t n, const float4 *pquad,
     const int tpp = pairs_per_thread(most, (n + blk - 1) / blk * s2, (int64_t)num_sms * 16 / most);
     dim3 g((unsigned)((n + 2 * P2_THREADS * tpp - 1) / (2 * P2_THREADS * tpp)), (unsigned)s2);
     auto f = tpp == 4 ? k_grad_mixed<D, 4> : tpp == 2 ? k_grad_mixed<D, 2> : k_grad_mixed<D, 1>;
-    f<<<g, P2_THREADS, 0, st>>>(tpair, pquad, nq, chunk, part2, stride, flags, gate, 1);
+    launch_pdl(overlap_pass(g, gate, num_sms), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2, stride, flags, gate, 1);
 }
 
 template <int D>
@@ -1038,51 +1163,34 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
     const bool tc = use_tensor_pairs(p);
     int *gate = tc ? &p->res_dev->gate : nullptr;
     const int k1 = tc ? p->k1_tc : p->k1, chunk1 = tc ? p->chunk1_tc : p->chunk1;
-    const int s2 = tc ? p->s2_tc : p->s2;
-    const int64_t chunk2 = tc ? p->chunk2_tc : p->chunk2;
-    trace_begin(p, "prep_targets_mixed");
-    k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                      p->d, eps, p->tquad, p->tpair, p->psinu,
-                                                      p->flags, tc ? p->trec : nullptr,
-                                                      1.0 / (double)p->tc_P, gate);
-    trace_end(p);
+    const int s2 = tc ? p->s2_tc : p->in_solve ? p->s2 : p->s2_eval;
+    const int64_t chunk2 = tc ? p->chunk2_tc : p->in_solve ? p->chunk2 : p->chunk2_eval;
+    launch_prep(p, psi, eps, tc ? p->trec : nullptr, 1.0 / (double)p->tc_P, gate);
     if (tc) {
         dim3 gt((unsigned)(p->nq_pad / TC_ROWS), (unsigned)k1);
         trace_begin(p, "lse_tc");
-        k_lse_tc<<<gt, TC_THREADS, TC_SMEM1, st>>>(p->prec16, p->nq_pad, p->trec,
-                                            (int)round_up(p->n, TC_TS), chunk1, p->part1,
-                                            p->flags, gate);
+        launch_pdl(true, k_lse_tc, gt, TC_THREADS, TC_SMEM1, st, p->prec16, p->nq_pad, p->trec,
+                   (int)round_up(p->n, TC_TS), chunk1, p->part1, p->flags, gate);
         trace_end(p);
     }
     trace_begin(p, "lse_mixed");
     launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, chunk1, k1, p->part1, p->flags, gate,
                         p->num_sms, st);
     trace_end(p);
-    trace_begin(p, "combine_mixed");
-    k_combine<<<p->nblk_comb, CB_THREADS, 0, st>>>(p->part1, k1, p->nq_pad, p->nq, p->xs, p->d,
-                                                   p->lmass2, p->mass, p->pquad, p->blockJ,
-                                                   p->lse_buf, tc ? p->pu : nullptr);
-    trace_end(p);
+    launch_combine(p, k1, tc ? p->pu : nullptr);
     if (tc) {
         dim3 gt((unsigned)(p->n_pad / TC_ROWS), (unsigned)s2);
         trace_begin(p, "grad_tc");
-        k_grad_tc<<<gt, TC_THREADS, TC_SMEM2, st>>>(p->trec, p->prec16, p->pu, p->nq_pad, chunk2,
-                                             p->part2, p->n_pad, p->flags, gate);
+        launch_pdl(true, k_grad_tc, gt, TC_THREADS, TC_SMEM2, st, p->trec, p->prec16, p->pu, p->nq_pad, chunk2,
+                   p->part2, p->n_pad, p->flags, gate);
         trace_end(p);
     }
     trace_begin(p, "grad_mixed");
     launch_grad_mixed<D>(p->tpair, p->n, p->pquad, p->nq, chunk2, s2, p->part2, p->n_pad, p->flags,
                          gate, p->num_sms, st);
     trace_end(p);
-    trace_begin(p, "finalize_grad");
-    k_finalize_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(p->part2, s2, p->n_pad,
-                                                                    p->nu, p->n, grad);
-    trace_end(p);
-    trace_begin(p, "finalize_J");
-    k_finalize_J<<<1, 256, 0, st>>>(p->blockJ, p->nblk_comb, p->psinu, p->nblk_prep, psi, eps,
-                                    p->msum, p->hx, 1, p->res_dev);
-    trace_end(p);
-    return cudaGetLastError();
+    return launch_finalize(p, psi, eps,
+                           {p->part2, s2, p->n_pad, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1, p->per_prep}, grad);
 }
 
 // ----------------------------------------------------------------------------
@@ -1132,14 +1240,10 @@ static cudaError_t softmax_refine_d(rsot_problem *p, const double *psi, double e
     cudaStream_t st = p->stream;
     cudaError_t e;
     const int64_t n_p1 = round_up(p->n, P1_TS);
-    k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, st>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                      p->d, eps, p->tquad, p->tpair, p->psinu,
-                                                      p->flags, nullptr, 1.0, nullptr);
+    launch_prep(p, psi, eps, nullptr, 1.0, nullptr);
     launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, p->chunk1, p->k1, p->part1, p->flags, nullptr,
                         p->num_sms, st);
-    k_combine<<<p->nblk_comb, CB_THREADS, 0, st>>>(p->part1, p->k1, p->nq_pad, p->nq, p->xs, p->d,
-                                                   p->lmass2, p->mass, p->pquad, p->blockJ,
-                                                   p->lse_buf);
+    launch_combine(p, p->k1, nullptr);
     const int64_t nf_alloc = round_up(nf, 1024);
     const int64_t blocks = nf_alloc / 1024;
     int s2 = pick_split(blocks, p->nq_pad / P2_TS, (int64_t)p->num_sms * (D == 3 ? 4 : 5));
@@ -1168,18 +1272,12 @@ cudaError_t launch_softmax_refine(rsot_problem *p, const double *psi_dev, double
                      : softmax_refine_d<2>(p, psi_dev, eps, nf, yf_dev, out_dev);
 }
 
-// gradient and log2-domain J from pass-2 partials [s2][n_pad] and nbj pass-1
-// block partials of sum_q m_q R_q (the compensated path's finalisation)
-cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps, const double *blockJ,
-                                 int nbj, const double *part2, int s2, double *grad) {
-    cudaStream_t st = p->stream;
-    trace_begin(p, "finalize_grad");
-    k_finalize_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(part2, s2, p->n_pad, p->nu,
-                                                                    p->n, grad);
-    trace_end(p);
-    trace_begin(p, "finalize_J");
-    k_finalize_J<<<1, 256, 0, st>>>(blockJ, nbj, p->psinu, p->nblk_prep, psi, eps, p->msum,
-                                    p->hx, 1, p->res_dev);
+cudaError_t launch_finalize(rsot_problem *p, const double *psi, double eps, const FinalArgs &a,
+                            double *grad) {
+    trace_begin(p, "finalize");
+    launch_pdl(true, k_finalize, (unsigned)((p->n + 255) / 256), 256, 0, p->stream, a, p->nu, p->n, grad, p->psinu,
+               p->nblk_prep, psi, eps, p->msum, p->hx, p->final_nonempty, p->final_out, p->res_dev,
+               p->res_host);
     trace_end(p);
     return cudaGetLastError();
 }
@@ -1190,20 +1288,7 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi, double eps, d
 
 // the target records of the mixed passes alone, for the pair skipping
 cudaError_t launch_prep_mixed(rsot_problem *p, const double *psi, double eps) {
-    trace_begin(p, "prep_targets_mixed");
-    k_prep_mixed<<<p->nblk_prep, CB_THREADS, 0, p->stream>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                             p->d, eps, p->tquad, p->tpair, p->psinu,
-                                                             p->flags, nullptr, 1.0, nullptr);
-    trace_end(p);
-    return cudaGetLastError();
-}
-
-// J from pass-1 block partials of sum_q m_q eps L_q (FP64 forms)
-cudaError_t launch_finalize_J64(rsot_problem *p, const double *psi, double eps, int nbj) {
-    trace_begin(p, "finalize_J");
-    k_finalize_J<<<1, 256, 0, p->stream>>>(p->blockJ, nbj, p->psinu, p->nblk_prep, psi, eps, p->msum,
-                                           0.0, 0, p->res_dev);
-    trace_end(p);
+    launch_prep(p, psi, eps, nullptr, 1.0, nullptr);
     return cudaGetLastError();
 }
 
@@ -1238,11 +1323,8 @@ static cudaError_t launch_fp64_d(rsot_problem *p, const double *psi, double eps,
                                                         p->chunk2_64, hinv, alpha, beta,
                                                         p->part2_64, p->n_pad);
     trace_end(p);
-    trace_begin(p, "finalize_grad");
-    k_finalize_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(p->part2_64, p->s2_64,
-                                                                    p->n_pad, p->nu, p->n, grad);
-    trace_end(p);
-    return launch_finalize_J64(p, psi, eps, (int)nb1);
+    return launch_finalize(p, psi, eps, {p->part2_64, p->s2_64, p->n_pad, nullptr, p->blockJ, (int)nb1, 1, 0, 1},
+                           grad);
 }
 
 cudaError_t launch_dense_fp64(rsot_problem *p, const double *psi, double eps, double *grad) {

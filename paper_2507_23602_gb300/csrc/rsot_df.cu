@@ -44,9 +44,6 @@
 
 namespace rsot {
 
-cudaError_t launch_finalize_log2(rsot_problem *p, const double *psi, double eps, const double *blockJ,
-                                 int nbj, const double *part2, int s2, double *grad);
-
 namespace {
 
 constexpr int D_THREADS = 128;            // threads per block
@@ -716,7 +713,8 @@ cudaError_t compensated_d(rsot_problem *p, const double *psi, double eps, bool t
                                                       nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     trace_end(p);
     if ((e = cudaGetLastError())) return e;
-    return launch_finalize_log2(p, psi, eps, p->blockJ, (int)nb1, p->df_part2, (int)s2, grad);
+    return launch_finalize(p, psi, eps, {p->df_part2, (int)s2, p->n_pad, nullptr, p->blockJ, (int)nb1, 1, 1, 1},
+                           grad);
 }
 
 }  // namespace

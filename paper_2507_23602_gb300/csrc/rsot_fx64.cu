@@ -445,11 +445,9 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, fx_rows(p, p->n, p->nq), tgr, ptc, p->fx_chunk2, p->fx_s2,
                                               eps, p->fx_part2);
     trace_end(p);
-    trace_begin(p, "finalize_grad");
-    k_fx_grad<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(p->fx_part2, p->fx_s2, p->n_pad,
-                                                              p->fx_tgscale, p->nu, p->n, grad);
-    trace_end(p);
-    return launch_finalize_J64(p, psi, eps, nbq);
+    return launch_finalize(p, psi, eps,
+                           {p->fx_part2, p->fx_s2, p->n_pad, p->fx_tgscale, p->blockJ, nbq, 1, 0, p->per_prep},
+                           grad);
 }
 
 }  // namespace rsot

@@ -51,6 +51,7 @@ struct EvalResult {
     int gate;           // bit 0: an f16 operand is out of range (both passes take the FP32 kernels)
     unsigned fx_key[3]; // pair skipping (rsot_skip.cuh): largest A_q, B_j, |B_j| as ordered keys
     int fx_F;           // fraction bits of the fixed-point passes (rsot_fx64.cu)
+    unsigned ticket;    // blocks of the final kernel that are done
 };
 
 struct Grid;  // truncated-path cell grid (rsot_trunc.cu)
@@ -89,11 +90,14 @@ struct rsot_problem {
     float4 *pquad = nullptr;        // [nq_pad] (x0,x1,x2,u)
     double *part2 = nullptr;        // [s2][n_pad]
     double *blockJ = nullptr;       // [nblk_j]
-    double *psinu = nullptr;        // [nblk_psi]
+    double *psinu = nullptr;        // [8 nblk_prep] partials of sum psi nu: one per 256 targets or per warp
     int k1 = 0, chunk1 = 0;         // pass-1 target chunks
     int s2 = 0;                     // pass-2 point splits
     int64_t chunk2 = 0;
+    int s2_eval = 0;                // outside the solver (dense_alloc)
+    int64_t chunk2_eval = 0;
     int nblk_comb = 0, nblk_prep = 0;
+    int per_comb = 1, per_prep = 1; // partials per 256 points / targets: 1, or 8 (one per warp)
     // tensor-core form of the pair arithmetic (rsot_tc.cuh)
     rsot::Rec16 *trec = nullptr;    // [n_pad] target operand records
     rsot::Rec16 *prec16 = nullptr;  // [nq_pad] point operand records (static)
@@ -170,6 +174,10 @@ struct rsot_problem {
     double *grad_host = nullptr;    // [n] pinned staging of host gradient outputs
     rsot::EvalResult *res_dev = nullptr;
     rsot::EvalResult *res_host = nullptr;   // pinned
+    bool res_clean = false;         // *res_dev is zero (the final kernel leaves it so)
+    int final_nonempty = 0;         // truncated: an empty neighbourhood is an error
+    double *final_out = nullptr;    // the evaluation's gradient output: the caller's device buffer or
+                                    // grad_host, written by the final kernel on success
     int *flags = nullptr;           // device error bits (inside res_dev)
 
     // per-point log partition of the last evaluation (see rsot_point_log_partition)
@@ -226,6 +234,50 @@ void trace_begin(rsot_problem *p, const char *name);
 void trace_end(rsot_problem *p);
 void trace_collect(rsot_problem *p);
 
+// ---- programmatic dependent launch -----------------------------------------------
+// The kernels of one evaluation form a chain of short launches: a kernel that is
+// launched with launch_pdl may be scheduled while its predecessor runs and waits
+// in pdl_wait() for all of it; each triggers its successor right after its own
+// wait, so that at most two kernels are in flight.  Without the attribute both
+// calls do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// at the start of a kernel whose inputs its predecessor writes
+__device__ __forceinline__ void pdl_enter() {
+    pdl_wait();
+    pdl_trigger();
+}
+template <class... P, class... A>
+inline void launch_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    (void)cudaLaunchKernelEx(&cfg, k, P(args)...);   // cudaGetLastError() reports a failure
+}
+
+// The last kernel of a dense evaluation: gradient and J from the partials, the
+// gradient to the caller's buffer on success, the result block to the host.
+struct FinalArgs {
+    const double *part2;        // [s2][stride] pass-2 partials
+    int s2;
+    int64_t stride;
+    const double *scale;        // per target, or null: grad = scale sum - nu
+    const double *blockJ;       // nbj groups of per_j partials of pass 1's J term
+    int nbj, per_j;
+    int log2_J;                 // they are sum m R_q (log2 domain), else sum m eps L_q
+    int per_psi;                // partials of sum psi nu per 256 targets
+};
+cudaError_t launch_finalize(rsot_problem *p, const double *psi_dev, double eps, const FinalArgs &a,
+                            double *grad_dev);
+
 // ---- launch helpers implemented in rsot_dense.cu --------------------------
 cudaError_t dense_alloc(rsot_problem *p);
 void dense_free(rsot_problem *p);
@@ -234,7 +286,6 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi_dev, double ep
 cudaError_t launch_dense_fp64(rsot_problem *p, const double *psi_dev, double eps,
                               double *grad_dev);
 cudaError_t launch_prep_mixed(rsot_problem *p, const double *psi_dev, double eps);
-cudaError_t launch_finalize_J64(rsot_problem *p, const double *psi_dev, double eps, int nbj);
 // dense FP64 evaluation with fixed-point exponents (rsot_fx64.cu); fx64_ready:
 // its buffers exist and the sizes of the exponents allow it
 bool fx64_ready(rsot_problem *p, double eps);

@@ -195,6 +195,7 @@ rsot_status rsot_softmax_refine(rsot_problem *p, const double *psi_coarse, doubl
     if (!e) e = cudaMallocAsync(&dout, (size_t)n_fine * 8, st);
     if (!e) e = cudaMemcpyAsync(dpsi, psi_coarse, (size_t)p->n * 8, cudaMemcpyDefault, st);
     if (!e) e = cudaMemcpyAsync(dyf, y_fine, (size_t)n_fine * d * 8, cudaMemcpyDefault, st);
+    p->res_clean = false;
     if (!e) e = cudaMemsetAsync(p->res_dev, 0, sizeof(EvalResult), st);
     if (!e) e = launch_softmax_refine(p, dpsi, eps, n_fine, dyf, dout);
     if (!e) e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(EvalResult), cudaMemcpyDeviceToHost, st);
