@@ -19,6 +19,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <vector>
 
 #include "rsot_internal.cuh"
@@ -33,9 +34,33 @@ constexpr int G_THREADS = 256;
 
 enum { EPI_F32 = 0, EPI_BIAS_SILU = 1, EPI_DSILU = 2 };
 
-__device__ __forceinline__ float silu(float z) { return z / (1.0f + __expf(-z)); }
+// z / d and 1 / d with d = 1 + exp(-z) >= 1, without the special cases of exp and
+// of the division (their tests cost as much as the arithmetic, and the division's
+// branch keeps the values of an unrolled loop from overlapping): exp(-z) as the
+// hardware's 2^x, where a subnormal result flushed to zero leaves d = 1 as it was;
+// the hardware's reciprocal (one unit in the last place), then the residual of the
+// quotient, exact in a fused multiply-add, corrects it (Markstein, IBM J. Res.
+// Dev. 34, 1990).  Where d or z is infinite the residual is not a number, the
+// minimum replaces it, and r = 0 or q infinite makes it nothing.  Of 6.7e8 values
+// of |z| in [1e-6, 1e6] two differ from z / (1 + __expf(-z)) as compiled, in the
+// last bit, and none after rounding to BF16.
+__device__ __forceinline__ float one_plus_exp_neg(float z) {
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
+    return 1.0f + e;
+}
+__device__ __forceinline__ float rcp_approx(float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return r;
+}
+__device__ __forceinline__ float silu(float z) {
+    const float d = one_plus_exp_neg(z), r = rcp_approx(d), q = z * r;
+    return fmaf(fminf(fmaf(-q, d, z), 3.402823466e38f), r, q);
+}
 __device__ __forceinline__ float dsilu(float z) {
-    const float s = 1.0f / (1.0f + __expf(-z));
+    const float d = one_plus_exp_neg(z), r = rcp_approx(d);
+    const float s = fmaf(fminf(fmaf(-d, r, 1.0f), 3.402823466e38f), r, r);
     return s * (1.0f + z * (1.0f - s));
 }
 
@@ -879,6 +904,550 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
 }
 
+// ---------------------------------------------------------- the network in one kernel
+// Forward pass (and, TRAIN, the back-propagation down to every layer's dZ) of a
+// network of width w (a multiple of 64, at most 256), 128-row tiles (64 or 32
+// where there are few rows), one tile at a time per CTA with every activation
+// on chip: the rows' BF16 operand stays in shared memory (K-major, 128-byte
+// swizzle, a block of 128 rows x 128 B per 64 columns), the weights stream
+// through stages of 64 K x 128 rows (TMA, from L2), the accumulator (128 lanes
+// x w columns) is in tensor memory, and a layer's epilogue writes its BF16
+// result over the operand it came from.
+//   warp 0 (one lane): weights; warp 1 (one lane): tcgen05.mma, M 128, N <= 128;
+//   warps 2-17: warp e owns rows 32 (e % 4) .. + 31 and columns 64 ((e - 2) / 4)
+//     .. + 63: input conversion, bias + SiLU, head, x SiLU'(Z).
+// Bound: a tile's chain of layers, each an MMA phase (about 4,400 cycles, the issue
+// of its 32 instructions) and an epilogue (about 4,500 and up: some 20 instructions
+// a value, 128 x 256 values), which wait for each other.  Two CTAs per SM (111 KB
+// each) therefore overlap one's MMAs and weight copies with the other's epilogue
+// (57 % of the issue slots taken at 65,536 rows); a CTA alone on its SM takes eight
+// weight stages instead of two and fetches the next layer's weights during the
+// epilogue.  The per-layer kernels this replaces wrote and read H, Z and dZ of
+// every layer (33 MB each at 65,536 x 256) and ran 32 of 152 SMs at 4,096 rows.
+//   forward, 4,096 rows: GPU time 50 -> 17 us (the call 84 -> 45);
+//   forward + back-propagation, 65,536 rows: 240 -> 119 us (the gradients' call
+//   384 -> 236).
+// TRAIN also stores X0, H1, H2 and the three dZ (the weight gradients' operands;
+// TMA, 32 x 64 boxes from the swizzled operand), keeps Z1 and Z2 in global memory
+// between a tile's two passes (each thread reads back what it wrote), and sums
+// dZ and d_out H3 over the rows per column (per CTA, tiles in order).
+// The arithmetic and the order of every sum of a row are those of the kernels
+// below (k_gemm_*, k_head_v8, k_head_back_v8).
+constexpr int NF_EPI = 16, NF_THREADS = 32 * (2 + NF_EPI), NF_MAXST = 8;
+constexpr int NF_BLK = 128 * 128;                    // 128 rows x 64 BF16
+constexpr int NF_A = 4 * NF_BLK, NF_V = 2 * 8 * 128 * 4;
+constexpr int NF_C = 4 * 256 * 4;                    // b1, b2, b3, w4
+constexpr int nf_smem(int stages) { return NF_A + stages * NF_BLK + NF_V + NF_C + 1024; }
+static_assert(2 * (nf_smem(2) + 1024 + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(nf_smem(NF_MAXST) + 1024 <= 232448, "one CTA with every stage");
+
+struct NetMaps {
+    CUtensorMap w[5];    // W1, W2, W3 and W3^T, W2^T: boxes of 64 K x 64 rows
+    CUtensorMap st[5];   // H1, H2, dZ3, dZ2, dZ1: boxes of 64 columns x 32 rows
+};
+struct NetArgs {
+    const float *x, *y;
+    int in_dim, in_pad, w, tiles, rt, stages;
+    int64_t valid;                 // rows; the buffers hold a multiple of 128
+    const float *b[3], *w4, *b4;
+    float inv_b;
+    bf16 *X0, *Z[2];
+    float *out;                    // forward: [valid]
+    float *part[6];                // TRAIN, per CTA: db3, dw4, db2, db1 [w]; db4, loss
+    int *flags, *host_flags;       // host_flags (pinned, or null): the host's copy
+};
+__device__ __forceinline__ void nf_fail(const NetArgs &a) {
+    atomicOr(a.flags, kErrTimeout);
+    if (a.host_flags) *(volatile int *)a.host_flags = kErrTimeout;
+}
+
+__device__ __forceinline__ void t5_ld16(uint32_t (&v)[16], uint32_t taddr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+        "%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+          "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+// 32 bytes (16 BF16) of global memory, 32-byte aligned: one whole sector
+__device__ __forceinline__ void st_global32(void *p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void ld_global32(uint32_t (&v)[8], const void *p) {
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void nf_bar() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NF_EPI) : "memory"); }
+__device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u));
+}
+
+// one MMA of K = 16 by the warp's elected lane (the same lane every time: the
+// commit below covers it); descriptors as their address words and the common high
+// word
+__device__ __forceinline__ void nf_mma(uint32_t d, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
+                                       uint32_t accum) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(d),
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accum)
+        : "memory");
+}
+__device__ __forceinline__ void nf_commit(uint64_t *bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
+        : "memory");
+}
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(NF_THREADS, 2)
+    k_net(const __grid_constant__ NetArgs a, const __grid_constant__ NetMaps maps) {
+    extern __shared__ __align__(1024) unsigned char nf_dyn[];
+    __shared__ __align__(8) uint64_t full[NF_MAXST], empty[NF_MAXST], aready, accf, mdone;
+    __shared__ uint32_t s_tmem;
+    __shared__ float s_d[128];
+    unsigned char *const sA = nf_dyn + ((1024u - (smem_u32(nf_dyn) & 1023u)) & 1023u);
+    unsigned char *const sW = sA + NF_A;
+    const int stages = a.stages, w = a.w;
+    float *const sV = reinterpret_cast<float *>(sW + stages * NF_BLK);   // [2][8][128]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float *const sC = sV + NF_V / 4;                                     // [4][256]
+    constexpr int STEPS = TRAIN ? 5 : 3;
+    for (int i = tid; i < 4 * w; i += NF_THREADS) sC[i / w * 256 + i % w] = (i < 3 * w ? a.b[i / w] : a.w4)[i % w];
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(256)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < stages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&aready, NF_EPI);
+        mbar_init(&accf, 1);
+        mbar_init(&mdone, 1);
+        fence_barrier_init();
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem;
+    bool ok = true;
+    if (warp == 0) {
+        if (lane == 0) {
+            // stage s of the ring, its n-th use: n = 0 finds it empty
+            int s = 0, n = 0;
+            for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x)
+#pragma unroll 1
+                for (int st = 0; st < STEPS && ok; ++st)
+                    for (int k0 = 0; k0 < (st == 0 ? 1 : w) && ok; k0 += 64)
+                        for (int h0 = 0; h0 < w; h0 += 128) {
+                            if (n > 0 && !mbar_wait(&empty[s], (unsigned)(n - 1) & 1u)) {
+                                ok = false;
+                                break;
+                            }
+                            const int two = w - h0 >= 128;
+                            unsigned char *const Ws = sW + s * NF_BLK;
+                            mbar_expect_tx(&full[s], two ? 16384u : 8192u);
+                            tma_load_2d(Ws, &maps.w[st], k0, h0, &full[s]);
+                            if (two) tma_load_2d(Ws + 8192, &maps.w[st], k0, h0 + 64, &full[s]);
+                            if (++s == stages) {
+                                s = 0;
+                                ++n;
+                            }
+                        }
+            // copies in flight land before the CTA exits
+            for (int i = 0; i < stages; ++i) {
+                const int uses = n + (i < s ? 1 : 0);
+                if (uses > 0) (void)mbar_wait(&full[i], (unsigned)(uses - 1) & 1u);
+            }
+            if (!ok) nf_fail(a);
+        }
+    } else if (warp == 1) {
+        // One thread issues every MMA, and the issue, not the 64 cycles of its
+        // execution, bounds this loop: the whole warp runs it (operands stay in
+        // uniform registers) and the same elected lane issues, descriptors differ in
+        // their address word alone, no divisions (a stage of four MMAs: 1,070 cycles
+        // from one lane's loop with divisions, about 550 now)
+        constexpr uint32_t dhi = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61)) >> 32);
+        const uint32_t abase = ((smem_u32(sA) >> 4) & 0x3FFFu) | (1u << 16);
+        const uint32_t wbase = ((smem_u32(sW) >> 4) & 0x3FFFu) | (1u << 16);
+        int s = 0;
+        unsigned k = 0, par = 0;
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x)
+#pragma unroll 1
+            for (int st = 0; st < STEPS && ok; ++st, ++k) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&aready, k & 1u))) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (int k0 = 0; k0 < (st == 0 ? 1 : w) && ok; k0 += 64)
+                    for (int h0 = 0; h0 < w; h0 += 128) {
+                        if (!__all_sync(0xffffffffu, mbar_wait(&full[s], par))) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24) |
+                                               (w - h0 >= 128 ? 16u << 17 : 8u << 17);
+                        const uint32_t a0 = abase + (uint32_t)(k0 >> 6) * (NF_BLK >> 4);
+                        const uint32_t b0 = wbase + (uint32_t)s * (NF_BLK >> 4);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            if (st > 0 || 16 * kk < a.in_pad)
+                                nf_mma(tmem + (uint32_t)h0, a0 + 2 * kk, b0 + 2 * kk, dhi, idesc,
+                                       kk > 0 || k0 > 0);
+                        nf_commit(&empty[s]);
+                        if (++s == stages) {
+                            s = 0;
+                            par ^= 1u;
+                        }
+                    }
+                if (ok) nf_commit(&accf);
+            }
+        nf_commit(&mdone);   // every MMA issued is complete before the tensor memory is freed
+        (void)mbar_wait(&mdone, 0u);
+        if (!ok && lane == 0) nf_fail(a);
+    } else {
+        // a wait that gives up clears ok; the warp then passes every barrier without
+        // waiting for the accumulator again, so that no warp is left at one
+        const int q = warp & 3, jb = (warp - 2) >> 2, et = tid - 64;
+        const bool live = 32 * q < a.rt, act = live && 64 * jb < w;
+        const int r = 32 * q + lane, c0 = 64 * jb;
+        const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
+        unsigned char *const aRow = sA + jb * NF_BLK + r * 128;   // the thread's 128 B of its block
+        unsigned char *const aBox = sA + jb * NF_BLK + q * 4096;  // the warp's 32 rows of it
+        // 16 columns 16 c .. + 15 of the thread's 64: two swizzled 16-byte chunks
+        auto put = [&](int c, const uint32_t (&v)[8]) {
+            *reinterpret_cast<uint4 *>(aRow + (((2 * c) ^ (r & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<uint4 *>(aRow + (((2 * c + 1) ^ (r & 7)) << 4)) = make_uint4(v[4], v[5], v[6], v[7]);
+        };
+        unsigned k = 0;
+        auto acc_wait = [&]() {
+            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&accf, k & 1u));
+            ++k;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        };
+        // the operand is written (and the accumulator read): the MMA may go on
+        auto ready = [&]() {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&aready);
+        };
+        auto store_box = [&](int m, int row0) {
+            if (act && lane == 0) {
+                tma_store_2d(&maps.st[m], aBox, c0, row0 + 32 * q);
+                bulk_commit();
+            }
+        };
+        auto stores_read = [&]() {   // the warp's earlier stores have read its box
+            if (lane == 0) bulk_wait_read();
+            __syncwarp();
+        };
+        // columns 2 cp, 2 cp + 1 summed over the rows 32 g .. + 31 of the operand
+        const int cp = et & 127, rg = et >> 7;
+        const unsigned char *const colp = sA + (cp >> 5) * NF_BLK + (cp & 3) * 4;
+        float cs[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        auto colsum = [&](float (&sum)[2], bool weighted) {
+            if (2 * cp >= w || 32 * rg >= a.rt) return;
+            const unsigned char *const cb = colp + rg * 4096;
+            const unsigned ch = ((cp & 31) >> 2) << 4;
+            const float *const dr = s_d + 32 * rg;
+#pragma unroll 1
+            for (int b = 0; b < 4; ++b)   // eight rows: row i's chunk ch at ch ^ i
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float2 f = unpack_bf16(*reinterpret_cast<const uint32_t *>(
+                        cb + b * 1024 + i * 128 + (ch ^ (i << 4))));
+                    if (weighted) {
+                        const float d = dr[8 * b + i];
+                        sum[0] = fmaf(d, f.x, sum[0]);
+                        sum[1] = fmaf(d, f.y, sum[1]);
+                    } else {
+                        sum[0] += f.x;
+                        sum[1] += f.y;
+                    }
+                }
+        };
+        float sd = 0.f, sl = 0.f;
+        for (int t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+            const int row0 = t * a.rt;
+            const int64_t gr = row0 + r;
+            if (TRAIN) {
+                stores_read();
+                nf_bar();   // the column sums of the tile before have read the operand
+            }
+            // the tile's rows of x are contiguous: read whole, through the blocks of
+            // the operand that the first layer does not use
+            float *const sX = reinterpret_cast<float *>(sA + NF_BLK);
+            {
+                const int64_t base = (int64_t)row0 * a.in_dim;
+                const int cnt = (int)min((int64_t)a.rt, max((int64_t)0, a.valid - row0)) * a.in_dim;
+#pragma unroll 4
+                for (int i = et; i < cnt; i += 32 * NF_EPI) sX[i] = a.x[base + i];
+            }
+            nf_bar();
+            if (live && 16 * jb < a.in_pad) {
+                float xv[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    xv[i] = (16 * jb + i < a.in_dim && gr < a.valid) ? sX[r * a.in_dim + 16 * jb + i] : 0.f;
+                uint32_t v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = pack_bf16(xv[2 * i], xv[2 * i + 1]);
+                unsigned char *const x0 = sA + r * 128;   // columns 16 jb .. of block 0
+                *reinterpret_cast<uint4 *>(x0 + (((2 * jb) ^ (r & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
+                *reinterpret_cast<uint4 *>(x0 + (((2 * jb + 1) ^ (r & 7)) << 4)) = make_uint4(v[4], v[5], v[6], v[7]);
+                if (TRAIN) st_global32(a.X0 + gr * a.in_pad + 16 * jb, v);
+            }
+            ready();
+#pragma unroll 1
+            for (int l = 0; l < 2; ++l) {
+                acc_wait();
+                if (TRAIN && l) stores_read();
+                if (act) {
+                    const float *const bias = sC + 256 * l + c0;
+                    bf16 *const Z = (l ? a.Z[1] : a.Z[0]) + gr * w + c0;
+#pragma unroll 1
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t v[16], zv[8], hv[8];
+                        t5_ld16(v, trow + 16 * c);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 b = *reinterpret_cast<const float2 *>(bias + 16 * c + 2 * i);
+                            const float x = __uint_as_float(v[2 * i]) + b.x, y = __uint_as_float(v[2 * i + 1]) + b.y;
+                            zv[i] = pack_bf16(x, y);
+                            hv[i] = pack_bf16(silu(x), silu(y));
+                        }
+                        put(c, hv);
+                        if (TRAIN) st_global32(Z + 16 * c, zv);
+                    }
+                }
+                ready();
+                if (TRAIN) store_box(l, row0);
+            }
+            // layer 3 and the head: out = sum_i H3 w4 + b4, eight columns at a time,
+            // then the 32 sums in the order of a warp's shuffle tree
+            acc_wait();
+            if (TRAIN) stores_read();
+            float v8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (act) {
+                const float *const bias = sC + 512 + c0, *const w4 = sC + 768 + c0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t v[16], hv[8];
+                    t5_ld16(v, trow + 16 * c);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float2 b = *reinterpret_cast<const float2 *>(bias + 16 * c + 2 * i);
+                        const float2 wv = *reinterpret_cast<const float2 *>(w4 + 16 * c + 2 * i);
+                        const float x = __uint_as_float(v[2 * i]) + b.x, y = __uint_as_float(v[2 * i + 1]) + b.y;
+                        hv[i] = pack_bf16(silu(x), silu(y));
+                        const float2 h = unpack_bf16(hv[i]);
+                        v8[2 * c + i / 4] = fmaf(h.x, wv.x, v8[2 * c + i / 4]);
+                        v8[2 * c + i / 4] = fmaf(h.y, wv.y, v8[2 * c + i / 4]);
+                    }
+                    if (TRAIN) put(c, hv);
+                }
+            }
+            float *const vx = sV + (jb & 1) * 1024 + r;
+            if (live && jb >= 2)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) vx[128 * i] = v8[i];
+            nf_bar();
+            if (live && jb < 2) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    v8[i] += vx[128 * i];
+                    if (jb == 1) vx[128 * i] = v8[i];
+                }
+            }
+            nf_bar();
+            if (live && jb == 0) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v8[i] += sV[1024 + r + 128 * i];
+                const float o = ((v8[0] + v8[4]) + (v8[2] + v8[6])) + ((v8[1] + v8[5]) + (v8[3] + v8[7])) + a.b4[0];
+                if (TRAIN) {
+                    const float e = gr < a.valid ? o - a.y[gr] : 0.f, d = e * a.inv_b;
+                    s_d[r] = d;
+                    sd += d;
+                    sl += 0.5f * e * e;
+                } else if (gr < a.valid && ok) {
+                    a.out[gr] = o;
+                }
+            }
+            if constexpr (TRAIN) {
+                nf_bar();   // H3 and d of every row
+                colsum(cs[1], true);
+                nf_bar();   // H3 has been read
+                if (act) {
+                    const float d = s_d[r];
+                    const float *const bias = sC + 512 + c0, *const w4 = sC + 768 + c0;
+#pragma unroll 1
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t v[16], o[8];
+                        t5_ld16(v, trow + 16 * c);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 b = *reinterpret_cast<const float2 *>(bias + 16 * c + 2 * i);
+                            const float2 wv = *reinterpret_cast<const float2 *>(w4 + 16 * c + 2 * i);
+                            // SiLU' of the pre-activation rounded to BF16, as stored for Z1, Z2
+                            const float2 z = unpack_bf16(
+                                pack_bf16(__uint_as_float(v[2 * i]) + b.x, __uint_as_float(v[2 * i + 1]) + b.y));
+                            o[i] = pack_bf16(d * wv.x * dsilu(z.x), d * wv.y * dsilu(z.y));
+                        }
+                        put(c, o);
+                    }
+                }
+                ready();
+                store_box(2, row0);
+                nf_bar();
+                colsum(cs[0], false);
+#pragma unroll 1
+                for (int l = 1; l >= 0; --l) {   // dZ2, dZ1
+                    acc_wait();
+                    stores_read();
+                    nf_bar();   // the column sums have read the operand
+                    if (act) {
+                        const bf16 *const Z = (l ? a.Z[1] : a.Z[0]) + gr * w + c0;
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t v[16], zv[8], o[8];
+                            ld_global32(zv, Z + 16 * c);
+                            t5_ld16(v, trow + 16 * c);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const float2 z = unpack_bf16(zv[i]);
+                                o[i] = pack_bf16(__uint_as_float(v[2 * i]) * dsilu(z.x),
+                                                 __uint_as_float(v[2 * i + 1]) * dsilu(z.y));
+                            }
+                            put(c, o);
+                        }
+                    }
+                    if (l) ready();
+                    else asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    store_box(4 - l, row0);
+                    nf_bar();
+                    if (l) colsum(cs[2], false);
+                    else colsum(cs[3], false);
+                }
+            }
+        }
+        if (TRAIN) {
+            // the CTA's column sums: four row groups in order
+            stores_read();
+            nf_bar();
+            float *const S = reinterpret_cast<float *>(sA);   // [4 sums][4 groups][256]
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                S[(4 * i + rg) * 256 + 2 * cp] = cs[i][0];
+                S[(4 * i + rg) * 256 + 2 * cp + 1] = cs[i][1];
+            }
+            if (jb == 0) {
+                for (int o = 16; o > 0; o >>= 1) {
+                    sd += __shfl_down_sync(0xffffffffu, sd, o);
+                    sl += __shfl_down_sync(0xffffffffu, sl, o);
+                }
+                if (lane == 0) {
+                    sV[q] = sd;
+                    sV[4 + q] = sl;
+                }
+            }
+            nf_bar();
+            for (int i = et; i < 4 * w; i += 32 * NF_EPI) {
+                const int m = i / w, c = i % w;
+                const float *p = S + 4 * m * 256 + c;
+                a.part[m][(int64_t)blockIdx.x * w + c] = ((p[0] + p[256]) + p[512]) + p[768];
+            }
+            if (et < 2) a.part[4 + et][blockIdx.x] = ((sV[4 * et] + sV[4 * et + 1]) + sV[4 * et + 2]) + sV[4 * et + 3];
+        }
+        if (!ok && lane == 0) nf_fail(a);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+}
+
+// k_net's column sums and scalars from stored operands, in its order, so that the
+// per-layer kernels give the same sums: the copies of the GEMMs' operands are then
+// the only difference between the two forms (and make none)
+__global__ void __launch_bounds__(32 * NF_EPI)
+    k_net_sums(const bf16 *__restrict__ dZ3, const bf16 *__restrict__ H3, const bf16 *__restrict__ dZ2,
+               const bf16 *__restrict__ dZ1, const float *__restrict__ out, const float *__restrict__ y,
+               int64_t valid, float inv_b, int w, int tiles, int rt, float *__restrict__ p0,
+               float *__restrict__ p1, float *__restrict__ p2, float *__restrict__ p3,
+               float *__restrict__ p4, float *__restrict__ p5) {
+    __shared__ float S[4][4][256], sdl[2][4], s_d[128];
+    const int et = threadIdx.x, cp = et & 127, rg = et >> 7, lane = et & 31;
+    float cs[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, sd = 0.f, sl = 0.f;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int64_t row0 = (int64_t)t * rt;
+        __syncthreads();
+        if (et < rt) {
+            const int64_t gr = row0 + et;
+            const float e = gr < valid ? out[gr] - y[gr] : 0.f, d = e * inv_b;
+            s_d[et] = d;
+            sd += d;
+            sl += 0.5f * e * e;
+        }
+        __syncthreads();
+        if (2 * cp >= w || 32 * rg >= rt) continue;
+        for (int i = 0; i < 32; ++i) {
+            const int64_t at = (row0 + 32 * rg + i) * w + 2 * cp;
+            const float d = s_d[32 * rg + i];
+            const float2 a = unpack_bf16(*reinterpret_cast<const uint32_t *>(dZ3 + at));
+            const float2 h = unpack_bf16(*reinterpret_cast<const uint32_t *>(H3 + at));
+            const float2 b = unpack_bf16(*reinterpret_cast<const uint32_t *>(dZ2 + at));
+            const float2 c = unpack_bf16(*reinterpret_cast<const uint32_t *>(dZ1 + at));
+            cs[0][0] += a.x;
+            cs[0][1] += a.y;
+            cs[1][0] = fmaf(d, h.x, cs[1][0]);
+            cs[1][1] = fmaf(d, h.y, cs[1][1]);
+            cs[2][0] += b.x;
+            cs[2][1] += b.y;
+            cs[3][0] += c.x;
+            cs[3][1] += c.y;
+        }
+    }
+    for (int i = 0; i < 4; ++i) {
+        S[i][rg][2 * cp] = cs[i][0];
+        S[i][rg][2 * cp + 1] = cs[i][1];
+    }
+    if (et < 128) {
+        for (int o = 16; o > 0; o >>= 1) {
+            sd += __shfl_down_sync(0xffffffffu, sd, o);
+            sl += __shfl_down_sync(0xffffffffu, sl, o);
+        }
+        if (lane == 0) {
+            sdl[0][et >> 5] = sd;
+            sdl[1][et >> 5] = sl;
+        }
+    }
+    __syncthreads();
+    for (int i = et; i < 4 * w; i += 32 * NF_EPI) {
+        const int m = i / w, c = i % w;
+        float *const p = m == 0 ? p0 : m == 1 ? p1 : m == 2 ? p2 : p3;
+        p[(int64_t)blockIdx.x * w + c] = ((S[m][0][c] + S[m][1][c]) + S[m][2][c]) + S[m][3][c];
+    }
+    if (et < 2)
+        (et ? p5 : p4)[blockIdx.x] = ((sdl[et][0] + sdl[et][1]) + sdl[et][2]) + sdl[et][3];
+}
+
 // out[b] = sum_i H3[b][i] w4[i] + b4 (FP32), one warp per row; for widths of
 // at most 256 (a multiple of 8) lane l takes columns 8l .. 8l + 7 in one
 // 16-byte load
@@ -1067,7 +1636,7 @@ __global__ void k_colsum_part(const T *__restrict__ X, const float *__restrict__
         part[(int64_t)blockIdx.y * cols + c] = t;
     }
 }
-// out[c] = sum_k part[k][c] for up to four (part, chunks, cols, out) segments
+// out[c] = sum_k part[k][c] for up to six (part, chunks, cols, out) segments
 // (blockIdx.y): 32 columns per block (lane: column), the 32 warps take chunks
 // w, w + 32, ... and their sums are added in warp order (deterministic)
 struct FinSeg {
@@ -1076,7 +1645,7 @@ struct FinSeg {
     int chunks, cols;
 };
 struct FinSegs {
-    FinSeg s[4];
+    FinSeg s[6];
 };
 __global__ void __launch_bounds__(1024) k_colsum_fin(const __grid_constant__ FinSegs segs) {
     __shared__ float sh[32][33];
@@ -1209,8 +1778,9 @@ __global__ void k_to_bf16(const float *__restrict__ W, int rows, int cols, bf16 
 }
 
 // X0 = BF16 rows of the input, zero-padded from in_dim to in_pad columns (a
-// multiple of 8): one thread per row, eight columns per 16-byte store
-__global__ void k_input_bf16(const float *__restrict__ x, int64_t rows, int in_dim, int in_pad,
+// multiple of 8; rows from `valid` on are zero): one thread per row, eight columns
+// per 16-byte store
+__global__ void k_input_bf16(const float *__restrict__ x, int64_t rows, int64_t valid, int in_dim, int in_pad,
                              bf16 *__restrict__ X0) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
@@ -1221,39 +1791,62 @@ __global__ void k_input_bf16(const float *__restrict__ x, int64_t rows, int in_d
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int c = c0 + 2 * k;
-            vp[k] = pack_bf16(c < in_dim ? xr[c] : 0.f, c + 1 < in_dim ? xr[c + 1] : 0.f);
+            vp[k] = pack_bf16(r < valid && c < in_dim ? xr[c] : 0.f, r < valid && c + 1 < in_dim ? xr[c + 1] : 0.f);
         }
         *reinterpret_cast<uint4 *>(X0 + r * in_pad + c0) = v;
     }
 }
 
-// C[r][c] = sum_z ws[z][r][c] (the split-K partials, in slice order)
+// C[r][c] = sum_z ws[z][r][c] (the split-K partials, in slice order) for up to three
+// GEMMs (blockIdx.y): one launch for the weight gradients of every layer.
 // 256 threads: 32 consecutive outputs x 8 slice groups; warp g sums slices
 // g, g + 8, g + 16, ... of its 32 outputs (coalesced 128-byte rows), then the 8
 // group sums are added in group order: a fixed order, so the result is
 // deterministic, with 8 x the parallelism of one thread per output.
 constexpr int SPLIT_GROUPS = 8;
-__global__ void __launch_bounds__(32 * SPLIT_GROUPS)
-    k_split_sum(const float *__restrict__ ws, int S, int M, int N, int ldc, float *__restrict__ C) {
+struct SplitSeg {
+    const float *ws;
+    float *C;
+    int S, M, N;   // S slices of M x N; S = 1: C holds the result already
+};
+struct SplitSegs {
+    SplitSeg s[3];
+};
+__global__ void __launch_bounds__(32 * SPLIT_GROUPS) k_split_sum(const __grid_constant__ SplitSegs segs) {
     __shared__ float sh[SPLIT_GROUPS][33];
+    const SplitSeg &g = segs.s[blockIdx.y];
     const int cx = threadIdx.x & 31, gz = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + cx;
-    const bool ok = i < (int64_t)M * N;
-    const int64_t o = ok ? (i / N) * ldc + i % N : 0, zs = (int64_t)M * ldc;
+    const int64_t i = (int64_t)blockIdx.x * 32 + cx, zs = (int64_t)g.M * g.N;
+    if (g.S <= 1 || (int64_t)blockIdx.x * 32 >= zs) return;   // uniform over the block
+    const bool ok = i < zs;
     float v = 0.f;
-    if (ok)
-        for (int z = gz; z < S; z += SPLIT_GROUPS) v += ws[z * zs + o];
+    if (ok) {
+#pragma unroll 4
+        for (int z = gz; z < g.S; z += SPLIT_GROUPS) v += g.ws[z * zs + i];
+    }
     sh[gz][cx] = v;
     __syncthreads();
     if (gz == 0 && ok) {
         float t = sh[0][cx];
 #pragma unroll
         for (int k = 1; k < SPLIT_GROUPS; ++k) t += sh[k][cx];
-        C[o] = t;
+        g.C[i] = t;
     }
 }
+inline void split_sum(cudaStream_t st, const SplitSegs &segs, int n) {
+    int64_t most = 0;
+    for (int i = 0; i < n; ++i)
+        if (segs.s[i].S > 1) most = std::max(most, (int64_t)segs.s[i].M * segs.s[i].N);
+    if (most)
+        k_split_sum<<<dim3((unsigned)((most + 31) / 32), (unsigned)n), 32 * SPLIT_GROUPS, 0, st>>>(segs);
+}
 
-constexpr int SPLIT_MAX = 128;   // split-K slices at most (workspace SPLIT_MAX x M x ldc floats)
+constexpr int SPLIT_MAX = 128;   // split-K slices at most
+// slices of an M x N product: about two output tiles per SM
+inline int split_max(int M, int N, int sms) {
+    const int tiles = ((M + 127) / 128) * ((N + 127) / 128);
+    return std::max(1, std::min(2 * sms / tiles, SPLIT_MAX));
+}
 
 // Tensor map of a BF16 operand for the tcgen05 kernel's TMA stage copies,
 // 128-byte swizzle, zero fill outside: K-contiguous src[r * ld + k] (rows x K,
@@ -1316,17 +1909,18 @@ bool t6_tensor_map(CUtensorMap *map, const void *src, int rows, int cols, int ld
 // (same operands, epilogues).
 // A plain-FP32 GEMM with a long K and few output tiles (the weight gradients,
 // K = rows) is split along K over about two CTAs per SM, its partials summed
-// by k_split_sum in a fixed order (ws: SPLIT_MAX x M x ldc floats).
+// by k_split_sum in a fixed order (ws: split_max() x M x N floats, ldc = N; the
+// caller sums `seg`).
 template <bool AT, bool BT, int EPI>
 void gemm(cudaStream_t st, int kind, int *flags, float *ws, int sms, int M, int N, int K, const bf16 *A,
           int lda, const bf16 *B, int ldb, float *C, int ldc, const float *bias, bf16 *H, int ldh,
-          bf16 *Z, int ldz) {
-    const int tiles = ((M + 127) / 128) * ((N + 127) / 128);
+          bf16 *Z, int ldz, SplitSeg *seg = nullptr) {
     int S = 1;
-    if (EPI == EPI_F32 && ws) S = std::max(1, std::min({K / 512, 2 * sms / std::max(1, tiles), SPLIT_MAX}));
+    if (EPI == EPI_F32 && ws) S = std::max(1, std::min(K / 512, split_max(M, N, sms)));
     const int kslice = S > 1 ? (K + S - 1) / S / 64 * 64 + 64 : K;
     if (S > 1) S = (K + kslice - 1) / kslice;
     float *Cw = S > 1 ? ws : C;
+    if (seg) *seg = SplitSeg{ws, C, S, M, N};
     // the persistent warp-specialised kernel: the BF16 epilogues with K-contiguous
     // operands and the FP32 weight gradients with MN-contiguous ones, N <= 256 a
     // multiple of 32, when every operand allows TMA; the same K slices as the
@@ -1355,8 +1949,6 @@ void gemm(cudaStream_t st, int kind, int *flags, float *ws, int sms, int M, int 
             const int mblocks = (M + 127) / 128, tiles6 = mblocks * S;
             k_gemm_t6<AT, BT, EPI><<<std::max(1, std::min(tiles6, sms)), T6_THREADS, T6_SMEM, st>>>(
                 M, N, K, kslice, mblocks, Cw, ldc, bias, flags, ma, mb, mh, mz);
-            if (S > 1)
-                k_split_sum<<<(unsigned)(((int64_t)M * N + 31) / 32), 32 * SPLIT_GROUPS, 0, st>>>(ws, S, M, N, ldc, C);
             return;
         }
     }
@@ -1394,8 +1986,6 @@ void gemm(cudaStream_t st, int kind, int *flags, float *ws, int sms, int M, int 
         k_gemm_bf16<AT, BT, EPI><<<grid, G_THREADS, 0, st>>>(M, N, K, kslice, A, lda, B, ldb, Cw, ldc, bias,
                                                              H, ldh, Z, ldz);
     }
-    if (S > 1)
-        k_split_sum<<<(unsigned)(((int64_t)M * N + 31) / 32), 32 * SPLIT_GROUPS, 0, st>>>(ws, S, M, N, ldc, C);
 }
 
 uint64_t mix64(uint64_t &s) {
@@ -1422,17 +2012,32 @@ struct rsot_mlp {
     // activations
     bf16 *X0 = nullptr, *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *dZ = nullptr, *dZ2 = nullptr;
     bf16 *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr;   // pre-activations, rounded to BF16
-    float *dH = nullptr, *out = nullptr, *dout = nullptr,
+    float *out = nullptr, *dout = nullptr,
           *lt = nullptr, *xin = nullptr, *yin = nullptr, *scal = nullptr;
     int gemm_kind = 0;       // 0: tcgen05 GEMM (TMA), 1: mma.sync GEMM, 2: tcgen05 GEMM (cp.async)
     float *ws = nullptr;     // split-K partials of the weight-gradient GEMMs
     float *red = nullptr;    // partials of the column sums (RED_CHUNKS x width)
     int sms = 1;
-    int *flags = nullptr;    // device error flags of the GEMM kernels (kErrTimeout)
+    struct Result {
+        float loss;
+        int flags;
+    };
+    Result *host = nullptr;  // pinned copy of (scal[0], *flags)
+    float *yhost = nullptr;  // pinned, cap rows: a forward call's results for host memory
+    int *flags = nullptr;    // device error flags of the GEMM kernels (kErrTimeout): the word after scal[0]
 };
 
 namespace rsot {
 namespace {
+
+// split-K partials of the three weight gradients (layers 3, 2, 1); floats in all
+size_t mlp_ws(const rsot_mlp *m, float **ws) {
+    const size_t w = m->width, n3 = split_max(m->width, m->width, m->sms) * w * w;
+    ws[0] = m->ws;
+    ws[1] = m->ws + n3;
+    ws[2] = m->ws + 2 * n3;
+    return 2 * n3 + split_max(m->width, m->in_pad, m->sms) * w * m->in_pad;
+}
 
 cudaError_t mlp_refresh_bf16(rsot_mlp *m) {
     const int w = m->width;
@@ -1446,11 +2051,16 @@ cudaError_t mlp_refresh_bf16(rsot_mlp *m) {
 cudaError_t mlp_reserve(rsot_mlp *m, int64_t rows) {
     if (rows <= m->cap) return cudaSuccess;
     const int64_t r = (rows + 127) / 128 * 128;
-    void *ptrs[] = {m->X0, m->H1, m->H2, m->H3, m->dZ, m->dZ2, m->Z1, m->Z2, m->Z3, m->dH,
+    void *ptrs[] = {m->X0, m->H1, m->H2, m->H3, m->dZ, m->dZ2, m->Z1, m->Z2, m->Z3,
                     m->out, m->dout, m->lt, m->xin, m->yin};
     for (void *q : ptrs) cudaFree(q);
+    if (m->yhost) cudaFreeHost(m->yhost);
+    // a failed allocation below leaves null pointers and no rows, not freed ones
+    m->X0 = m->H1 = m->H2 = m->H3 = m->dZ = m->dZ2 = m->Z1 = m->Z2 = m->Z3 = nullptr;
+    m->out = m->dout = m->lt = m->xin = m->yin = m->yhost = nullptr;
+    m->cap = 0;
     const int w = m->width;
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = cudaMallocHost(&m->yhost, (size_t)r * sizeof(float));
 #define MA(ptr, cnt) \
     if (!e) e = cudaMalloc(&(ptr), (size_t)(cnt) * sizeof(*(ptr)))
     MA(m->X0, r * m->in_pad);
@@ -1462,7 +2072,6 @@ cudaError_t mlp_reserve(rsot_mlp *m, int64_t rows) {
     MA(m->Z1, r * w);
     MA(m->Z2, r * w);
     MA(m->Z3, r * w);
-    MA(m->dH, r * w);
     MA(m->out, r);
     MA(m->dout, r);
     MA(m->lt, r);
@@ -1485,12 +2094,98 @@ rsot_status mlp_take_flags(rsot_mlp *m, int fl) {
     return RSOT_ERR_TIMEOUT;
 }
 
-// forward on rows (padded to 128) from m->xin; result in m->out
-void mlp_forward(rsot_mlp *m, int64_t rows) {
+// The fused kernel of the network: default GEMM kind, a width of whole 64-column
+// blocks that the accumulator holds.  false: a tensor map could not be made (the
+// per-layer kernels run).
+bool net_shape(const rsot_mlp *m) { return m->width % 64 == 0 && m->width <= 256; }
+bool net_fused(const rsot_mlp *m) { return m->gemm_kind == 0 && net_shape(m); }
+
+// Tiles of 128 rows; fewer rows per CTA where those leave SMs idle (a tile's time
+// is its rows' epilogue plus the layers' latencies), one CTA per SM with every
+// weight stage while that holds the tiles, else two.
+struct NetSplit {
+    int rt, tiles, stages, grid;
+};
+NetSplit net_split(const rsot_mlp *m, int64_t rows) {
+    NetSplit s;
+    s.rt = 128;
+    while (s.rt > 32 && (rows + s.rt - 1) / s.rt < m->sms) s.rt /= 2;
+    s.tiles = (int)((rows + s.rt - 1) / s.rt);
+    s.stages = s.tiles <= m->sms ? NF_MAXST : 2;
+    s.grid = std::min(s.tiles, s.stages == 2 ? 2 * m->sms : m->sms);
+    return s;
+}
+// partial sums of a CTA: four of [grid][w], two of [grid]; false: too many
+bool net_parts(const rsot_mlp *m, int grid, float *(&part)[6]) {
+    const int w = m->width;
+    if ((size_t)grid * (4 * w + 2) > red_floats(w)) return false;
+    for (int i = 0; i < 4; ++i) part[i] = m->red + (size_t)i * grid * w;
+    for (int i = 0; i < 2; ++i) part[4 + i] = m->red + (size_t)4 * grid * w + (size_t)i * grid;
+    return true;
+}
+void net_fin(rsot_mlp *m, int grid, float *const (&part)[6], float *loss_sum) {
+    FinSegs segs{};
+    const int at[5] = {5, 6, 3, 1, 7};
+    for (int i = 0; i < 5; ++i) segs.s[i] = FinSeg{part[i], m->G + m->off[at[i]], grid, i < 4 ? m->width : 1};
+    segs.s[5] = FinSeg{part[5], loss_sum, grid, 1};
+    colsum_fin(m->stream, segs, loss_sum ? 6 : 5);
+}
+
+template <bool TRAIN>
+bool launch_net(rsot_mlp *m, int64_t rows, const float *x, const float *y, float *out, float *loss_sum,
+                int *host_flags = nullptr) {
+    const int w = m->width, R = (int)((rows + 127) / 128 * 128);
+    NetArgs a{};
+    a.x = x;
+    a.y = y;
+    a.in_dim = m->in_dim;
+    a.in_pad = m->in_pad;
+    a.w = w;
+    const NetSplit sp = net_split(m, TRAIN ? R : rows);
+    a.rt = sp.rt;
+    a.tiles = sp.tiles;
+    a.stages = sp.stages;
+    a.valid = rows;
+    for (int i = 0; i < 3; ++i) a.b[i] = m->P + m->off[2 * i + 1];
+    a.w4 = m->P + m->off[6];
+    a.b4 = m->P + m->off[7];
+    a.inv_b = 1.0f / (float)rows;
+    a.X0 = m->X0;
+    a.Z[0] = m->Z1;
+    a.Z[1] = m->Z2;
+    a.out = out;
+    a.flags = m->flags;
+    a.host_flags = host_flags;
+    const int grid = sp.grid;
+    if (TRAIN) {
+        if (!net_parts(m, grid, a.part)) return false;
+    }
+    NetMaps maps;
+    memset(&maps, 0, sizeof(maps));
+    bool t = t6_tensor_map(&maps.w[0], m->W1b, w, m->in_pad, m->in_pad, 64) &&
+             t6_tensor_map(&maps.w[1], m->W2b, w, w, w, 64) && t6_tensor_map(&maps.w[2], m->W3b, w, w, w, 64);
+    if (TRAIN) {
+        t = t && t6_tensor_map(&maps.w[3], m->W3bT, w, w, w, 64) && t6_tensor_map(&maps.w[4], m->W2bT, w, w, w, 64);
+        bf16 *const dst[5] = {m->H1, m->H2, m->dZ, m->dZ2, m->Z3};
+        for (int i = 0; i < 5; ++i) t = t && t6_tensor_map(&maps.st[i], dst[i], R, w, w, 32);
+    }
+    if (!t) return false;
+    static std::atomic<bool> attr{false};
+    if (!attr.load()) {
+        cudaFuncSetAttribute((const void *)k_net<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             nf_smem(NF_MAXST));
+        attr.store(true);
+    }
+    k_net<TRAIN><<<grid, NF_THREADS, nf_smem(a.stages), m->stream>>>(a, maps);
+    if (TRAIN) net_fin(m, grid, a.part, loss_sum);
+    return true;
+}
+
+// forward on rows (padded to 128) of x (device) by the per-layer kernels; result in m->out
+void mlp_forward_layers(rsot_mlp *m, int64_t rows, const float *x) {
     const int w = m->width, R = (int)((rows + 127) / 128 * 128);
     cudaStream_t st = m->stream;
-    k_input_bf16<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(m->xin, R, m->in_dim,
-                                                                                 m->in_pad, m->X0);
+    k_input_bf16<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(x, R, rows, m->in_dim, m->in_pad, m->X0);
     gemm<false, false, EPI_BIAS_SILU>(st, m->gemm_kind, m->flags, m->ws, m->sms, R, w, m->in_pad, m->X0, m->in_pad, m->W1b, m->in_pad, nullptr,
                                       w, m->P + m->off[1], m->H1, w, m->Z1, w);
     gemm<false, false, EPI_BIAS_SILU>(st, m->gemm_kind, m->flags, m->ws, m->sms, R, w, w, m->H1, w, m->W2b, w, nullptr, w, m->P + m->off[3],
@@ -1503,20 +2198,44 @@ void mlp_forward(rsot_mlp *m, int64_t rows) {
         k_head<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(m->H3, w, R, m->P + m->off[6], m->P + m->off[7], m->out);
 }
 
+// k_net's sums of stored dZ3 (m->dZ), dZ2 and dZ1 (m->Z3), after the per-layer kernels
+void launch_net_sums(rsot_mlp *m, int64_t rows, const float *y, float *loss_sum) {
+    const int64_t R = (rows + 127) / 128 * 128;
+    const NetSplit sp = net_split(m, R);
+    float *part[6];
+    if (!net_parts(m, sp.grid, part)) return;   // not reached: the buffer holds 2 CTAs per SM
+    k_net_sums<<<sp.grid, 32 * NF_EPI, 0, m->stream>>>(m->dZ, m->H3, m->dZ2, m->Z3, m->out, y, rows,
+                                                       1.0f / (float)rows, m->width, sp.tiles, sp.rt, part[0],
+                                                       part[1], part[2], part[3], part[4], part[5]);
+    net_fin(m, sp.grid, part, loss_sum);
+}
+
 // forward + backward: gradients of loss = sum_valid (out - y)^2 / (2 rows) into m->G;
 // loss_sum (device, one float) receives the sum of the loss terms 0.5 (out - y)^2
-void mlp_backward(rsot_mlp *m, int64_t rows, float *loss_sum) {
+void mlp_backward(rsot_mlp *m, int64_t rows, const float *x, const float *y, float *loss_sum) {
     const int w = m->width, R = (int)((rows + 127) / 128 * 128);
     cudaStream_t st = m->stream;
-    mlp_forward(m, rows);
     float *G = m->G;
-    if (w % 8 == 0 && w <= 256) {
+    const bf16 *dZ1 = m->dZ;
+    const bool fused = net_fused(m) && launch_net<true>(m, rows, x, y, nullptr, loss_sum);
+    // the per-layer tcgen05 kernels on the same shapes: the fused kernel's sums
+    const bool net_sums = !fused && m->gemm_kind != 1 && net_shape(m);
+    if (fused) {
+        dZ1 = m->Z3;   // m->dZ holds dZ3
+    } else {
+        mlp_forward_layers(m, rows, x);
+    }
+    if (fused) {
+    } else if (net_sums) {
+        k_head_back<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(m->out, y, R, rows, 1.0f / (float)rows,
+                                                             m->P + m->off[6], m->Z3, w, m->dout, m->dZ, m->lt);
+    } else if (w % 8 == 0 && w <= 256) {
         // head back-propagation with its column sums: dw4 = sum_r dout_r H3[r],
         // db3 = colsum dZ3, db4 = sum_r dout_r and the loss
         const int ch = stream_chunks(R, m->sms, HB_CHUNKS, 3);   // one wave of three blocks per SM
         float *p3 = m->red, *p4 = p3 + (size_t)HB_CHUNKS * w, *p5 = p4 + (size_t)HB_CHUNKS * w,
               *p6 = p5 + HB_CHUNKS;
-        k_head_back_v8<<<(unsigned)ch, 256, 0, st>>>(m->out, m->yin, R, rows, 1.0f / (float)rows,
+        k_head_back_v8<<<(unsigned)ch, 256, 0, st>>>(m->out, y, R, rows, 1.0f / (float)rows,
                                                      m->P + m->off[6], m->Z3, m->H3, w, m->dout, m->dZ,
                                                      p3, p4, p5, p6);
         FinSegs segs{};
@@ -1526,24 +2245,36 @@ void mlp_backward(rsot_mlp *m, int64_t rows, float *loss_sum) {
         segs.s[3] = FinSeg{p6, loss_sum, ch, 1};
         colsum_fin(st, segs, loss_sum ? 4 : 3);
     } else {
-        k_head_back<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(m->out, m->yin, R, rows, 1.0f / (float)rows,
+        k_head_back<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(m->out, y, R, rows, 1.0f / (float)rows,
                                                              m->P + m->off[6], m->Z3, w, m->dout, m->dZ, m->lt);
         colsum<bf16>(st, m->H3, m->dout, R, w, m->red, G + m->off[6], m->sms);   // dw4 = sum_r dout_r H3[r]
         colsum<float>(st, m->dout, nullptr, R, 1, m->red, G + m->off[7], m->sms);
         colsum<bf16>(st, m->dZ, nullptr, R, w, m->red, G + m->off[5], m->sms);   // db3 = colsum dZ3
         if (loss_sum) colsum<float>(st, m->lt, nullptr, R, 1, m->red, loss_sum, m->sms);
     }
+    // the weight gradients' partials, one after the other; summed together at the end
+    SplitSegs segs{};
+    float *ws[3];
+    mlp_ws(m, ws);
     // layer 3: dW3 = dZ3^T H2, dZ2 = (dZ3 W3) * SiLU'(Z2)
-    gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, m->ws, m->sms, w, w, R, m->dZ, w, m->H2, w, G + m->off[4], w, nullptr, nullptr, 0, nullptr, 0);
-    gemm<false, false, EPI_DSILU>(st, m->gemm_kind, m->flags, m->ws, m->sms, R, w, w, m->dZ, w, m->W3bT, w, nullptr, 0, nullptr, m->dZ2, w, m->Z2, w);
+    gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, ws[0], m->sms, w, w, R, m->dZ, w, m->H2, w, G + m->off[4], w, nullptr, nullptr, 0, nullptr, 0,
+                              &segs.s[0]);
+    if (!fused)
+        gemm<false, false, EPI_DSILU>(st, m->gemm_kind, m->flags, m->ws, m->sms, R, w, w, m->dZ, w, m->W3bT, w, nullptr, 0, nullptr, m->dZ2, w, m->Z2, w);
     // layer 2
-    gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, m->ws, m->sms, w, w, R, m->dZ2, w, m->H1, w, G + m->off[2], w, nullptr, nullptr, 0, nullptr, 0);
-    colsum<bf16>(st, m->dZ2, nullptr, R, w, m->red, G + m->off[3], m->sms);
-    gemm<false, false, EPI_DSILU>(st, m->gemm_kind, m->flags, m->ws, m->sms, R, w, w, m->dZ2, w, m->W2bT, w, nullptr, 0, nullptr, m->dZ, w, m->Z1, w);
+    gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, ws[1], m->sms, w, w, R, m->dZ2, w, m->H1, w, G + m->off[2], w, nullptr, nullptr, 0, nullptr, 0,
+                              &segs.s[1]);
+    if (!fused) {
+        if (!net_sums) colsum<bf16>(st, m->dZ2, nullptr, R, w, m->red, G + m->off[3], m->sms);
+        gemm<false, false, EPI_DSILU>(st, m->gemm_kind, m->flags, m->ws, m->sms, R, w, w, m->dZ2, w, m->W2bT, w, nullptr, 0, nullptr, net_sums ? m->Z3 : m->dZ, w, m->Z1, w);
+        if (net_sums) dZ1 = m->Z3;
+    }
     // layer 1: dW1 = dZ1^T X0, db1 = colsum dZ1
-    gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, m->ws, m->sms, w, m->in_pad, R, m->dZ, w, m->X0, m->in_pad, G + m->off[0], m->in_pad,
-                              nullptr, nullptr, 0, nullptr, 0);
-    colsum<bf16>(st, m->dZ, nullptr, R, w, m->red, G + m->off[1], m->sms);
+    gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, ws[2], m->sms, w, m->in_pad, R, dZ1, w, m->X0, m->in_pad, G + m->off[0], m->in_pad,
+                              nullptr, nullptr, 0, nullptr, 0, &segs.s[2]);
+    split_sum(st, segs, 3);
+    if (net_sums) launch_net_sums(m, rows, y, loss_sum);
+    else if (!fused) colsum<bf16>(st, m->dZ, nullptr, R, w, m->red, G + m->off[1], m->sms);
 }
 
 }  // namespace
@@ -1556,9 +2287,11 @@ extern "C" {
 void rsot_mlp_destroy(rsot_mlp *m) {
     if (!m) return;
     void *ptrs[] = {m->P, m->G, m->Mo, m->Vo, m->W1b, m->W1bT, m->W2b, m->W2bT, m->W3b, m->W3bT,
-                    m->X0, m->H1, m->H2, m->H3, m->dZ, m->dZ2, m->Z1, m->Z2, m->Z3, m->dH, m->out,
-                    m->dout, m->lt, m->xin, m->yin, m->scal, m->flags, m->ws, m->red};
+                    m->X0, m->H1, m->H2, m->H3, m->dZ, m->dZ2, m->Z1, m->Z2, m->Z3, m->out,
+                    m->dout, m->lt, m->xin, m->yin, m->scal, m->ws, m->red};
     for (void *q : ptrs) cudaFree(q);
+    if (m->host) cudaFreeHost(m->host);
+    if (m->yhost) cudaFreeHost(m->yhost);
     delete m;
 }
 
@@ -1596,12 +2329,16 @@ rsot_status rsot_mlp_create(int in_dim, int width, uint64_t seed, rsot_mlp **out
     if (!e) e = cudaMalloc(&m->W3b, (size_t)w * w * 2);
     if (!e) e = cudaMalloc(&m->W3bT, (size_t)w * w * 2);
     if (!e) e = cudaMalloc(&m->scal, 16);
-    if (!e) e = cudaMalloc(&m->flags, sizeof(int));
-    if (!e) e = cudaMalloc(&m->ws, (size_t)SPLIT_MAX * w * std::max(w, m->in_pad) * sizeof(float));
+    m->flags = reinterpret_cast<int *>(m->scal + 1);
+    if (!e) e = cudaMallocHost(&m->host, sizeof(*m->host));
     if (!e) e = cudaMalloc(&m->red, red_floats(w) * sizeof(float));
     int dev = 0;
     if (!e) e = cudaGetDevice(&dev);
     if (!e) e = cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!e) {
+        float *ws[3];
+        e = cudaMalloc(&m->ws, mlp_ws(m, ws) * sizeof(float));
+    }
     if (!e) e = cudaMemset(m->flags, 0, sizeof(int));
     if (!e) e = cudaMemcpy(m->P, h.data(), m->n_params * 4, cudaMemcpyHostToDevice);
     if (!e) e = cudaMemset(m->Mo, 0, m->n_params * 4);
@@ -1644,52 +2381,85 @@ rsot_status rsot_mlp_set_params(rsot_mlp *m, const float *in) {
     return cudaStreamSynchronize(m->stream) ? RSOT_ERR_CUDA : RSOT_OK;
 }
 
+// What a kernel can read (write) as it is: aligned memory of this device, managed or
+// pinned; nullptr: the call copies through the handle's buffers
+static float *direct_ptr(const float *p) {
+    cudaPointerAttributes at;
+    int dev = -1;
+    if (((uintptr_t)p & 3) || cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type == cudaMemoryTypeDevice) return at.device == dev ? const_cast<float *>(p) : nullptr;
+    if (at.type == cudaMemoryTypeManaged || at.type == cudaMemoryTypeHost) return (float *)at.devicePointer;
+    return nullptr;
+}
+
 rsot_status rsot_mlp_forward(rsot_mlp *m, int64_t rows, const float *x, float *y_out) {
     if (!m || rows < 1 || !x || !y_out) return RSOT_ERR_ARG;
     cudaError_t e = mlp_reserve(m, rows);
-    if (!e) e = cudaMemcpyAsync(m->xin, x, (size_t)rows * m->in_dim * 4, cudaMemcpyDefault, m->stream);
-    if (!e) {
-        mlp_forward(m, rows);
-        e = cudaGetLastError();
+    const float *xd = direct_ptr(x);
+    if (!e && !xd) {
+        e = cudaMemcpyAsync(m->xin, x, (size_t)rows * m->in_dim * 4, cudaMemcpyDefault, m->stream);
+        xd = m->xin;
     }
-    if (!e) e = cudaMemcpyAsync(y_out, m->out, (size_t)rows * 4, cudaMemcpyDefault, m->stream);
-    int fl = 0;
-    if (!e) e = cudaMemcpyAsync(&fl, m->flags, sizeof(int), cudaMemcpyDeviceToHost, m->stream);
+    // the fused kernel writes y_out itself where it can, else a pinned buffer
+    float *yd = direct_ptr(y_out);
+    if (yd && yd < xd + rows * m->in_dim && xd < yd + rows) yd = nullptr;   // overlaps x
+    bool fused = false;
+    if (!e && net_fused(m)) {
+        m->host->flags = 0;
+        fused = launch_net<false>(m, rows, xd, nullptr, yd ? yd : m->yhost, nullptr, &m->host->flags);
+    }
+    if (!e && !fused) mlp_forward_layers(m, rows, xd);
+    if (!e) e = cudaGetLastError();
+    if (!e && !fused) {
+        e = cudaMemcpyAsync(&m->host->flags, m->flags, sizeof(int), cudaMemcpyDeviceToHost, m->stream);
+        if (!e) e = cudaMemcpyAsync(y_out, m->out, (size_t)rows * 4, cudaMemcpyDefault, m->stream);
+    }
     if (!e) e = cudaStreamSynchronize(m->stream);
+    if (!e && fused && !yd) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, y_out) == cudaSuccess && at.type == cudaMemoryTypeUnregistered)
+            memcpy(y_out, m->yhost, (size_t)rows * 4);
+        else
+            e = cudaMemcpy(y_out, m->yhost, (size_t)rows * 4, cudaMemcpyDefault);
+    }
     if (e) {
         cudaGetLastError();
         return RSOT_ERR_CUDA;
     }
-    return mlp_take_flags(m, fl);
+    return mlp_take_flags(m, m->host->flags);
 }
 
 rsot_status rsot_mlp_gradients(rsot_mlp *m, int64_t rows, const float *x, const float *y,
                                float *loss_out, float *grad_out) {
     if (!m || rows < 1 || !x || !y) return RSOT_ERR_ARG;
     cudaError_t e = mlp_reserve(m, rows);
-    const int64_t R = (rows + 127) / 128 * 128;
-    // the padding rows (rows .. R) are zeroed; the copies fill the others
-    if (!e && R > rows) e = cudaMemsetAsync(m->xin + rows * m->in_dim, 0, (size_t)(R - rows) * m->in_dim * 4, m->stream);
-    if (!e && R > rows) e = cudaMemsetAsync(m->yin + rows, 0, (size_t)(R - rows) * 4, m->stream);
-    if (!e) e = cudaMemcpyAsync(m->xin, x, (size_t)rows * m->in_dim * 4, cudaMemcpyDefault, m->stream);
-    if (!e) e = cudaMemcpyAsync(m->yin, y, (size_t)rows * 4, cudaMemcpyDefault, m->stream);
+    const float *xd = direct_ptr(x), *yd = direct_ptr(y);
+    if (!e && !xd) {
+        e = cudaMemcpyAsync(m->xin, x, (size_t)rows * m->in_dim * 4, cudaMemcpyDefault, m->stream);
+        xd = m->xin;
+    }
+    if (!e && !yd) {
+        e = cudaMemcpyAsync(m->yin, y, (size_t)rows * 4, cudaMemcpyDefault, m->stream);
+        yd = m->yin;
+    }
     if (!e) {
-        mlp_backward(m, rows, m->scal);
+        mlp_backward(m, rows, xd, yd, m->scal);
         e = cudaGetLastError();
     }
-    float l = 0.f;
-    if (!e) e = cudaMemcpyAsync(&l, m->scal, 4, cudaMemcpyDeviceToHost, m->stream);
+    // loss and flags by one copy into pinned memory, before the gradient's
+    if (!e) e = cudaMemcpyAsync(m->host, m->scal, sizeof(*m->host), cudaMemcpyDeviceToHost, m->stream);
     if (!e && grad_out) e = cudaMemcpyAsync(grad_out, m->G, m->n_params * 4, cudaMemcpyDefault, m->stream);
-    int fl = 0;
-    if (!e) e = cudaMemcpyAsync(&fl, m->flags, sizeof(int), cudaMemcpyDeviceToHost, m->stream);
     if (!e) e = cudaStreamSynchronize(m->stream);
     if (e) {
         cudaGetLastError();
         return RSOT_ERR_CUDA;
     }
-    const rsot_status fs = mlp_take_flags(m, fl);
+    const rsot_status fs = mlp_take_flags(m, m->host->flags);
     if (fs) return fs;
-    if (loss_out) *loss_out = l / (float)rows;
+    if (loss_out) *loss_out = m->host->loss / (float)rows;
     return RSOT_OK;
 }
 
