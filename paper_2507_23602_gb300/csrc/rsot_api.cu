@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <vector>
 
 #include "rsot_internal.cuh"
@@ -177,6 +178,8 @@ void rsot_destroy(rsot_problem *p) {
     cudaFree(p->res_dev);
     if (p->res_host) cudaFreeHost(p->res_host);
     if (p->grad_host) cudaFreeHost(p->grad_host);
+    cudaFree(p->plan_dev);
+    if (p->plan_host) cudaFreeHost(p->plan_host);
     for (cudaEvent_t e : p->tr_events) cudaEventDestroy(e);
     delete p;
 }
@@ -321,7 +324,7 @@ rsot_status rsot_set_pair_kernel(rsot_problem *p, rsot_pair_kernel kind) {
 // tail = arg, rsot_cutoff.cu).
 static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int mode, double arg,
                              rsot_precision prec, double *J_out, double *grad_out,
-                             int64_t *pairs_out) {
+                             int64_t *pairs_out, const std::function<cudaError_t()> &then = nullptr) {
     if (!p || !psi || !J_out || !grad_out) return RSOT_ERR_ARG;
     if (!(eps > 0.0) || !isfinite(eps) || isnan(arg)) return RSOT_ERR_ARG;
     if (prec != RSOT_FP64 && prec != RSOT_MIXED && prec != RSOT_COMPENSATED) return RSOT_ERR_ARG;
@@ -384,6 +387,7 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
         if (!e && !gdev) e = cudaMemcpyAsync(p->grad_host, gd, nb, cudaMemcpyDeviceToHost, st);
         if (!e) e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(EvalResult), cudaMemcpyDeviceToHost, st);
     }
+    if (!e && then) e = then();   // launches that follow a dense evaluation on the stream
     if (!e) e = cudaStreamSynchronize(st);
     if (!e && alt && (p->res_host->flags & kErrRange64)) {
         e = prec == RSOT_FP64 ? launch_dense_fp64(p, psid, eps, gd)
@@ -512,46 +516,78 @@ rsot_status rsot_point_log_partition(rsot_problem *p, double *L_out) {
 
 // Runs a dense mixed evaluation at (psi, eps) -- its records feed the maps and
 // centroid kernels -- then `what` (0: maps, 1: centroids) into device or host
-// outputs.
+// outputs, all on the stream before one wait: the last kernel writes its outputs
+// when the evaluation has succeeded.  Host outputs come through buffers kept with
+// the handle: up to kPlanPinned bytes in pinned memory that the kernel writes, up
+// to kPlanKept in device memory (a pool allocation and its return to the system at
+// the next wait cost 100 us a call), else allocated for the call.
+constexpr size_t kPlanPinned = (size_t)1 << 20, kPlanKept = (size_t)64 << 20;
+
 static rsot_status plan_sums(rsot_problem *p, const double *psi, double eps, int what, double *T_out,
                              int64_t *j_out, double *mass_out) {
-    double J = 0.0;
-    rsot_status s = rsot_eval_dual_grad(p, psi, eps, 0.0, RSOT_MIXED, &J, p->grad_dev, nullptr);
-    if (s) return s;
     cudaStream_t st = p->stream;
     const int64_t rows = what == 0 ? p->nq : p->n;
-    const size_t tb = (size_t)rows * p->d * sizeof(double);
-    const bool tdev = !T_out || is_device_ptr(T_out);
-    const bool jdev = !j_out || is_device_ptr(j_out);
-    const bool mdev = !mass_out || is_device_ptr(mass_out);
-    double *Td = tdev ? T_out : nullptr, *md = mdev ? mass_out : nullptr, *org = nullptr;
-    int64_t *jd = jdev ? j_out : nullptr;
-    cudaError_t e = cudaMallocAsync(&org, 3 * sizeof(double), st);
-    if (!e) e = cudaMemcpyAsync(org, p->origin, 3 * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (!e && !tdev) e = cudaMallocAsync(&Td, tb, st);
-    if (!e && !jdev) e = cudaMallocAsync(&jd, (size_t)rows * sizeof(int64_t), st);
-    if (!e && !mdev) e = cudaMallocAsync(&md, (size_t)rows * sizeof(double), st);
-    if (!e) {
-        trace_begin(p, what == 0 ? "maps" : "centroids");
-        e = what == 0 ? launch_maps(p, eps, Td, jd, org) : launch_centroids(p, Td, md, org);
-        trace_end(p);
+    // the outputs in host memory: sizes, then places in the call's buffer
+    void *const out[3] = {T_out, j_out, mass_out};
+    const size_t bytes[3] = {(size_t)rows * p->d * sizeof(double), (size_t)rows * sizeof(int64_t),
+                             (size_t)rows * sizeof(double)};
+    void *dst[3];
+    size_t at[3], total = 0;
+    for (int i = 0; i < 3; ++i) {
+        dst[i] = out[i];
+        at[i] = total;
+        if (out[i] && !is_device_ptr(out[i])) {
+            dst[i] = nullptr;
+            total += (bytes[i] + 255) / 256 * 256;
+        }
     }
-    if (!e && !tdev) e = cudaMemcpyAsync(T_out, Td, tb, cudaMemcpyDeviceToHost, st);
-    if (!e && !jdev) e = cudaMemcpyAsync(j_out, jd, (size_t)rows * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-    if (!e && !mdev) e = cudaMemcpyAsync(mass_out, md, (size_t)rows * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (org) cudaFreeAsync(org, st);
-    if (!tdev && Td) cudaFreeAsync(Td, st);
-    if (!jdev && jd) cudaFreeAsync(jd, st);
-    if (!mdev && md) cudaFreeAsync(md, st);
-    if (!e) e = cudaStreamSynchronize(st);
+    const bool pinned = total <= kPlanPinned, kept = total <= kPlanKept;
+    char *buf = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (total && kept) {
+        char *&b = pinned ? p->plan_host : p->plan_dev;
+        size_t &have = pinned ? p->plan_host_bytes : p->plan_dev_bytes;
+        if (have < total) {
+            e = pinned ? cudaFreeHost(b) : cudaFree(b);
+            b = nullptr;
+            have = 0;
+            if (!e) e = pinned ? cudaMallocHost(&b, total) : cudaMalloc(&b, total);
+            if (!e) have = total;
+            else b = nullptr;
+        }
+        buf = b;
+    } else if (total) {
+        e = cudaMallocAsync(&buf, total, st);
+    }
+    if (!e && what == 1) e = cent_ready(p);
     if (e) {
         cudaGetLastError();
-        p->tr_open.clear();
-        p->tr_used = 0;
         return from_cuda(e);
     }
-    trace_collect(p);
-    return RSOT_OK;
+    for (int i = 0; i < 3; ++i)
+        if (out[i] && !dst[i]) dst[i] = buf + at[i];
+    double J = 0.0;
+    p->cent_now = what == 1;
+    const rsot_status s = eval_impl(p, psi, eps, 1, 0.0, RSOT_MIXED, &J, p->grad_dev, nullptr, [&]() {
+        trace_begin(p, what == 0 ? "maps" : "centroids");
+        const cudaError_t r = what == 0 ? launch_maps(p, eps, (double *)dst[0], (int64_t *)dst[1])
+                                        : launch_centroids(p, (double *)dst[0], (double *)dst[2]);
+        trace_end(p);
+        return r;
+    });
+    p->cent_now = false;
+    for (int i = 0; !s && !e && i < 3; ++i) {
+        if (!out[i] || dst[i] == out[i]) continue;
+        if (pinned) memcpy(out[i], dst[i], bytes[i]);
+        else e = cudaMemcpyAsync(out[i], dst[i], bytes[i], cudaMemcpyDeviceToHost, st);
+    }
+    if (total && !kept) cudaFreeAsync(buf, st);
+    if (!pinned && !e) e = cudaStreamSynchronize(st);
+    if (e) {
+        cudaGetLastError();
+        return from_cuda(e);
+    }
+    return s;
 }
 
 rsot_status rsot_transport_maps(rsot_problem *p, const double *psi, double eps, double *T_out,

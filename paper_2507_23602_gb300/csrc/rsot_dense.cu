@@ -278,8 +278,12 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
 // ----------------------------------------------------------------------------
 // Pass 2: per-target sum over one point chunk of m_q p_qj (step a3).
 // ----------------------------------------------------------------------------
-template <int D, int TPP>
-__global__ void __launch_bounds__(P2_THREADS, P2_MINB)
+// CENT: with the conditional centroids' sums (Eq. barycenter_fixed_point), whose
+// pair exponents are the same: rows 1 .. D + 1 of the split's partials at part2 are
+// sum e x'_k and sum e.  One pass instead of two (98,304 x 4,096: 80 + 139 -> 141
+// us); bound like pass 2 by the packed FP32 instructions' register reads.
+template <int D, int TPP, bool CENT = false>
+__global__ void __launch_bounds__(P2_THREADS, CENT ? (TPP == 1 ? 6 : 4) : P2_MINB)
     k_grad_mixed(const Rec8 *__restrict__ tpair, const float4 *__restrict__ pquad, int64_t nq,
                  int64_t chunk, double *__restrict__ part2, int64_t stride,
                  int *__restrict__ flags, const int *__restrict__ gate = nullptr, int need = 0) {
@@ -304,9 +308,13 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
     const int64_t p_count = min(chunk, nq - p_begin);   // < 0 in a chunk of padding alone
     const int ntile = p_count > 0 ? (int)((p_count + P2_TS - 1) / P2_TS) : 0;
 
-    double2 acc64[TPP];
+    double2 acc64[TPP], cen[TPP][D + 1];
 #pragma unroll
-    for (int tp = 0; tp < TPP; ++tp) acc64[tp] = make_double2(0.0, 0.0);
+    for (int tp = 0; tp < TPP; ++tp) {
+        acc64[tp] = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k <= D; ++k) cen[tp][k] = make_double2(0.0, 0.0);
+    }
 
     if (tid == 0) {
         s_abort[0] = s_abort[1] = 0;
@@ -330,8 +338,11 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
             s_abort[it & 1] = 1;
             atomicOr(flags, kErrTimeout);
         } else {
-            grad_stage<D, TPP>(sm[s], (int)min((int64_t)P2_TS, p_count - (int64_t)it * P2_TS), W0, W1, W2, C,
-                               acc64);
+            const int cnt = (int)min((int64_t)P2_TS, p_count - (int64_t)it * P2_TS);
+            if constexpr (CENT)
+                cent_stage<D, TPP>(sm[s], cnt, W0, W1, W2, C, acc64, cen);
+            else
+                grad_stage<D, TPP>(sm[s], cnt, W0, W1, W2, C, acc64);
         }
         __syncthreads();
         aborted = s_abort[it & 1] != 0;
@@ -353,7 +364,15 @@ __global__ void __launch_bounds__(P2_THREADS, P2_MINB)
 #pragma unroll
     for (int tp = 0; tp < TPP; ++tp) {
         const int64_t j = 2 * (g0 + tp * P2_THREADS + tid);
-        *reinterpret_cast<double2 *>(part2 + (int64_t)blockIdx.y * stride + j) = acc64[tp];
+        if constexpr (CENT) {
+            const int64_t row = stride / (D + 2);   // the split's rows: gradient, e x', e
+            double *const o = part2 + (int64_t)blockIdx.y * stride + j;
+            *reinterpret_cast<double2 *>(o) = acc64[tp];
+#pragma unroll
+            for (int k = 0; k <= D; ++k) *reinterpret_cast<double2 *>(o + (k + 1) * row) = cen[tp][k];
+        } else {
+            *reinterpret_cast<double2 *>(part2 + (int64_t)blockIdx.y * stride + j) = acc64[tp];
+        }
     }
 }
 
@@ -688,6 +707,7 @@ __global__ void __launch_bounds__(256)
             res->flags = res->gate = 0;
             res->fx_key[0] = res->fx_key[1] = res->fx_key[2] = 0;
             res->ticket = 0;
+            res->ok = s_ok;   // read by the kernels that follow the evaluation
         }
     }
 }
@@ -1089,6 +1109,7 @@ void dense_free(rsot_problem *p) {
     cudaFree(p->a64);
     cudaFree(p->prec64);
     cudaFree(p->lse_buf);
+    cudaFree(p->cent_part);
 }
 
 // Point pairs (pass 1) or target pairs (pass 2) per thread: `most` where the grid
@@ -1155,6 +1176,30 @@ static void launch_grad_mixed(const Rec8 *tpair, int64_t n, const float4 *pquad,
 }
 
 template <int D>
+static void launch_grad_cent(rsot_problem *p) {
+    const int64_t stride = (D + 2) * p->n_pad;
+    dim3 g((unsigned)((p->n + 2 * P2_THREADS * p->cent_tpp - 1) / (2 * P2_THREADS * p->cent_tpp)),
+           (unsigned)p->cent_s2);
+    auto f = p->cent_tpp == 2 ? k_grad_mixed<D, 2, true> : k_grad_mixed<D, 1, true>;
+    launch_pdl(overlap_pass(g, nullptr, p->num_sms), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad, p->nq,
+               p->cent_chunk, p->cent_part, stride, p->flags, (const int *)nullptr, 0);
+}
+
+// buffers of the centroids' pass, once per problem: two target pairs per thread
+// where that fills the slots, else one; splits as in pass 2
+cudaError_t cent_ready(rsot_problem *p) {
+    if (p->cent_part) return cudaSuccess;
+    const int64_t tiles = p->nq_pad / P2_TS;
+    p->cent_tpp = (p->n + 2 * P2_THREADS - 1) / (2 * P2_THREADS) * tiles >= (int64_t)p->num_sms * 12 ? 2 : 1;
+    const int64_t blk = 2 * P2_THREADS * p->cent_tpp, units = (p->n + blk - 1) / blk;
+    p->cent_s2 = pick_split(units, tiles, (int64_t)p->num_sms * (p->cent_tpp == 2 ? 4 : 6));
+    if (units * tiles <= (int64_t)p->num_sms * 6) p->cent_s2 = (int)std::min<int64_t>(tiles, 64);
+    p->cent_chunk = round_up((p->nq_pad + p->cent_s2 - 1) / p->cent_s2, P2_TS);
+    p->cent_s2 = (int)((p->nq_pad + p->cent_chunk - 1) / p->cent_chunk);
+    return cudaMalloc(&p->cent_part, (size_t)p->cent_s2 * (p->d + 2) * p->n_pad * sizeof(double));
+}
+
+template <int D>
 static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps, double *grad) {
     cudaStream_t st = p->stream;
     const int64_t n_p1 = round_up(p->n, P1_TS);
@@ -1185,12 +1230,30 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
                    p->part2, p->n_pad, p->flags, gate);
         trace_end(p);
     }
+    if (p->cent_now && !tc) {   // the centroids' sums with pass 2
+        trace_begin(p, "grad_centroids");
+        launch_grad_cent<D>(p);
+        trace_end(p);
+        const int64_t stride = (D + 2) * p->n_pad;
+        return launch_finalize(p, psi, eps,
+                               {p->cent_part, p->cent_s2, stride, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1,
+                                p->per_prep},
+                               grad);
+    }
     trace_begin(p, "grad_mixed");
     launch_grad_mixed<D>(p->tpair, p->n, p->pquad, p->nq, chunk2, s2, p->part2, p->n_pad, p->flags,
                          gate, p->num_sms, st);
     trace_end(p);
-    return launch_finalize(p, psi, eps,
-                           {p->part2, s2, p->n_pad, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1, p->per_prep}, grad);
+    cudaError_t e = launch_finalize(
+        p, psi, eps, {p->part2, s2, p->n_pad, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1, p->per_prep}, grad);
+    // after tensor-core passes: the FP32 pass for the centroids alone
+    if (!e && p->cent_now) {
+        trace_begin(p, "grad_centroids");
+        launch_grad_cent<D>(p);
+        trace_end(p);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 // ----------------------------------------------------------------------------

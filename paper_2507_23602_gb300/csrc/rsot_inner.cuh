@@ -176,4 +176,65 @@ __device__ __forceinline__ void grad_stage(const float4 *__restrict__ T, int cnt
     }
 }
 
+// The same with the sums of the conditional centroids: cen[tp][k] += sum over the
+// half stage of e x'_k, cen[tp][D] += sum of e, in FP32 per 256 points; acc runs on
+// over the stage's two halves (whose first sum it is) as in grad_stage.
+template <int D, int TPP, bool FIRST>
+__device__ __forceinline__ void cent_half(const float4 *__restrict__ T, int cnt, const float2 (&W0)[TPP],
+                                          const float2 (&W1)[TPP], const float2 (&W2)[TPP],
+                                          const float2 (&C)[TPP], float2 (&acc)[TPP],
+                                          double2 (&cen)[TPP][D + 1]) {
+    float2 s[TPP], sx[TPP][D];
+#pragma unroll
+    for (int tp = 0; tp < TPP; ++tp) {
+        s[tp] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < D; ++k) sx[tp][k] = make_float2(0.f, 0.f);
+    }
+#pragma unroll 4
+    for (int i = 0; i < cnt; ++i) {
+        const float4 p = T[i];
+        const float2 x0 = both(p.x), x1 = both(p.y), x2 = both(p.z), u = both(p.w);
+#pragma unroll
+        for (int tp = 0; tp < TPP; ++tp) {
+            float2 t = C[tp];
+            if (D == 3) t = __ffma2_rn(x2, W2[tp], t);
+            t = __ffma2_rn(x1, W1[tp], t);
+            t = __ffma2_rn(x0, W0[tp], t);
+            t = __fadd2_rn(t, u);
+            const float2 e = make_float2(ex2_approx(t.x), ex2_approx(t.y));
+            acc[tp] = __fadd2_rn(acc[tp], e);
+            if (!FIRST) s[tp] = __fadd2_rn(s[tp], e);
+            sx[tp][0] = __ffma2_rn(e, x0, sx[tp][0]);
+            sx[tp][1] = __ffma2_rn(e, x1, sx[tp][1]);
+            if (D == 3) sx[tp][2] = __ffma2_rn(e, x2, sx[tp][2]);
+        }
+    }
+#pragma unroll
+    for (int tp = 0; tp < TPP; ++tp) {
+        const float2 a = FIRST ? acc[tp] : s[tp];
+        cen[tp][D].x += a.x, cen[tp][D].y += a.y;
+#pragma unroll
+        for (int k = 0; k < D; ++k) cen[tp][k].x += sx[tp][k].x, cen[tp][k].y += sx[tp][k].y;
+    }
+}
+template <int D, int TPP>
+__device__ __forceinline__ void cent_stage(const float4 *__restrict__ T, int cnt, const float2 (&W0)[TPP],
+                                           const float2 (&W1)[TPP], const float2 (&W2)[TPP],
+                                           const float2 (&C)[TPP], double2 (&acc64)[TPP],
+                                           double2 (&cen)[TPP][D + 1]) {
+    constexpr int HALF = 256;   // points per FP32 sum of the centroids
+    static_assert(P2_TS == 2 * HALF, "two halves per stage");
+    float2 acc[TPP];
+#pragma unroll
+    for (int tp = 0; tp < TPP; ++tp) acc[tp] = make_float2(0.f, 0.f);
+    cent_half<D, TPP, true>(T, min(cnt, HALF), W0, W1, W2, C, acc, cen);
+    if (cnt > HALF) cent_half<D, TPP, false>(T + HALF, cnt - HALF, W0, W1, W2, C, acc, cen);
+#pragma unroll
+    for (int tp = 0; tp < TPP; ++tp) {
+        acc64[tp].x += (double)acc[tp].x;
+        acc64[tp].y += (double)acc[tp].y;
+    }
+}
+
 }  // namespace rsot

@@ -52,6 +52,7 @@ struct EvalResult {
     unsigned fx_key[3]; // pair skipping (rsot_skip.cuh): largest A_q, B_j, |B_j| as ordered keys
     int fx_F;           // fraction bits of the fixed-point passes (rsot_fx64.cu)
     unsigned ticket;    // blocks of the final kernel that are done
+    int ok;             // the last evaluation that ended with the final kernel succeeded
 };
 
 struct Grid;  // truncated-path cell grid (rsot_trunc.cu)
@@ -94,6 +95,13 @@ struct rsot_problem {
     int k1 = 0, chunk1 = 0;         // pass-1 target chunks
     int s2 = 0;                     // pass-2 point splits
     int64_t chunk2 = 0;
+    bool cent_now = false;          // this evaluation also forms the centroids' sums
+    int cent_tpp = 0, cent_s2 = 0;  // target pairs per thread, point splits of that pass
+    int64_t cent_chunk = 0;
+    double *cent_part = nullptr;    // [cent_s2][d + 2][n_pad]
+    char *plan_dev = nullptr;       // outputs of maps and centroids for host memory (rsot_api.cu)
+    char *plan_host = nullptr;      // pinned
+    size_t plan_dev_bytes = 0, plan_host_bytes = 0;
     int s2_eval = 0;                // outside the solver (dense_alloc)
     int64_t chunk2_eval = 0;
     int nblk_comb = 0, nblk_prep = 0;
@@ -328,10 +336,9 @@ void compensated_free(rsot_problem *p);
 constexpr double kCompGradRel = 6.5e-7;
 
 // ---- transport maps and centroids (rsot_maps.cu), after a dense mixed evaluation
-cudaError_t launch_maps(rsot_problem *p, double eps, double *T_dev, int64_t *j_dev,
-                        const double *origin_dev);
-cudaError_t launch_centroids(rsot_problem *p, double *T_dev, double *mass_dev,
-                             const double *origin_dev);
+cudaError_t launch_maps(rsot_problem *p, double eps, double *T_dev, int64_t *j_dev);
+cudaError_t cent_ready(rsot_problem *p);   // before an evaluation with cent_now
+cudaError_t launch_centroids(rsot_problem *p, double *T_dev, double *mass_dev);
 
 // ---- truncated path (rsot_trunc.cu) ----------------------------------------
 // truncated by the cutoffs in p->alpha / p->beta
