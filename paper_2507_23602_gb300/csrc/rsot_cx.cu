@@ -83,6 +83,7 @@ __global__ void k_cx_targets(const double *__restrict__ psi, const double *__res
                              const double *__restrict__ lnu, int64_t n, int64_t n_pad, int d, double eps,
                              double P, double Q, double kappa_diam2, CxRec *__restrict__ trec,
                              EvalResult *__restrict__ res) {
+    pdl_enter();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_pad) return;
     const double k = kLog2e / (2.0 * eps);
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(CX_THREADS)
     k_cx_pass(CxRows rows, CxCols cols, int64_t chunk, const float *__restrict__ pmax, float kappa,
               float kdiam2, double *__restrict__ out, float *__restrict__ shift,
               const EvalResult *__restrict__ res) {
+    pdl_enter();
     if (res->flags & kErrRange64) return;
     __shared__ CxRec s_rec[CX_TS];
     __shared__ __align__(16) float4 s_f[CX_TS];
@@ -293,7 +295,7 @@ __global__ void k_cx_combine(const double *__restrict__ part, const float *__res
                              const float4 *__restrict__ ptrow, CxRec *__restrict__ prec,
                              float4 *__restrict__ ptcol, float *__restrict__ ptA,
                              double *__restrict__ lse_buf, double *__restrict__ blockJ) {
-    __shared__ double sh[32];
+    pdl_enter();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double contrib = 0.0;
     if (q < nq) {
@@ -321,8 +323,7 @@ __global__ void k_cx_combine(const double *__restrict__ part, const float *__res
         ptcol[q] = col;
         ptA[q] = A;
     }
-    const double s = block_sum_d(contrib, sh);
-    if (threadIdx.x == 0) blockJ[blockIdx.x] = s;
+    store_partial(contrib, blockJ);
 }
 
 }  // namespace
@@ -336,8 +337,11 @@ static bool cx_alloc(rsot_problem *p, double P) {
     if (p->cx_buf) return true;
     auto chunked = [&](int64_t rows, int64_t cols, int &split, int64_t &chunk) {
         const int64_t tiles = (cols + CX_TS - 1) / CX_TS;
-        split = split_for_slots((rows + CX_ROWS - 1) / CX_ROWS, tiles, (int64_t)p->num_sms * 5);
-        chunk = (tiles + split - 1) / split * CX_TS;
+        // 40 CTAs per SM: skipped columns leave their work uneven (98,304 x 65,536:
+        // pass 2 2.44 ms with 5 per SM, 2.34 with 20, 2.31 with 40)
+        const int64_t units = (rows + CX_ROWS - 1) / CX_ROWS;
+        const int64_t want = std::min({tiles, (40 * p->num_sms + units - 1) / units, (int64_t)256});
+        chunk = (tiles + want - 1) / want * CX_TS;
         split = (int)((cols + chunk - 1) / chunk);
     };
     chunked(p->n, p->nq, p->cx_s2, p->cx_chunk2);
@@ -397,7 +401,8 @@ static void cx_passes(rsot_problem *p, double eps, float t1, float kd) {
                             p->res_dev);
     trace_end(p);
     trace_begin(p, "combine_cx");
-    k_cx_combine<<<(unsigned)(p->nq_pad / 256), 256, 0, st>>>(p->cx_part1, p->cx_shift, p->sk_k, p->nq,
+    const unsigned th = p->per_comb == 1 ? 256 : kSmall;
+    launch_pdl(true, k_cx_combine, (unsigned)(p->nq_pad / th), th, 0, st, p->cx_part1, p->cx_shift, p->sk_k, p->nq,
                                                               p->nq_pad, t1, p->lmass2, p->mass, p->sk_ptrow, prec,
                                                               p->sk_ptcol, p->sk_ptA, p->lse_buf, p->blockJ);
     trace_end(p);
@@ -416,7 +421,8 @@ cudaError_t launch_compensated_cx(rsot_problem *p, const double *psi, double eps
     cudaError_t e = launch_skip(p, psi, eps);
     if (e) return e;
     trace_begin(p, "prep_cx");
-    k_cx_targets<<<(unsigned)(p->n_pad / 256), 256, 0, st>>>(psi, p->y64, p->lnu, p->n, p->n_pad, p->d,
+    const unsigned tt = small_threads(p->n_pad, p->num_sms);
+    launch_pdl(true, k_cx_targets, (unsigned)(p->n_pad / tt), tt, 0, st, psi, p->y64, p->lnu, p->n, p->n_pad, p->d,
                                                             eps, P, Q, kd,
                                                             reinterpret_cast<CxRec *>(p->cx_trec),
                                                             p->res_dev);
@@ -424,7 +430,7 @@ cudaError_t launch_compensated_cx(rsot_problem *p, const double *psi, double eps
     (p->d == 3 ? cx_passes<3> : cx_passes<2>)(p, eps, (float)skip_t1(p), (float)kd);
     if ((e = cudaGetLastError())) return e;
     return launch_finalize(p, psi, eps,
-                           {p->cx_part2, p->cx_s2, p->n_pad, nullptr, p->blockJ, (int)(p->nq_pad / 256), 1, 1,
+                           {p->cx_part2, p->cx_s2, p->n_pad, nullptr, p->blockJ, (int)(p->nq_pad / 256), p->per_comb, 1,
                             p->per_prep},
                            grad);
 }

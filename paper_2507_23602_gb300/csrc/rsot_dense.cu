@@ -48,22 +48,6 @@ constexpr int F_TS = 128;
 
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
-// Partial sums of v: one per block of 256 threads, or one per warp in smaller
-// blocks (kSmall), which final_term() adds in the order of block_sum_d -- the
-// same bits either way.  Smaller blocks spread the FP64 work of few targets or
-// points over more SMs: 16 blocks of 256 threads kept 16 SMs' two FP64 lanes busy
-// for 7 us.
-constexpr int kSmall = 64;
-__device__ __forceinline__ void store_partial(double v, double *__restrict__ out) {
-    if (blockDim.x == 256) {
-        __shared__ double sh[32];
-        const double s = block_sum_d(v, sh);
-        if (threadIdx.x == 0) out[blockIdx.x] = s;
-    } else {
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) out[blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)] = v;
-    }
-}
 __device__ __forceinline__ double final_term(const double *__restrict__ p, int per, int i) {
     if (per == 1) return p[i];
     const double2 *q = reinterpret_cast<const double2 *>(p + 8 * (int64_t)i);
@@ -661,19 +645,34 @@ __global__ void __launch_bounds__(256)
     __shared__ double s_J;
     __shared__ int s_ok;
     pdl_enter();
-    const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    // a.groups threads per target, each with every groups-th partial
+    const int tpb = 256 / a.groups, grp = threadIdx.x / tpb;
+    const int64_t j = (int64_t)blockIdx.x * tpb + threadIdx.x % tpb;
+    const bool mine = j < n && grp == 0;
     double g = 0.0;
     if (j < n) {
         const double *p = a.part2 + j;
-        int s = 0;
-        for (; s + 8 <= a.s2; s += 8) {   // eight loads in flight, added in order
+        const int64_t step = (int64_t)a.groups * a.stride;
+        int s = grp;
+        p += (int64_t)grp * a.stride;
+        for (; s + 7 * a.groups < a.s2; s += 8 * a.groups) {   // eight loads in flight, added in order
             double v[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = p[(int64_t)(s + k) * a.stride];
+            for (int k = 0; k < 8; ++k) v[k] = p[k * step];
+            p += 8 * step;
 #pragma unroll
             for (int k = 0; k < 8; ++k) g += v[k];
         }
-        for (; s < a.s2; ++s) g += p[(int64_t)s * a.stride];
+        for (; s < a.s2; s += a.groups, p += step) g += *p;
+    }
+    if (a.groups > 1) {
+        __shared__ double shg[256];
+        shg[threadIdx.x] = g;
+        __syncthreads();
+        if (mine)
+            for (int k = 1; k < a.groups; ++k) g += shg[k * tpb + threadIdx.x];
+    }
+    if (mine) {
         g = a.scale ? fma(g, a.scale[j], -nu[j]) : g - nu[j];
         grad[j] = g;
     }
@@ -689,7 +688,7 @@ __global__ void __launch_bounds__(256)
                !(nonempty && *(volatile long long *)&res->empty > 0);
     }
     __syncthreads();
-    if (s_ok && out && j < n) out[j] = g;
+    if (s_ok && out && mine) out[j] = g;
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(&res->ticket, 1u) == gridDim.x - 1) {   // every block has read the flags
@@ -1144,15 +1143,6 @@ static void launch_combine(rsot_problem *p, int k1, float *pu) {
     trace_end(p);
 }
 
-// The passes overlap their predecessor's end (launch_pdl) only where their CTAs
-// are at most one per SM, or where they run as the tensor-core passes' fallback
-// and mostly return at once: CTAs placed while the short kernel before still holds
-// slots leave some SMs with more of the single wave than others (61,206 x 5,003:
-// the call 160 -> 225 us, 2,400 x 30,000: 88 -> 144; 1,536 x 128: 63 -> 60).
-static bool overlap_pass(const dim3 &g, const int *gate, int num_sms) {
-    return gate || (int64_t)g.x * g.y <= num_sms;
-}
-
 template <int D>
 static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tquad, int64_t n, int chunk,
                              int k1, float2 *part, int *flags, const int *gate, int num_sms,
@@ -1160,7 +1150,8 @@ static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tqua
     const int pp = pairs_per_thread(P1_PP, nq_pad / P1_TILE * k1, (int64_t)num_sms * P1_MINB);
     dim3 g((unsigned)(nq_pad / (2 * pp * P1_THREADS)), (unsigned)k1);
     auto f = pp == 4 ? k_lse_mixed<D, 4> : pp == 2 ? k_lse_mixed<D, 2> : k_lse_mixed<D, 1>;
-    launch_pdl(overlap_pass(g, gate, num_sms), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk, part, flags, gate, 1);
+    // the tensor-core passes' fallback mostly returns at once
+    launch_pdl(gate || overlap_pass(g, num_sms), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk, part, flags, gate, 1);
 }
 
 template <int D>
@@ -1172,7 +1163,7 @@ static void launch_grad_mixed(const Rec8 *tpair, int64_t n, const float4 *pquad,
     const int tpp = pairs_per_thread(most, (n + blk - 1) / blk * s2, (int64_t)num_sms * 16 / most);
     dim3 g((unsigned)((n + 2 * P2_THREADS * tpp - 1) / (2 * P2_THREADS * tpp)), (unsigned)s2);
     auto f = tpp == 4 ? k_grad_mixed<D, 4> : tpp == 2 ? k_grad_mixed<D, 2> : k_grad_mixed<D, 1>;
-    launch_pdl(overlap_pass(g, gate, num_sms), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2, stride, flags, gate, 1);
+    launch_pdl(gate || overlap_pass(g, num_sms), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2, stride, flags, gate, 1);
 }
 
 template <int D>
@@ -1181,7 +1172,7 @@ static void launch_grad_cent(rsot_problem *p) {
     dim3 g((unsigned)((p->n + 2 * P2_THREADS * p->cent_tpp - 1) / (2 * P2_THREADS * p->cent_tpp)),
            (unsigned)p->cent_s2);
     auto f = p->cent_tpp == 2 ? k_grad_mixed<D, 2, true> : k_grad_mixed<D, 1, true>;
-    launch_pdl(overlap_pass(g, nullptr, p->num_sms), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad, p->nq,
+    launch_pdl(overlap_pass(g, p->num_sms), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad, p->nq,
                p->cent_chunk, p->cent_part, stride, p->flags, (const int *)nullptr, 0);
 }
 
@@ -1337,8 +1328,13 @@ cudaError_t launch_softmax_refine(rsot_problem *p, const double *psi_dev, double
 
 cudaError_t launch_finalize(rsot_problem *p, const double *psi, double eps, const FinalArgs &a,
                             double *grad) {
+    // Many splits are of few targets: eight threads a target outside the solver,
+    // whose sums keep their order (512 targets, 192 splits: 14 -> 9 us).
+    FinalArgs f = a;
+    f.groups = !p->in_solve && a.s2 > 16 ? 8 : 1;
+    const int tpb = 256 / f.groups;
     trace_begin(p, "finalize");
-    launch_pdl(true, k_finalize, (unsigned)((p->n + 255) / 256), 256, 0, p->stream, a, p->nu, p->n, grad, p->psinu,
+    launch_pdl(true, k_finalize, (unsigned)((p->n + tpb - 1) / tpb), 256, 0, p->stream, f, p->nu, p->n, grad, p->psinu,
                p->nblk_prep, psi, eps, p->msum, p->hx, p->final_nonempty, p->final_out, p->res_dev,
                p->res_host);
     trace_end(p);

@@ -51,8 +51,11 @@ struct FxRec {
 namespace {
 
 constexpr int FX_THREADS = 128;
-constexpr int FX_TS = 128;        // columns per shared-memory tile
+constexpr int FX_TS = 64;         // columns per shared-memory tile
 constexpr int FX_TAB = 2048;      // 2^(-i/2048)
+constexpr int FX_U = 4;           // columns at once where a thread has one row (24,576 x 512,
+                                  // with tiles of 128 columns: 63, 55, 47 us a pass for 1, 2, 4;
+                                  // 41 with tiles of 64, half the chain of a CTA)
 constexpr int FX_FMAX = 52, FX_FMIN = 46;
 
 // 2^F (hi + lo) modulo 2^64, |hi| < 2^52
@@ -84,6 +87,7 @@ __global__ void k_fx_records(const double *__restrict__ x64, int64_t nq, int64_t
                              FxRec *__restrict__ trec, int *__restrict__ tgshift,
                              double *__restrict__ tgscale, double *__restrict__ tab,
                              EvalResult *__restrict__ res) {
+    pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const double amax = from_key(res->fx_key[0]), bmax = from_key(res->fx_key[1]);
     const double E = skip_error(res, (float)kappa_diam2);
@@ -98,7 +102,8 @@ __global__ void k_fx_records(const double *__restrict__ x64, int64_t nq, int64_t
     }
     const int s = (F + 62) / 2;
     if (bad) return;
-    if (i < nq_pad) {
+    // one part per block (blockIdx.y): a thread's chains of FP64 would add up
+    if (blockIdx.y == 0 && i < nq_pad) {
         int2 c[3] = {};
         if (i < nq)
             for (int t = 0; t < d; ++t) c[t] = fx_coord(x64[i * d + t], c0, c1, s);
@@ -108,7 +113,7 @@ __global__ void k_fx_records(const double *__restrict__ x64, int64_t nq, int64_t
         prec[i] = r;
         ptshift[i] = i < nq ? -(int)rintf(ptA[i]) : 0;   // the point's largest exponent
     }
-    if (i < n_pad) {
+    if (blockIdx.y == 1 && i < n_pad) {
         int2 c[3] = {};
         long long C = 0;
         int sh = 0;
@@ -129,7 +134,7 @@ __global__ void k_fx_records(const double *__restrict__ x64, int64_t nq, int64_t
         tgshift[i] = -sh;
         tgscale[i] = scale;
     }
-    if (i < FX_TAB) {
+    if (blockIdx.y == 2 && i < FX_TAB) {
         // 2^(-i/2048) = 2^(j/64) e^r / 2 with 2048 - i = 32 j + 2048 r / ln 2
         const int m = FX_TAB - (int)i, j = m >> 5;
         const double r = (double)(m & 31) * (kLn2 / 2048.0);
@@ -171,11 +176,59 @@ struct FxCols {
 // 2^(C_col - kappa d^2 - shift_row).  Pass 1: rows = points, columns = targets;
 // pass 2: rows = targets (in the order of perm), columns = points.
 // ----------------------------------------------------------------------------
+// the pair's FP32 exponent reaches the row's threshold
+template <int D>
+__device__ __forceinline__ bool pair_on(const float4 &f, const float4 &x) {
+    float e = f.w;
+    if (D == 3) e = fmaf(f.z, x.z, e);
+    e = fmaf(f.x, x.x, fmaf(f.y, x.y, e));
+    return e >= x.w;
+}
+
+// 2^(C_col - kappa d^2 - shift_row) = Ts q
+template <int D>
+__device__ __forceinline__ void fx_term(const FxRec &rec, const int (&H)[3], const int (&Lo)[3], int rs, int shE,
+                                        int shI, int shG, const double *s_tab, double &Ts, double &q) {
+    const int4 a = rec.a, b = rec.b;
+    const long long nc = (long long)(((unsigned long long)(unsigned)b.w << 32) | (unsigned)b.z);
+    const int h0 = H[0] - a.x, h1 = H[1] - a.z;
+    const int l0 = Lo[0] - a.y, l1 = Lo[1] - a.w;
+    long long hh = (long long)h0 * h0 + nc;
+    long long mid = (long long)h0 * l0;
+    hh += (long long)h1 * h1;
+    mid += (long long)h1 * l1;
+    if (D == 3) {
+        const int h2 = H[2] - b.x, l2 = Lo[2] - b.y;
+        hh += (long long)h2 * h2;
+        mid += (long long)h2 * l2;
+    }
+    hh += mid >> 30;
+    const unsigned lo = (unsigned)hh;
+    const int hi = (int)(hh >> 32) + rs;
+    const int ex = hi >> shE;                       // integer part
+    const unsigned off = ((unsigned)hi >> shI) & ((FX_TAB - 1u) << 3);
+    const double T = *reinterpret_cast<const double *>(reinterpret_cast<const char *>(s_tab) + off);
+    const unsigned G = __funnelshift_l(lo, (unsigned)hi, shG);   // g 2^43
+    const unsigned Gl = lo << shG;
+    // z = g ln 2 in units of 2^-75 (2^21: rounds the shift below)
+    constexpr unsigned kL1 = 0xB17217F7u, kL2 = 0xD1CF79ABu;
+    unsigned long long z = (unsigned long long)G * kL1 + (1u << 21);
+    z += __umulhi(G, kL2);
+    z += __umulhi(Gl, kL1);
+    const unsigned zh = (unsigned)(z >> 32);                     // 2^-43
+    const unsigned s2 = __umulhi(zh, zh);                        // 2^-54
+    const unsigned y = zh - __umulhi(s2, 698996u);
+    z -= (unsigned long long)__umulhi(zh, y) << 20;
+    q = __longlong_as_double(0x3FF0000000000000ll - (long long)(z >> 22));
+    Ts = __hiloint2double(__double2hiint(T) - (ex << 20), __double2loint(T));
+}
+
 template <int D, int R>
 __global__ void __launch_bounds__(FX_THREADS)
     k_fx_pass(FxRows rows, FxCols cols, int64_t chunk, float kappa, float kdiam2,
               const double *__restrict__ tab, double *__restrict__ out,
               const EvalResult *__restrict__ res) {
+    pdl_enter();
     if (res->flags & kErrRange64) return;
     __shared__ __align__(16) FxRec s_rec[FX_TS];
     __shared__ __align__(16) float4 s_f[FX_TS];
@@ -191,6 +244,7 @@ __global__ void __launch_bounds__(FX_THREADS)
     float4 xf[R];
     float val[R];
     double acc[R];
+    constexpr int U = FX_U;
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         const int64_t i = (int64_t)blockIdx.x * (FX_THREADS * R) + R * tid + k;
@@ -214,7 +268,8 @@ __global__ void __launch_bounds__(FX_THREADS)
         H[k][2] = r.b.x, Lo[k][2] = r.b.y;
     }
     // where k diam^2 is a few times the depth of the sums, few columns are skipped
-    // whole: the pair test alone (24,576 x 512, eps 1e-2: 51 us a pass, 63 with)
+    // whole: the pair test alone (24,576 x 512, eps 1e-2, one column at a time: 51 us
+    // a pass, 63 with)
     const bool use_ball = kdiam2 > 4.0f * rows.slack;
     RowBall ball = {};
     if (use_ball) ball = row_ball(xf[0], val[0], xf[R - 1], val[R - 1], rows.scale);
@@ -233,49 +288,41 @@ __global__ void __launch_bounds__(FX_THREADS)
             unsigned need = __ballot_sync(
                 0xffffffffu, g + lane < cnt && (!use_ball || ball_needs(ball, s_f[g + lane], s_v[g + lane],
                                                                         cols.scale, kappa)));
-            for (; need; need &= need - 1) {
-                const int c = g + __ffs(need) - 1;
-                const float4 f = s_f[c];
-                const int4 a = s_rec[c].a, b = s_rec[c].b;
-                const long long nc = (long long)(((unsigned long long)(unsigned)b.w << 32) | (unsigned)b.z);
+            if constexpr (R == 1) {
+                // U columns at once, straight through for every lane of the warp:
+                // the chain of one pair (about 330 cycles) overlaps the others'
+                while (need) {
+                    int c[U];
+                    bool on[U];
+                    unsigned any = 0;
 #pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    float e = f.w;
-                    if (D == 3) e = fmaf(f.z, xf[k].z, e);
-                    e = fmaf(f.x, xf[k].x, fmaf(f.y, xf[k].y, e));
-                    if (!(e >= xf[k].w)) continue;
-                    const int h0 = H[k][0] - a.x, h1 = H[k][1] - a.z;
-                    const int l0 = Lo[k][0] - a.y, l1 = Lo[k][1] - a.w;
-                    long long hh = (long long)h0 * h0 + nc;
-                    long long mid = (long long)h0 * l0;
-                    hh += (long long)h1 * h1;
-                    mid += (long long)h1 * l1;
-                    if (D == 3) {
-                        const int h2 = H[k][2] - b.x, l2 = Lo[k][2] - b.y;
-                        hh += (long long)h2 * h2;
-                        mid += (long long)h2 * l2;
+                    for (int u = 0; u < U; ++u) {
+                        const bool has = need != 0;
+                        c[u] = has ? g + __ffs(need) - 1 : c[0];
+                        need &= need - 1;
+                        on[u] = has && pair_on<D>(s_f[c[u]], xf[0]);
+                        any |= on[u];
                     }
-                    hh += mid >> 30;
-                    const unsigned lo = (unsigned)hh;
-                    const int hi = (int)(hh >> 32) + rs[k];
-                    const int ex = hi >> shE;                       // integer part
-                    const unsigned off = ((unsigned)hi >> shI) & ((FX_TAB - 1u) << 3);
-                    const double T = *reinterpret_cast<const double *>(
-                        reinterpret_cast<const char *>(s_tab) + off);
-                    const unsigned G = __funnelshift_l(lo, (unsigned)hi, shG);   // g 2^43
-                    const unsigned Gl = lo << shG;
-                    // z = g ln 2 in units of 2^-75 (2^21: rounds the shift below)
-                    constexpr unsigned kL1 = 0xB17217F7u, kL2 = 0xD1CF79ABu;
-                    unsigned long long z = (unsigned long long)G * kL1 + (1u << 21);
-                    z += __umulhi(G, kL2);
-                    z += __umulhi(Gl, kL1);
-                    const unsigned zh = (unsigned)(z >> 32);                     // 2^-43
-                    const unsigned s2 = __umulhi(zh, zh);                        // 2^-54
-                    const unsigned y = zh - __umulhi(s2, 698996u);
-                    z -= (unsigned long long)__umulhi(zh, y) << 20;
-                    const double q = __longlong_as_double(0x3FF0000000000000ll - (long long)(z >> 22));
-                    const double Ts = __hiloint2double(__double2hiint(T) - (ex << 20), __double2loint(T));
-                    acc[k] = fma(Ts, q, acc[k]);
+                    if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        double Ts, q;
+                        fx_term<D>(s_rec[c[u]], H[0], Lo[0], rs[0], shE, shI, shG, s_tab, Ts, q);
+                        acc[0] = fma(on[u] ? Ts : 0.0, q, acc[0]);
+                    }
+                }
+            } else {
+                for (; need; need &= need - 1) {
+                    const int c = g + __ffs(need) - 1;
+                    const float4 f = s_f[c];
+                    const FxRec rec = s_rec[c];
+#pragma unroll
+                    for (int k = 0; k < R; ++k) {
+                        if (!pair_on<D>(f, xf[k])) continue;
+                        double Ts, q;
+                        fx_term<D>(rec, H[k], Lo[k], rs[k], shE, shI, shG, s_tab, Ts, q);
+                        acc[k] = fma(Ts, q, acc[k]);
+                    }
                 }
             }
         }
@@ -294,7 +341,7 @@ __global__ void k_fx_combine(const double *__restrict__ part, int k1, int64_t nq
                              float4 *__restrict__ ptcol, float *__restrict__ ptA,
                              double *__restrict__ lse_buf, double *__restrict__ blockJ,
                              const EvalResult *__restrict__ res) {
-    __shared__ double sh[32];
+    pdl_enter();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double contrib = 0.0;
     if (res->flags & kErrRange64) return;
@@ -322,23 +369,12 @@ __global__ void k_fx_combine(const double *__restrict__ part, int k1, int64_t nq
         ptcol[q] = col;
         ptA[q] = A;
     }
-    const double s = block_sum_d(contrib, sh);
-    if (threadIdx.x == 0) blockJ[blockIdx.x] = s;
-}
-
-__global__ void k_fx_grad(const double *__restrict__ part2, int s2, int64_t stride,
-                          const double *__restrict__ scale, const double *__restrict__ nu, int64_t n,
-                          double *__restrict__ grad) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double g = 0.0;
-    for (int s = 0; s < s2; ++s) g += part2[(int64_t)s * stride + j];
-    grad[j] = fma(g, scale[j], -nu[j]);
+    store_partial(contrib, blockJ);
 }
 
 // rows per thread: 2 share a column's loads, 1 where that leaves SMs idle
 inline int fx_rows(const rsot_problem *p, int64_t rows, int64_t cols) {
-    return rows / (2 * FX_THREADS) * (cols / (4 * FX_TS)) >= 5 * p->num_sms ? 2 : 1;
+    return rows / (2 * FX_THREADS) * (cols / 512) >= 5 * p->num_sms ? 2 : 1;
 }
 
 template <int D>
@@ -347,23 +383,22 @@ void fx_launch(rsot_problem *p, int R, const FxRows &rows, const FxCols &cols, i
     const float kappa = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
     // blocks of padding rows alone are not launched
     dim3 g((unsigned)((rows.count + FX_THREADS * R - 1) / (FX_THREADS * R)), (unsigned)splits);
-    if (R == 2)
-        k_fx_pass<D, 2><<<g, FX_THREADS, 0, p->stream>>>(rows, cols, chunk, kappa, kd, p->fx_tab, out,
-                                                         p->res_dev);
-    else
-        k_fx_pass<D, 1><<<g, FX_THREADS, 0, p->stream>>>(rows, cols, chunk, kappa, kd, p->fx_tab, out,
-                                                         p->res_dev);
+    launch_pdl(overlap_pass(g, p->num_sms), R == 2 ? k_fx_pass<D, 2> : k_fx_pass<D, 1>, g, FX_THREADS, 0, p->stream,
+               rows, cols, chunk, kappa, kd, p->fx_tab, out, p->res_dev);
 }
 
 // buffers of the fixed-point passes, once per problem; false: no memory (the
 // FP64 passes need none of them)
 bool fx_alloc(rsot_problem *p) {
     if (p->fx_buf) return true;
-    const int64_t slots = (int64_t)p->num_sms * 5;
     auto chunked = [&](int64_t rows, int64_t cols, int &split, int64_t &chunk) {
         const int64_t blk = FX_THREADS * fx_rows(p, rows, cols), tiles = (cols + FX_TS - 1) / FX_TS;
-        split = split_for_slots((rows + blk - 1) / blk, tiles, slots);
-        chunk = (tiles + split - 1) / split * FX_TS;
+        // about 60 CTAs per SM: skipped columns leave their work uneven (98,304 x
+        // 16,384: 8.9 ms with 5 per SM, 8.8 with 20, 8.4 with 60, 8.3 with 100; 61,206 x
+        // 5,003: 1.69, 1.58, 1.55, 1.55); 256 splits bound the last kernel's sums
+        const int64_t units = (rows + blk - 1) / blk;
+        const int64_t s = std::min({tiles, (60 * p->num_sms + units - 1) / units, (int64_t)256});
+        chunk = (tiles + s - 1) / s * FX_TS;
         split = (int)((cols + chunk - 1) / chunk);
     };
     chunked(p->nq, p->n, p->fx_k1, p->fx_chunk1);
@@ -418,10 +453,11 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     const double tmax = std::max(t1, 60.0 + log2(p->msum / p->nu_min));   // largest slack of a row
     cudaError_t e = launch_skip(p, psi, eps);
     if (e) return e;
-    const unsigned nb = (unsigned)((std::max(p->nq_pad, p->n_pad) + 255) / 256);
+    const int64_t most = std::max({p->nq_pad, p->n_pad, (int64_t)FX_TAB});
+    const unsigned tr = small_threads(most, p->num_sms);
     trace_begin(p, "fx_records");
-    k_fx_records<<<std::max(nb, (unsigned)(FX_TAB / 256)), 256, 0, st>>>(
-        p->x64, p->nq, p->nq_pad, p->y64, p->n, p->n_pad, p->d, c0, c1, kappa * p->diam2, tmax, psi,
+    launch_pdl(
+        true, k_fx_records, dim3((unsigned)(most / tr), 3), tr, 0, st, p->x64, p->nq, p->nq_pad, p->y64, p->n, p->n_pad, p->d, c0, c1, kappa * p->diam2, tmax, psi,
         eps, p->nu, p->sk_ptA, p->fx_prec, p->fx_ptshift, p->fx_trec, p->fx_tgshift, p->fx_tgscale,
         p->fx_tab, p->res_dev);
     trace_end(p);
@@ -433,8 +469,9 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
                                               eps, p->fx_part1);
     trace_end(p);
     trace_begin(p, "fx_combine");
-    const int nbq = (int)((p->nq_pad + 255) / 256);
-    k_fx_combine<<<nbq, 256, 0, st>>>(p->fx_part1, p->fx_k1, p->nq, p->nq_pad, p->fx_ptshift, p->mass,
+    const int nbq = (int)(p->nq_pad / 256);
+    const unsigned tc = p->per_comb == 1 ? 256 : kSmall;
+    launch_pdl(true, k_fx_combine, (unsigned)(p->nq_pad / tc), tc, 0, st, p->fx_part1, p->fx_k1, p->nq, p->nq_pad, p->fx_ptshift, p->mass,
                                       psi, eps, (float)t1, p->sk_ptrow, p->fx_prec, p->sk_ptcol,
                                       p->sk_ptA, p->lse_buf, p->blockJ, p->res_dev);
     trace_end(p);
@@ -446,7 +483,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
                                               eps, p->fx_part2);
     trace_end(p);
     return launch_finalize(p, psi, eps,
-                           {p->fx_part2, p->fx_s2, p->n_pad, p->fx_tgscale, p->blockJ, nbq, 1, 0, p->per_prep},
+                           {p->fx_part2, p->fx_s2, p->n_pad, p->fx_tgscale, p->blockJ, nbq, p->per_comb, 0, p->per_prep},
                            grad);
 }
 

@@ -271,6 +271,12 @@ inline void launch_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t 
     (void)cudaLaunchKernelEx(&cfg, k, P(args)...);   // cudaGetLastError() reports a failure
 }
 
+// A pass overlaps its predecessor's end only where its CTAs are at most one per SM:
+// CTAs placed while the short kernel before still holds slots leave some SMs with
+// more of a single wave than others (mixed passes, 61,206 x 5,003: the call
+// 160 -> 225 us, 2,400 x 30,000: 88 -> 144; 1,536 x 128: 63 -> 60).
+inline bool overlap_pass(const dim3 &g, int num_sms) { return (int64_t)g.x * g.y <= num_sms; }
+
 // The last kernel of a dense evaluation: gradient and J from the partials, the
 // gradient to the caller's buffer on success, the result block to the host.
 struct FinalArgs {
@@ -282,6 +288,7 @@ struct FinalArgs {
     int nbj, per_j;
     int log2_J;                 // they are sum m R_q (log2 domain), else sum m eps L_q
     int per_psi;                // partials of sum psi nu per 256 targets
+    int groups = 1;             // threads per target (launch_finalize)
 };
 cudaError_t launch_finalize(rsot_problem *p, const double *psi_dev, double eps, const FinalArgs &a,
                             double *grad_dev);
@@ -478,6 +485,24 @@ __device__ __forceinline__ double block_sum_d(double v, double *sh /* >= 32 */) 
     }
     __syncthreads();
     return r;
+}
+
+// Partial sums of v: one per block of 256 threads, or one per warp in smaller
+// blocks (kSmall), which final_term() adds in the order of block_sum_d -- the
+// same bits either way.  Smaller blocks spread the FP64 work of few targets or
+// points over more SMs: 16 blocks of 256 threads kept 16 SMs' two FP64 lanes busy
+// for 7 us.
+constexpr int kSmall = 64;
+inline unsigned small_threads(int64_t rows, int num_sms) { return rows / 256 < 2 * num_sms ? kSmall : 256; }
+__device__ __forceinline__ void store_partial(double v, double *__restrict__ out) {
+    if (blockDim.x == 256) {
+        __shared__ double sh[32];
+        const double s = block_sum_d(v, sh);
+        if (threadIdx.x == 0) out[blockIdx.x] = s;
+    } else {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) out[blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)] = v;
+    }
 }
 
 }  // namespace rsot

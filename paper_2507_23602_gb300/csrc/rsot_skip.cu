@@ -22,6 +22,7 @@ template <int D, int PP>
 __global__ void __launch_bounds__(RM_THREADS)
     k_row_max(const float *__restrict__ xs, int64_t nq_pad, const float4 *__restrict__ tquad, int64_t n,
               int64_t chunk, float *__restrict__ out) {
+    pdl_enter();
     __shared__ __align__(16) float4 sm[RM_TS];
     const int64_t q0 = (int64_t)blockIdx.x * (2 * PP * RM_THREADS);
     float2 X[PP][3], m[PP];
@@ -79,9 +80,11 @@ __global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t 
                                 const float4 *__restrict__ tquad, float4 *__restrict__ ptrow,
                                 float *__restrict__ ptA, float4 *__restrict__ tgrow,
                                 float *__restrict__ tgB, EvalResult *__restrict__ res) {
+    pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float amax = -INFINITY, bmax = -INFINITY, babs = -INFINITY;
-    if (i < nq_pad) {
+    // points or targets per block (blockIdx.y): a thread's FP64 chains would add up
+    if (blockIdx.y == 0 && i < nq_pad) {
         float4 row = make_float4(0.f, 0.f, 0.f, INFINITY);
         float A = -INFINITY;
         if (i < nq) {
@@ -99,7 +102,7 @@ __global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t 
         ptrow[i] = row;
         ptA[i] = A;
     }
-    if (i < n_pad) {
+    if (blockIdx.y == 1 && i < n_pad) {
         float4 r = tquad[i];
         float B = -INFINITY;
         r.w = INFINITY;
@@ -113,9 +116,12 @@ __global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t 
         tgrow[i] = r;
         tgB[i] = B;
     }
-    block_max_key(amax, &res->fx_key[0]);
-    block_max_key(bmax, &res->fx_key[1]);
-    block_max_key(babs, &res->fx_key[2]);
+    if (blockIdx.y == 0) {
+        block_max_key(amax, &res->fx_key[0]);
+    } else {
+        block_max_key(bmax, &res->fx_key[1]);
+        block_max_key(babs, &res->fx_key[2]);
+    }
 }
 
 // Order of the target rows of pass 2: by cells of a 2^b grid in Morton order
@@ -169,12 +175,8 @@ __global__ void k_cell_scatter(const int *__restrict__ cell, int64_t n, int64_t 
 template <int D>
 void row_max(rsot_problem *p) {
     dim3 g((unsigned)(p->nq_pad / (2 * p->sk_pp * RM_THREADS)), (unsigned)p->sk_k);
-    if (p->sk_pp == 4)
-        k_row_max<D, 4><<<g, RM_THREADS, 0, p->stream>>>(p->xs, p->nq_pad, p->tquad, p->n, p->sk_chunk,
-                                                        p->sk_part);
-    else
-        k_row_max<D, 1><<<g, RM_THREADS, 0, p->stream>>>(p->xs, p->nq_pad, p->tquad, p->n, p->sk_chunk,
-                                                        p->sk_part);
+    launch_pdl(overlap_pass(g, p->num_sms), p->sk_pp == 4 ? k_row_max<D, 4> : k_row_max<D, 1>, g, RM_THREADS, 0,
+               p->stream, p->xs, p->nq_pad, p->tquad, p->n, p->sk_chunk, p->sk_part);
 }
 
 }  // namespace
@@ -207,7 +209,9 @@ bool skip_ready(rsot_problem *p, double eps) {
     if (p->sk_buf) return true;
     const int64_t tiles = (p->n + RM_TS - 1) / RM_TS;
     p->sk_pp = p->nq_pad / 1024 * tiles >= 4 * p->num_sms ? 4 : 1;
-    p->sk_k = split_for_slots(p->nq_pad / (2 * p->sk_pp * RM_THREADS), tiles, (int64_t)p->num_sms * 6);
+    // also the chunks of the compensated pass 1, whose work skipping leaves uneven
+    // (98,304 x 65,536: 2.06 ms with 6 CTAs per SM, 1.95 with 24)
+    p->sk_k = split_for_slots(p->nq_pad / (2 * p->sk_pp * RM_THREADS), tiles, (int64_t)p->num_sms * 24);
     p->sk_chunk = (tiles + p->sk_k - 1) / p->sk_k * RM_TS;
     p->sk_k = (int)((p->n + p->sk_chunk - 1) / p->sk_chunk);
     size_t at = 0;
@@ -257,9 +261,10 @@ cudaError_t launch_skip(rsot_problem *p, const double *psi, double eps) {
     trace_begin(p, "row_max");
     (p->d == 3 ? row_max<3> : row_max<2>)(p);
     trace_end(p);
-    const unsigned nb = (unsigned)((std::max(p->nq_pad, p->n_pad) + 255) / 256);
+    const int64_t most = std::max(p->nq_pad, p->n_pad);
+    const unsigned t = small_threads(most, p->num_sms);
     trace_begin(p, "skip_operands");
-    k_skip_operands<<<nb, 256, 0, st>>>(p->sk_part, p->sk_k, p->nq_pad, p->nq, p->xs, p->x64, p->d,
+    launch_pdl(true, k_skip_operands, dim3((unsigned)(most / t), 2), t, 0, st, p->sk_part, p->sk_k, p->nq_pad, p->nq, p->xs, p->x64, p->d,
                                         kLog2e / (2.0 * eps), (float)skip_t1(p), psi, eps, p->nu, p->msum,
                                         p->n, p->n_pad, p->tquad, p->sk_ptrow, p->sk_ptA, p->sk_tgrow,
                                         p->sk_tgB, p->res_dev);
