@@ -178,6 +178,7 @@ void rsot_destroy(rsot_problem *p) {
     cudaFree(p->res_dev);
     if (p->res_host) cudaFreeHost(p->res_host);
     if (p->grad_host) cudaFreeHost(p->grad_host);
+    if (p->psi_host) cudaFreeHost(p->psi_host);
     cudaFree(p->plan_dev);
     if (p->plan_host) cudaFreeHost(p->plan_host);
     for (cudaEvent_t e : p->tr_events) cudaEventDestroy(e);
@@ -296,6 +297,7 @@ rsot_status rsot_create(int d, int64_t nq, const double *x, const double *mass, 
     if (!e) e = cudaMalloc(&p->res_dev, sizeof(EvalResult) + 8 * sizeof(double));
     if (!e) e = cudaMallocHost(&p->res_host, sizeof(EvalResult) + 8 * sizeof(double));
     if (!e) e = cudaMallocHost(&p->grad_host, (size_t)n * 8);
+    if (!e) e = cudaMallocHost(&p->psi_host, (size_t)n * 8);
     if (e) {
         cudaGetLastError();
         rsot_destroy(p);
@@ -322,6 +324,8 @@ rsot_status rsot_set_pair_kernel(rsot_problem *p, rsot_pair_kernel kind) {
 // One evaluation: dense (mode 0), truncated by a radius (mode 1, cutoff C =
 // arg^2 / 2 for every pair) or by the separable psi-aware cutoffs (mode 2,
 // tail = arg, rsot_cutoff.cu).
+constexpr int64_t kPsiDirect = 65536;   // largest host potential that a kernel reads in place
+
 static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int mode, double arg,
                              rsot_precision prec, double *J_out, double *grad_out,
                              int64_t *pairs_out, const std::function<cudaError_t()> &then = nullptr) {
@@ -340,13 +344,12 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     const size_t nb = (size_t)p->n * sizeof(double);
     const double *psid = psi;
     cudaError_t e = cudaSuccess;
-    // the handle's copy of psi: from host memory (through the pinned buffer), and
+    // the handle's copy of psi: from host memory (through a pinned buffer), and
     // where the caller's gradient overlaps it (the final kernel reads psi[0])
     const bool gdev = wgrad == 1;
     if (wpsi == 0) {
-        memcpy(p->grad_host, psi, nb);
+        memcpy(p->psi_host, psi, nb);
         psid = p->psi_dev;
-        e = cudaMemcpyAsync(p->psi_dev, p->grad_host, nb, cudaMemcpyHostToDevice, st);
     } else if (gdev && psi < grad_out + p->n && grad_out < psi + p->n) {
         psid = p->psi_dev;
         e = cudaMemcpyAsync(p->psi_dev, psi, nb, cudaMemcpyDeviceToDevice, st);
@@ -360,6 +363,8 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     // a radius beyond the diameter of the data keeps every pair: dense
     const bool dense = mode == 0 || (mode == 1 && (!(arg > 0.0) || isinf(arg) ||
                                                     arg * arg > p->diam2 * (1.0 + 1e-12)));
+    const auto upload = [&]() { return cudaMemcpyAsync(p->psi_dev, p->psi_host, nb, cudaMemcpyHostToDevice, st); };
+    if (!e && !dense && wpsi == 0) e = upload();
     if (!e && !dense) e = mode == 1 ? cutoffs_uniform(p, 0.5 * arg * arg) : cutoffs_separable(p, psid, eps, arg);
     // dense FP64: fixed-point exponents where they can hold the range, the FP64
     // passes otherwise (or when the device finds that they cannot, kErrRange64)
@@ -367,6 +372,13 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     p->final_nonempty = dense ? 0 : 1;
     const bool alt = !e && dense && ((prec == RSOT_FP64 && fx64_ready(p, eps)) ||
                                      (prec == RSOT_COMPENSATED && cx_ready(p, eps)));
+    // evaluations that begin with the mixed passes' target records read a small host
+    // potential from the pinned buffer (a copy on the stream takes 5 us more)
+    p->psi_src = nullptr;
+    if (!e && dense && wpsi == 0) {
+        if (p->n <= kPsiDirect && (prec == RSOT_MIXED || alt)) p->psi_src = p->psi_host;
+        else e = upload();
+    }
     if (!e) {
         if (alt)
             e = prec == RSOT_FP64 ? launch_dense_fx64(p, psid, eps, gd)

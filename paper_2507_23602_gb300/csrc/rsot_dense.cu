@@ -64,7 +64,8 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
                              int64_t n, int64_t n_alloc, int d, double eps,
                              float4 *__restrict__ tquad, Rec8 *__restrict__ tpair,
                              double *__restrict__ psinu_part, int *__restrict__ flags,
-                             Rec16 *__restrict__ trec, double inv_P, int *__restrict__ gate) {
+                             Rec16 *__restrict__ trec, double inv_P, int *__restrict__ gate,
+                             double *__restrict__ psi_copy) {
     pdl_trigger();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const double psic = psi[0];
@@ -77,6 +78,7 @@ __global__ void k_prep_mixed(const double *__restrict__ psi, const double *__res
         float C = -256.0f * TC_RANGE;
         if (j < n) {
             const double ps = psi[j];
+            if (psi_copy) psi_copy[j] = ps;   // psi is host memory: for the kernels that follow
             if (!isfinite(ps)) atomicOr(flags, kErrNonfinitePsi);
             const double b = ((ps - psic) / eps + lnu[j]) * kLog2e;
             double yy = 0.0;
@@ -641,7 +643,7 @@ __global__ void __launch_bounds__(256)
                const double *__restrict__ psinu, int npn, const double *__restrict__ psi,
                double eps, double msum, double hx, int nonempty, double *__restrict__ out,
                EvalResult *__restrict__ res, EvalResult *__restrict__ host) {
-    __shared__ double sh[32];
+    __shared__ double sh[64];
     __shared__ double s_J;
     __shared__ int s_ok;
     pdl_enter();
@@ -649,21 +651,23 @@ __global__ void __launch_bounds__(256)
     const int tpb = 256 / a.groups, grp = threadIdx.x / tpb;
     const int64_t j = (int64_t)blockIdx.x * tpb + threadIdx.x % tpb;
     const bool mine = j < n && grp == 0;
-    double g = 0.0;
-    if (j < n) {
-        const double *p = a.part2 + j;
-        const int64_t step = (int64_t)a.groups * a.stride;
-        int s = grp;
-        p += (int64_t)grp * a.stride;
-        for (; s + 7 * a.groups < a.s2; s += 8 * a.groups) {   // eight loads in flight, added in order
-            double v[8];
+    double g = 0.0, v[8], sa = 0.0, sb = 0.0;
+    const double *p = a.part2 + (int64_t)grp * a.stride + j;
+    const int64_t step = (int64_t)a.groups * a.stride;
+    const int mine2 = j < n ? (a.s2 - grp + a.groups - 1) / a.groups : 0;   // partials of this thread
+    // eight loads in flight, the first with those of J; added in order
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = p[k * step];
-            p += 8 * step;
+    for (int k = 0; k < 8; ++k) v[k] = k < mine2 ? p[k * step] : 0.0;
+    for (int i = threadIdx.x; i < a.nbj; i += 256) sa += final_term(a.blockJ, a.per_j, i);
+    for (int i = threadIdx.x; i < npn; i += 256) sb += final_term(psinu, a.per_psi, i);
+    for (int s = 0; s < mine2; s += 8) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) g += v[k];
-        }
-        for (; s < a.s2; s += a.groups, p += step) g += *p;
+        for (int k = 0; k < 8; ++k)
+            if (s + k < mine2) g += v[k];
+        p += 8 * step;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (s + 8 + k < mine2) v[k] = p[k * step];
     }
     if (a.groups > 1) {
         __shared__ double shg[256];
@@ -676,11 +680,7 @@ __global__ void __launch_bounds__(256)
         g = a.scale ? fma(g, a.scale[j], -nu[j]) : g - nu[j];
         grad[j] = g;
     }
-    double sa = 0.0, sb = 0.0;
-    for (int i = threadIdx.x; i < a.nbj; i += 256) sa += final_term(a.blockJ, a.per_j, i);
-    for (int i = threadIdx.x; i < npn; i += 256) sb += final_term(psinu, a.per_psi, i);
-    sa = block_sum_d(sa, sh);
-    sb = block_sum_d(sb, sh);
+    block_sum2_d(sa, sb, sh);
     if (threadIdx.x == 0) {
         // log2_J: sa = sum_q m_q R_q (log2, translated frame), else sum_q m_q eps L_q
         s_J = a.log2_J ? (psi[0] * msum - hx + eps * kLn2 * sa - sb) : (sa - sb);
@@ -699,7 +699,6 @@ __global__ void __launch_bounds__(256)
             host->empty = res->empty;
             host->flags = flags;
             host->gate = gate;
-            __threadfence_system();
             res->J = s_J;
             res->psic = psi[0];   // read by k_point_L
             res->pairs = res->empty = 0;
@@ -1129,9 +1128,11 @@ static int pairs_per_thread(int most, int64_t items, int64_t slots) {
 static void launch_prep(rsot_problem *p, const double *psi, double eps, Rec16 *trec, double inv_P, int *gate) {
     const int t = p->per_prep == 1 ? CB_THREADS : kSmall;
     trace_begin(p, "prep_targets_mixed");
-    k_prep_mixed<<<(unsigned)(p->n_pad / t), t, 0, p->stream>>>(psi, p->y64, p->lnu, p->nu, p->n, p->n_pad,
-                                                                p->d, eps, p->tquad, p->tpair, p->psinu,
-                                                                p->flags, trec, inv_P, gate);
+    const double *const src = p->psi_src ? p->psi_src : psi;
+    k_prep_mixed<<<(unsigned)(p->n_pad / t), t, 0, p->stream>>>(
+        src, p->y64, p->lnu, p->nu, p->n, p->n_pad, p->d, eps, p->tquad, p->tpair, p->psinu, p->flags, trec, inv_P,
+        gate, p->psi_src ? p->psi_dev : nullptr);
+    p->psi_src = nullptr;
     trace_end(p);
 }
 

@@ -177,6 +177,8 @@ struct rsot_problem {
 
     // staging for host psi / grad
     double *psi_dev = nullptr;      // [n]
+    double *psi_host = nullptr;     // pinned [n]: a host potential on its way
+    const double *psi_src = nullptr;   // set: the next prep kernel reads psi there and fills psi_dev
     bool borrowed = false;          // mass and nu are the caller's device arrays (not freed)
     double *grad_dev = nullptr;     // [n] gradient of the last evaluation
     double *grad_host = nullptr;    // [n] pinned staging of host gradient outputs
@@ -485,6 +487,28 @@ __device__ __forceinline__ double block_sum_d(double v, double *sh /* >= 32 */) 
     }
     __syncthreads();
     return r;
+}
+// block_sum_d of two values at once (thread 0 has the sums)
+__device__ __forceinline__ void block_sum2_d(double &a, double &b, double *sh /* >= 64 */) {
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        sh[threadIdx.x >> 5] = a;
+        sh[32 + (threadIdx.x >> 5)] = b;
+    }
+    __syncthreads();
+    const int nw = (blockDim.x + 31) / 32;
+    if (threadIdx.x < 32) {
+        a = (int)threadIdx.x < nw ? sh[threadIdx.x] : 0.0;
+        b = (int)threadIdx.x < nw ? sh[32 + threadIdx.x] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, o);
+            b += __shfl_down_sync(0xffffffffu, b, o);
+        }
+    }
 }
 
 // Partial sums of v: one per block of 256 threads, or one per warp in smaller

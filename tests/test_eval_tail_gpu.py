@@ -75,3 +75,19 @@ def test_split_of_small_problems(d, nq, n):
         P.close()
     assert abs(J - J64) <= 1e-6 * 1e-2 * 154 + 1e-12
     assert np.all(np.abs(g - g64) <= 3e-5 * (g64 + nu))
+
+
+# host potentials of at most 65,536 entries are read in place by the target records' kernel
+@pytest.mark.parametrize("prec", ["FP64", "MIXED", "COMPENSATED"])
+@pytest.mark.parametrize("n", [65536, 65537])
+def test_host_potential_read_or_copied(n, prec):
+    import torch
+    rs, P, psi, _ = _problem(3, 64, n)
+    try:
+        for k in range(2):
+            psi = psi + 0.001 * k
+            J, g, _ = P.eval(psi, 1e-2, 0.0, getattr(rs, prec))
+            Jd, gd, _ = P.eval(torch.tensor(psi, device="cuda"), 1e-2, 0.0, getattr(rs, prec))
+            assert J == Jd and np.array_equal(g, gd.cpu().numpy())
+    finally:
+        P.close()
