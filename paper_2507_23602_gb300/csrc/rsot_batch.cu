@@ -291,14 +291,7 @@ __global__ void k_bcombine(const BProb *__restrict__ probs, const int *__restric
         const int64_t tile = ql / P1_TILE;
         const int l = (int)(ql % P1_TILE);
         const int64_t it0 = P.item1_base + tile * P.nck1;
-        float mx = kPadC;
-        for (int c = 0; c < P.nck1; ++c) mx = fmaxf(mx, part1[(it0 + c) * P1_TILE + l].x);
-        double tot = 0.0;
-        for (int c = 0; c < P.nck1; ++c) {
-            const float2 v = part1[(it0 + c) * P1_TILE + l];
-            tot += (double)v.y * pow2_int_d(v.x - mx);
-        }
-        const double R = (double)mx + log2(tot);
+        const double R = merge_partials(P.nck1, [&](int c) { return part1[(it0 + c) * P1_TILE + l]; });
         if (mass[g] > 0.0) {
             contrib = mass[g] * R;
             u = (float)fmax(lm2[g] - R, -1.0e30);

@@ -215,14 +215,6 @@ __global__ void __launch_bounds__(P1_THREADS, p1_minb(PP))
     }
 }
 
-// (double)v 2^k for an integer-valued k <= 0, by the bits of a normal v > 0 (the
-// conversion and the product would each take the FP64 pipe); else as written
-__device__ __forceinline__ double scaled_d(float v, float k) {
-    const unsigned b = __float_as_uint(v);
-    if (b - 0x00800000u >= 0x7f000000u || !(k >= -896.0f)) return (double)v * pow2_int_d(k);
-    return __hiloint2double((int)((b >> 3) + (896u << 20)) + ((int)k << 20), (int)(b << 29));
-}
-
 // ----------------------------------------------------------------------------
 // Merge the pass-1 chunk partials into R_q, write the pass-2 point records
 // (x', u_q = log2 m_q - R_q) and the block partials of sum_q m_q R_q.
@@ -239,14 +231,7 @@ __global__ void k_combine(const float2 *__restrict__ part, int k1, int64_t nq_pa
         float x[3] = {0.f, 0.f, 0.f};
         float u = kPadC;
         if (q < nq) {
-            float mx = kPadC;
-            for (int k = 0; k < k1; ++k) mx = fmaxf(mx, part[(int64_t)k * nq_pad + q].x);
-            double tot = 0.0;
-            for (int k = 0; k < k1; ++k) {
-                const float2 v = part[(int64_t)k * nq_pad + q];
-                tot += scaled_d(v.y, v.x - mx);
-            }
-            const double R = (double)mx + log2(tot);
+            const double R = merge_partials(k1, [&](int k) { return part[(int64_t)k * nq_pad + q]; });
             lse_buf[q] = R;
             const double lm = lmass2[q];
             if (mass[q] > 0.0) {

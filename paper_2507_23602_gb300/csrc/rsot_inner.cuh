@@ -237,4 +237,39 @@ __device__ __forceinline__ void cent_stage(const float4 *__restrict__ T, int cnt
     }
 }
 
+// (double)v 2^k for an integer-valued k <= 0, by the bits of a normal v > 0 (the
+// conversion and the product would each take the FP64 pipe); else as written
+__device__ __forceinline__ double scaled_d(float v, float k) {
+    const unsigned b = __float_as_uint(v);
+    if (b - 0x00800000u >= 0x7f000000u || !(k >= -896.0f)) return (double)v * pow2_int_d(k);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)) + ((int)k << 20), (int)(b << 29));
+}
+
+// log2 of the sum of k1 pass-1 partials (M, S): S 2^M each.  The first eight loads are
+// in flight together and held for the sum (a load after the other, twice, took
+// half of the combining kernels: 61,206 points of a 61,206 x 5,003 problem: 18 -> 14 us, the FP64 logarithm is
+// most of the rest).
+template <class F>
+__device__ __forceinline__ double merge_partials(int k1, F load) {
+    constexpr int HELD = 8;
+    float2 v[HELD];
+    float mx = kPadC;
+#pragma unroll
+    for (int k = 0; k < HELD; ++k) v[k] = k < k1 ? load(k) : make_float2(kPadC, 0.f);
+#pragma unroll
+    for (int k = 0; k < HELD; ++k) mx = fmaxf(mx, v[k].x);
+#pragma unroll 4
+    for (int k = HELD; k < k1; ++k) mx = fmaxf(mx, load(k).x);
+    double tot = 0.0;
+#pragma unroll
+    for (int k = 0; k < HELD; ++k)
+        if (k < k1) tot += scaled_d(v[k].y, v[k].x - mx);
+#pragma unroll 4
+    for (int k = HELD; k < k1; ++k) {
+        const float2 w = load(k);
+        tot += scaled_d(w.y, w.x - mx);
+    }
+    return (double)mx + log2(tot);
+}
+
 }  // namespace rsot

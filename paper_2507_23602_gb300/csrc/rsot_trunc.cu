@@ -1881,7 +1881,7 @@ __global__ void k_combine_trunc(const float2 *__restrict__ part1, const int *__r
             double tot = 0.0;
             for (int it = a; it < e; ++it) {
                 const float2 v = part1[(int64_t)it * PT + l];
-                if (v.y > 0.f) tot += (double)v.y * pow2_int_d(v.x - mx);
+                if (v.y > 0.f) tot += scaled_d(v.y, v.x - mx);
             }
             if (tot > 0.0) {
                 const double R = (double)mx + log2(tot);
