@@ -165,6 +165,7 @@ void rsot_destroy(rsot_problem *p) {
     skip_free(p);
     fx64_free(p);
     cx_free(p);
+    mskip_free(p);
     dense_free(p);
     cudaFree(p->xs);
     cudaFree(p->x64);
@@ -178,7 +179,6 @@ void rsot_destroy(rsot_problem *p) {
     cudaFree(p->res_dev);
     if (p->res_host) cudaFreeHost(p->res_host);
     if (p->grad_host) cudaFreeHost(p->grad_host);
-    if (p->psi_host) cudaFreeHost(p->psi_host);
     cudaFree(p->plan_dev);
     if (p->plan_host) cudaFreeHost(p->plan_host);
     for (cudaEvent_t e : p->tr_events) cudaEventDestroy(e);
@@ -296,8 +296,8 @@ rsot_status rsot_create(int d, int64_t nq, const double *x, const double *mass, 
     if (!e) e = cudaMalloc(&p->grad_dev, (size_t)n * 8);
     if (!e) e = cudaMalloc(&p->res_dev, sizeof(EvalResult) + 8 * sizeof(double));
     if (!e) e = cudaMallocHost(&p->res_host, sizeof(EvalResult) + 8 * sizeof(double));
-    if (!e) e = cudaMallocHost(&p->grad_host, (size_t)n * 8);
-    if (!e) e = cudaMallocHost(&p->psi_host, (size_t)n * 8);
+    if (!e) e = cudaMallocHost(&p->grad_host, (size_t)n * 16);
+    if (!e) p->psi_host = p->grad_host + n;
     if (e) {
         cudaGetLastError();
         rsot_destroy(p);

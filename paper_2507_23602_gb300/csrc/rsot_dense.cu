@@ -1195,9 +1195,13 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
                    (int)round_up(p->n, TC_TS), chunk1, p->part1, p->flags, gate);
         trace_end(p);
     }
-    trace_begin(p, "lse_mixed");
-    launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, chunk1, k1, p->part1, p->flags, gate,
-                        p->num_sms, st);
+    const int skip = tc ? 0 : mskip_ready(p, eps);
+    trace_begin(p, skip & 1 ? "lse_skip" : "lse_mixed");
+    if (skip & 1)
+        mskip_lse(p, eps);
+    else
+        launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, chunk1, k1, p->part1, p->flags, gate, p->num_sms,
+                            st);
     trace_end(p);
     launch_combine(p, k1, tc ? p->pu : nullptr);
     if (tc) {
@@ -1214,6 +1218,15 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
         const int64_t stride = (D + 2) * p->n_pad;
         return launch_finalize(p, psi, eps,
                                {p->cent_part, p->cent_s2, stride, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1,
+                                p->per_prep},
+                               grad);
+    }
+    if (skip & 2) {
+        trace_begin(p, "grad_skip");
+        mskip_grad(p, eps);
+        trace_end(p);
+        return launch_finalize(p, psi, eps,
+                               {p->ms_part2, p->ms_s2, p->n_pad, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1,
                                 p->per_prep},
                                grad);
     }

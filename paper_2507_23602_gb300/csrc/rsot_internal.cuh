@@ -95,6 +95,11 @@ struct rsot_problem {
     int k1 = 0, chunk1 = 0;         // pass-1 target chunks
     int s2 = 0;                     // pass-2 point splits
     int64_t chunk2 = 0;
+    char *ms_buf = nullptr;         // skipping mixed passes (rsot_mskip.cu): orders of the rows, partials
+    int *ms_perm_q = nullptr, *ms_perm_t = nullptr;
+    double *ms_part2 = nullptr;     // [ms_s2][n_pad]
+    int ms_s2 = 0;
+    int64_t ms_chunk2 = 0;
     bool cent_now = false;          // this evaluation also forms the centroids' sums
     int cent_tpp = 0, cent_s2 = 0;  // target pairs per thread, point splits of that pass
     int64_t cent_chunk = 0;
@@ -315,6 +320,15 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi_dev, double eps
 void fx64_free(rsot_problem *p);
 // the smallest column split whose CTAs fill the resident slots
 int split_for_slots(int64_t units, int64_t tiles, int64_t slots);
+// rows 0 .. n (row j at pos[j step][d]) by the cells of a grid along the Morton curve, then
+// n .. n_pad as they are; scratch: n_pad + 4,096 integers
+cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_pad, int *perm, int *scratch,
+                       int step = 1);
+// dense mixed passes without the pairs that cannot matter (rsot_mskip.cu)
+int mskip_ready(rsot_problem *p, double eps);   // bit 0: pass 1, bit 1: pass 2
+void mskip_lse(rsot_problem *p, double eps);
+void mskip_grad(rsot_problem *p, double eps);
+void mskip_free(rsot_problem *p);
 // compensated dense evaluation outside the solver (rsot_cx.cu)
 bool cx_ready(rsot_problem *p, double eps);
 cudaError_t launch_compensated_cx(rsot_problem *p, const double *psi_dev, double eps, double *grad_dev);

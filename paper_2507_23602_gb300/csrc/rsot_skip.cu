@@ -130,14 +130,14 @@ __global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t 
 // (98,304 x 16,384) the FP64 pass 2 takes 1.6 ms, 3.7 in the caller's order.
 // The order inside a cell is whatever the atomics give; a row's sum does not
 // depend on it.
-__global__ void k_cell_count(const double *__restrict__ y64, int64_t n, int d, double half,
+__global__ void k_cell_count(const double *__restrict__ y64, int64_t n, int step, int d, double half,
                              int *__restrict__ cell, int *__restrict__ count) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const int bits = d == 3 ? 4 : 6;
     int id = 0;
     for (int t = 0; t < d; ++t) {
-        const double u = half > 0.0 ? (y64[j * d + t] / half + 1.0) * 0.5 : 0.0;
+        const double u = half > 0.0 ? (y64[j * step * d + t] / half + 1.0) * 0.5 : 0.0;
         const int c = min(max((int)(u * (1 << bits)), 0), (1 << bits) - 1);
         for (int b = 0; b < bits; ++b) id |= ((c >> b) & 1) << (d * b + t);
     }
@@ -200,6 +200,18 @@ void skip_free(rsot_problem *p) {
     p->sk_buf = nullptr;
 }
 
+cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_pad, int *perm, int *scratch,
+                       int step) {
+    int *cell = scratch, *count = cell + n_pad;
+    const unsigned nb = (unsigned)((n_pad + 255) / 256);
+    const cudaError_t e = cudaMemsetAsync(count, 0, SORT_CELLS * 4, p->stream);
+    if (e) return e;
+    k_cell_count<<<nb, 256, 0, p->stream>>>(pos, n, step, p->d, p->half_ext, cell, count);
+    k_cell_scan<<<1, 1024, 0, p->stream>>>(count);
+    k_cell_scatter<<<nb, 256, 0, p->stream>>>(cell, n, n_pad, count, perm);
+    return cudaGetLastError();
+}
+
 // buffers and the target order, once per problem; false: not for these sizes,
 // or no memory (the callers have passes that need none of it)
 bool skip_ready(rsot_problem *p, double eps) {
@@ -237,14 +249,9 @@ bool skip_ready(rsot_problem *p, double eps) {
     p->sk_tgrow = reinterpret_cast<float4 *>(b + o_trow);
     p->sk_tgB = reinterpret_cast<float *>(b + o_tB);
     p->sk_perm = reinterpret_cast<int *>(b + o_perm);
-    int *cell = reinterpret_cast<int *>(b + o_cell), *count = cell + nt;
-    cudaMemsetAsync(count, 0, SORT_CELLS * 4, p->stream);
-    const unsigned nb = (unsigned)((p->n_pad + 255) / 256);
-    k_cell_count<<<nb, 256, 0, p->stream>>>(p->y64, p->n, p->d, p->half_ext, cell, count);
-    k_cell_scan<<<1, 1024, 0, p->stream>>>(count);
-    k_cell_scatter<<<nb, 256, 0, p->stream>>>(cell, p->n, p->n_pad, count, p->sk_perm);
+    const cudaError_t e = cell_order(p, p->y64, p->n, p->n_pad, p->sk_perm, reinterpret_cast<int *>(b + o_cell));
     // once per problem: a later evaluation may run on another stream
-    if (cudaStreamSynchronize(p->stream) != cudaSuccess) {
+    if (e || cudaStreamSynchronize(p->stream) != cudaSuccess) {
         cudaGetLastError();
         skip_free(p);
         return false;
