@@ -217,7 +217,14 @@ __global__ void __launch_bounds__(CX_THREADS)
     const int tid = threadIdx.x, lane = tid & 31;
     const float margin = 2.0f * skip_error(res, kdiam2);
     const int64_t i0 = (int64_t)blockIdx.x * CX_ROWS + 2 * tid;   // < rows.pad, a multiple of 1,024
-    const int64_t at0 = rows.perm ? rows.perm[i0] : i0, at1 = rows.perm ? rows.perm[i0 + 1] : i0 + 1;
+    // pass 1: order of point pairs, pass 2: of targets (null: as stored); points in cell
+    // order, pass 1 of 98,304 x 65,536 at eps 1e-3: 1.95 -> 1.77 ms
+    int64_t at0 = i0, at1 = i0 + 1;
+    if (rows.perm) {
+        at0 = PASS == 1 ? 2 * rows.perm[i0 >> 1] : rows.perm[i0];
+        at1 = PASS == 1 ? at0 + 1 : rows.perm[i0 + 1];
+    }
+    const bool in0 = (PASS == 1 ? at0 : i0) < rows.count, in1 = (PASS == 1 ? at1 : i0 + 1) < rows.count;
     CxOp W;
     f2 C1, C2, C3, X[3], thr, M;
     RowBall ball;
@@ -231,14 +238,14 @@ __global__ void __launch_bounds__(CX_THREADS)
         X[0] = make_float2(fa.x, fb.x);
         X[1] = make_float2(fa.y, fb.y);
         X[2] = make_float2(fa.z, fb.z);
-        const float va = i0 < rows.count ? rows.val[at0] + rows.slack + margin : -INFINITY;
-        const float vb = i0 + 1 < rows.count ? rows.val[at1] + rows.slack + margin : -INFINITY;
+        const float va = in0 ? rows.val[at0] + rows.slack + margin : -INFINITY;
+        const float vb = in1 ? rows.val[at1] + rows.slack + margin : -INFINITY;
         ball = row_ball(fa, va, fb, vb, rows.scale);
         thr = make_float2(fa.w - margin, fb.w - margin);   // +inf: padding
         M = make_float2(-INFINITY, -INFINITY);
         if (PASS == 1)
             for (int k = 0; k < (int)blockIdx.y; ++k) {
-                const float2 m = *reinterpret_cast<const float2 *>(pmax + (int64_t)k * rows.pad + i0);
+                const float2 m = *reinterpret_cast<const float2 *>(pmax + (int64_t)k * rows.pad + at0);
                 M = make_float2(fmaxf(M.x, ceilf(m.x)), fmaxf(M.y, ceilf(m.y)));
             }
     }
@@ -284,7 +291,7 @@ __global__ void __launch_bounds__(CX_THREADS)
     }
     out[(int64_t)blockIdx.y * rows.pad + at0] = acc0;
     out[(int64_t)blockIdx.y * rows.pad + at1] = acc1;
-    if (PASS == 1) *reinterpret_cast<float2 *>(shift + (int64_t)blockIdx.y * rows.pad + i0) = M;
+    if (PASS == 1) *reinterpret_cast<float2 *>(shift + (int64_t)blockIdx.y * rows.pad + at0) = M;
 }
 
 // R_q, the J term of the point's mass, and the column of pass 2: u_q = log2 m_q
@@ -393,7 +400,7 @@ static void cx_passes(rsot_problem *p, double eps, float t1, float kd) {
     const float kappa = (float)k, inv2k = (float)(0.5 / k);
     const float tmax = (float)(60.0 + log2(p->msum / p->nu_min));   // largest slack of a target
     trace_begin(p, "lse_cx");
-    const CxRows pr = {prec, p->sk_ptrow, p->sk_ptA, nullptr, t1, 1.f, p->nq, p->nq_pad};
+    const CxRows pr = {prec, p->sk_ptrow, p->sk_ptA, p->sk_perm_q, t1, 1.f, p->nq, p->nq_pad};
     const CxCols tc = {trec, p->tquad, p->sk_tgB, inv2k, p->n};
     // the column chunks of the maximum's kernel: a chunk's shift starts from theirs
     k_cx_pass<D, 1><<<dim3((unsigned)((p->nq + CX_ROWS - 1) / CX_ROWS), (unsigned)p->sk_k), CX_THREADS, 0,

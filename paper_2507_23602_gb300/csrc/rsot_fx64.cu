@@ -159,6 +159,7 @@ struct FxRows {
     const float *val;
     const int *shift;   // integral, added to the exponent's negative
     const int *perm;    // row order (null: as stored)
+    bool pairs;         // of pairs of rows
     float slack;        // added to val in the ball test
     float scale;
     int64_t count, pad;
@@ -255,8 +256,11 @@ __global__ void __launch_bounds__(FX_THREADS)
         at[k] = -1;
         FxRec r;
         r.a = r.b = make_int4(0, 0, 0, 0);
-        if (i < rows.count) {
-            at[k] = rows.perm ? rows.perm[i] : (int)i;
+        int64_t a = i;   // a pair's second row may be padding
+        if (rows.perm && rows.pairs && (i & ~(int64_t)1) < rows.count) a = 2 * rows.perm[i >> 1] + (i & 1);
+        else if (rows.perm && i < rows.count) a = rows.perm[i];
+        if (a < rows.count) {
+            at[k] = (int)a;
             r = rows.rec[at[k]];
             xf[k] = rows.f[at[k]];
             xf[k].w -= margin;
@@ -461,7 +465,9 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
         eps, p->nu, p->sk_ptA, p->fx_prec, p->fx_ptshift, p->fx_trec, p->fx_tgshift, p->fx_tgscale,
         p->fx_tab, p->res_dev);
     trace_end(p);
-    const FxRows pts = {p->fx_prec, p->sk_ptrow, p->sk_ptA, p->fx_ptshift, nullptr,
+    // compact warps where columns are skipped whole (use_ball)
+    const int *const order = kappa * p->diam2 > 4.0 * t1 ? p->sk_perm_q : nullptr;
+    const FxRows pts = {p->fx_prec, p->sk_ptrow, p->sk_ptA, p->fx_ptshift, order, true,
                         (float)t1,  1.f,         p->nq,     p->nq_pad};
     const FxCols tgt = {p->fx_trec, p->tquad, p->sk_tgB, inv2k, p->n};
     trace_begin(p, "fx_lse");
@@ -475,7 +481,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
                                       psi, eps, (float)t1, p->sk_ptrow, p->fx_prec, p->sk_ptcol,
                                       p->sk_ptA, p->lse_buf, p->blockJ, p->res_dev);
     trace_end(p);
-    const FxRows tgr = {p->fx_trec,  p->sk_tgrow, p->sk_tgB, p->fx_tgshift, p->sk_perm,
+    const FxRows tgr = {p->fx_trec,  p->sk_tgrow, p->sk_tgB, p->fx_tgshift, p->sk_perm, false,
                         (float)tmax, inv2k,       p->n,      p->n_pad};
     const FxCols ptc = {p->fx_prec, p->sk_ptcol, p->sk_ptA, 1.f, p->nq};
     trace_begin(p, "fx_grad");

@@ -142,6 +142,7 @@ struct rsot_problem {
     float *sk_ptA = nullptr, *sk_tgB = nullptr;            // values of the ball test
     int *sk_perm = nullptr;                                // order of the target rows
     int sk_pp = 0, sk_k = 0;
+    int *sk_perm_q = nullptr;       // order of the point pairs (large problems)
     int64_t sk_chunk = 0;
     // fixed-point passes of the dense FP64 path (rsot_fx64.cu): one allocation on first use
     void *fx_buf = nullptr;

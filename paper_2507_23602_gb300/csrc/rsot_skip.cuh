@@ -89,4 +89,37 @@ __device__ __forceinline__ void target_B(double ps, double psic, double eps, dou
     lo = ((p - (a - ab)) + ((double)e - ab)) + pe + f;
 }
 
+// The warp's rows: their box in the columns' units (centre and half edges, 2k or 1
+// times positions) and the factor of the distance.
+struct Box {
+    float c[3], h[3], f;
+};
+
+// this lane's column at (x, y, z): value - k dist^2
+template <int D>
+__device__ __forceinline__ float box_bound(const Box &b, float4 col, float value) {
+    const float x[3] = {col.x, col.y, col.z};
+    float d2 = 0.f;
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+        const float d = fmaxf(fabsf(x[t] - b.c[t]) - b.h[t], 0.f);
+        d2 = fmaf(d, d, d2);
+    }
+    return fmaf(-d2, b.f, value);
+}
+
+// box of the warp's rows, lo and hi per lane; widened for the rounding of both sides
+template <int D>
+__device__ __forceinline__ Box make_box(const float (&lo)[3], const float (&hi)[3], float scale, float f) {
+    Box b;
+    b.f = f * 0.9999f;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const float H = t < D ? warp_max_f(hi[t]) : 0.f, L = t < D ? -warp_max_f(-lo[t]) : 0.f;
+        b.c[t] = 0.5f * (H + L) * scale;
+        b.h[t] = (0.5f * (H - L) + 1e-6f * (fabsf(H) + fabsf(L))) * scale;
+    }
+    return b;
+}
+
 }  // namespace rsot

@@ -76,3 +76,10 @@ def test_solves_keep_the_general_passes():
     finally:
         P.close()
     assert "grad_df" in names and "grad_cx" not in names
+
+
+# from 1e9 pairs on the points' maxima leave out targets and the points are taken in cell order by pairs:
+# an odd number of points in no order, one chunk of targets and many, clusters apart
+@pytest.mark.parametrize("d,nq,n,eps", [(3, 100001, 10007, 1e-3), (2, 400003, 2503, 1e-3), (3, 5121, 200001, 2e-3)])
+def test_large(d, nq, n, eps):
+    _check(d, nq, n, eps, 2 * eps, seed=nq)

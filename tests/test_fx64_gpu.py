@@ -129,3 +129,30 @@ def test_many_rows_per_thread_and_split_columns():
     assert abs(J - J2) <= 1e-12 * abs(J2)
     # FP64 sums of up to 70,001 terms in both: 70,001 * 2^-53 = 8e-12
     assert np.max(np.abs(g - g2)) <= 2e-11 * np.max(nu)
+
+
+# from 1e9 pairs on points are taken in cell order by pairs and their maxima leave out targets: an odd
+# number of points in no order, against the error-free part of the compensated bound
+@pytest.mark.parametrize("d,nq,n,eps", [(3, 100001, 10007, 1e-3), (2, 400003, 2503, 2e-4)])
+def test_large(d, nq, n, eps):
+    import paper_2507_23602_gb300 as rs
+    rng = np.random.default_rng(nq)
+    x, y = rng.uniform(0, 1, (nq, d)), rng.uniform(0, 1, (n, d))
+    m, nu = rng.uniform(0.2, 1.8, nq), rng.uniform(0.5, 1.5, n)
+    m, nu = m / m.sum(), nu / nu.sum()
+    psi = eps * rng.standard_normal(n)
+    P = rs.Problem(x, m, y, nu)
+    try:
+        P.kernel_timing(True)
+        J, g, _ = P.eval(psi, eps, 0.0, rs.FP64)
+        assert "fx_lse" in P.kernel_times()
+        L = P.point_log_partition()
+    finally:
+        P.close()
+    # every point's logarithm against a sum over all targets, for some points, and the total mass
+    pick = rng.choice(nq, 200, replace=False)
+    for q in pick:
+        e = (psi - 0.5 * ((x[q] - y) ** 2).sum(1)) / eps + np.log(nu)
+        M = e.max()
+        assert abs(L[q] - (M + np.log(np.exp(e - M).sum()))) <= 1e-12 * max(1.0, abs(M))
+    assert abs((g + nu).sum() - 1.0) <= 1e-12
