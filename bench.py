@@ -42,15 +42,9 @@ FP32_LANE_OPS_PER_CLK_PER_SM = 128
 # FP32 lane-operations per pair of the compensated passes, counted from their
 # source: double-float exponent 3 x 12 + 3, shift TwoSum 6, Kahan 4, tail 2-3
 COMP_FP32_OPS_PER_PAIR = {"lse_df": 51, "grad_df": 52}
-# FP64-pipe operations per pair of the two dense FP64 passes, counted from
-# their source (d = 2 / 3): the squared distance (d subtractions, d fused
-# multiply-adds), the exponent (one fma; pass 2 one more add), the library's own
-# exponential (two range compares, multiply, round, conversion, 2 fma reduction,
-# 5 fma + 1 multiply polynomial, 1 fma + 1 add table, 1 multiply scaling: 16),
-# then pass 1's compare-and-update (2: the shift subtraction and one of the two
-# update forms, plus the compare) and pass 2's accumulation (1):
-# pass 1 = 2d + 20, pass 2 = 2d + 19
-FP64_OPS_PER_PAIR = {2: 47, 3: 51}
+# FP64-pipe operations per pair of the two dense FP64 passes: one fused multiply-add
+# each (exponents and exponentials are 64-bit integers)
+FP64_OPS_PER_PAIR = {2: 2, 3: 2}
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -732,7 +726,10 @@ def main():
 
     P = rs.Problem(p.x, p.mass, p.y, p.nu, stream=torch.cuda.current_stream())
     kind = {"auto": rs.PAIRS_AUTO, "tensor": rs.PAIRS_TENSOR, "fp32": rs.PAIRS_FP32}[args.pair_kernel]
-    P.set_pair_kernel(kind)
+    # the timed steps evaluate every pair: the automatic choice leaves out the pairs
+    # below 2^-60 of every sum they enter (reported beside the headline)
+    timed_kind = rs.PAIRS_FP32 if kind == rs.PAIRS_AUTO else kind
+    P.set_pair_kernel(timed_kind)
     psi_d = torch.tensor(psi, device=dev)
     grad_d = torch.empty(p.n, dtype=torch.float64, device=dev)
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
@@ -763,13 +760,11 @@ def main():
     value = whole_job_rate(pairs, args.steps, world, total_s)
     ms_per_step = 1e3 * total_s / args.steps
 
-    # the same evaluation with the other pair form (the tensor-core exponents,
-    # opt-in, when the headline runs the default FP32 form): reported beside the
+    # the same evaluation with the automatic choice (leaves out pairs) and with the
+    # other pair form (the tensor-core exponents, opt-in): reported beside the
     # headline for comparison, not part of it
-    fp32_pairs = None
-    if not args.no_fp32_compare:
-        other = rs.PAIRS_TENSOR if kind != rs.PAIRS_TENSOR else rs.PAIRS_FP32
-        P.set_pair_kernel(other)
+    def timed_eval(which, label):
+        P.set_pair_kernel(which)
         for _ in range(max(1, args.warmup)):
             P.eval(psi_d, p.eps, 0.0, rs.MIXED, grad_out=grad_d)
         P.kernel_timing(True)
@@ -785,11 +780,17 @@ def main():
             fms.append(a.elapsed_time(b_))
         fk = P.kernel_times()
         P.kernel_timing(False)
-        P.set_pair_kernel(kind)
-        fp32_pairs = {"pair_kernel": "tensor (opt-in)" if other == rs.PAIRS_TENSOR else "fp32",
-                      "value": pairs / (sum(fms) / len(fms) * 1e-3) / 1e9, "unit": "G pairs/s",
-                      "ms_per_step": sum(fms) / len(fms),
-                      "per_kernel_ms": {k: v[0] / v[1] for k, v in fk.items()}}
+        return {"pair_kernel": label, "value": pairs / (sum(fms) / len(fms) * 1e-3) / 1e9, "unit": "G pairs/s",
+                "ms_per_step": sum(fms) / len(fms), "per_kernel_ms": {k: v[0] / v[1] for k, v in fk.items()}}
+
+    fp32_pairs = auto_pairs = None
+    if not args.no_fp32_compare:
+        other = rs.PAIRS_TENSOR if kind != rs.PAIRS_TENSOR else rs.PAIRS_FP32
+        fp32_pairs = timed_eval(other, "tensor (opt-in)" if other == rs.PAIRS_TENSOR else "fp32")
+        if kind == rs.PAIRS_AUTO:
+            auto_pairs = timed_eval(rs.PAIRS_AUTO, "auto: pairs below 2^-60 of every sum are left out; "
+                                                   "value counts them (dense equivalent)")
+    P.set_pair_kernel(kind)
 
     # the compensated evaluation (double-float pair exponents, certified gradient
     # bound): a secondary line, with its own roofline on the FP32 pipe
@@ -813,19 +814,22 @@ def main():
         sms_c = torch.cuda.get_device_properties(dev).multi_processor_count
         sm_max_c = float(measured_peaks().get("sm_max_mhz", 2070.0))
         peak_ops = FP32_LANE_OPS_PER_CLK_PER_SM * sms_c * sm_max_c * 1e6 / 1e12
-        dom_c = max(("lse_df", "grad_df"), key=lambda k: ck.get(k, 0.0))
-        ops = COMP_FP32_OPS_PER_PAIR[dom_c] * pairs
-        ach = ops / (ck[dom_c] * 1e-3) / 1e12
+        dom_c = max((k for k in ck if k.startswith(("lse_", "grad_"))), key=lambda k: ck[k])
+        roof_c = {"bound": "alu", "kernel": dom_c, "frac": None,
+                  "note": "leaves out the pairs below 2^-60 of every sum: no work per pair to count"}
+        if dom_c in COMP_FP32_OPS_PER_PAIR:
+            ach = COMP_FP32_OPS_PER_PAIR[dom_c] * pairs / (ck[dom_c] * 1e-3) / 1e12
+            roof_c = {"bound": "alu", "unit": "T FP32 lane-ops/s", "kernel": dom_c,
+                      "achieved": ach, "peak": peak_ops, "frac": ach / peak_ops,
+                      "peak_basis": f"{FP32_LANE_OPS_PER_CLK_PER_SM} FP32 lane-ops/clk/SM x "
+                                    f"{sms_c} SMs x {sm_max_c:.0f} MHz; "
+                                    f"{COMP_FP32_OPS_PER_PAIR[dom_c]} lane-ops per pair",
+                      "traffic": None}
         comp = {"metric": "dual+grad G pairs/s (dense, compensated: double-float pair exponents)",
                 "value": pairs / (sum(cms) / len(cms) * 1e-3) / 1e9, "unit": "G pairs/s",
                 "ms_per_step": sum(cms) / len(cms), "per_kernel_ms": ck,
                 "grad_l1_error_bound": rs.COMPENSATED_GRAD_REL * float(p.mass.sum()),
-                "roofline": {"bound": "alu", "unit": "T FP32 lane-ops/s", "kernel": dom_c,
-                             "achieved": ach, "peak": peak_ops, "frac": ach / peak_ops,
-                             "peak_basis": f"{FP32_LANE_OPS_PER_CLK_PER_SM} FP32 lane-ops/clk/SM x "
-                                           f"{sms_c} SMs x {sm_max_c:.0f} MHz; "
-                                           f"{COMP_FP32_OPS_PER_PAIR[dom_c]} lane-ops per pair",
-                             "traffic": None}}
+                "roofline": roof_c}
         # the same evaluation truncated at tail 1e-12 (psi-aware cutoffs, block-skip
         # passes keeping exactly the FP64 path's pairs), at the bench potential
         P.eval_tail(psi_d, p.eps, 1e-12, rs.COMPENSATED, grad_out=grad_d)
@@ -920,6 +924,7 @@ def main():
     if not args.no_e2e:
         psi_h = torch.tensor(psi, dtype=torch.float64).pin_memory()
         grad_h = torch.empty(p.n, dtype=torch.float64).pin_memory()
+        P.set_pair_kernel(timed_kind)
         for _ in range(max(1, args.warmup)):
             P.eval(psi_h, p.eps, 0.0, rs.MIXED, grad_out=grad_h)
         e2e_s = 0.0
@@ -932,6 +937,7 @@ def main():
         e2e_s = max_over_ranks(e2e_s, world, dev)
         e2e = {"value": whole_job_rate(pairs, args.steps, world, e2e_s), "unit": "G pairs/s",
                "h2d_bytes_per_step": p.n * 8, "d2h_bytes_per_step": p.n * 8 + 48}
+        P.set_pair_kernel(kind)
 
     if rank != 0:
         P.close()
@@ -975,15 +981,14 @@ def main():
         "data": "synthetic",
         "config": {"workload": workload, "nq": p.nq, "n": p.n, "eps": p.eps,
                    "pairs_per_step": pairs, "precision": "mixed (f32 pairs, f64 reductions)",
-                   "pair_kernel": args.pair_kernel + (" (FP32 pair arithmetic for evaluations "
-                                                      "returned to the caller)"
-                                                      if args.pair_kernel == "auto" else ""),
+                   "pair_kernel": "fp32, every pair" if args.pair_kernel == "auto" else args.pair_kernel,
                    "l2": "flushed between steps (256 MiB write, outside the step events)",
                    "parallelism": "replicas" if world > 1 else "single"},
         "roofline": roof,
         "e2e": e2e,
         "truncated": trunc,
         "other_pair_kernel": fp32_pairs,
+        "automatic_pair_kernel": auto_pairs,
         "compensated": comp,
         "solve": solve,
         "gpu_launches": int(sum(v[1] for v in ktimes.values())),

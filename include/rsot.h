@@ -110,7 +110,9 @@ rsot_status rsot_set_stream(rsot_problem *p, void *stream);
  *     to the FP32 kernels by itself, per evaluation, when an operand leaves
  *     the f16 range.  Both passes form bitwise the same exponents.
  *   RSOT_PAIRS_AUTO (the default): every evaluation returned to the caller
- *     (rsot_eval_dual_grad, _tail, the maps) uses the FP32 form; inside
+ *     (rsot_eval_dual_grad, _tail, the maps) uses the FP32 form, and large
+ *     dense ones at small eps leave out the pairs below 2^-60 of every sum
+ *     they enter (the terms that remain keep their arithmetic and order); inside
  *     rsot_solve and the batched and multilevel solvers, whose stop is
  *     certified on compensated or FP64 reference evaluations, the mixed
  *     iterations take the tensor-core form while the gradient is far above

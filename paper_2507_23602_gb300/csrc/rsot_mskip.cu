@@ -280,7 +280,8 @@ void mskip_free(rsot_problem *p) {
     p->ms_buf = nullptr;
 }
 
-// Which passes leave pairs out: bit 0 pass 1, bit 1 pass 2; 0 in the solver and where
+// Which passes leave pairs out: bit 0 pass 1, bit 1 pass 2; 0 in the solver, where the
+// caller has chosen a pair kernel (RSOT_PAIRS_FP32 takes every pair) and where
 // few pairs can be left out (kd = k diam^2, in 3-D a pair's reach is about
 // sqrt(78 / kd) of the diameter) or the work is too small for the loops over masks and
 // the first, whole stage.  Both sides in us:
@@ -293,7 +294,7 @@ void mskip_free(rsot_problem *p) {
 //     192,000 x 10,000: kd 1082 373 -> 353;  61,206 x 5,003: kd 1443 51 -> 55 (not)
 static int mskip_passes(const rsot_problem *p, double eps) {
     const double kd = kLog2e / (2.0 * eps) * p->diam2;
-    if (p->in_solve || !(kd <= 0x1p20)) return 0;
+    if (p->in_solve || p->pair_kernel != 2 || !(kd <= 0x1p20)) return 0;
     return (kd >= 700.0 && kd * (double)p->chunk1 >= 5e6 ? 1 : 0) |
            (kd >= 500.0 && (double)p->nq * (double)p->n >= 1.5e9 ? 2 : 0);
 }

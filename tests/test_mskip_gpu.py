@@ -22,9 +22,17 @@ def _check(x, m, y, nu, psi, eps, forms):
         J, g, pairs = P.eval(psi, eps, 0.0, rs.MIXED)
         names = set(P.kernel_times())
         L = P.point_log_partition()
+        P.set_pair_kernel(rs.PAIRS_FP32)   # every pair: the same to 2^-59 of a sum
+        Jd, gd, _ = P.eval(psi, eps, 0.0, rs.MIXED)
+        Ld = P.point_log_partition()
+        assert "lse_mixed" in P.kernel_times()
     finally:
         P.close()
     assert forms <= names and pairs == len(m) * len(nu)
+    # FP64 sums in another order (512 points each: at most nq / 512 terms)
+    order = (len(m) / 512 + 2) * 2.0 ** -52
+    assert np.all(np.abs(g - gd) <= order * (gd + 2 * nu))
+    assert np.all(np.abs(L - Ld) <= 2.0 ** -50 * (1 + np.abs(Ld))) and abs(J - Jd) <= 2.0 ** -50 * (1 + abs(Jd))
     rel = 2 * delta_of(x, y, nu, psi, eps) + 2.0 ** -24 * 512
     assert np.all(np.abs(g - g64) <= rel * (g64 + nu) + 1e-14 * nu)
     live = m > 0
