@@ -381,8 +381,9 @@ def run_solve_workloads(args):
                "steps": args.steps, "warmup": args.warmup, "ms_per_step": kt["maps"],
                "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
                "data": "synthetic", "config": {"workload": f"cube-{p.nq}x{p.n}-maps-eps{args.eps:g}"},
-               "centroids": {"value": pairs / (kt["centroids"] * 1e-3) / 1e9, "unit": "G pairs/s",
-                             "ms": kt["centroids"]},
+               # pass 2 of the evaluation with the centroids' sums, and their last kernel
+               "centroids": {"value": pairs / ((kt["grad_centroids"] + kt["centroids"]) * 1e-3) / 1e9,
+                             "unit": "G pairs/s", "ms": kt["grad_centroids"] + kt["centroids"]},
                "per_kernel_ms": kt}
         print(json.dumps(out))
         return
