@@ -407,6 +407,7 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
         if (!e) e = cudaStreamSynchronize(st);
     }
     p->final_out = nullptr;
+    p->psi_src = nullptr;   // also where an error came before the kernel that takes it
     if (e) {
         cudaGetLastError();
         p->tr_open.clear();
