@@ -924,7 +924,7 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
 // weight stages instead of two and fetches the next layer's weights during the
 // epilogue.  The per-layer kernels this replaces wrote and read H, Z and dZ of
 // every layer (33 MB each at 65,536 x 256) and ran 32 of 152 SMs at 4,096 rows.
-//   forward, 4,096 rows: GPU time 50 -> 17 us (the call 84 -> 45);
+//   forward, 4,096 rows: GPU time 50 -> 12 us (the call 84 -> 40);
 //   forward + back-propagation, 65,536 rows: 240 -> 119 us (the gradients' call
 //   384 -> 236).
 // TRAIN also stores X0, H1, H2 and the three dZ (the weight gradients' operands;
@@ -1008,8 +1008,13 @@ __device__ __forceinline__ void nf_commit(uint64_t *bar) {
         : "memory");
 }
 
-template <bool TRAIN>
-__global__ void __launch_bounds__(NF_THREADS, 2)
+// REP (forward of 32-row tiles): the operand's rows are kept four times, so that every
+// quarter of the tensor memory's lanes holds the tile and each of the 16 epilogue warps
+// takes 16 of a block's 64 columns: a quarter of the epilogue's chain for a fourfold store.
+// PAIR (width 256, every stage): one MMA takes two stages, 256 columns, which halves the
+// issue.  Forward of 4,096 rows: 17.1 us without, 12.1 with both.
+template <bool TRAIN, bool REP, bool PAIR>
+__global__ void __launch_bounds__(NF_THREADS, REP ? 1 : 2)
     k_net(const __grid_constant__ NetArgs a, const __grid_constant__ NetMaps maps) {
     extern __shared__ __align__(1024) unsigned char nf_dyn[];
     __shared__ __align__(8) uint64_t full[NF_MAXST], empty[NF_MAXST], aready, accf, mdone;
@@ -1083,6 +1088,7 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
         constexpr uint32_t dhi = (uint32_t)((((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61)) >> 32);
         const uint32_t abase = ((smem_u32(sA) >> 4) & 0x3FFFu) | (1u << 16);
         const uint32_t wbase = ((smem_u32(sW) >> 4) & 0x3FFFu) | (1u << 16);
+        constexpr int hstep = PAIR ? 256 : 128;
         int s = 0;
         unsigned k = 0, par = 0;
         for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x)
@@ -1094,14 +1100,15 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int k0 = 0; k0 < (st == 0 ? 1 : w) && ok; k0 += 64)
-                    for (int h0 = 0; h0 < w; h0 += 128) {
-                        if (!__all_sync(0xffffffffu, mbar_wait(&full[s], par))) {
+                    for (int h0 = 0; h0 < w; h0 += hstep) {
+                        if (!__all_sync(0xffffffffu, mbar_wait(&full[s], par) &&
+                                                         (hstep == 128 || mbar_wait(&full[s + 1], par)))) {
                             ok = false;
                             break;
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24) |
-                                               (w - h0 >= 128 ? 16u << 17 : 8u << 17);
+                                               ((uint32_t)(min(hstep, w - h0) >> 3) << 17);
                         const uint32_t a0 = abase + (uint32_t)(k0 >> 6) * (NF_BLK >> 4);
                         const uint32_t b0 = wbase + (uint32_t)s * (NF_BLK >> 4);
 #pragma unroll
@@ -1110,6 +1117,7 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
                                 nf_mma(tmem + (uint32_t)h0, a0 + 2 * kk, b0 + 2 * kk, dhi, idesc,
                                        kk > 0 || k0 > 0);
                         nf_commit(&empty[s]);
+                        if (hstep == 256) nf_commit(&empty[++s]);
                         if (++s == stages) {
                             s = 0;
                             par ^= 1u;
@@ -1124,13 +1132,26 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
         // a wait that gives up clears ok; the warp then passes every barrier without
         // waiting for the accumulator again, so that no warp is left at one
         const int q = warp & 3, jb = (warp - 2) >> 2, et = tid - 64;
-        const bool live = 32 * q < a.rt, act = live && 64 * jb < w;
+        const bool live = REP || 32 * q < a.rt, act = live && 64 * jb < w;
+        const int src = REP ? lane : 32 * q + lane;   // the row's place in the tile
+        const int cfirst = REP ? q : 0, clast = REP ? q + 1 : 4;   // 16-column pieces of the thread's block
         const int r = 32 * q + lane, c0 = 64 * jb;
         const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
         unsigned char *const aRow = sA + jb * NF_BLK + r * 128;   // the thread's 128 B of its block
         unsigned char *const aBox = sA + jb * NF_BLK + q * 4096;  // the warp's 32 rows of it
         // 16 columns 16 c .. + 15 of the thread's 64: two swizzled 16-byte chunks
         auto put = [&](int c, const uint32_t (&v)[8]) {
+            if constexpr (REP) {   // rows lane, lane + 32, ... alike
+                unsigned char *const p = sA + jb * NF_BLK + lane * 128;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    *reinterpret_cast<uint4 *>(p + k * 4096 + (((2 * c) ^ (lane & 7)) << 4)) =
+                        make_uint4(v[0], v[1], v[2], v[3]);
+                    *reinterpret_cast<uint4 *>(p + k * 4096 + (((2 * c + 1) ^ (lane & 7)) << 4)) =
+                        make_uint4(v[4], v[5], v[6], v[7]);
+                }
+                return;
+            }
             *reinterpret_cast<uint4 *>(aRow + (((2 * c) ^ (r & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
             *reinterpret_cast<uint4 *>(aRow + (((2 * c + 1) ^ (r & 7)) << 4)) = make_uint4(v[4], v[5], v[6], v[7]);
         };
@@ -1185,7 +1206,7 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
         float sd = 0.f, sl = 0.f;
         for (int t = blockIdx.x; t < a.tiles; t += gridDim.x) {
             const int row0 = t * a.rt;
-            const int64_t gr = row0 + r;
+            const int64_t gr = row0 + src;
             if (TRAIN) {
                 stores_read();
                 nf_bar();   // the column sums of the tile before have read the operand
@@ -1204,7 +1225,7 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
                 float xv[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    xv[i] = (16 * jb + i < a.in_dim && gr < a.valid) ? sX[r * a.in_dim + 16 * jb + i] : 0.f;
+                    xv[i] = (16 * jb + i < a.in_dim && gr < a.valid) ? sX[src * a.in_dim + 16 * jb + i] : 0.f;
                 uint32_t v[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) v[i] = pack_bf16(xv[2 * i], xv[2 * i + 1]);
@@ -1222,7 +1243,7 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
                     const float *const bias = sC + 256 * l + c0;
                     bf16 *const Z = (l ? a.Z[1] : a.Z[0]) + gr * w + c0;
 #pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = cfirst; c < clast; ++c) {
                         uint32_t v[16], zv[8], hv[8];
                         t5_ld16(v, trow + 16 * c);
 #pragma unroll
@@ -1243,6 +1264,36 @@ __global__ void __launch_bounds__(NF_THREADS, 2)
             // then the 32 sums in the order of a warp's shuffle tree
             acc_wait();
             if (TRAIN) stores_read();
+            if constexpr (REP) {
+                float p2[2] = {0.f, 0.f};
+                if (act) {
+                    const float *const bias = sC + 512 + c0 + 16 * q, *const w4 = sC + 768 + c0 + 16 * q;
+                    uint32_t v[16];
+                    t5_ld16(v, trow + 16 * q);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float2 b = *reinterpret_cast<const float2 *>(bias + 2 * i);
+                        const float2 wv = *reinterpret_cast<const float2 *>(w4 + 2 * i);
+                        const float2 h = unpack_bf16(pack_bf16(silu(__uint_as_float(v[2 * i]) + b.x),
+                                                               silu(__uint_as_float(v[2 * i + 1]) + b.y)));
+                        p2[i / 4] = fmaf(h.x, wv.x, p2[i / 4]);
+                        p2[i / 4] = fmaf(h.y, wv.y, p2[i / 4]);
+                    }
+                }
+                sV[(8 * jb + 2 * q) * 32 + lane] = p2[0];
+                sV[(8 * jb + 2 * q + 1) * 32 + lane] = p2[1];
+                nf_bar();
+                if (warp == 4) {   // rows of the tile: jb = 0, q = 0
+                    float t[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        t[i] = (sV[i * 32 + lane] + sV[(i + 16) * 32 + lane]) +
+                               (sV[(i + 8) * 32 + lane] + sV[(i + 24) * 32 + lane]);
+                    const float o = ((t[0] + t[4]) + (t[2] + t[6])) + ((t[1] + t[5]) + (t[3] + t[7])) + a.b4[0];
+                    if (gr < a.valid && ok) a.out[gr] = o;
+                }
+                continue;
+            }
             float v8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             if (act) {
                 const float *const bias = sC + 512 + c0, *const w4 = sC + 768 + c0;
@@ -2170,13 +2221,17 @@ bool launch_net(rsot_mlp *m, int64_t rows, const float *x, const float *y, float
         for (int i = 0; i < 5; ++i) t = t && t6_tensor_map(&maps.st[i], dst[i], R, w, w, 32);
     }
     if (!t) return false;
+    const bool alone = a.stages == NF_MAXST, pair = alone && w == 256, rep = !TRAIN && alone && a.rt == 32;
+    auto f = rep ? (pair ? k_net<TRAIN, !TRAIN, true> : k_net<TRAIN, !TRAIN, false>)
+                 : (pair ? k_net<TRAIN, false, true> : k_net<TRAIN, false, false>);
     static std::atomic<bool> attr{false};
     if (!attr.load()) {
-        cudaFuncSetAttribute((const void *)k_net<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             nf_smem(NF_MAXST));
+        for (auto g : {k_net<TRAIN, !TRAIN, true>, k_net<TRAIN, !TRAIN, false>, k_net<TRAIN, false, true>,
+                       k_net<TRAIN, false, false>})
+            cudaFuncSetAttribute((const void *)g, cudaFuncAttributeMaxDynamicSharedMemorySize, nf_smem(NF_MAXST));
         attr.store(true);
     }
-    k_net<TRAIN><<<grid, NF_THREADS, nf_smem(a.stages), m->stream>>>(a, maps);
+    f<<<grid, NF_THREADS, nf_smem(a.stages), m->stream>>>(a, maps);
     if (TRAIN) net_fin(m, grid, a.part, loss_sum);
     return true;
 }
