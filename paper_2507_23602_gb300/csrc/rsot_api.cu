@@ -185,6 +185,8 @@ void rsot_destroy(rsot_problem *p) {
     delete p;
 }
 
+static constexpr int64_t kPsiDirect = 65536;   // largest host potential that a kernel reads in place
+
 rsot_status rsot_create(int d, int64_t nq, const double *x, const double *mass, int64_t n,
                         const double *y, const double *nu, int device_ptrs, rsot_problem **out) {
     if (!out) return RSOT_ERR_ARG;
@@ -296,7 +298,7 @@ rsot_status rsot_create(int d, int64_t nq, const double *x, const double *mass, 
     if (!e) e = cudaMalloc(&p->grad_dev, (size_t)n * 8);
     if (!e) e = cudaMalloc(&p->res_dev, sizeof(EvalResult) + 8 * sizeof(double));
     if (!e) e = cudaMallocHost(&p->res_host, sizeof(EvalResult) + 8 * sizeof(double));
-    if (!e) e = cudaMallocHost(&p->grad_host, (size_t)n * 16);
+    if (!e) e = cudaMallocHost(&p->grad_host, (size_t)(n + std::min(n, kPsiDirect)) * 8);
     if (!e) p->psi_host = p->grad_host + n;
     if (e) {
         cudaGetLastError();
@@ -324,8 +326,6 @@ rsot_status rsot_set_pair_kernel(rsot_problem *p, rsot_pair_kernel kind) {
 // One evaluation: dense (mode 0), truncated by a radius (mode 1, cutoff C =
 // arg^2 / 2 for every pair) or by the separable psi-aware cutoffs (mode 2,
 // tail = arg, rsot_cutoff.cu).
-constexpr int64_t kPsiDirect = 65536;   // largest host potential that a kernel reads in place
-
 static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int mode, double arg,
                              rsot_precision prec, double *J_out, double *grad_out,
                              int64_t *pairs_out, const std::function<cudaError_t()> &then = nullptr) {
@@ -348,7 +348,7 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     // where the caller's gradient overlaps it (the final kernel reads psi[0])
     const bool gdev = wgrad == 1;
     if (wpsi == 0) {
-        memcpy(p->psi_host, psi, nb);
+        if (p->n <= kPsiDirect) memcpy(p->psi_host, psi, nb);
         psid = p->psi_dev;
     } else if (gdev && psi < grad_out + p->n && grad_out < psi + p->n) {
         psid = p->psi_dev;
@@ -363,7 +363,9 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     // a radius beyond the diameter of the data keeps every pair: dense
     const bool dense = mode == 0 || (mode == 1 && (!(arg > 0.0) || isinf(arg) ||
                                                     arg * arg > p->diam2 * (1.0 + 1e-12)));
-    const auto upload = [&]() { return cudaMemcpyAsync(p->psi_dev, p->psi_host, nb, cudaMemcpyHostToDevice, st); };
+    const auto upload = [&]() {
+        return cudaMemcpyAsync(p->psi_dev, p->n <= kPsiDirect ? p->psi_host : psi, nb, cudaMemcpyHostToDevice, st);
+    };
     if (!e && !dense && wpsi == 0) e = upload();
     if (!e && !dense) e = mode == 1 ? cutoffs_uniform(p, 0.5 * arg * arg) : cutoffs_separable(p, psid, eps, arg);
     // dense FP64: fixed-point exponents where they can hold the range, the FP64

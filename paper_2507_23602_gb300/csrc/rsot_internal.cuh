@@ -183,7 +183,7 @@ struct rsot_problem {
 
     // staging for host psi / grad
     double *psi_dev = nullptr;      // [n]
-    double *psi_host = nullptr;     // pinned [n]: a host potential on its way
+    double *psi_host = nullptr;     // pinned (behind grad_host): a small host potential on its way
     const double *psi_src = nullptr;   // set: the next prep kernel reads psi there and fills psi_dev
     bool borrowed = false;          // mass and nu are the caller's device arrays (not freed)
     double *grad_dev = nullptr;     // [n] gradient of the last evaluation
