@@ -23,8 +23,8 @@
 // Both tests carry a margin of 2^-19 (|terms|), twice the bound of the FP32
 // exponents' error (rsot_skip.cuh).
 // Bound: the packed FP32 instructions of the pairs that remain, and about ten
-// instructions a column for the loop over a mask's bits (shared by 256 rows).  786,432 x 65,536, eps 1e-3: 8.4 -> 3.6 and 8.5 -> 3.8 ms, the
-// call 17.0 -> 7.5.
+// instructions a column for the loop over a mask's bits (shared by 128 rows).
+// 786,432 x 65,536, eps 1e-3: 8.4 -> 3.4 and 8.5 -> 3.4 ms, the call 17.0 -> 7.05.
 #include <math.h>
 
 #include <algorithm>
@@ -39,7 +39,7 @@ namespace {
 constexpr int MS_WARPS = 4, MS_THREADS = 32 * MS_WARPS;
 
 template <int D, int PP>
-__global__ void __launch_bounds__(MS_THREADS, PP == 4 ? 4 : PP == 2 ? 6 : 8)
+__global__ void __launch_bounds__(MS_THREADS, 8)
     k_lse_skip(const float *__restrict__ xs, const int *__restrict__ perm, int64_t nq, int64_t nq_pad,
                const float4 *__restrict__ tquad, int n, int chunk, float k, float kdiam2, float t1,
                float2 *__restrict__ part) {
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(MS_THREADS, PP == 4 ? 4 : PP == 2 ? 6 : 8)
 }
 
 template <int D, int TPP>
-__global__ void __launch_bounds__(MS_THREADS, TPP == 4 ? 4 : TPP == 2 ? 6 : 8)
+__global__ void __launch_bounds__(MS_THREADS, TPP == 2 ? 6 : 8)
     k_grad_skip(const float4 *__restrict__ tquad, const int *__restrict__ perm, const double *__restrict__ nu,
                 int64_t n, const float4 *__restrict__ pquad, int64_t nq, int64_t chunk, float k, float kdiam2,
                 float t2, double *__restrict__ part2, int64_t stride) {
@@ -266,9 +266,11 @@ __global__ void __launch_bounds__(MS_THREADS, TPP == 4 ? 4 : TPP == 2 ? 6 : 8)
     }
 }
 
-// rows (pairs) per thread: most where that leaves a few warps per scheduler
+// pairs of rows per thread: two where that leaves a few warps per scheduler, else one
+// (four: fewer tests, but wider boxes and half the warps; 786,432 x 65,536 at eps 1e-3:
+// 3.58 and 3.76 ms with four, 3.39 and 3.43 with two, 6.35 and 6.04 with one)
 int rows_per_thread(int64_t rows, int64_t splits, int num_sms) {
-    int pp = 4;
+    int pp = 2;
     while (pp > 1 && (rows + 64 * pp - 1) / (64 * pp) * splits < (int64_t)num_sms * 32) pp /= 2;
     return pp;
 }
@@ -285,29 +287,30 @@ void mskip_free(rsot_problem *p) {
 // few pairs can be left out (kd = k diam^2, in 3-D a pair's reach is about
 // sqrt(78 / kd) of the diameter) or the work is too small for the loops over masks and
 // the first, whole stage.  Both sides in us:
-//   pass 1, kd >= 700 and kd x targets per chunk >= 5e6:
-//     786,432 x 65,536: kd 2164 8435 -> 3562, 721 8385 -> 7614, 433 8376 -> 9544 (not)
-//     194,400 x 30,000: kd 721 804 -> 772;  192,000 x 10,000: kd 2164 (3,584 per chunk)
-//     363 -> 316, 1082 352 -> 371 (not);  61,206 x 5,003: kd 1443 55 -> 78 (not)
-//   pass 2, kd >= 500 and 1.5e9 pairs:
-//     786,432 x 65,536: kd 2164 8460 -> 3751, 721 8454 -> 6777, 433 8455 -> 8310 (not)
-//     192,000 x 10,000: kd 1082 373 -> 353;  61,206 x 5,003: kd 1443 51 -> 55 (not)
+//   pass 1, kd >= 700 and kd x targets per chunk >= 2e6:
+//     786,432 x 65,536: kd 2164 8439 -> 3392, 721 8382 -> 7107, 433 8375 -> 9096 (not)
+//     331,776 x 16,384 (2,048 per chunk): kd 2164 970 -> 568, 1082 952 -> 785, 721 946 -> 935
+//     192,000 x 10,000 (1,024): kd 2164 364 -> 267;  61,206 x 5,003 (512): kd 2885 61 -> 73 (not)
+//   pass 2, kd >= 500 and 1e9 pairs:
+//     786,432 x 65,536: kd 2164 8458 -> 3428, 721 8456 -> 6669, 433 8457 -> 8452 (not)
+//     192,000 x 10,000: kd 1082 373 -> 346;  60,000 x 20,000: kd 2885 188 -> 92
+//     61,206 x 5,003: kd 2885 51.1 -> 51.2 (not)
 static int mskip_passes(const rsot_problem *p, double eps) {
     const double kd = kLog2e / (2.0 * eps) * p->diam2;
     if (p->in_solve || p->pair_kernel != 2 || !(kd <= 0x1p20)) return 0;
-    return (kd >= 700.0 && kd * (double)p->chunk1 >= 5e6 ? 1 : 0) |
-           (kd >= 500.0 && (double)p->nq * (double)p->n >= 1.5e9 ? 2 : 0);
+    return (kd >= 700.0 && kd * (double)p->chunk1 >= 2e6 ? 1 : 0) |
+           (kd >= 500.0 && (double)p->nq * (double)p->n >= 1e9 ? 2 : 0);
 }
 
 static bool mskip_alloc(rsot_problem *p) {
     if (p->ms_buf) return true;
-    const int64_t blk = 256 * MS_WARPS, tiles = p->nq_pad / P2_TS, units = (p->n + blk - 1) / blk;
+    const int64_t blk = 128 * MS_WARPS, tiles = p->nq_pad / P2_TS, units = (p->n + blk - 1) / blk;
     // pass 2 in about 60 CTAs per SM where that many stages exist: skipping leaves
     // their work uneven; at most 64 splits (the last kernel's sums)
     const int64_t want = std::min({tiles, (60 * p->num_sms + units - 1) / units, (int64_t)64});
     p->ms_chunk2 = (tiles + want - 1) / want * P2_TS;
     p->ms_s2 = (int)((p->nq_pad + p->ms_chunk2 - 1) / p->ms_chunk2);
-    // rows are read in whole warps of 256: the orders are padded to that (1,024s)
+    // rows are read in whole warps of 64 or 128: the orders are padded to that (1,024s)
     const size_t np = (size_t)p->nq_pad, nt = (size_t)p->n_pad;
     const size_t scratch = (std::max(np, nt) + 4096) * 4;
     char *b = nullptr;
@@ -345,7 +348,7 @@ static void mskip_lse_d(rsot_problem *p, double eps) {
     const float k = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
     const int pp = rows_per_thread(p->nq, p->k1, p->num_sms);
     dim3 g((unsigned)((p->nq + 64 * pp * MS_WARPS - 1) / (64 * pp * MS_WARPS)), (unsigned)p->k1);
-    auto f = pp == 4 ? k_lse_skip<D, 4> : pp == 2 ? k_lse_skip<D, 2> : k_lse_skip<D, 1>;
+    auto f = pp == 2 ? k_lse_skip<D, 2> : k_lse_skip<D, 1>;
     launch_pdl(overlap_pass(g, p->num_sms), f, g, MS_THREADS, 0, p->stream, p->xs, p->ms_perm_q, p->nq, p->nq_pad,
                p->tquad, (int)p->n, p->chunk1, k, kd, (float)(61.0 + log2((double)p->n)), p->part1);
 }
@@ -356,7 +359,7 @@ static void mskip_grad_d(rsot_problem *p, double eps) {
     const float k = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
     const int pp = rows_per_thread(p->n, p->ms_s2, p->num_sms);
     dim3 g((unsigned)((p->n + 64 * pp * MS_WARPS - 1) / (64 * pp * MS_WARPS)), (unsigned)p->ms_s2);
-    auto f = pp == 4 ? k_grad_skip<D, 4> : pp == 2 ? k_grad_skip<D, 2> : k_grad_skip<D, 1>;
+    auto f = pp == 2 ? k_grad_skip<D, 2> : k_grad_skip<D, 1>;
     launch_pdl(overlap_pass(g, p->num_sms), f, g, MS_THREADS, 0, p->stream, p->tquad, p->ms_perm_t, p->nu, p->n,
                p->pquad, p->nq, p->ms_chunk2, k, kd, (float)(61.0 + log2((double)p->nq)), p->ms_part2, p->n_pad);
 }

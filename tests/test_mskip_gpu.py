@@ -70,3 +70,10 @@ def test_shifts_and_ranges(case):
         x[:20000] += [4.0, 0.0, 0.0]
         y[:300] -= [0.0, 3.0, 0.0]
     _check(x, m / m.sum(), y, nu, psi, eps, {"lse_skip", "grad_skip"})
+
+
+# the smallest work that leaves pairs out: many chunks of targets, few warps per scheduler
+@pytest.mark.parametrize("d,nq,n,eps", [(3, 331777, 16383, 1e-3), (3, 98305, 16385, 1e-3), (2, 153601, 10001, 5e-4)])
+def test_smaller_work(d, nq, n, eps):
+    x, m, y, nu, rng = _problem(d, nq, n, nq + n)
+    _check(x, m, y, nu, 0.5 * eps * rng.standard_normal(n), eps, {"lse_skip", "grad_skip"})
