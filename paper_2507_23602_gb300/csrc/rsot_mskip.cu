@@ -287,19 +287,21 @@ void mskip_free(rsot_problem *p) {
 // few pairs can be left out (kd = k diam^2, in 3-D a pair's reach is about
 // sqrt(78 / kd) of the diameter) or the work is too small for the loops over masks and
 // the first, whole stage.  Both sides in us:
+//   either, 1e9 pairs: with less, a problem's first call pays for the orders (~0.3 ms)
+//     what many later ones save (98,304 x 4,096: kd 4328 105 -> 95 and 84 -> 79)
 //   pass 1, kd >= 700 and kd x targets per chunk >= 2e6:
 //     786,432 x 65,536: kd 2164 8439 -> 3392, 721 8382 -> 7107, 433 8375 -> 9096 (not)
 //     331,776 x 16,384 (2,048 per chunk): kd 2164 970 -> 568, 1082 952 -> 785, 721 946 -> 935
 //     192,000 x 10,000 (1,024): kd 2164 364 -> 267;  61,206 x 5,003 (512): kd 2885 61 -> 73 (not)
-//   pass 2, kd >= 500 and 1e9 pairs:
+//   pass 2, kd >= 500:
 //     786,432 x 65,536: kd 2164 8458 -> 3428, 721 8456 -> 6669, 433 8457 -> 8452 (not)
 //     192,000 x 10,000: kd 1082 373 -> 346;  60,000 x 20,000: kd 2885 188 -> 92
 //     61,206 x 5,003: kd 2885 51.1 -> 51.2 (not)
 static int mskip_passes(const rsot_problem *p, double eps) {
     const double kd = kLog2e / (2.0 * eps) * p->diam2;
     if (p->in_solve || p->pair_kernel != 2 || !(kd <= 0x1p20)) return 0;
-    return (kd >= 700.0 && kd * (double)p->chunk1 >= 2e6 ? 1 : 0) |
-           (kd >= 500.0 && (double)p->nq * (double)p->n >= 1e9 ? 2 : 0);
+    if ((double)p->nq * (double)p->n < 1e9) return 0;
+    return (kd >= 700.0 && kd * (double)p->chunk1 >= 2e6 ? 1 : 0) | (kd >= 500.0 ? 2 : 0);
 }
 
 static bool mskip_alloc(rsot_problem *p) {
