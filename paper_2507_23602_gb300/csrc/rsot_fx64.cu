@@ -21,6 +21,11 @@
 //     1 - z + z^2/2 (1 - c z), z = g ln 2, in 32-bit integer multiplications
 //     (c is 1/3 less the value that centres the dropped z^4/24: error below
 //     2^-54); its FP64 bits are those of 1.0 minus the integer 2^53 (1 - q).
+//   * A term of pass 2 is m_q p_qj, and the exponent field of its FP64 value has no
+//     lower end to stop at, so every term that is summed has to stay above 2^-1020:
+//     points whose mass is below 2^-61 of the smallest weight over their number are
+//     left out of pass 2 (all of them together stay below 2^-61 nu_j), which bounds
+//     the others from below by the weights (fx_exponents_fit).
 //   * Pairs that cannot change a sum by 2^-60 of it are skipped (rsot_skip.cuh).
 //     The wrapped integers are only read for pairs that are not, whose exponents
 //     lie inside the range that F allows.
@@ -29,7 +34,7 @@
 //
 // Where the skipping's estimate could be off by more than 16 or the exponents
 // need F < 46 the records kernel raises kErrRange64 and the caller runs the FP64
-// passes.
+// passes; they also run where the weights reach further down than that allows.
 //
 // A pair and pass takes about 55 instructions: the FP64 pipe (one fma) is 63 %
 // busy, the FMA pipe with the multiplications 76 %.
@@ -336,11 +341,11 @@ __global__ void __launch_bounds__(FX_THREADS)
         if (at[k] >= 0) out[(int64_t)blockIdx.y * rows.pad + at[k]] = acc[k];
 }
 
-// Per point: L_q, the mass's J term, and the column of pass 2: u_q = log2(m_q /
-// S_q) - shift_q, (x', -R_q) and A_q.
+// Per point: L_q, the mass's J term, and, for masses from m_least on, the column of
+// pass 2: u_q = log2(m_q / S_q) - shift_q, (x', -R_q) and A_q.
 __global__ void k_fx_combine(const double *__restrict__ part, int k1, int64_t nq, int64_t nq_pad,
                              const int *__restrict__ shift, const double *__restrict__ mass,
-                             const double *__restrict__ psi, double eps, float t1,
+                             double m_least, const double *__restrict__ psi, double eps, float t1,
                              const float4 *__restrict__ ptrow, FxRec *__restrict__ prec,
                              float4 *__restrict__ ptcol, float *__restrict__ ptA,
                              double *__restrict__ lse_buf, double *__restrict__ blockJ,
@@ -360,8 +365,8 @@ __global__ void k_fx_combine(const double *__restrict__ part, int k1, int64_t nq
         const float rise = (float)M + ptA[q] + __log2f((float)S);   // R_q - max_j r_qj
         float4 col = make_float4(x.x, x.y, x.z, kPadC);
         float A = -INFINITY;
-        if (m > 0.0) {
-            contrib = m * (psi[0] + eps * L);
+        if (m > 0.0) contrib = m * (psi[0] + eps * L);
+        if (m >= m_least) {
             int em, es;
             const double fm = log2_split(m, em), fs = log2_split(S, es);
             const long long C = 1 - to_fixed((double)(em - es - M), fm - fs, res->fx_F);
@@ -441,7 +446,19 @@ void fx64_free(rsot_problem *p) {
     p->fx_buf = nullptr;
 }
 
-bool fx64_ready(rsot_problem *p, double eps) { return skip_ready(p, eps) && fx_alloc(p); }
+// the smallest mass that takes part in pass 2
+static double fx_least_mass(const rsot_problem *p) { return ldexp(p->nu_min, -61) / (double)p->nq; }
+
+// A term of pass 2 that is summed is at least fx_least_mass() times the smallest p_qj
+// of a pair that is kept, 2^-60 nu_j / sum m less four errors E <= 16 of the estimate:
+// its exponent stays above -1020 (weights down to about 1e-120 of a total mass of 1).
+static bool fx_exponents_fit(const rsot_problem *p) {
+    return log2(fx_least_mass(p)) + (log2(p->nu_min) - log2(p->msum)) - 60.0 - 4.0 * 16.0 >= -1020.0;
+}
+
+bool fx64_ready(rsot_problem *p, double eps) {
+    return fx_exponents_fit(p) && skip_ready(p, eps) && fx_alloc(p);
+}
 
 cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, double *grad) {
     cudaStream_t st = p->stream;
@@ -478,7 +495,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     const int nbq = (int)(p->nq_pad / 256);
     const unsigned tc = p->per_comb == 1 ? 256 : kSmall;
     launch_pdl(true, k_fx_combine, (unsigned)(p->nq_pad / tc), tc, 0, st, p->fx_part1, p->fx_k1, p->nq, p->nq_pad, p->fx_ptshift, p->mass,
-                                      psi, eps, (float)t1, p->sk_ptrow, p->fx_prec, p->sk_ptcol,
+                                      fx_least_mass(p), psi, eps, (float)t1, p->sk_ptrow, p->fx_prec, p->sk_ptcol,
                                       p->sk_ptA, p->lse_buf, p->blockJ, p->res_dev);
     trace_end(p);
     const FxRows tgr = {p->fx_trec,  p->sk_tgrow, p->sk_tgB, p->fx_tgshift, p->sk_perm, false,
