@@ -1211,15 +1211,16 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
                    p->part2, p->n_pad, p->flags, gate);
         trace_end(p);
     }
-    if (p->cent_now && !tc) {   // the centroids' sums with pass 2
+    if (p->cent_now) {   // the centroids' sums with pass 2; after tensor-core passes for themselves
         trace_begin(p, "grad_centroids");
         launch_grad_cent<D>(p);
         trace_end(p);
         const int64_t stride = (D + 2) * p->n_pad;
-        return launch_finalize(p, psi, eps,
-                               {p->cent_part, p->cent_s2, stride, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1,
-                                p->per_prep},
-                               grad);
+        if (!tc)
+            return launch_finalize(p, psi, eps,
+                                   {p->cent_part, p->cent_s2, stride, nullptr, p->blockJ, p->nblk_comb, p->per_comb,
+                                    1, p->per_prep},
+                                   grad);
     }
     if (skip & 2) {
         trace_begin(p, "grad_skip");
@@ -1234,16 +1235,8 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
     launch_grad_mixed<D>(p->tpair, p->n, p->pquad, p->nq, chunk2, s2, p->part2, p->n_pad, p->flags,
                          gate, p->num_sms, st);
     trace_end(p);
-    cudaError_t e = launch_finalize(
+    return launch_finalize(
         p, psi, eps, {p->part2, s2, p->n_pad, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1, p->per_prep}, grad);
-    // after tensor-core passes: the FP32 pass for the centroids alone
-    if (!e && p->cent_now) {
-        trace_begin(p, "grad_centroids");
-        launch_grad_cent<D>(p);
-        trace_end(p);
-        e = cudaGetLastError();
-    }
-    return e;
 }
 
 // ----------------------------------------------------------------------------
