@@ -321,9 +321,10 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi_dev, double eps
 void fx64_free(rsot_problem *p);
 // the smallest column split whose CTAs fill the resident slots
 int split_for_slots(int64_t units, int64_t tiles, int64_t slots);
-// rows 0 .. n (row j at pos[j step][d]) by the cells of a grid along the Morton curve, then
-// n .. n_pad as they are; scratch: n_pad + 4,096 integers
-cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_pad, int *perm, int *scratch,
+// rows 0 .. n (row j at pos[j step][d]) by the cells of a grid along the Morton curve, those of
+// a cell in their own order, then n .. n_pad as they are; scratch: cell_order_scratch(n) bytes
+size_t cell_order_scratch(int64_t n);
+cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_pad, int *perm, void *scratch,
                        int step = 1);
 // dense mixed passes without the pairs that cannot matter (rsot_mskip.cu)
 int mskip_ready(rsot_problem *p, double eps);   // bit 0: pass 1, bit 1: pass 2

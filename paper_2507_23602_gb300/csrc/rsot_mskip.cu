@@ -314,20 +314,20 @@ static bool mskip_alloc(rsot_problem *p) {
     p->ms_s2 = (int)((p->nq_pad + p->ms_chunk2 - 1) / p->ms_chunk2);
     // rows are read in whole warps of 64 or 128: the orders are padded to that (1,024s)
     const size_t np = (size_t)p->nq_pad, nt = (size_t)p->n_pad;
-    const size_t scratch = (std::max(np, nt) + 4096) * 4;
+    // the orders, then pass 2's partials, whose place is scratch while the orders are made
+    const size_t part = std::max({nt * 8 * p->ms_s2, cell_order_scratch(p->n), cell_order_scratch((p->nq + 1) / 2)});
     char *b = nullptr;
-    if (cudaMalloc(&b, np * 4 + nt * 4 + nt * 8 * p->ms_s2 + scratch) != cudaSuccess) {
+    if (cudaMalloc(&b, np / 2 * 4 + nt * 4 + part) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     p->ms_buf = b;
-    p->ms_part2 = reinterpret_cast<double *>(b);
-    p->ms_perm_q = reinterpret_cast<int *>(b + nt * 8 * p->ms_s2);
-    p->ms_perm_t = p->ms_perm_q + np;
-    int *tmp = p->ms_perm_t + nt;
+    p->ms_perm_q = reinterpret_cast<int *>(b);
+    p->ms_perm_t = p->ms_perm_q + np / 2;
+    p->ms_part2 = reinterpret_cast<double *>(p->ms_perm_t + nt);
     // points by pairs, which share a raise of their shifts
-    cudaError_t e = cell_order(p, p->x64, (p->nq + 1) / 2, p->nq_pad / 2, p->ms_perm_q, tmp, 2);
-    if (!e) e = cell_order(p, p->y64, p->n, p->n_pad, p->ms_perm_t, tmp);
+    cudaError_t e = cell_order(p, p->x64, (p->nq + 1) / 2, p->nq_pad / 2, p->ms_perm_q, p->ms_part2, 2);
+    if (!e) e = cell_order(p, p->y64, p->n, p->n_pad, p->ms_perm_t, p->ms_part2);
     // once per problem: a later evaluation may run on another stream
     if (!e) e = cudaStreamSynchronize(p->stream);
     if (e) {

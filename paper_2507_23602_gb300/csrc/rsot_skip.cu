@@ -124,25 +124,52 @@ __global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t 
     }
 }
 
-// Order of the target rows of pass 2: by cells of a 2^b grid in Morton order
-// (counting sort, once per problem), so that a warp's targets are near each
-// other and most of a far point's pairs are skipped by whole warps: at eps 1e-3
-// (98,304 x 16,384) the FP64 pass 2 takes 1.6 ms, 3.7 in the caller's order.
-// The order inside a cell is whatever the atomics give; a row's sum does not
-// depend on it.
-__global__ void k_cell_count(const double *__restrict__ y64, int64_t n, int step, int d, double half,
-                             int *__restrict__ cell, int *__restrict__ count) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
+// Order of the target rows of pass 2: by cells of a 2^b grid in Morton order, so
+// that a warp's targets are near each other and most of a far point's pairs are
+// skipped by whole warps: at eps 1e-3 (98,304 x 16,384) the FP64 pass 2 takes 1.6
+// ms, 3.7 in the caller's order.  Which rows share a warp decides which columns
+// below 2^-60 of a sum enter it in the compensated and mixed passes, so the order is
+// a function of the data: a stable counting sort, once per problem.  Chunks of
+// rows count their cells (k_cell_count), a cell's counts are summed over the chunks
+// (k_cell_chunks) and the cells (k_cell_scan), and one warp per chunk places its
+// rows in their order (k_cell_scatter).
+__global__ void __launch_bounds__(128)
+    k_cell_count(const double *__restrict__ pos, int64_t n, int64_t rows, int step, int d, double half,
+                 int *__restrict__ cell, int *__restrict__ hist) {
+    __shared__ int cnt[SORT_CELLS];
+    for (int i = threadIdx.x; i < SORT_CELLS; i += 128) cnt[i] = 0;
+    __syncthreads();
+    const int64_t j0 = (int64_t)blockIdx.x * rows, j1 = min(n, j0 + rows);
     const int bits = d == 3 ? 4 : 6;
-    int id = 0;
-    for (int t = 0; t < d; ++t) {
-        const double u = half > 0.0 ? (y64[j * step * d + t] / half + 1.0) * 0.5 : 0.0;
-        const int c = min(max((int)(u * (1 << bits)), 0), (1 << bits) - 1);
-        for (int b = 0; b < bits; ++b) id |= ((c >> b) & 1) << (d * b + t);
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += 128) {
+        int id = 0;
+        for (int t = 0; t < d; ++t) {
+            const double u = half > 0.0 ? (pos[j * step * d + t] / half + 1.0) * 0.5 : 0.0;
+            const int c = min(max((int)(u * (1 << bits)), 0), (1 << bits) - 1);
+            for (int b = 0; b < bits; ++b) id |= ((c >> b) & 1) << (d * b + t);
+        }
+        cell[j] = id;
+        atomicAdd(&cnt[id], 1);
     }
-    cell[j] = id;
-    atomicAdd(&count[id], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < SORT_CELLS; i += 128) hist[(int64_t)blockIdx.x * SORT_CELLS + i] = cnt[i];
+}
+
+// a cell's counts become its rows in the chunks before; total: all of its rows
+__global__ void k_cell_chunks(int *__restrict__ hist, int chunks, int *__restrict__ total) {
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    int sum = 0;
+    for (int b0 = 0; b0 < chunks; b0 += 16) {
+        int v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = b0 + i < chunks ? hist[(int64_t)(b0 + i) * SORT_CELLS + id] : 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if (b0 + i < chunks) hist[(int64_t)(b0 + i) * SORT_CELLS + id] = sum;
+            sum += v[i];
+        }
+    }
+    total[id] = sum;
 }
 
 // exclusive scan of the 4,096 counts (one block of 1,024 threads)
@@ -165,11 +192,25 @@ __global__ void k_cell_scan(int *__restrict__ count) {
     for (int k = 0; k < 4; ++k) count[threadIdx.x * 4 + k] = base + v[k];
 }
 
-__global__ void k_cell_scatter(const int *__restrict__ cell, int64_t n, int64_t n_pad,
-                               int *__restrict__ offset, int *__restrict__ perm) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) perm[atomicAdd(&offset[cell[j]], 1)] = (int)j;
-    else if (j < n_pad) perm[j] = (int)j;
+__global__ void __launch_bounds__(32)
+    k_cell_scatter(const int *__restrict__ cell, int64_t n, int64_t n_pad, int64_t rows,
+                   const int *__restrict__ hist, const int *__restrict__ base, int *__restrict__ perm) {
+    __shared__ int next[SORT_CELLS];
+    const int lane = threadIdx.x;
+    for (int i = lane; i < SORT_CELLS; i += 32) next[i] = base[i] + hist[(int64_t)blockIdx.x * SORT_CELLS + i];
+    __syncwarp();
+    const int64_t j0 = (int64_t)blockIdx.x * rows, j1 = min(n, j0 + rows);
+    for (int64_t g = j0; g < j1; g += 32) {
+        const int64_t j = g + lane;
+        const int id = j < j1 ? cell[j] : SORT_CELLS;
+        const unsigned same = __match_any_sync(0xffffffffu, id);
+        const int rank = __popc(same & ((1u << lane) - 1u));
+        if (j < j1) perm[next[id] + rank] = (int)j;
+        __syncwarp();
+        if (j < j1 && rank == 0) next[id] += __popc(same);
+        __syncwarp();
+    }
+    for (int64_t j = n + (int64_t)blockIdx.x * 32 + lane; j < n_pad; j += (int64_t)gridDim.x * 32) perm[j] = (int)j;
 }
 
 // The same maxima where the work is large: a warp holds 256 neighbouring points (by
@@ -277,15 +318,20 @@ void skip_free(rsot_problem *p) {
     p->sk_buf = nullptr;
 }
 
-cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_pad, int *perm, int *scratch,
+// chunks of at least 1,024 rows, at most 512 of them
+static int64_t sort_chunks(int64_t n) { return std::max<int64_t>(1, std::min<int64_t>(512, (n + 1023) / 1024)); }
+
+size_t cell_order_scratch(int64_t n) { return ((size_t)n + (size_t)(sort_chunks(n) + 1) * SORT_CELLS) * sizeof(int); }
+
+cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_pad, int *perm, void *scratch,
                        int step) {
-    int *cell = scratch, *count = cell + n_pad;
-    const unsigned nb = (unsigned)((n_pad + 255) / 256);
-    const cudaError_t e = cudaMemsetAsync(count, 0, SORT_CELLS * 4, p->stream);
-    if (e) return e;
-    k_cell_count<<<nb, 256, 0, p->stream>>>(pos, n, step, p->d, p->half_ext, cell, count);
-    k_cell_scan<<<1, 1024, 0, p->stream>>>(count);
-    k_cell_scatter<<<nb, 256, 0, p->stream>>>(cell, n, n_pad, count, perm);
+    const int64_t chunks = sort_chunks(n), rows = (n + chunks - 1) / chunks;
+    int *const total = static_cast<int *>(scratch), *const hist = total + SORT_CELLS,
+               *const cell = hist + chunks * SORT_CELLS;
+    k_cell_count<<<(unsigned)chunks, 128, 0, p->stream>>>(pos, n, rows, step, p->d, p->half_ext, cell, hist);
+    k_cell_chunks<<<SORT_CELLS / 64, 64, 0, p->stream>>>(hist, (int)chunks, total);
+    k_cell_scan<<<1, 1024, 0, p->stream>>>(total);
+    k_cell_scatter<<<(unsigned)chunks, 32, 0, p->stream>>>(cell, n, n_pad, rows, hist, total, perm);
     return cudaGetLastError();
 }
 
@@ -310,11 +356,12 @@ bool skip_ready(rsot_problem *p, double eps) {
         return o;
     };
     const size_t np = (size_t)p->nq_pad, nt = (size_t)p->n_pad;
-    const size_t o_part = take(np * 4 * p->sk_k), o_prow = take(np * 16), o_pcol = take(np * 16);
-    const size_t o_pA = take(np * 4), o_trow = take(nt * 16), o_tB = take(nt * 4), o_perm = take(nt * 4);
-    const size_t o_cell = take(std::max(nt, np / 2) * 4 + SORT_CELLS * 4);
     const bool skip_max = p->sk_pp == 4 && (double)p->nq * (double)p->n >= 1e9;   // k_row_max_skip
-    const size_t o_pq = take(skip_max ? np / 2 * 4 : 0);
+    const size_t o_perm = take(nt * 4), o_pq = take(skip_max ? np / 2 * 4 : 0);
+    const size_t o_part = take(np * 4 * p->sk_k), o_prow = take(np * 16), o_pcol = take(np * 16);
+    const size_t o_pA = take(np * 4), o_trow = take(nt * 16), o_tB = take(nt * 4);
+    // while the orders are made, all that follows them is scratch
+    at = std::max(at, o_part + std::max(cell_order_scratch(p->n), cell_order_scratch((p->nq + 1) / 2)));
     char *b = nullptr;
     if (cudaMalloc(&b, at) != cudaSuccess) {
         cudaGetLastError();
@@ -328,10 +375,9 @@ bool skip_ready(rsot_problem *p, double eps) {
     p->sk_tgrow = reinterpret_cast<float4 *>(b + o_trow);
     p->sk_tgB = reinterpret_cast<float *>(b + o_tB);
     p->sk_perm = reinterpret_cast<int *>(b + o_perm);
-    int *const tmp = reinterpret_cast<int *>(b + o_cell);
     p->sk_perm_q = skip_max ? reinterpret_cast<int *>(b + o_pq) : nullptr;
-    cudaError_t e = cell_order(p, p->y64, p->n, p->n_pad, p->sk_perm, tmp);
-    if (!e && skip_max) e = cell_order(p, p->x64, (p->nq + 1) / 2, p->nq_pad / 2, p->sk_perm_q, tmp, 2);
+    cudaError_t e = cell_order(p, p->y64, p->n, p->n_pad, p->sk_perm, b + o_part);
+    if (!e && skip_max) e = cell_order(p, p->x64, (p->nq + 1) / 2, p->nq_pad / 2, p->sk_perm_q, b + o_part, 2);
     // once per problem: a later evaluation may run on another stream
     if (e || cudaStreamSynchronize(p->stream) != cudaSuccess) {
         cudaGetLastError();
