@@ -187,6 +187,17 @@ void rsot_destroy(rsot_problem *p) {
 
 static constexpr int64_t kPsiDirect = 65536;   // largest host potential that a kernel reads in place
 
+// Ordinary host memory, which a copy on a stream reads at the call as well.  Pinned
+// memory is read when the stream gets there: earlier work on it may write it.
+static bool is_pageable(const void *ptr) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return a.type == cudaMemoryTypeUnregistered;
+}
+
 rsot_status rsot_create(int d, int64_t nq, const double *x, const double *mass, int64_t n,
                         const double *y, const double *nu, int device_ptrs, rsot_problem **out) {
     if (!out) return RSOT_ERR_ARG;
@@ -347,8 +358,9 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     // the handle's copy of psi: from host memory (through a pinned buffer), and
     // where the caller's gradient overlaps it (the final kernel reads psi[0])
     const bool gdev = wgrad == 1;
+    const bool staged = wpsi == 0 && p->n <= kPsiDirect && is_pageable(psi);
     if (wpsi == 0) {
-        if (p->n <= kPsiDirect) memcpy(p->psi_host, psi, nb);
+        if (staged) memcpy(p->psi_host, psi, nb);
         psid = p->psi_dev;
     } else if (gdev && psi < grad_out + p->n && grad_out < psi + p->n) {
         psid = p->psi_dev;
@@ -364,7 +376,7 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     const bool dense = mode == 0 || (mode == 1 && (!(arg > 0.0) || isinf(arg) ||
                                                     arg * arg > p->diam2 * (1.0 + 1e-12)));
     const auto upload = [&]() {
-        return cudaMemcpyAsync(p->psi_dev, p->n <= kPsiDirect ? p->psi_host : psi, nb, cudaMemcpyHostToDevice, st);
+        return cudaMemcpyAsync(p->psi_dev, staged ? p->psi_host : psi, nb, cudaMemcpyHostToDevice, st);
     };
     if (!e && !dense && wpsi == 0) e = upload();
     if (!e && !dense) e = mode == 1 ? cutoffs_uniform(p, 0.5 * arg * arg) : cutoffs_separable(p, psid, eps, arg);
@@ -378,7 +390,7 @@ static rsot_status eval_impl(rsot_problem *p, const double *psi, double eps, int
     // potential from the pinned buffer (a copy on the stream takes 5 us more)
     p->psi_src = nullptr;
     if (!e && dense && wpsi == 0) {
-        if (p->n <= kPsiDirect && (prec == RSOT_MIXED || alt)) p->psi_src = p->psi_host;
+        if (staged && (prec == RSOT_MIXED || alt)) p->psi_src = p->psi_host;
         else e = upload();
     }
     if (!e) {
