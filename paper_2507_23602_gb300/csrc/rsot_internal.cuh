@@ -313,6 +313,7 @@ cudaError_t launch_prep_mixed(rsot_problem *p, const double *psi_dev, double eps
 // its buffers exist and the sizes of the exponents allow it
 bool fx64_ready(rsot_problem *p, double eps);
 // pair skipping (rsot_skip.cu)
+bool skip_estimate_fits(const rsot_problem *p, double kappa);
 bool skip_ready(rsot_problem *p, double eps);
 double skip_t1(const rsot_problem *p);
 cudaError_t launch_skip(rsot_problem *p, const double *psi_dev, double eps);

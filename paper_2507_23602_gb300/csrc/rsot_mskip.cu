@@ -298,8 +298,8 @@ void mskip_free(rsot_problem *p) {
 //     192,000 x 10,000: kd 1082 373 -> 346;  60,000 x 20,000: kd 2885 188 -> 92
 //     61,206 x 5,003: kd 2885 51.1 -> 51.2 (not)
 static int mskip_passes(const rsot_problem *p, double eps) {
-    const double kd = kLog2e / (2.0 * eps) * p->diam2;
-    if (p->in_solve || p->pair_kernel != 2 || !(kd <= 0x1p20)) return 0;
+    const double kappa = kLog2e / (2.0 * eps), kd = kappa * p->diam2;
+    if (p->in_solve || p->pair_kernel != 2 || !(kd <= 0x1p20) || !skip_estimate_fits(p, kappa)) return 0;
     if ((double)p->nq * (double)p->n < 1e9) return 0;
     return (kd >= 700.0 && kd * (double)p->chunk1 >= 2e6 ? 1 : 0) | (kd >= 500.0 ? 2 : 0);
 }

@@ -335,12 +335,21 @@ cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_
     return cudaGetLastError();
 }
 
+// The estimates of the pair skipping work on squared distances, on k and on weights
+// in FP32, here and in rsot_mskip.cu: units of length in which these leave its range,
+// or so nearly that a squared length of 1e-6 of the data's does, take the passes
+// without them.
+bool skip_estimate_fits(const rsot_problem *p, double kappa) {
+    return (p->diam2 == 0.0 || (p->diam2 >= 0x1p-64 && p->diam2 <= 0x1p100)) && kappa >= 0x1p-90 && kappa <= 0x1p88 &&
+           p->nu_max <= 0x1p127;
+}
+
 // buffers and the target order, once per problem; false: not for these sizes,
 // or no memory (the callers have passes that need none of it)
 bool skip_ready(rsot_problem *p, double eps) {
     const double kappa = kLog2e / (2.0 * eps);
     // the estimate's error bound must allow a decision
-    if (!(kappa * p->diam2 <= 0x1p23) || !(p->msum > 0.0)) return false;
+    if (!(kappa * p->diam2 <= 0x1p23) || !skip_estimate_fits(p, kappa) || !(p->msum > 0.0)) return false;
     if (p->sk_buf) return true;
     const int64_t tiles = (p->n + RM_TS - 1) / RM_TS;
     p->sk_pp = p->nq_pad / 1024 * tiles >= 4 * p->num_sms ? 4 : 1;
