@@ -2254,11 +2254,8 @@ void mlp_forward_layers(rsot_mlp *m, int64_t rows, const float *x) {
 }
 
 // k_net's sums of stored dZ3 (m->dZ), dZ2 and dZ1 (m->Z3), after the per-layer kernels
-void launch_net_sums(rsot_mlp *m, int64_t rows, const float *y, float *loss_sum) {
-    const int64_t R = (rows + 127) / 128 * 128;
-    const NetSplit sp = net_split(m, R);
-    float *part[6];
-    if (!net_parts(m, sp.grid, part)) return;   // not reached: the buffer holds 2 CTAs per SM
+void launch_net_sums(rsot_mlp *m, int64_t rows, const float *y, const NetSplit &sp, float *const (&part)[6],
+                     float *loss_sum) {
     k_net_sums<<<sp.grid, 32 * NF_EPI, 0, m->stream>>>(m->dZ, m->H3, m->dZ2, m->Z3, m->out, y, rows,
                                                        1.0f / (float)rows, m->width, sp.tiles, sp.rt, part[0],
                                                        part[1], part[2], part[3], part[4], part[5]);
@@ -2273,8 +2270,11 @@ void mlp_backward(rsot_mlp *m, int64_t rows, const float *x, const float *y, flo
     float *G = m->G;
     const bf16 *dZ1 = m->dZ;
     const bool fused = net_fused(m) && launch_net<true>(m, rows, x, y, nullptr, loss_sum);
-    // the per-layer tcgen05 kernels on the same shapes: the fused kernel's sums
-    const bool net_sums = !fused && m->gemm_kind != 1 && net_shape(m);
+    // the per-layer tcgen05 kernels on the same shapes: the fused kernel's sums, where
+    // the buffer holds a partial per CTA (two CTAs per SM, up to 256 SMs)
+    const NetSplit sp = net_split(m, R);
+    float *part[6];
+    const bool net_sums = !fused && m->gemm_kind != 1 && net_shape(m) && net_parts(m, sp.grid, part);
     if (fused) {
         dZ1 = m->Z3;   // m->dZ holds dZ3
     } else {
@@ -2328,7 +2328,7 @@ void mlp_backward(rsot_mlp *m, int64_t rows, const float *x, const float *y, flo
     gemm<true, true, EPI_F32>(st, m->gemm_kind, m->flags, ws[2], m->sms, w, m->in_pad, R, dZ1, w, m->X0, m->in_pad, G + m->off[0], m->in_pad,
                               nullptr, nullptr, 0, nullptr, 0, &segs.s[2]);
     split_sum(st, segs, 3);
-    if (net_sums) launch_net_sums(m, rows, y, loss_sum);
+    if (net_sums) launch_net_sums(m, rows, y, sp, part, loss_sum);
     else if (!fused) colsum<bf16>(st, m->dZ, nullptr, R, w, m->red, G + m->off[1], m->sms);
 }
 
