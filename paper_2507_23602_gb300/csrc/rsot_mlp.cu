@@ -19,7 +19,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <atomic>
 #include <vector>
 
 #include "rsot_internal.cuh"
@@ -1991,12 +1990,6 @@ void gemm(cudaStream_t st, int kind, int *flags, float *ws, int sms, int M, int 
         if (t6 && EPI == EPI_F32)   // the FP32 results: S slices of M rows, boxes 32 x 32
             t6 = t6_tensor_map(&mh, Cw, S * M, N, ldc, 32, true);
         if (t6) {
-            static bool attr6 = false;   // 225 KB of dynamic shared memory, set once per instance
-            if (!attr6) {
-                cudaFuncSetAttribute((const void *)k_gemm_t6<AT, BT, EPI>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, T6_SMEM);
-                attr6 = true;
-            }
             const int mblocks = (M + 127) / 128, tiles6 = mblocks * S;
             k_gemm_t6<AT, BT, EPI><<<std::max(1, std::min(tiles6, sms)), T6_THREADS, T6_SMEM, st>>>(
                 M, N, K, kslice, mblocks, Cw, ldc, bias, flags, ma, mb, mh, mz);
@@ -2004,12 +1997,6 @@ void gemm(cudaStream_t st, int kind, int *flags, float *ws, int sms, int M, int 
         }
     }
     if (kind == 0 || kind == 2) {
-        static bool attr = false;   // 69 KB of dynamic shared memory, set once per instance
-        if (!attr) {
-            cudaFuncSetAttribute((const void *)k_gemm_t5<AT, BT, EPI>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, T5_SMEM);
-            attr = true;
-        }
         // TMA operand copies: a box (64 K) never crosses a K slice's end, since
         // slices start and end on multiples of 64 or at K, where zero fill begins
         CUtensorMap ma, mb, mh, mz;
@@ -2069,6 +2056,7 @@ struct rsot_mlp {
     float *ws = nullptr;     // split-K partials of the weight-gradient GEMMs
     float *red = nullptr;    // partials of the column sums (RED_CHUNKS x width)
     int sms = 1;
+    bool net_smem = false;   // the fused kernel may use its shared memory on this device
     struct Result {
         float loss;
         int flags;
@@ -2145,11 +2133,33 @@ rsot_status mlp_take_flags(rsot_mlp *m, int fl) {
     return RSOT_ERR_TIMEOUT;
 }
 
+// Dynamic shared memory beyond 48 KB is an attribute of a kernel on a device: set for
+// the handle's device when the handle is made.  The layers' GEMMs in their three forms
+// and, returned, whether every form of the fused kernel has it.
+template <bool AT, bool BT, int EPI>
+cudaError_t gemm_smem() {
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_gemm_t6<AT, BT, EPI>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, T6_SMEM);
+    if (!e)
+        e = cudaFuncSetAttribute((const void *)k_gemm_t5<AT, BT, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 T5_SMEM);
+    return e;
+}
+bool net_smem() {
+    for (auto g : {k_net<false, true, true>, k_net<false, true, false>, k_net<false, false, true>,
+                   k_net<false, false, false>, k_net<true, false, true>, k_net<true, false, false>})
+        if (cudaFuncSetAttribute((const void *)g, cudaFuncAttributeMaxDynamicSharedMemorySize, nf_smem(NF_MAXST))) {
+            cudaGetLastError();
+            return false;
+        }
+    return true;
+}
+
 // The fused kernel of the network: default GEMM kind, a width of whole 64-column
 // blocks that the accumulator holds.  false: a tensor map could not be made (the
 // per-layer kernels run).
 bool net_shape(const rsot_mlp *m) { return m->width % 64 == 0 && m->width <= 256; }
-bool net_fused(const rsot_mlp *m) { return m->gemm_kind == 0 && net_shape(m); }
+bool net_fused(const rsot_mlp *m) { return m->gemm_kind == 0 && net_shape(m) && m->net_smem; }
 
 // Tiles of 128 rows; fewer rows per CTA where those leave SMs idle (a tile's time
 // is its rows' epilogue plus the layers' latencies), one CTA per SM with every
@@ -2224,13 +2234,6 @@ bool launch_net(rsot_mlp *m, int64_t rows, const float *x, const float *y, float
     const bool alone = a.stages == NF_MAXST, pair = alone && w == 256, rep = !TRAIN && alone && a.rt == 32;
     auto f = rep ? (pair ? k_net<TRAIN, !TRAIN, true> : k_net<TRAIN, !TRAIN, false>)
                  : (pair ? k_net<TRAIN, false, true> : k_net<TRAIN, false, false>);
-    static std::atomic<bool> attr{false};
-    if (!attr.load()) {
-        for (auto g : {k_net<TRAIN, !TRAIN, true>, k_net<TRAIN, !TRAIN, false>, k_net<TRAIN, false, true>,
-                       k_net<TRAIN, false, false>})
-            cudaFuncSetAttribute((const void *)g, cudaFuncAttributeMaxDynamicSharedMemorySize, nf_smem(NF_MAXST));
-        attr.store(true);
-    }
     f<<<grid, NF_THREADS, nf_smem(a.stages), m->stream>>>(a, maps);
     if (TRAIN) net_fin(m, grid, a.part, loss_sum);
     return true;
@@ -2390,6 +2393,10 @@ rsot_status rsot_mlp_create(int in_dim, int width, uint64_t seed, rsot_mlp **out
     int dev = 0;
     if (!e) e = cudaGetDevice(&dev);
     if (!e) e = cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!e) e = gemm_smem<false, false, EPI_BIAS_SILU>();
+    if (!e) e = gemm_smem<false, false, EPI_DSILU>();
+    if (!e) e = gemm_smem<true, true, EPI_F32>();
+    if (!e) m->net_smem = net_smem();
     if (!e) {
         float *ws[3];
         e = cudaMalloc(&m->ws, mlp_ws(m, ws) * sizeof(float));
