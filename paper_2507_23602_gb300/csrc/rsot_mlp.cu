@@ -2062,7 +2062,8 @@ struct rsot_mlp {
         int flags;
     };
     Result *host = nullptr;  // pinned copy of (scal[0], *flags)
-    float *yhost = nullptr;  // pinned, cap rows: a forward call's results for host memory
+    float *yhost = nullptr;  // pinned, ycap rows: a forward call's results for host memory
+    int64_t ycap = 0;
     int *flags = nullptr;    // device error flags of the GEMM kernels (kErrTimeout): the word after scal[0]
 };
 
@@ -2093,13 +2094,12 @@ cudaError_t mlp_reserve(rsot_mlp *m, int64_t rows) {
     void *ptrs[] = {m->X0, m->H1, m->H2, m->H3, m->dZ, m->dZ2, m->Z1, m->Z2, m->Z3,
                     m->out, m->dout, m->lt, m->xin, m->yin};
     for (void *q : ptrs) cudaFree(q);
-    if (m->yhost) cudaFreeHost(m->yhost);
     // a failed allocation below leaves null pointers and no rows, not freed ones
     m->X0 = m->H1 = m->H2 = m->H3 = m->dZ = m->dZ2 = m->Z1 = m->Z2 = m->Z3 = nullptr;
-    m->out = m->dout = m->lt = m->xin = m->yin = m->yhost = nullptr;
+    m->out = m->dout = m->lt = m->xin = m->yin = nullptr;
     m->cap = 0;
     const int w = m->width;
-    cudaError_t e = cudaMallocHost(&m->yhost, (size_t)r * sizeof(float));
+    cudaError_t e = cudaSuccess;
 #define MA(ptr, cnt) \
     if (!e) e = cudaMalloc(&(ptr), (size_t)(cnt) * sizeof(*(ptr)))
     MA(m->X0, r * m->in_pad);
@@ -2124,6 +2124,22 @@ cudaError_t mlp_reserve(rsot_mlp *m, int64_t rows) {
         cudaMemset(m->yin, 0, r * sizeof(float));
     }
     return e;
+}
+
+// the pinned buffer of forward calls whose results go to host memory; false: none
+bool mlp_host_rows(rsot_mlp *m, int64_t rows) {
+    if (rows <= m->ycap) return true;
+    const int64_t r = (rows + 127) / 128 * 128;
+    if (m->yhost) cudaFreeHost(m->yhost);
+    m->yhost = nullptr;
+    m->ycap = 0;
+    if (cudaMallocHost(&m->yhost, (size_t)r * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        m->yhost = nullptr;
+        return false;
+    }
+    m->ycap = r;
+    return true;
 }
 
 // a GEMM wait that gave up (flag read with the call's results): cleared, reported
@@ -2465,11 +2481,12 @@ rsot_status rsot_mlp_forward(rsot_mlp *m, int64_t rows, const float *x, float *y
         e = cudaMemcpyAsync(m->xin, x, (size_t)rows * m->in_dim * 4, cudaMemcpyDefault, m->stream);
         xd = m->xin;
     }
-    // the fused kernel writes y_out itself where it can, else a pinned buffer
+    // the fused kernel writes y_out itself where it can, else a pinned buffer; without
+    // memory for that the per-layer kernels run
     float *yd = direct_ptr(y_out);
     if (yd && yd < xd + rows * m->in_dim && xd < yd + rows) yd = nullptr;   // overlaps x
     bool fused = false;
-    if (!e && net_fused(m)) {
+    if (!e && net_fused(m) && (yd || mlp_host_rows(m, rows))) {
         m->host->flags = 0;
         fused = launch_net<false>(m, rows, xd, nullptr, yd ? yd : m->yhost, nullptr, &m->host->flags);
     }
