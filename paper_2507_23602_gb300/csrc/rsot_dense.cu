@@ -1111,10 +1111,9 @@ static int pairs_per_thread(int most, int64_t items, int64_t slots) {
 
 // the targets' records and the partials of sum psi nu
 static void launch_prep(rsot_problem *p, const double *psi, double eps, Rec16 *trec, double inv_P, int *gate) {
-    const int t = p->per_prep == 1 ? CB_THREADS : kSmall;
     trace_begin(p, "prep_targets_mixed");
     const double *const src = p->psi_src ? p->psi_src : psi;
-    k_prep_mixed<<<(unsigned)(p->n_pad / t), t, 0, p->stream>>>(
+    k_prep_mixed<<<(unsigned)prep_blocks(p), prep_threads(p), 0, p->stream>>>(
         src, p->y64, p->lnu, p->nu, p->n, p->n_pad, p->d, eps, p->tquad, p->tpair, p->psinu, p->flags, trec, inv_P,
         gate, p->psi_src ? p->psi_dev : nullptr);
     p->psi_src = nullptr;
@@ -1122,9 +1121,8 @@ static void launch_prep(rsot_problem *p, const double *psi, double eps, Rec16 *t
 }
 
 static void launch_combine(rsot_problem *p, int k1, float *pu) {
-    const int t = p->per_comb == 1 ? CB_THREADS : kSmall;
     trace_begin(p, "combine_mixed");
-    launch_pdl(true, k_combine, (unsigned)(p->nq_pad / t), t, 0, p->stream, p->part1, k1, p->nq_pad, p->nq, p->xs,
+    launch_pdl(true, k_combine, (unsigned)combine_blocks(p), combine_threads(p), 0, p->stream, p->part1, k1, p->nq_pad, p->nq, p->xs,
                p->d, p->lmass2, p->mass, p->pquad, p->blockJ, p->lse_buf, pu);
     trace_end(p);
 }
@@ -1132,24 +1130,26 @@ static void launch_combine(rsot_problem *p, int k1, float *pu) {
 template <int D>
 static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tquad, int64_t n, int chunk,
                              int k1, float2 *part, int *flags, const int *gate, int num_sms,
-                             cudaStream_t st) {
+                             int64_t before, cudaStream_t st) {
     const int pp = pairs_per_thread(P1_PP, nq_pad / P1_TILE * k1, (int64_t)num_sms * P1_MINB);
     dim3 g((unsigned)(nq_pad / (2 * pp * P1_THREADS)), (unsigned)k1);
     auto f = pp == 4 ? k_lse_mixed<D, 4> : pp == 2 ? k_lse_mixed<D, 2> : k_lse_mixed<D, 1>;
     // the tensor-core passes' fallback mostly returns at once
-    launch_pdl(gate || overlap_pass(g, num_sms), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk, part, flags, gate, 1);
+    launch_pdl(gate || overlap_pass(g, before, num_sms, true), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk,
+               part, flags, gate, 1);
 }
 
 template <int D>
 static void launch_grad_mixed(const Rec8 *tpair, int64_t n, const float4 *pquad, int64_t nq,
                               int64_t chunk, int s2, double *part2, int64_t stride, int *flags,
-                              const int *gate, int num_sms, cudaStream_t st) {
+                              const int *gate, int num_sms, int64_t before, cudaStream_t st) {
     const int most = pick_tpp(n);
     const int64_t blk = (int64_t)P2_THREADS * 2 * most;
     const int tpp = pairs_per_thread(most, (n + blk - 1) / blk * s2, (int64_t)num_sms * 16 / most);
     dim3 g((unsigned)((n + 2 * P2_THREADS * tpp - 1) / (2 * P2_THREADS * tpp)), (unsigned)s2);
     auto f = tpp == 4 ? k_grad_mixed<D, 4> : tpp == 2 ? k_grad_mixed<D, 2> : k_grad_mixed<D, 1>;
-    launch_pdl(gate || overlap_pass(g, num_sms), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2, stride, flags, gate, 1);
+    launch_pdl(gate || overlap_pass(g, before, num_sms), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2,
+               stride, flags, gate, 1);
 }
 
 template <int D>
@@ -1158,8 +1158,8 @@ static void launch_grad_cent(rsot_problem *p) {
     dim3 g((unsigned)((p->n + 2 * P2_THREADS * p->cent_tpp - 1) / (2 * P2_THREADS * p->cent_tpp)),
            (unsigned)p->cent_s2);
     auto f = p->cent_tpp == 2 ? k_grad_mixed<D, 2, true> : k_grad_mixed<D, 1, true>;
-    launch_pdl(overlap_pass(g, p->num_sms), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad, p->nq,
-               p->cent_chunk, p->cent_part, stride, p->flags, (const int *)nullptr, 0);
+    launch_pdl(overlap_pass(g, combine_blocks(p), p->num_sms), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad,
+               p->nq, p->cent_chunk, p->cent_part, stride, p->flags, (const int *)nullptr, 0);
 }
 
 // buffers of the centroids' pass, once per problem: two target pairs per thread
@@ -1201,7 +1201,7 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
         mskip_lse(p, eps);
     else
         launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, chunk1, k1, p->part1, p->flags, gate, p->num_sms,
-                            st);
+                            prep_blocks(p), st);
     trace_end(p);
     launch_combine(p, k1, tc ? p->pu : nullptr);
     if (tc) {
@@ -1233,7 +1233,7 @@ static cudaError_t launch_mixed_d(rsot_problem *p, const double *psi, double eps
     }
     trace_begin(p, "grad_mixed");
     launch_grad_mixed<D>(p->tpair, p->n, p->pquad, p->nq, chunk2, s2, p->part2, p->n_pad, p->flags,
-                         gate, p->num_sms, st);
+                         gate, p->num_sms, combine_blocks(p), st);
     trace_end(p);
     return launch_finalize(
         p, psi, eps, {p->part2, s2, p->n_pad, nullptr, p->blockJ, p->nblk_comb, p->per_comb, 1, p->per_prep}, grad);
@@ -1288,7 +1288,7 @@ static cudaError_t softmax_refine_d(rsot_problem *p, const double *psi, double e
     const int64_t n_p1 = round_up(p->n, P1_TS);
     launch_prep(p, psi, eps, nullptr, 1.0, nullptr);
     launch_lse_mixed<D>(p->xs, p->nq_pad, p->tquad, p->n, p->chunk1, p->k1, p->part1, p->flags, nullptr,
-                        p->num_sms, st);
+                        p->num_sms, prep_blocks(p), st);
     launch_combine(p, p->k1, nullptr);
     const int64_t nf_alloc = round_up(nf, 1024);
     const int64_t blocks = nf_alloc / 1024;
@@ -1663,7 +1663,7 @@ cudaError_t na_launch(unsigned char *base, int64_t nq, const double *x, const do
     int k1 = pick_split(tiles1, std::min<int64_t>(n_p1 / P1_TS, NA_K1_ROWS / nq_pad), slots1);
     const int chunk1 = (int)round_up((n_p1 + k1 - 1) / k1, P1_TS);
     k1 = (int)((n_p1 + chunk1 - 1) / chunk1);
-    launch_lse_mixed<D>(xs, nq_pad, tquad, n, chunk1, k1, part1, &res->flags, nullptr, num_sms, st);
+    launch_lse_mixed<D>(xs, nq_pad, tquad, n, chunk1, k1, part1, &res->flags, nullptr, num_sms, nb_prep, st);
     k_combine<<<nb_pts, CB_THREADS, 0, st>>>(part1, k1, nq_pad, nq, xs, D, lm2, mass, pquad, blockJ,
                                              lse);
     const int tpp = pick_tpp(n);
@@ -1673,7 +1673,8 @@ cudaError_t na_launch(unsigned char *base, int64_t nq, const double *x, const do
                         (int64_t)num_sms * (D == 3 ? 4 : 5));
     const int64_t chunk2 = round_up((nq_pad + s2 - 1) / s2, P2_TS);
     s2 = (int)((nq_pad + chunk2 - 1) / chunk2);
-    launch_grad_mixed<D>(tpair, n, pquad, nq, chunk2, s2, part2, n_alloc, &res->flags, nullptr, num_sms, st);
+    launch_grad_mixed<D>(tpair, n, pquad, nq, chunk2, s2, part2, n_alloc, &res->flags, nullptr, num_sms,
+                         nb_pts, st);
     // the gradient goes to the scratch first; the caller's buffer receives it
     // only when the evaluation succeeded
     k_finalize_grad<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part2, s2, n_alloc, nu, n, gscr);

@@ -388,11 +388,11 @@ inline int fx_rows(const rsot_problem *p, int64_t rows, int64_t cols) {
 
 template <int D>
 void fx_launch(rsot_problem *p, int R, const FxRows &rows, const FxCols &cols, int64_t chunk, int splits,
-               double eps, double *out) {
+               double eps, double *out, int64_t before) {
     const float kappa = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
     // blocks of padding rows alone are not launched
     dim3 g((unsigned)((rows.count + FX_THREADS * R - 1) / (FX_THREADS * R)), (unsigned)splits);
-    launch_pdl(overlap_pass(g, p->num_sms), R == 2 ? k_fx_pass<D, 2> : k_fx_pass<D, 1>, g, FX_THREADS, 0, p->stream,
+    launch_pdl(overlap_pass(g, before, p->num_sms), R == 2 ? k_fx_pass<D, 2> : k_fx_pass<D, 1>, g, FX_THREADS, 0, p->stream,
                rows, cols, chunk, kappa, kd, p->fx_tab, out, p->res_dev);
 }
 
@@ -489,7 +489,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     const FxCols tgt = {p->fx_trec, p->tquad, p->sk_tgB, inv2k, p->n};
     trace_begin(p, "fx_lse");
     (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, fx_rows(p, p->nq, p->n), pts, tgt, p->fx_chunk1, p->fx_k1,
-                                              eps, p->fx_part1);
+                                              eps, p->fx_part1, 3 * (most / tr));
     trace_end(p);
     trace_begin(p, "fx_combine");
     const int nbq = (int)(p->nq_pad / 256);
@@ -503,7 +503,7 @@ cudaError_t launch_dense_fx64(rsot_problem *p, const double *psi, double eps, do
     const FxCols ptc = {p->fx_prec, p->sk_ptcol, p->sk_ptA, 1.f, p->nq};
     trace_begin(p, "fx_grad");
     (p->d == 3 ? fx_launch<3> : fx_launch<2>)(p, fx_rows(p, p->n, p->nq), tgr, ptc, p->fx_chunk2, p->fx_s2,
-                                              eps, p->fx_part2);
+                                              eps, p->fx_part2, p->nq_pad / tc);
     trace_end(p);
     return launch_finalize(p, psi, eps,
                            {p->fx_part2, p->fx_s2, p->n_pad, p->fx_tgscale, p->blockJ, nbq, p->per_comb, 0, p->per_prep},

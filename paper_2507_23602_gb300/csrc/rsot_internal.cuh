@@ -279,11 +279,19 @@ inline void launch_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t 
     (void)cudaLaunchKernelEx(&cfg, k, P(args)...);   // cudaGetLastError() reports a failure
 }
 
-// A pass overlaps its predecessor's end only where its CTAs are at most one per SM:
-// CTAs placed while the short kernel before still holds slots leave some SMs with
-// more of a single wave than others (mixed passes, 61,206 x 5,003: the call
-// 160 -> 225 us, 2,400 x 30,000: 88 -> 144; 1,536 x 128: 63 -> 60).
-inline bool overlap_pass(const dim3 &g, int num_sms) { return (int64_t)g.x * g.y <= num_sms; }
+// A pass overlaps the end of the short kernel before it only where its CTAs and that
+// kernel's blocks (`before`) together are at most one per SM: CTAs placed while those
+// still hold slots leave some SMs with more of a single wave than others.  Calls without
+// and with the overlap, in us: 1,536 x 128 43 -> 40, 1,000 x 8,000 (160 in all) 55 -> 55,
+// 1,536 x 8,000 (192) 53 -> 60, 16 x 16,000 (320) 52 -> 110, 61,206 x 5,003 160 -> 225;
+// FP64 1,536 x 128 (120) 76 -> 70, 6,000 x 128 (382) 79 -> 103.
+// Also where it has a CTA on every second SM at most, unless that kernel is the one of
+// the target records (after_prep), which lets it start at once: 60,000 x 16 (59 CTAs
+// after 944 blocks) 55 -> 51, FP64 3,000 x 128 (48 after 144) 74 -> 70.
+inline bool overlap_pass(const dim3 &g, int64_t before, int num_sms, bool after_prep = false) {
+    const int64_t own = (int64_t)g.x * g.y;
+    return own + before <= num_sms || (!after_prep && 2 * own <= num_sms);
+}
 
 // The last kernel of a dense evaluation: gradient and J from the partials, the
 // gradient to the caller's buffer on success, the result block to the host.
@@ -309,6 +317,11 @@ cudaError_t launch_dense_mixed(rsot_problem *p, const double *psi_dev, double ep
 cudaError_t launch_dense_fp64(rsot_problem *p, const double *psi_dev, double eps,
                               double *grad_dev);
 cudaError_t launch_prep_mixed(rsot_problem *p, const double *psi_dev, double eps);
+// threads and blocks of the target records' and of the combining kernels
+inline int prep_threads(const rsot_problem *p) { return p->per_prep == 1 ? 256 : 64; }
+inline int64_t prep_blocks(const rsot_problem *p) { return p->n_pad / prep_threads(p); }
+inline int combine_threads(const rsot_problem *p) { return p->per_comb == 1 ? 256 : 64; }
+inline int64_t combine_blocks(const rsot_problem *p) { return p->nq_pad / combine_threads(p); }
 // dense FP64 evaluation with fixed-point exponents (rsot_fx64.cu); fx64_ready:
 // its buffers exist and the sizes of the exponents allow it
 bool fx64_ready(rsot_problem *p, double eps);

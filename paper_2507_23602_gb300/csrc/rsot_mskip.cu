@@ -351,7 +351,7 @@ static void mskip_lse_d(rsot_problem *p, double eps) {
     const int pp = rows_per_thread(p->nq, p->k1, p->num_sms);
     dim3 g((unsigned)((p->nq + 64 * pp * MS_WARPS - 1) / (64 * pp * MS_WARPS)), (unsigned)p->k1);
     auto f = pp == 2 ? k_lse_skip<D, 2> : k_lse_skip<D, 1>;
-    launch_pdl(overlap_pass(g, p->num_sms), f, g, MS_THREADS, 0, p->stream, p->xs, p->ms_perm_q, p->nq, p->nq_pad,
+    launch_pdl(false, f, g, MS_THREADS, 0, p->stream, p->xs, p->ms_perm_q, p->nq, p->nq_pad,
                p->tquad, (int)p->n, p->chunk1, k, kd, (float)(61.0 + log2((double)p->n)), p->part1);
 }
 void mskip_lse(rsot_problem *p, double eps) { (p->d == 3 ? mskip_lse_d<3> : mskip_lse_d<2>)(p, eps); }
@@ -362,7 +362,7 @@ static void mskip_grad_d(rsot_problem *p, double eps) {
     const int pp = rows_per_thread(p->n, p->ms_s2, p->num_sms);
     dim3 g((unsigned)((p->n + 64 * pp * MS_WARPS - 1) / (64 * pp * MS_WARPS)), (unsigned)p->ms_s2);
     auto f = pp == 2 ? k_grad_skip<D, 2> : k_grad_skip<D, 1>;
-    launch_pdl(overlap_pass(g, p->num_sms), f, g, MS_THREADS, 0, p->stream, p->tquad, p->ms_perm_t, p->nu, p->n,
+    launch_pdl(false, f, g, MS_THREADS, 0, p->stream, p->tquad, p->ms_perm_t, p->nu, p->n,
                p->pquad, p->nq, p->ms_chunk2, k, kd, (float)(61.0 + log2((double)p->nq)), p->ms_part2, p->n_pad);
 }
 void mskip_grad(rsot_problem *p, double eps) { (p->d == 3 ? mskip_grad_d<3> : mskip_grad_d<2>)(p, eps); }

@@ -289,11 +289,12 @@ template <int D>
 void row_max(rsot_problem *p, double eps) {
     dim3 g((unsigned)(p->nq_pad / (2 * p->sk_pp * RM_THREADS)), (unsigned)p->sk_k);
     const float k = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
+    const bool over = overlap_pass(g, prep_blocks(p), p->num_sms, true);
     if (p->sk_perm_q)
-        launch_pdl(overlap_pass(g, p->num_sms), k_row_max_skip<D>, g, RM_THREADS, 0, p->stream, p->xs, p->sk_perm_q,
+        launch_pdl(over, k_row_max_skip<D>, g, RM_THREADS, 0, p->stream, p->xs, p->sk_perm_q,
                    p->nq, p->nq_pad, p->tquad, p->n, p->sk_chunk, k, kd, p->sk_part);
     else
-        launch_pdl(overlap_pass(g, p->num_sms), p->sk_pp == 4 ? k_row_max<D, 4> : k_row_max<D, 1>, g, RM_THREADS, 0,
+        launch_pdl(over, p->sk_pp == 4 ? k_row_max<D, 4> : k_row_max<D, 1>, g, RM_THREADS, 0,
                    p->stream, p->xs, p->nq_pad, p->tquad, p->n, p->sk_chunk, p->sk_part);
 }
 
