@@ -1135,7 +1135,7 @@ static void launch_lse_mixed(const float *xs, int64_t nq_pad, const float4 *tqua
     dim3 g((unsigned)(nq_pad / (2 * pp * P1_THREADS)), (unsigned)k1);
     auto f = pp == 4 ? k_lse_mixed<D, 4> : pp == 2 ? k_lse_mixed<D, 2> : k_lse_mixed<D, 1>;
     // the tensor-core passes' fallback mostly returns at once
-    launch_pdl(gate || overlap_pass(g, before, num_sms, true), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk,
+    launch_pdl(gate || overlap_pass(g, before, num_sms, 0), f, g, P1_THREADS, 0, st, xs, nq_pad, tquad, (int)n, chunk,
                part, flags, gate, 1);
 }
 
@@ -1148,7 +1148,7 @@ static void launch_grad_mixed(const Rec8 *tpair, int64_t n, const float4 *pquad,
     const int tpp = pairs_per_thread(most, (n + blk - 1) / blk * s2, (int64_t)num_sms * 16 / most);
     dim3 g((unsigned)((n + 2 * P2_THREADS * tpp - 1) / (2 * P2_THREADS * tpp)), (unsigned)s2);
     auto f = tpp == 4 ? k_grad_mixed<D, 4> : tpp == 2 ? k_grad_mixed<D, 2> : k_grad_mixed<D, 1>;
-    launch_pdl(gate || overlap_pass(g, before, num_sms), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2,
+    launch_pdl(gate || overlap_pass(g, before, num_sms, num_sms * 2 / 3), f, g, P2_THREADS, 0, st, tpair, pquad, nq, chunk, part2,
                stride, flags, gate, 1);
 }
 
@@ -1158,7 +1158,7 @@ static void launch_grad_cent(rsot_problem *p) {
     dim3 g((unsigned)((p->n + 2 * P2_THREADS * p->cent_tpp - 1) / (2 * P2_THREADS * p->cent_tpp)),
            (unsigned)p->cent_s2);
     auto f = p->cent_tpp == 2 ? k_grad_mixed<D, 2, true> : k_grad_mixed<D, 1, true>;
-    launch_pdl(overlap_pass(g, combine_blocks(p), p->num_sms), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad,
+    launch_pdl(overlap_pass(g, combine_blocks(p), p->num_sms, p->num_sms * 2 / 3), f, g, P2_THREADS, 0, p->stream, p->tpair, p->pquad,
                p->nq, p->cent_chunk, p->cent_part, stride, p->flags, (const int *)nullptr, 0);
 }
 

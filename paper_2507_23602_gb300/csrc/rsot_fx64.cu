@@ -392,7 +392,7 @@ void fx_launch(rsot_problem *p, int R, const FxRows &rows, const FxCols &cols, i
     const float kappa = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
     // blocks of padding rows alone are not launched
     dim3 g((unsigned)((rows.count + FX_THREADS * R - 1) / (FX_THREADS * R)), (unsigned)splits);
-    launch_pdl(overlap_pass(g, before, p->num_sms), R == 2 ? k_fx_pass<D, 2> : k_fx_pass<D, 1>, g, FX_THREADS, 0, p->stream,
+    launch_pdl(overlap_pass(g, before, p->num_sms, p->num_sms / 2), R == 2 ? k_fx_pass<D, 2> : k_fx_pass<D, 1>, g, FX_THREADS, 0, p->stream,
                rows, cols, chunk, kappa, kd, p->fx_tab, out, p->res_dev);
 }
 

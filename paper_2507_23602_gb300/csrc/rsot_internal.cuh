@@ -285,12 +285,14 @@ inline void launch_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t 
 // and with the overlap, in us: 1,536 x 128 43 -> 40, 1,000 x 8,000 (160 in all) 55 -> 55,
 // 1,536 x 8,000 (192) 53 -> 60, 16 x 16,000 (320) 52 -> 110, 61,206 x 5,003 160 -> 225;
 // FP64 1,536 x 128 (120) 76 -> 70, 6,000 x 128 (382) 79 -> 103.
-// Also where it has a CTA on every second SM at most, unless that kernel is the one of
-// the target records (after_prep), which lets it start at once: 60,000 x 16 (59 CTAs
-// after 944 blocks) 55 -> 51, FP64 3,000 x 128 (48 after 144) 74 -> 70.
-inline bool overlap_pass(const dim3 &g, int64_t before, int num_sms, bool after_prep = false) {
+// A kernel of few blocks leaves room for a pass of one CTA per SM (3,000 x 4,096: 96 CTAs
+// after 64 blocks 56 -> 54, 6,000 x 2,000: 53 -> 49), and a pass of few CTAs (`few`) may
+// follow any but the target records' kernel, which lets it start at once: 60,000 x 16 (59
+// after 944 blocks) 55 -> 51, 24,576 x 300 (96 after 384) 48 -> 45, centroids 60,000 x 300
+// (118 after 944) 73 -> 77, FP64 3,000 x 128 (48 after 144) 74 -> 70.
+inline bool overlap_pass(const dim3 &g, int64_t before, int num_sms, int few) {
     const int64_t own = (int64_t)g.x * g.y;
-    return own + before <= num_sms || (!after_prep && 2 * own <= num_sms);
+    return own + before <= num_sms || (2 * before <= num_sms && own <= num_sms) || own <= few;
 }
 
 // The last kernel of a dense evaluation: gradient and J from the partials, the

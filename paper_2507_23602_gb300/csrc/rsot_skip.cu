@@ -289,7 +289,7 @@ template <int D>
 void row_max(rsot_problem *p, double eps) {
     dim3 g((unsigned)(p->nq_pad / (2 * p->sk_pp * RM_THREADS)), (unsigned)p->sk_k);
     const float k = (float)(kLog2e / (2.0 * eps)), kd = (float)(kLog2e / (2.0 * eps) * p->diam2);
-    const bool over = overlap_pass(g, prep_blocks(p), p->num_sms, true);
+    const bool over = overlap_pass(g, prep_blocks(p), p->num_sms, 0);
     if (p->sk_perm_q)
         launch_pdl(over, k_row_max_skip<D>, g, RM_THREADS, 0, p->stream, p->xs, p->sk_perm_q,
                    p->nq, p->nq_pad, p->tquad, p->n, p->sk_chunk, k, kd, p->sk_part);
