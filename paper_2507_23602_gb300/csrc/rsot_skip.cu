@@ -301,11 +301,15 @@ void row_max(rsot_problem *p, double eps) {
 }  // namespace
 
 // the smallest column split whose CTAs fill the resident slots (at most 5 % idle
-// in the last wave)
+// in the last wave); where a CTA per tile does not fill them, that, up to 64 splits (of
+// few row blocks one more split fills hardly more slots, and there was none: compensated
+// 1,000 x 1,000 173 -> 94 us, 64 x 2,000 266 -> 100; more partials than 64 cost what the
+// shorter passes save, 1,000 x 65,536 with 256: 291 -> 331)
 int split_for_slots(int64_t units, int64_t tiles, int64_t slots) {
-    int best = 1;
-    double best_eff = 0.0;
-    for (int64_t s = 1; s <= std::min<int64_t>(tiles, 256); ++s) {
+    const int64_t least = units * tiles <= slots ? std::min<int64_t>(tiles, 64) : 1;
+    int best = (int)least;
+    double best_eff = least > 1 ? (double)(units * least) / (double)slots : 0.0;
+    for (int64_t s = least; s <= std::min<int64_t>(tiles, 256); ++s) {
         const int64_t items = units * s, waves = (items + slots - 1) / slots;
         const double eff = (double)items / (double)(waves * slots);
         if (eff > best_eff + 0.01) best_eff = eff, best = (int)s;
