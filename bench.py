@@ -42,9 +42,6 @@ FP32_LANE_OPS_PER_CLK_PER_SM = 128
 # FP32 lane-operations per pair of the compensated passes, counted from their
 # source: double-float exponent 3 x 12 + 3, shift TwoSum 6, Kahan 4, tail 2-3
 COMP_FP32_OPS_PER_PAIR = {"lse_df": 51, "grad_df": 52}
-# FP64-pipe operations per pair of the two dense FP64 passes: one fused multiply-add
-# each (exponents and exponentials are 64-bit integers)
-FP64_OPS_PER_PAIR = {2: 2, 3: 2}
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -539,20 +536,18 @@ def run_solve_workloads(args):
         return
 
 
-def eval_roofline_seconds(pairs_prec, sms, sm_mhz, dfma_per_s=None, d=3):
+def eval_roofline_seconds(pairs_prec, sms, sm_mhz):
     """Roofline time of a solve's evaluations: per precision, the algorithmic
     work of its pairs over its binding unit's peak -- mixed: 2 ex2 per pair on
-    the SFU; compensated: the FP32 lane-ops per pair of both passes; FP64: the
-    FP64 operations per pair of both passes at the measured DFMA rate (None when
-    the FP64 rate is not known).  Index = rsot_precision (FP64, MIXED,
-    COMPENSATED)."""
+    the SFU; compensated: the FP32 lane-ops per pair of both passes.  None with
+    FP64 evaluations among them: their passes are bound by integer work on the
+    pairs that can matter (the others are left out), which the count of pairs
+    does not give.  Index = rsot_precision (FP64, MIXED, COMPENSATED)."""
+    if pairs_prec[0]:
+        return None
     clk = sm_mhz * 1e6
     t = 2.0 * pairs_prec[1] / (SFU_EX2_PER_CLK_PER_SM * sms * clk)
     t += pairs_prec[2] * sum(COMP_FP32_OPS_PER_PAIR.values()) / (FP32_LANE_OPS_PER_CLK_PER_SM * sms * clk)
-    if pairs_prec[0]:
-        if not dfma_per_s:
-            return None
-        t += pairs_prec[0] * FP64_OPS_PER_PAIR[d] / dfma_per_s
     return t
 
 
@@ -590,7 +585,7 @@ def warmstart_network(args, log):
                  "cached": False, "loss_history": hist}
 
 
-def solve_metrics(args, P, p, dev, dfma_per_s):
+def solve_metrics(args, P, p, dev):
     """The metric's solve-time half: (a) the cube solve eps 0.1 -> 1e-3 to
     ||grad J||_1 <= 1e-6 (mixed evaluations, refinement on compensated
     evaluations with the certified stop); (b) on the same held-out warm-start
@@ -614,16 +609,15 @@ def solve_metrics(args, P, p, dev, dfma_per_s):
            "roofline_basis": f"evaluations' roofline time / wall: mixed 2 ex2 per pair at "
                              f"{SFU_EX2_PER_CLK_PER_SM} ex2/clk/SM, compensated "
                              f"{sum(COMP_FP32_OPS_PER_PAIR.values())} FP32 lane-ops per pair at "
-                             f"{FP32_LANE_OPS_PER_CLK_PER_SM}/clk/SM, FP64 {FP64_OPS_PER_PAIR} (by d) "
-                             f"FP64-pipe ops per pair at the measured DFMA rate "
-                             f"({dfma_per_s:.4g}/s); {sms} SMs x {sm_max:.0f} MHz"}
+                             f"{FP32_LANE_OPS_PER_CLK_PER_SM}/clk/SM, none with FP64 evaluations "
+                             f"(integer work on the pairs that can matter); {sms} SMs x {sm_max:.0f} MHz"}
     # (a) cube solve
     torch.cuda.synchronize()
     t = time.perf_counter()
     psi_c, st = P.solve(eps=p.eps, eps_start=0.1, eps_factor=0.5, tol_l1=1e-6, precision=rs.MIXED,
                         raise_on_error=False, max_iter=20000)
     wall = time.perf_counter() - t
-    rt = eval_roofline_seconds(st.pairs_prec, sms, sm_max, dfma_per_s)
+    rt = eval_roofline_seconds(st.pairs_prec, sms, sm_max)
     out["cube"] = {"workload": f"cube-{p.nq}x{p.n}, eps 0.1 -> {p.eps:g} (x0.5), tol 1e-6",
                    "seconds": wall, "iters": st.iters, "evals": st.evals, "stages": st.stages,
                    "status": st.status, "converged": int(st.status == 0),
@@ -659,7 +653,7 @@ def solve_metrics(args, P, p, dev, dfma_per_s):
         net.close()
 
     def arm(st_, wall_):
-        rt_ = eval_roofline_seconds(st_["pairs_prec"], sms, sm_max, dfma_per_s, d=2)
+        rt_ = eval_roofline_seconds(st_["pairs_prec"], sms, sm_max)
         return {"seconds": wall_, "rounds": st_["rounds"], "evals": st_["evals"],
                 "converged": st_["converged"], "max_grad_l1_reported": st_["max_grad_l1"],
                 "evals_by_precision": dict(zip(("fp64", "mixed", "compensated"), st_["evals_prec"])),
@@ -971,9 +965,8 @@ def main():
 
     # the metric's solve-time half (after every timed evaluation above)
     solve = None
-    dfma = rs.probe_dfma_rate()
     if not args.no_solve and world == 1:
-        solve = solve_metrics(args, P, p, dev, dfma)
+        solve = solve_metrics(args, P, p, dev)
 
     out = {
         "metric": "dual+grad G pairs/s (dense)", "value": value, "unit": "G pairs/s",
