@@ -14,7 +14,7 @@ namespace {
 
 constexpr int RM_THREADS = 128;
 constexpr int RM_TS = 256;   // targets per shared-memory tile
-constexpr int SORT_CELLS = 4096;
+constexpr int SORT_CELLS = 4096, SORT_THREADS = 256;
 
 // max_j r_qj over a chunk of targets, two points per lane pair and PP pairs a
 // thread (4 share a target's load; 1 where that leaves SMs idle)
@@ -131,17 +131,17 @@ __global__ void k_skip_operands(const float *__restrict__ part, int k1, int64_t 
 // below 2^-60 of a sum enter it in the compensated and mixed passes, so the order is
 // a function of the data: a stable counting sort, once per problem.  Chunks of
 // rows count their cells (k_cell_count), a cell's counts are summed over the chunks
-// (k_cell_chunks) and the cells (k_cell_scan), and one warp per chunk places its
-// rows in their order (k_cell_scatter).
-__global__ void __launch_bounds__(128)
+// (k_cell_chunks) and the cells (k_cell_scan), and one warp of each chunk's block places
+// its rows in their order (k_cell_scatter).
+__global__ void __launch_bounds__(SORT_THREADS)
     k_cell_count(const double *__restrict__ pos, int64_t n, int64_t rows, int step, int d, double half,
                  int *__restrict__ cell, int *__restrict__ hist) {
     __shared__ int cnt[SORT_CELLS];
-    for (int i = threadIdx.x; i < SORT_CELLS; i += 128) cnt[i] = 0;
+    for (int i = threadIdx.x; i < SORT_CELLS; i += SORT_THREADS) cnt[i] = 0;
     __syncthreads();
     const int64_t j0 = (int64_t)blockIdx.x * rows, j1 = min(n, j0 + rows);
     const int bits = d == 3 ? 4 : 6;
-    for (int64_t j = j0 + threadIdx.x; j < j1; j += 128) {
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += SORT_THREADS) {
         int id = 0;
         for (int t = 0; t < d; ++t) {
             const double u = half > 0.0 ? (pos[j * step * d + t] / half + 1.0) * 0.5 : 0.0;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(128)
         atomicAdd(&cnt[id], 1);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < SORT_CELLS; i += 128) hist[(int64_t)blockIdx.x * SORT_CELLS + i] = cnt[i];
+    for (int i = threadIdx.x; i < SORT_CELLS; i += SORT_THREADS) hist[(int64_t)blockIdx.x * SORT_CELLS + i] = cnt[i];
 }
 
 // a cell's counts become its rows in the chunks before; total: all of its rows
@@ -192,25 +192,33 @@ __global__ void k_cell_scan(int *__restrict__ count) {
     for (int k = 0; k < 4; ++k) count[threadIdx.x * 4 + k] = base + v[k];
 }
 
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(SORT_THREADS)
     k_cell_scatter(const int *__restrict__ cell, int64_t n, int64_t n_pad, int64_t rows,
                    const int *__restrict__ hist, const int *__restrict__ base, int *__restrict__ perm) {
-    __shared__ int next[SORT_CELLS];
-    const int lane = threadIdx.x;
-    for (int i = lane; i < SORT_CELLS; i += 32) next[i] = base[i] + hist[(int64_t)blockIdx.x * SORT_CELLS + i];
-    __syncwarp();
+    __shared__ int next[SORT_CELLS], ids[1024];
+    const int tid = threadIdx.x, lane = tid & 31;
+#pragma unroll 4
+    for (int i = tid; i < SORT_CELLS; i += SORT_THREADS) next[i] = base[i] + hist[(int64_t)blockIdx.x * SORT_CELLS + i];
     const int64_t j0 = (int64_t)blockIdx.x * rows, j1 = min(n, j0 + rows);
-    for (int64_t g = j0; g < j1; g += 32) {
-        const int64_t j = g + lane;
-        const int id = j < j1 ? cell[j] : SORT_CELLS;
-        const unsigned same = __match_any_sync(0xffffffffu, id);
-        const int rank = __popc(same & ((1u << lane) - 1u));
-        if (j < j1) perm[next[id] + rank] = (int)j;
-        __syncwarp();
-        if (j < j1 && rank == 0) next[id] += __popc(same);
-        __syncwarp();
+    for (int64_t t0 = j0; t0 < j1; t0 += 1024) {
+        const int cnt = (int)min((int64_t)1024, j1 - t0);
+        __syncthreads();
+        for (int i = tid; i < cnt; i += SORT_THREADS) ids[i] = cell[t0 + i];
+        __syncthreads();
+        if (tid < 32)
+            for (int g = 0; g < cnt; g += 32) {
+                const bool in = g + lane < cnt;
+                const int id = in ? ids[g + lane] : SORT_CELLS;
+                const unsigned same = __match_any_sync(0xffffffffu, id);
+                const int rank = __popc(same & ((1u << lane) - 1u));
+                if (in) perm[next[id] + rank] = (int)(t0 + g + lane);
+                __syncwarp();
+                if (in && rank == 0) next[id] += __popc(same);
+                __syncwarp();
+            }
     }
-    for (int64_t j = n + (int64_t)blockIdx.x * 32 + lane; j < n_pad; j += (int64_t)gridDim.x * 32) perm[j] = (int)j;
+    for (int64_t j = n + (int64_t)blockIdx.x * SORT_THREADS + tid; j < n_pad; j += (int64_t)gridDim.x * SORT_THREADS)
+        perm[j] = (int)j;
 }
 
 // The same maxima where the work is large: a warp holds 256 neighbouring points (by
@@ -323,8 +331,11 @@ void skip_free(rsot_problem *p) {
     p->sk_buf = nullptr;
 }
 
-// chunks of at least 1,024 rows, at most 512 of them
-static int64_t sort_chunks(int64_t n) { return std::max<int64_t>(1, std::min<int64_t>(512, (n + 1023) / 1024)); }
+// Chunks of rows: counting and placing 1,024 rows take 10 us each, a chunk's counts 0.1 us
+// of k_cell_chunks (sorting 16,384 rows 35 us with 16 chunks, 13 without the stable order).
+static int64_t sort_chunks(int64_t n) {
+    return std::max<int64_t>(1, std::min<int64_t>(512, (int64_t)sqrt((double)n / 5.0)));
+}
 
 size_t cell_order_scratch(int64_t n) { return ((size_t)n + (size_t)(sort_chunks(n) + 1) * SORT_CELLS) * sizeof(int); }
 
@@ -333,10 +344,10 @@ cudaError_t cell_order(rsot_problem *p, const double *pos, int64_t n, int64_t n_
     const int64_t chunks = sort_chunks(n), rows = (n + chunks - 1) / chunks;
     int *const total = static_cast<int *>(scratch), *const hist = total + SORT_CELLS,
                *const cell = hist + chunks * SORT_CELLS;
-    k_cell_count<<<(unsigned)chunks, 128, 0, p->stream>>>(pos, n, rows, step, p->d, p->half_ext, cell, hist);
+    k_cell_count<<<(unsigned)chunks, SORT_THREADS, 0, p->stream>>>(pos, n, rows, step, p->d, p->half_ext, cell, hist);
     k_cell_chunks<<<SORT_CELLS / 64, 64, 0, p->stream>>>(hist, (int)chunks, total);
     k_cell_scan<<<1, 1024, 0, p->stream>>>(total);
-    k_cell_scatter<<<(unsigned)chunks, 32, 0, p->stream>>>(cell, n, n_pad, rows, hist, total, perm);
+    k_cell_scatter<<<(unsigned)chunks, SORT_THREADS, 0, p->stream>>>(cell, n, n_pad, rows, hist, total, perm);
     return cudaGetLastError();
 }
 
@@ -376,6 +387,9 @@ bool skip_ready(rsot_problem *p, double eps) {
     const size_t o_pA = take(np * 4), o_trow = take(nt * 16), o_tB = take(nt * 4);
     // while the orders are made, all that follows them is scratch
     at = std::max(at, o_part + std::max(cell_order_scratch(p->n), cell_order_scratch((p->nq + 1) / 2)));
+    // in steps of 256 KiB, of which the allocator more often has a block left from a handle
+    // before (24,576 x 512 in a loop of new handles: cudaMalloc 77 -> 5 us)
+    at = (at + 262143) / 262144 * 262144;
     char *b = nullptr;
     if (cudaMalloc(&b, at) != cudaSuccess) {
         cudaGetLastError();
