@@ -383,8 +383,11 @@ static double pow2_above(double v) {   // the power of two in (v, 2 v]
 
 bool cx_ready(rsot_problem *p, double eps) {
     if (p->in_solve || !(p->half_ext > 0.0)) return false;
-    // smaller problems are bound by the launches, three more than rsot_df.cu's
-    // (3,456 x 181: 121 us against 87; 8,232 x 2,337: 179 against 293)
+    // smaller problems are bound by the launches, three more than rsot_df.cu's, against
+    // its chains over the targets (us there and here: 16 x 500 71 and 78, 1,000 x 500 76 and
+    // 90, 12,000 x 300 84 and 94; 16 x 1,000 97 and 79, 1,000 x 1,000 104 and 93, 12,000 x
+    // 1,000 121 and 111, 3,000 x 1,500 164 and 104, 16 x 65,536 3,713 and 169; from 2.5e7
+    // pairs 200,000 x 128 487 and 231)
     if (p->n < 1000 && (double)p->nq * (double)p->n < 2.5e7) return false;
     const double P = pow2_above(p->half_ext), Q = pow2_above(kLog2e / eps * p->half_ext);
     // all grids and sums inside FP32's range; the estimate's error bound below 16

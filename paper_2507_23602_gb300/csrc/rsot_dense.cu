@@ -622,7 +622,7 @@ __global__ void k_finalize_grad(const double *__restrict__ part2, int s2, int64_
 // the next evaluation.  Bound by latency (a launch, the loads of the partials, a
 // write to the host): one launch instead of gradient, J, conditional copy, result
 // copy and clearing.  With the overlapped launches, the small blocks and the
-// finer pass-2 split a call on 1,536 x 128 took 76 us before and 48 now.
+// finer pass-2 split a call on 1,536 x 128 took 76 us before and 39 now.
 __global__ void __launch_bounds__(256)
     k_finalize(FinalArgs a, const double *__restrict__ nu, int64_t n, double *__restrict__ grad,
                const double *__restrict__ psinu, int npn, const double *__restrict__ psi,

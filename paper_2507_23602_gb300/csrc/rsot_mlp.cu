@@ -41,8 +41,9 @@ enum { EPI_F32 = 0, EPI_BIAS_SILU = 1, EPI_DSILU = 2 };
 // quotient, exact in a fused multiply-add, corrects it (Markstein, IBM J. Res.
 // Dev. 34, 1990).  Where d or z is infinite the residual is not a number, the
 // minimum replaces it, and r = 0 or q infinite makes it nothing.  Of 6.7e8 values
-// of |z| in [1e-6, 1e6] two differ from z / (1 + __expf(-z)) as compiled, in the
-// last bit, and none after rounding to BF16.
+// of |z| in [1e-6, 1e6] two differ from z / (1 + __expf(-z)) as compiled by more than
+// 1e-30, in the last bit, and none of those after rounding to BF16; from z = -87.3
+// down, where 1 / d is subnormal and flushed, the result is 0 (1e-36 at most there).
 __device__ __forceinline__ float one_plus_exp_neg(float z) {
     float e;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
@@ -925,7 +926,8 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
 // every layer (33 MB each at 65,536 x 256) and ran 32 of 152 SMs at 4,096 rows.
 //   forward, 4,096 rows: GPU time 50 -> 12 us (the call 84 -> 40);
 //   forward + back-propagation, 65,536 rows: 240 -> 119 us (the gradients' call
-//   384 -> 236).
+//   384 -> 236).  TRAIN needs more than its 56 registers (two CTAs of 576 threads per
+//   SM) and spills 28 bytes.
 // TRAIN also stores X0, H1, H2 and the three dZ (the weight gradients' operands;
 // TMA, 32 x 64 boxes from the swizzled operand), keeps Z1 and Z2 in global memory
 // between a tile's two passes (each thread reads back what it wrote), and sums
