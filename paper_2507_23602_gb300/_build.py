@@ -31,7 +31,8 @@ def nvcc_path() -> str:
 
 
 def _headers():
-    return glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    return [h for d, p in ((CSRC, "*.cuh"), (CSRC, "*.h"), (os.path.join(ROOT, "include"), "*.h"))
+            for h in glob.glob(os.path.join(d, p))]
 
 
 def _compile(src: str, verbose_ptxas: bool) -> str:
